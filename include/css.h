@@ -293,10 +293,10 @@ int css_batch_free(css_batch* batch);
  * face outside [0, nf) or a barycentric triple that is not finite, has an entry below
  * -1e-12 or does not sum to 1 within 1e-9 gives CSS_ERR_INVALID_ARG, as does a stream of
  * another device.
- * Limits: n <= 262144 particles, at most 1048576 faces, 2048 windows per source and
- * warp; beyond them it returns CSS_ERR_CAPACITY (sizes) or CSS_ERR_QUEUE_OVERFLOW (a
- * source needing more windows), and css_compute_forces should be used instead; a device
- * loop cap gives CSS_ERR_ITER_LIMIT.
+ * Limits: n <= 262144 particles, at most 1048576 faces; beyond them it returns
+ * CSS_ERR_CAPACITY.  A source whose patch overflows the array's tables (4096 windows waiting
+ * at a time, 14336 vertices) gives CSS_ERR_QUEUE_OVERFLOW, and css_compute_forces should be
+ * used instead; a device loop cap gives CSS_ERR_ITER_LIMIT.
  * The first call on a device looks up the array's device address (set-up): make it
  * before any stream capture.  Every call shares the array, which keeps the previous
  * call's contents, so calls that overlap on the GPU (other streams, other host threads)
@@ -319,31 +319,28 @@ int css_fma_peak(css_ctx* ctx, int precision, double* flops_per_s);
 /* ---------------------------------------------------------------- tuning
  * Launch shape of the neighbour/force evaluation (no counterpart in the paper, whose
  * method runs one source per CPU process).  Every source runs in a first pass: one
- * warp per source, per-warp hash tables (edges, pseudo-source vertices, faces) in
- * shared memory and a window pool in global memory.  A source whose patch overflows
- * them is deferred, and a second pass re-runs the deferred sources with global-memory
- * tables and a larger pool on fewer warps.  Results do not depend on the shape.
+ * warp per source, with its working memory -- a ring of windows waiting to be unfolded, a
+ * table of vertices, a table of targets -- in shared memory.  A source that overflows it is
+ * deferred, and a second pass re-runs the deferred sources with larger working memory in
+ * global memory on fewer warps.  Results do not depend on the shape.
  *   warps_per_cta      first pass, 1..8
  *   ctas_per_sm        first pass resident CTAs per SM, 0 = as many as fit, else a cap
- *                      (fewer resident warps keep more of each warp's pool in L2)
  *   tile               work items (sources) a warp claims per atomic, 1..64
- *   shared_scale       first-pass table size, 0 (global tables), 1, 2, 4 or 8 times
- *                      512 edges / 256 vertices / 512 faces per warp
- *   window_capacity    first-pass windows per warp, 64..2^20 (rounded up to 2^k)
- *   window_capacity2   second-pass windows per warp (grown on overflow)
+ *   shared_scale       first-pass working memory in shared memory: 1, 2, 4 or 8 times 256
+ *                      vertices, 64 targets and a ring of at most 128 windows (1024 in the team
+ *                      form; halved until the shape fits an SM); 0 = in global memory
+ *   window_capacity    first-pass windows, 64..2^20 (rounded up to 2^k): the ring holds a sixteenth
+ *                      of them (a quarter in the team form), at least 32
+ *   window_capacity2   the same for the second pass (grown on overflow)
  *   warps2_per_sm      second-pass warps per SM, 1..8
- *   occupancy          first-pass register budget: 1 = up to 255 registers a thread (at
- *                      most 8 resident warps per SM, no spills), 2 = at most 128 (twice
- *                      the resident warps, some spills to local memory)
- *   table_capacity     first pass with global tables (shared_scale 0): edge and face table
- *                      slots per warp, vertex slots half of it (rounded up to 2^k, 64..2^20);
- *                      0 = tied to window_capacity.  Tables sized for the patches of the
- *                      workload keep each source's entries on few cache lines; a source
- *                      that overflows them is deferred to the second pass
+ *   occupancy          1 or 2: accepted and kept; the kernel's register budget (at most 128 a
+ *                      thread) suits both
+ *   table_capacity     working memory in global memory (shared_scale 0): half as many vertices, a
+ *                      quarter as many targets and at most a quarter as many waiting windows
+ *                      (rounded up to 2^k, 64..2^20); 0 = tied to window_capacity
  *   team               0: one warp per source; 1: all warps of a CTA (warps_per_cta >= 2) work
  *                      on one source together -- each wave unfolds up to 32 x warps_per_cta
- *                      windows and the insertions are spread over the warps by edge and vertex
- *                      id -- for sets with fewer sources than resident warps
+ *                      windows -- for sets with fewer sources than resident warps
  * css_set_launch fails with CSS_ERR_INVALID_ARG when a value is out of range or the
  * shape's shared memory does not fit an SM.  Until a shape is set or tuned, a context
  * starts from {4, 0, 1, 1, 2048, 16384, 2, 1, 0, 0} and adapts by itself: after an evaluation

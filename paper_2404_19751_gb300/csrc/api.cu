@@ -19,7 +19,7 @@
 #include "css_internal.h"
 
 using cssi::GeoJob;
-using cssi::GeoWs;
+using cssi::WaveWs;
 
 namespace {
 
@@ -69,47 +69,44 @@ int next_pow2(int x) {
     return p;
 }
 
-// ---- workspaces of the two passes of the persistent neighbour/force kernel
+// ---- the two passes of the persistent neighbour/force kernel
 struct GeoPlan {
-    GeoWs g1, g2;
+    WaveWs g1, g2;
     int wpc1 = 0, nctas1 = 0, wpc2 = 0, nctas2 = 0;
-    int team = 0;   // first pass in the team form (one source per CTA)
 };
 
-// size (and zero on a layout change, so old bytes never look like valid hash tags) one
-// pass's workspace
-int ensure_buf(css_ctx* c, cssi::WsBuf& b, int precision, int win_cap, int tab_cap, int shared, int nwarps,
-               GeoWs* out) {
-    GeoWs g{};
-    g.shared = shared;
-    g.stride = cssi::geo_ws_bytes_per_warp(precision, win_cap, shared ? 0 : tab_cap, &g.log_eh, &g.log_vh, &g.log_fh,
-                                           &g.fcap, &g.emcap);
-    g.wcap = win_cap;
-    g.nwarps = nwarps;
-    const size_t need = g.stride * (size_t)nwarps;
-    const int64_t key = (((int64_t)precision * 1000003 + (int64_t)win_cap * 31 + nwarps) * 16 + shared) * 2097152 +
-                        (shared ? 0 : tab_cap);
-    const bool relayout = (need > b.bytes) || (b.warps < nwarps) || (b.key != key);
-    if (need > b.bytes) {
-        cudaFree(b.ws);
-        b.ws = nullptr;
-        b.bytes = 0;
-        TRY(c, "workspace", cudaMalloc(&b.ws, need));
-        b.bytes = need;
+// one pass: layout, grid and (for tables in global memory) its workspace
+int plan_pass(css_ctx* c, cssi::WsBuf& b, int precision, int win_cap, int tab_cap, int shared, int warps, int team,
+              int max_ctas, WaveWs* out, int* nctas) {
+    WaveWs g{};
+    g.lay = cssi::wave_layout(precision, win_cap, tab_cap, shared, warps, team);
+    g.shared = shared != 0;
+    g.team = team;
+    // the occupancy query costs host time on every call: cached per shape
+    const int64_t key = ((((int64_t)g.lay.bytes * 16 + warps) * 2 + precision) * 2 + team) * 2 + g.shared;
+    auto hit = c->bps_cache.find(key);
+    int bps = hit != c->bps_cache.end()
+                  ? hit->second
+                  : (c->bps_cache[key] = cssi::waves_blocks_per_sm(precision, g.lay, warps, g.shared, team));
+    if (bps < 1) {
+        c->err = "launch shape does not fit an SM (" + std::to_string(warps) + " warps per CTA, shared scale " +
+                 std::to_string(shared) + ")";
+        return CSS_ERR_INVALID_ARG;
     }
-    if (b.warps < nwarps) {
-        cudaFree(b.gen);
-        b.gen = nullptr;
-        TRY(c, "workspace", cudaMalloc(&b.gen, nwarps * sizeof(uint32_t)));
-        b.warps = nwarps;
+    if (max_ctas > 0) bps = std::min(bps, max_ctas);
+    *nctas = c->sm_count * bps;
+    if (!g.shared) {
+        g.stride = (size_t)g.lay.bytes;
+        const size_t need = g.stride * (size_t)*nctas * (team ? 1 : warps);
+        if (need > b.bytes) {
+            cudaFree(b.ws);
+            b.ws = nullptr;
+            b.bytes = 0;
+            TRY(c, "workspace", cudaMalloc(&b.ws, need));
+            b.bytes = need;
+        }
+        g.base = (char*)b.ws;
     }
-    if (relayout) {
-        TRY(c, "workspace", cudaMemsetAsync(b.ws, 0, b.bytes, c->stream));
-        TRY(c, "workspace", cudaMemsetAsync(b.gen, 0, b.warps * sizeof(uint32_t), c->stream));
-        b.key = key;
-    }
-    g.base = (char*)b.ws;
-    g.gen = b.gen;
     *out = g;
     return CSS_OK;
 }
@@ -117,34 +114,13 @@ int ensure_buf(css_ctx* c, cssi::WsBuf& b, int precision, int win_cap, int tab_c
 // both passes for the context's launch shape and up to `nitems` work items
 int ensure_plan(css_ctx* c, int precision, int64_t nitems, GeoPlan* P) {
     const cssi::LaunchCfg& L = c->cfg;
-    // the occupancy query costs host time on every call: cached per shape
-    const int64_t bkey = (((int64_t)precision * 64 + L.warps_per_cta) * 64 + L.shared_scale * 4 + L.occupancy) * 2 + L.team;
-    auto hit = c->bps_cache.find(bkey);
-    int bps = hit != c->bps_cache.end()
-                  ? hit->second
-                  : (c->bps_cache[bkey] = L.team ? cssi::geodesic_team_blocks_per_sm(precision, L.warps_per_cta,
-                                                                                     L.shared_scale, L.occupancy)
-                                                 : cssi::geodesic_blocks_per_sm(precision, L.warps_per_cta,
-                                                                                L.shared_scale, L.occupancy));
-    if (bps < 1) {
-        c->err = "launch shape does not fit an SM (" + std::to_string(L.warps_per_cta) + " warps per CTA, shared scale " +
-                 std::to_string(L.shared_scale) + ")";
-        return CSS_ERR_INVALID_ARG;
-    }
-    if (L.ctas_per_sm > 0) bps = std::min(bps, L.ctas_per_sm);
     P->wpc1 = L.warps_per_cta;
-    P->nctas1 = c->sm_count * bps;
-    P->team = L.team;
-    // one workspace slice per warp, or per CTA in the team form
-    int rc = ensure_buf(c, c->ws1, precision, L.win_cap, L.tab_cap, L.shared_scale,
-                        L.team ? P->nctas1 : P->nctas1 * P->wpc1, &P->g1);
+    int rc = plan_pass(c, c->ws1, precision, L.win_cap, L.tab_cap, L.shared_scale, L.warps_per_cta, L.team,
+                       L.ctas_per_sm, &P->g1, &P->nctas1);
     if (rc) return rc;
-    P->g1.occupancy = L.occupancy;
     P->wpc2 = L.warps2_per_sm;
-    P->nctas2 = c->sm_count;
-    rc = ensure_buf(c, c->ws2, precision, L.win_cap2, 0, 0, P->nctas2 * P->wpc2, &P->g2);
+    rc = plan_pass(c, c->ws2, precision, L.win_cap2, 0, 0, L.warps2_per_sm, 0, 1, &P->g2, &P->nctas2);
     if (rc) return rc;
-    P->g2.occupancy = 1;
     if (c->defer_cap < nitems) {
         cudaFree(c->defer);
         c->defer = nullptr;
@@ -157,10 +133,11 @@ int ensure_plan(css_ctx* c, int precision, int64_t nitems, GeoPlan* P) {
 
 // the plan's identity, for keying captured graphs
 std::string plan_key(const css_ctx* c, const GeoPlan& P) {
-    const int64_t v[8] = {c->ws1.key, c->ws2.key, (int64_t)(uintptr_t)c->ws1.ws, (int64_t)(uintptr_t)c->ws2.ws,
-                          (int64_t)(uintptr_t)c->defer, P.nctas1, (c->cfg.tile * 8 + c->cfg.occupancy) * 2 + P.team,
-                          P.nctas2};
-    return std::string((const char*)v, sizeof(v));
+    std::string k((const char*)&P.g1, sizeof(P.g1));
+    k.append((const char*)&P.g2, sizeof(P.g2));
+    const int64_t v[6] = {(int64_t)(uintptr_t)c->defer, P.wpc1, P.nctas1, P.wpc2, P.nctas2, c->cfg.tile};
+    k.append((const char*)v, sizeof(v));
+    return k;
 }
 
 int ensure_pairs(css_parts* p, int cap) {
@@ -216,15 +193,11 @@ int enqueue_passes(css_ctx* c, const GeoJob& j0, const GeoJob* djobs, const int3
     TRY(c, "reset", cudaMemsetAsync(c->dscal + 2, 0, 2 * sizeof(int), st));
     TRY(c, "event", record_ev(c, c->ev_geo0));
     cssi::GeoQueue q1{job_of_item, src_of_item, nitems, nullptr, nullptr, c->defer, c->dscal + 2, c->cfg.tile};
-    if (P.team)
-        TRY(c, "geodesic", cssi::launch_geodesic_team(j0, djobs, q1, prec, P.g1, P.wpc1, P.nctas1, c->dscal,
-                                                      c->dscal + 1, c->dcount, st));
-    else
-        TRY(c, "geodesic", cssi::launch_geodesic(j0, djobs, q1, prec, P.g1, P.wpc1, P.nctas1, c->dscal, c->dscal + 1,
-                                                 c->dcount, st));
+    TRY(c, "geodesic", cssi::launch_waves(j0, djobs, q1, prec, P.g1, P.wpc1, P.nctas1, c->dscal, c->dscal + 1,
+                                          c->dcount, st));
     cssi::GeoQueue q2{job_of_item, src_of_item, nitems, c->defer, c->dscal + 2, nullptr, nullptr, 1};
-    TRY(c, "geodesic", cssi::launch_geodesic(j0, djobs, q2, prec, P.g2, P.wpc2, P.nctas2, c->dscal + 3, c->dscal + 1,
-                                             c->dcount, st));
+    TRY(c, "geodesic", cssi::launch_waves(j0, djobs, q2, prec, P.g2, P.wpc2, P.nctas2, c->dscal + 3, c->dscal + 1,
+                                          c->dcount, st));
     TRY(c, "event", record_ev(c, c->ev_geo1));
     return CSS_OK;
 }
@@ -372,9 +345,7 @@ int css_create(css_ctx** out, int device, void* stream) {
 int css_destroy(css_ctx* c) {
     if (!c) return CSS_ERR_INVALID_ARG;
     cudaFree(c->ws1.ws);
-    cudaFree(c->ws1.gen);
     cudaFree(c->ws2.ws);
-    cudaFree(c->ws2.gen);
     cudaFree(c->defer);
     cudaFree(c->dscal);
     cudaFree(c->dcount);
@@ -412,6 +383,11 @@ int css_fma_peak(css_ctx* c, int precision, double* flops_per_s) {
     return CSS_OK;
 }
 
+static bool shape_fits(int prec, int win_cap, int tab_cap, int scale, int warps, int team) {
+    return cssi::waves_blocks_per_sm(prec, cssi::wave_layout(prec, win_cap, tab_cap, scale, warps, team), warps,
+                                     scale != 0, team) >= 1;
+}
+
 static bool launch_ok(const css_launch* l) {
     const int s = l->shared_scale;
     return l->warps_per_cta >= 1 && l->warps_per_cta <= 8 && l->ctas_per_sm >= 0 && l->ctas_per_sm <= 32 &&
@@ -426,8 +402,8 @@ static bool launch_ok(const css_launch* l) {
 int css_set_launch(css_ctx* c, const css_launch* l) {
     if (!c || !l || !launch_ok(l)) return CSS_ERR_INVALID_ARG;
     for (int prec : {CSS_FP32, CSS_FP64})
-        if ((l->team ? cssi::geodesic_team_blocks_per_sm(prec, l->warps_per_cta, l->shared_scale, l->occupancy)
-                     : cssi::geodesic_blocks_per_sm(prec, l->warps_per_cta, l->shared_scale, l->occupancy)) < 1) {
+        if (!shape_fits(prec, next_pow2(l->window_capacity), l->table_capacity ? next_pow2(l->table_capacity) : 0,
+                        l->shared_scale, l->warps_per_cta, l->team)) {
             c->err = "launch shape does not fit an SM";
             return CSS_ERR_INVALID_ARG;
         }
@@ -489,6 +465,7 @@ int css_mesh_free(css_mesh* m) {
     cudaFree(m->ring_start); cudaFree(m->ring); cudaFree(m->X); cudaFree(m->he32); cudaFree(m->lay32);
     cudaFree(m->frank);
     cudaFree(m->cang);
+    cudaFree(m->htop);
     cssi::vhm_free(m);
     delete m;
     return CSS_OK;
@@ -1127,7 +1104,8 @@ int css_autotune(css_ctx* c, css_parts* const* sets, int32_t n_sets, const css_p
     int rc = CSS_OK;
     for (int s : {1, 2, 4, 0}) {
         for (int wpc : {2, 4, 8}) {
-            const int bps = cssi::geodesic_blocks_per_sm(precision, wpc, s, 1);
+            const int bps = cssi::waves_blocks_per_sm(
+                precision, cssi::wave_layout(precision, POOL_UNIT * (s ? s : 4), 0, s, wpc, 0), wpc, s != 0, 0);
             if (bps < 1) continue;
             for (int cps : {0, 1}) {
                 if (cps == 1 && bps == 1) continue;   // same shape as "as many as fit"
@@ -1181,7 +1159,7 @@ int css_autotune(css_ctx* c, css_parts* const* sets, int32_t n_sets, const css_p
                 L.ctas_per_sm = 0;
                 L.tile = 1;
                 L.tab_cap = T.shared_scale ? 0 : tab;
-                if (cssi::geodesic_blocks_per_sm(precision, wpc, L.shared_scale, 2) < 1) continue;
+                if (!shape_fits(precision, L.win_cap, L.tab_cap, L.shared_scale, wpc, 0)) continue;
                 double t = 0.0;
                 rc = measure(L, &t);
                 if (rc) break;
@@ -1196,7 +1174,7 @@ int css_autotune(css_ctx* c, css_parts* const* sets, int32_t n_sets, const css_p
         for (int s : {1, 4, 0}) {
             for (int wpc : {2, 4, 8}) {
                 for (int occ : {1, 2}) {
-                    if (cssi::geodesic_team_blocks_per_sm(precision, wpc, s, occ) < 1) continue;
+                    if (!shape_fits(precision, POOL_UNIT * (s ? s : 4), 0, s, wpc, 1)) continue;
                     cssi::LaunchCfg L = base;
                     L.team = 1;
                     L.occupancy = occ;

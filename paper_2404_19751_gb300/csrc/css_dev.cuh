@@ -28,6 +28,10 @@ struct __align__(16) HeRec32 {
     int32_t pad;
 };
 
+// Half-edge topology for unfolding (16 B): the vertices at the start, the end and the far corner
+// (bit 30: shortest paths may bend there, see EMITS), and the face's rank (bucket index)
+constexpr int32_t EMITS = 1 << 30, VMASK = EMITS - 1;
+
 struct DMesh {
     int32_t nv, nf;
     int32_t periodic;
@@ -49,6 +53,8 @@ struct DMesh {
     const float2* cang;           // 3 nf: (start, width) of corner h around its vertex, angles
                                   // counted counter-clockwise from one fixed edge; NaN on boundary
                                   // and non-manifold vertices
+    const int4* htop;             // 3 nf: (start, end, far corner, face rank); vertices that are on the
+                                  // boundary, non-manifold or of an angle sum above 2 pi carry EMITS
 };
 
 __device__ __forceinline__ double cross2(double ax, double ay, double bx, double by) { return ax * by - ay * bx; }

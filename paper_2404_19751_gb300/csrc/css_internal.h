@@ -27,13 +27,10 @@ struct LaunchCfg {
     int tab_cap = 0;         // first pass with global tables: table slots (0: tied to win_cap)
     int team = 0;            // 1: the warps of a CTA work on one source together (team form)
 };
-// a second-pass workspace (global tables)
+// one pass's workspace (global tables and rings), grown on demand
 struct WsBuf {
     void* ws = nullptr;
     size_t bytes = 0;
-    uint32_t* gen = nullptr;
-    int warps = 0;
-    int64_t key = -1;        // layout the bytes were zeroed for
 };
 }  // namespace cssi
 
@@ -94,6 +91,7 @@ struct css_mesh {
     float* lay32 = nullptr;
     int32_t* frank = nullptr;   // nf: Morton rank of each face
     float2* cang = nullptr;     // 3 nf: corner (start, width) around its vertex
+    int4* htop = nullptr;       // 3 nf: half-edge topology (css::DMesh::htop)
     cssi::VhmOp* vhm = nullptr;
     css::DMesh view() const;
 };
@@ -211,6 +209,39 @@ struct GeoWs {
     char* lbase = nullptr;   // path launches: per-warp vertex link arrays (lstride bytes a warp)
     size_t lstride = 0;
 };
+
+// One source's working memory in k_waves: capacities (powers of two of ring, vertex and target
+// tables, and the fills at which they count as full) and byte offsets of its arrays; e_*: a
+// warp's queued target tests.
+struct WaveLay {
+    int ring_log, vh_log, th_log;
+    int v_most, t_most, em_cap, lg_cap, max_waves;
+    int sx, sy, ra, rb, d0x, d0y, d1x, d1y, b0, b1, key, he, vs;   // ring
+    int vkey, vdist, vtan, vflag;                                  // vertices
+    int tkey, tdist, tvert, tlist;                                        // targets
+    int emit;                                                      // vertices waiting to start windows
+    int ldist, lcmp, ltan, lslot;                                        // improvements of target distances
+    int bytes;
+    int e_sx, e_sy, e_ra, e_rb, e_d0x, e_d0y, e_d1x, e_d1y, e_he, e_vs, e_j;
+    int e_bytes;
+};
+struct WaveWs {
+    WaveLay lay;
+    int shared;      // working memory in shared memory (else base + group * stride)
+    int team;        // the warps of a CTA work on one source
+    char* base;
+    size_t stride;
+};
+
+// waves.cu
+constexpr size_t WAVE_SHARED_MAX = 224 * 1024;   // dynamic shared memory a CTA may ask for
+WaveLay wave_layout(int precision, int win_cap, int tab_cap, int shared_scale, int warps, int team);
+// the layout for given table sizes (logarithms), in global memory
+WaveLay wave_layout_of(int precision, int ring_log, int vh_log, int th_log);
+int waves_blocks_per_sm(int precision, const WaveLay& y, int warps, int shared, int team);
+cudaError_t launch_waves(const GeoJob& job0, const GeoJob* djobs, const GeoQueue& q, int precision, const WaveWs& g,
+                         int warps, int nctas, int* work_counter, int* status, unsigned long long* counters,
+                         cudaStream_t st);
 
 // geodesic.cu
 size_t geo_ws_bytes_per_warp(int precision, int win_cap, int tab_cap, int* log_eh, int* log_vh, int* log_fh,

@@ -32,11 +32,21 @@
 #include <stdint.h>
 
 #include "css_internal.h"
+#include "geo_common.cuh"
 
 namespace {
 
 using css::DMesh;
 using css::HeRec;
+using geo::BACK_OFF;
+using geo::BACK_STEP;
+using geo::SHADOW_TOL;
+using geo::back_angle;
+using geo::pack_back;
+using geo::pot_dudl;
+using geo::pot_u;
+using geo::scan_owner;
+using geo::warp_incl_scan;
 
 constexpr int WIN_ALIVE = 1;
 constexpr int WIN_DONE = 2;    // already unfolded
@@ -434,15 +444,6 @@ struct VCand : VLink<L> {
     float back;      // direction of the path's last leg, seen from the vertex, as a cumulative
                      // corner angle (DMesh::cang); NaN where it is not known
 };
-
-// Cumulative angle at a vertex of the direction g, given the vertex's corner hc whose first
-// edge runs along e (both in one face layout); NaN when g is too short to have a reliable
-// direction or the corner has no cumulative angle.
-__device__ __forceinline__ float back_angle(const DMesh& m, int hc, double ex, double ey, double gx, double gy,
-                                            double scale) {
-    if (hc < 0 || !(gx * gx + gy * gy > 1e-12 * scale * scale)) return __int_as_float(0x7fffffff);
-    return m.cang[hc].x + atan2f((float)(ex * gy - ey * gx), (float)(ex * gx + ey * gy));
-}
 
 // The link of the point (X, Y) of window W's half-edge frame straight back to W's
 // pseudo-source: which = 2 the far corner of the face W enters (the direction lies in that
@@ -1057,12 +1058,6 @@ __device__ __forceinline__ int group_rounds(bool has, int key, int lane, int& ra
 // Vertex table flags: bit 0 queued for emission, bit 1 distance from a pseudo-source path,
 // bits 16..31 the back direction of the recorded path (DMesh::cang units) in steps of 1/4096
 // rad offset by 4 rad; 0xffff where it is unknown or out of range.
-constexpr float BACK_STEP = 4096.0f, BACK_OFF = 4.0f;
-__device__ __forceinline__ unsigned pack_back(float b) {
-    const float t = (b + BACK_OFF) * BACK_STEP;
-    return (t >= 0.0f && t < 65535.0f) ? (unsigned)__float2int_rn(t) : 0xffffu;   // NaN -> unknown
-}
-
 template <class R, int SH>
 __device__ __noinline__ void vertex_round(const DMesh& m, Ws<R, SH>& ws, WarpSm& sm, bool has,
                                           const VCand<R, SH == 2>& c, double rc, int lane) {
@@ -1166,7 +1161,6 @@ __device__ __noinline__ void child_round(const DMesh& m, Ws<R, SH>& ws, WarpSm& 
 // where it is below pi, so the continuation is not shortest).  The range is widened by
 // SHADOW_TOL for the rounding of b and of the corner angles; vertices without a known back
 // direction, boundary and non-manifold vertices emit on every corner.
-constexpr float SHADOW_TOL = 1e-3f;
 template <class R, int SH>
 __device__ __noinline__ int emit_round(const DMesh& m, Ws<R, SH>& ws, WarpSm& sm, double rc, double kmin, int lane,
                                        Win<R>* stage = nullptr, int cap = 0, int* nstaged = nullptr) {
@@ -1303,26 +1297,6 @@ __device__ __noinline__ int emit_round(const DMesh& m, Ws<R, SH>& ws, WarpSm& sm
     }
     __syncwarp();
     return emitted;
-}
-
-__device__ __forceinline__ double pot_dudl(const css_potential& p, double l) {
-    if (!(l < p.r_cut)) return 0.0;
-    if (p.kind == CSS_POT_HARMONIC) return -2.0 * p.eps * (1.0 - l / p.sigma) / p.sigma;
-    if (p.kind == CSS_POT_WCA) {
-        const double q = p.sigma / l, q2 = q * q, q6 = q2 * q2 * q2;
-        return 24.0 * p.eps * (q6 - 2.0 * q6 * q6) / l;
-    }
-    return -(l / (p.sigma * p.sigma)) * p.A * exp(-l * l / (2.0 * p.sigma * p.sigma));
-}
-
-__device__ __forceinline__ double pot_u(const css_potential& p, double l) {
-    if (!(l < p.r_cut)) return 0.0;
-    if (p.kind == CSS_POT_HARMONIC) { const double u = 1.0 - l / p.sigma; return p.eps * u * u; }
-    if (p.kind == CSS_POT_WCA) {
-        const double q = p.sigma / l, q2 = q * q, q6 = q2 * q2 * q2;
-        return 4.0 * p.eps * (q6 * q6 - q6) + p.eps;
-    }
-    return p.A * exp(-l * l / (2.0 * p.sigma * p.sigma));
 }
 
 // distance + source tangent (source-face layout) of particle j of face fl
@@ -1686,27 +1660,6 @@ __device__ __forceinline__ void eval_face_block(const cssi::GeoJob& J, int i, co
         if (t < total) j = J.fitems[o_st + (t - o_ex)];
         eval_targets<R>(J, i, ws, f0, qx, qy, t < total && j != i, o_fl, j, lane, item, slots, fx, fy, en);
     }
-}
-
-// Inclusive prefix sum of x over the warp.
-__device__ __forceinline__ int warp_incl_scan(int x, int lane) {
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(CSS_FULL, x, o);
-        if (lane >= o) x += t;
-    }
-    return x;
-}
-
-// The lane whose inclusive-scan range holds item t (31 for t beyond the total).
-__device__ __forceinline__ int scan_owner(int incl, int t) {
-    int owner = 0;
-#pragma unroll
-    for (int step = 16; step >= 1; step >>= 1) {
-        const int v = __shfl_sync(CSS_FULL, incl, owner + step - 1);
-        if (v <= t) owner += step;
-    }
-    return min(owner, 31);
 }
 
 // Per-warp staging (shared memory) of a wave's vertex candidates and then of its children,
@@ -2583,33 +2536,32 @@ cudaError_t launch_pairs_compact(int32_t n, const int32_t* pcnt, const int32_t* 
 // inside a host callback or a framework that forbids device allocation on its hot path,
 // or an embedding that must not change the device memory footprint after start-up. For
 // them css_compute_forces_noalloc runs the same neighbour/force kernel as
-// css_compute_forces, but all of its scratch (the per-warp window workspace, the face
-// buckets and the launch counters) lives in the one file-scope device array below, of a
-// fixed size that every GPU loading this library holds until the process exits.
+// css_compute_forces, but all of its scratch (the per-warp tables, the face buckets and the launch
+// counters) lives in the one file-scope device array below, of a fixed size that every GPU
+// loading this library holds until the process exits.
 namespace {
 
-constexpr size_t NA_WS_BYTES = 48ull << 20;        // per-warp window workspaces
-constexpr int NA_MAX_WARPS = 1024;
-constexpr int NA_WIN_CAP = 2048;                    // windows per warp
+constexpr size_t NA_WS_BYTES = 48ull << 20;        // working memory in global memory
 constexpr int64_t NA_MAX_FACES = 1 << 20;
 constexpr int64_t NA_MAX_PARTICLES = 1 << 18;
 constexpr int NA_WARPS_PER_CTA = 4;
-constexpr size_t NA_OFF_GEN = NA_WS_BYTES;
-constexpr size_t NA_OFF_FCNT = NA_OFF_GEN + NA_MAX_WARPS * 4;
+constexpr size_t NA_OFF_FCNT = NA_WS_BYTES;
 constexpr size_t NA_OFF_FSTART = NA_OFF_FCNT + (NA_MAX_FACES + 1) * 4;
 constexpr size_t NA_OFF_FITEMS = NA_OFF_FSTART + (NA_MAX_FACES + 1) * 4;
 constexpr size_t NA_OFF_SCAN = NA_OFF_FITEMS + NA_MAX_PARTICLES * 4;
 constexpr size_t NA_SCAN_INTS = (NA_MAX_FACES + 1) / 2048 + 2;
 constexpr size_t NA_OFF_PCNT = NA_OFF_SCAN + NA_SCAN_INTS * 4;
-constexpr size_t NA_OFF_SCAL = (NA_OFF_PCNT + NA_MAX_PARTICLES * 4 + 255) & ~(size_t)255;  // work, status
-constexpr size_t NA_OFF_COUNT = NA_OFF_SCAL + 256;                                         // 8 counters
-constexpr size_t NA_BYTES = NA_OFF_COUNT + 8 * 8;   // ~59 MB in all
+constexpr size_t NA_OFF_DEFER = NA_OFF_PCNT + NA_MAX_PARTICLES * 4;   // two lists of sources left to a later pass
+constexpr size_t NA_OFF_SCAL = (NA_OFF_DEFER + 2 * NA_MAX_PARTICLES * 4 + 255) & ~(size_t)255;  // work, status
+constexpr size_t NA_OFF_COUNT = NA_OFF_SCAL + 256;                                              // 8 counters
+constexpr size_t NA_BYTES = NA_OFF_COUNT + 8 * 8;   // ~61 MB in all
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NA_BYTES];
 
 struct NaDevice {
     char* base = nullptr;   // device address of g_noalloc_scratch on this device
-    int layout = -1;        // precision whose workspace layout the bytes currently hold
+    int bps[2] = {0, 0};    // resident CTAs per SM of the shared-memory pass, by precision
+    bool zeroed = false;    // the face counts start from zero (every call leaves them so)
 };
 NaDevice g_na[64];
 
@@ -2649,8 +2601,7 @@ int na_status_error(css_ctx* c, int status) {
         return CSS_ERR_INVALID_ARG;
     }
     if (status & (css::ST_WIN_OVERFLOW | css::ST_HASH_OVERFLOW)) {
-        c->err = "compute_forces_noalloc: a source needs more than the fixed window workspace (" +
-                 std::to_string(NA_WIN_CAP) + " windows per warp); use css_compute_forces";
+        c->err = "compute_forces_noalloc: a source needs more than the fixed workspace; use css_compute_forces";
         return CSS_ERR_QUEUE_OVERFLOW;
     }
     if (status & (css::ST_ITER_LIMIT | css::ST_WALK_LIMIT)) {
@@ -2701,13 +2652,6 @@ int css_compute_forces_noalloc(const css_mesh* mesh, int64_t n, const int32_t* f
         e = cudaGetSymbolAddress((void**)&D.base, g_noalloc_scratch);
         if (e != cudaSuccess) { D.base = nullptr; c->err = std::string("noalloc set-up: ") + cudaGetErrorString(e); return CSS_ERR_CUDA; }
     }
-    cssi::GeoWs g{};
-    g.stride = cssi::geo_ws_bytes_per_warp(precision, NA_WIN_CAP, 0, &g.log_eh, &g.log_vh, &g.log_fh, &g.fcap, &g.emcap);
-    g.wcap = NA_WIN_CAP;
-    g.nwarps = (int)std::min<size_t>(NA_MAX_WARPS, NA_WS_BYTES / g.stride);
-    g.nwarps -= g.nwarps % NA_WARPS_PER_CTA;
-    g.base = D.base;
-    g.gen = (uint32_t*)(D.base + NA_OFF_GEN);
     int32_t* fcnt = (int32_t*)(D.base + NA_OFF_FCNT);
     int32_t* fstart = (int32_t*)(D.base + NA_OFF_FSTART);
     int32_t* fitems = (int32_t*)(D.base + NA_OFF_FITEMS);
@@ -2719,11 +2663,9 @@ int css_compute_forces_noalloc(const css_mesh* mesh, int64_t n, const int32_t* f
     // read here) comes first; the event was made with the context, so nothing is allocated
     e = cudaEventRecord(c->ev_order, c->stream);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(st, c->ev_order, 0);
-    if (e == cudaSuccess && D.layout != precision) {
-        // the array keeps the previous call's bytes; a new workspace layout starts from zero so
-        // no stale bytes look like hash entries, and the face counts start from zero
-        e = cudaMemsetAsync(D.base, 0, NA_OFF_FSTART, st);
-        if (e == cudaSuccess) D.layout = precision;
+    if (e == cudaSuccess && !D.zeroed) {
+        e = cudaMemsetAsync(fcnt, 0, (NA_MAX_FACES + 1) * 4, st);
+        if (e == cudaSuccess) D.zeroed = true;
     }
     if (e == cudaSuccess) e = cudaMemsetAsync(scal, 0, 256 + 8 * 8, st);
     int status = 0;
@@ -2754,10 +2696,35 @@ int css_compute_forces_noalloc(const css_mesh* mesh, int64_t n, const int32_t* f
     j.pot = *pot;
     j.force = forces;
     j.epot = e_pot;
-    if (e == cudaSuccess) {   // one pass, global tables; a source overflowing them is reported
-        const cssi::GeoQueue q{nullptr, nullptr, (int32_t)n, nullptr, nullptr, nullptr, nullptr, 1};
-        e = cssi::launch_geodesic(j, nullptr, q, precision, g, NA_WARPS_PER_CTA, g.nwarps / NA_WARPS_PER_CTA, scal,
-                                  scal + 1, cnt, st);
+    // three passes, each over the sources the one before could not hold: shared-memory tables; the
+    // scratch array in slices for up to 1792 vertices and 896 targets; the same array in fewer
+    // slices that hold every particle as a target.  What overflows the last one is reported.
+    int32_t* defer = (int32_t*)(D.base + NA_OFF_DEFER);
+    for (int pass = 0; pass < 3 && e == cudaSuccess; ++pass) {
+        cssi::WaveWs g{};
+        g.shared = pass == 0;
+        g.base = D.base;
+        int tl = 10;
+        while (pass == 2 && (7ll << tl) / 8 < n + 1) ++tl;
+        g.lay = pass == 0 ? cssi::wave_layout(precision, 2048, 0, 1, NA_WARPS_PER_CTA, 0)
+                          : cssi::wave_layout_of(precision, pass == 1 ? 10 : 12, pass == 1 ? 11 : 14, tl);
+        g.stride = (size_t)g.lay.bytes;
+        int warps = NA_WARPS_PER_CTA, ctas = 0;
+        if (pass) {
+            const int slices = (int)std::min<size_t>(1024, NA_WS_BYTES / g.stride);
+            warps = std::min(warps, slices);
+            ctas = slices / warps;
+        } else {
+            int& bps = D.bps[precision];
+            if (!bps) bps = cssi::waves_blocks_per_sm(precision, g.lay, warps, 1, 0);
+            if (bps < 1) e = cudaErrorInvalidConfiguration;
+            ctas = c->sm_count * bps;
+        }
+        const cssi::GeoQueue q{nullptr, nullptr, (int32_t)n,
+                               pass ? defer + (pass - 1) * NA_MAX_PARTICLES : nullptr, pass ? scal + 1 + 2 * pass : nullptr,
+                               pass < 2 ? defer + pass * NA_MAX_PARTICLES : nullptr, pass < 2 ? scal + 3 + 2 * pass : nullptr, 1};
+        if (e == cudaSuccess)
+            e = cssi::launch_waves(j, nullptr, q, precision, g, warps, ctas, pass ? scal + 2 * pass : scal, scal + 1, cnt, st);
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(&status, scal + 1, sizeof(int), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);

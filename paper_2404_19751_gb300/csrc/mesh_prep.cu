@@ -219,6 +219,25 @@ __global__ void k_vertices(int64_t nv, const int32_t* ring_start, int32_t* ring,
         for (int i = s; i < e; ++i) cang[ring[i]] = make_float2(NAN, NAN);
 }
 
+// Topology records of the half-edges.  A shortest path bends only at a boundary, non-manifold or
+// saddle vertex.  An interior vertex of angle sum 2 pi (within 1e-12, a flat one) needs no windows
+// of its own: the straight lines on its two sides meet behind it.
+__global__ void k_htop(int64_t nf, const int32_t* fv, const uint8_t* pseudo, const double* theta,
+                       const float2* cang, const int32_t* ring_start, const int32_t* ring, const int32_t* frank,
+                       int4* htop) {
+    const int64_t h = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (h >= 3 * nf) return;
+    const int64_t f = h / 3;
+    const int k = (int)(h - 3 * f);
+    int32_t o[3];
+    for (int q = 0; q < 3; ++q) {
+        const int32_t v = fv[3 * f + (k + q) % 3];
+        const bool fan = !isnan(cang[ring[ring_start[v]]].x);   // one closed fan of faces
+        o[q] = v | (pseudo[v] && !(fan && theta[v] <= TWO_PI + 1e-12) ? css::EMITS : 0);
+    }
+    htop[h] = make_int4(o[0], o[1], o[2], frank[f]);
+}
+
 inline unsigned nblk(int64_t n, int b = 256) { return (unsigned)((n + b - 1) / b); }
 
 }  // namespace
@@ -265,6 +284,7 @@ css::DMesh css_mesh::view() const {
     d.lay32 = lay32;
     d.frank = frank;
     d.cang = cang;
+    d.htop = htop;
     return d;
 }
 
@@ -321,6 +341,7 @@ int build_mesh(css_ctx* ctx, const double* dX, int64_t nv, const int32_t* dF, in
     CK(cudaMalloc(&m->lay32, 3 * nf * sizeof(float)));
     CK(cudaMalloc(&m->frank, nf * sizeof(int32_t)));
     CK(cudaMalloc(&m->cang, nh * sizeof(float2)));
+    CK(cudaMalloc(&m->htop, nh * sizeof(int4)));
     CK(cudaMalloc(&ring_cnt, (nv + 1) * sizeof(int32_t)));
     CK(cudaMalloc(&tmp, scan_tmp_ints(nv + 1) * sizeof(int32_t)));
     CK(cudaMemcpyAsync(m->X, dX, 3 * nv * sizeof(double), cudaMemcpyDeviceToDevice, st));
@@ -383,6 +404,9 @@ int build_mesh(css_ctx* ctx, const double* dX, int64_t nv, const int32_t* dF, in
         std::vector<int32_t> rank(nf);
         for (int64_t r = 0; r < nf; ++r) rank[(int64_t)(key[r] & 0xffffffffu)] = (int32_t)r;
         CK(cudaMemcpyAsync(m->frank, rank.data(), nf * sizeof(int32_t), cudaMemcpyHostToDevice, st));
+        k_htop<<<nblk(nh), 256, 0, st>>>(nf, m->fv, m->pseudo, m->theta, m->cang, m->ring_start, m->ring,
+                                         m->frank, m->htop);
+        CK(cudaGetLastError());
         CK(cudaStreamSynchronize(st));
     }
 done:
