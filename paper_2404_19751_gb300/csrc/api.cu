@@ -83,7 +83,7 @@ int plan_pass(css_ctx* c, cssi::WsBuf& b, int precision, int win_cap, int tab_ca
     g.shared = shared != 0;
     g.team = team;
     // the occupancy query costs host time on every call: cached per shape
-    const int64_t key = ((((int64_t)g.lay.bytes * 16 + warps) * 2 + precision) * 2 + team) * 2 + g.shared;
+    const int64_t key = (((((int64_t)g.lay.t_bytes << 20) + g.lay.h_bytes) * 16 + warps) * 2 + precision) * 4 + team * 2 + g.shared;
     auto hit = c->bps_cache.find(key);
     int bps = hit != c->bps_cache.end()
                   ? hit->second
@@ -95,18 +95,16 @@ int plan_pass(css_ctx* c, cssi::WsBuf& b, int precision, int win_cap, int tab_ca
     }
     if (max_ctas > 0) bps = std::min(bps, max_ctas);
     *nctas = c->sm_count * bps;
-    if (!g.shared) {
-        g.stride = (size_t)g.lay.bytes;
-        const size_t need = g.stride * (size_t)*nctas * (team ? 1 : warps);
-        if (need > b.bytes) {
-            cudaFree(b.ws);
-            b.ws = nullptr;
-            b.bytes = 0;
-            TRY(c, "workspace", cudaMalloc(&b.ws, need));
-            b.bytes = need;
-        }
-        g.base = (char*)b.ws;
+    g.stride = cssi::waves_global_bytes(g.lay, g.shared);
+    const size_t need = g.stride * (size_t)*nctas * (team ? 1 : warps);
+    if (need > b.bytes) {
+        cudaFree(b.ws);
+        b.ws = nullptr;
+        b.bytes = 0;
+        TRY(c, "workspace", cudaMalloc(&b.ws, need));
+        b.bytes = need;
     }
+    g.base = (char*)b.ws;
     *out = g;
     return CSS_OK;
 }

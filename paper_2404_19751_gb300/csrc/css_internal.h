@@ -210,26 +210,29 @@ struct GeoWs {
     size_t lstride = 0;
 };
 
-// One source's working memory in k_waves: capacities (powers of two of ring, vertex and target
-// tables, and the fills at which they count as full) and byte offsets of its arrays; e_*: a
-// warp's queued target tests.
+// One source's working memory in k_waves: capacities (powers of two of the vertex and target tables
+// and of the spill area, the fills at which they count as full) and byte offsets of its arrays.
+// A window record is six arrays: pseudo-source, rotation, two rims, (half-edge, vertex, key,
+// interval), slots of the edge's ends.
 struct WaveLay {
-    int ring_log, vh_log, th_log;
-    int v_most, t_most, em_cap, lg_cap, max_waves;
-    int sx, sy, ra, rb, d0x, d0y, d1x, d1y, b0, b1, key, he, vs;   // ring
-    int vkey, vdist, vtan, vflag;                                  // vertices
-    int tkey, tdist, tvert, tlist;                                        // targets
-    int emit;                                                      // vertices waiting to start windows
-    int ldist, lcmp, ltan, lslot;                                        // improvements of target distances
-    int bytes;
-    int e_sx, e_sy, e_ra, e_rb, e_d0x, e_d0y, e_d1x, e_d1y, e_he, e_vs, e_j;
-    int e_bytes;
+    int r_mask, s_cap, vh_log, th_log;
+    int v_most, t_most, i_cap, lg_cap, max_waves;
+    int r[6], h_bytes;                                 // ring (shared memory)
+    int vkey, vdist, vinfo;                            // vertices
+    int itan, iback, ihc;                              // path records of vertices that start windows
+    int emit;                                          // vertices waiting to start windows
+    int tkey, tdist, tvert, tlist;                     // targets
+    int ttan, tcmp;                                    // their directions and compared lengths (a team: its log's)
+    int ldist, lslot;                                  // a team's log of improvements
+    int t_bytes;                                       // tables
+    int s[6], s_bytes;                                 // spill area (global memory)
+    int e[6], e_task, e_bytes;                         // a warp's queued tests and child tasks (shared memory)
 };
 struct WaveWs {
     WaveLay lay;
-    int shared;      // working memory in shared memory (else base + group * stride)
+    int shared;      // tables in shared memory
     int team;        // the warps of a CTA work on one source
-    char* base;
+    char* base;      // global memory of group k: base + k * stride
     size_t stride;
 };
 
@@ -237,7 +240,8 @@ struct WaveWs {
 constexpr size_t WAVE_SHARED_MAX = 224 * 1024;   // dynamic shared memory a CTA may ask for
 WaveLay wave_layout(int precision, int win_cap, int tab_cap, int shared_scale, int warps, int team);
 // the layout for given table sizes (logarithms), in global memory
-WaveLay wave_layout_of(int precision, int ring_log, int vh_log, int th_log);
+WaveLay wave_layout_of(int precision, int spill_log, int vh_log, int th_log);
+size_t waves_global_bytes(const WaveLay& y, int shared);   // of one group
 int waves_blocks_per_sm(int precision, const WaveLay& y, int warps, int shared, int team);
 cudaError_t launch_waves(const GeoJob& job0, const GeoJob* djobs, const GeoQueue& q, int precision, const WaveWs& g,
                          int warps, int nctas, int* work_counter, int* status, unsigned long long* counters,

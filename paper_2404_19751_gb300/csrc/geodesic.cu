@@ -2706,9 +2706,9 @@ int css_compute_forces_noalloc(const css_mesh* mesh, int64_t n, const int32_t* f
         g.base = D.base;
         int tl = 10;
         while (pass == 2 && (7ll << tl) / 8 < n + 1) ++tl;
-        g.lay = pass == 0 ? cssi::wave_layout(precision, 2048, 0, 1, NA_WARPS_PER_CTA, 0)
+        g.lay = pass == 0 ? cssi::wave_layout(precision, 256, 0, 1, NA_WARPS_PER_CTA, 0)
                           : cssi::wave_layout_of(precision, pass == 1 ? 10 : 12, pass == 1 ? 11 : 14, tl);
-        g.stride = (size_t)g.lay.bytes;
+        g.stride = cssi::waves_global_bytes(g.lay, g.shared);
         int warps = NA_WARPS_PER_CTA, ctas = 0;
         if (pass) {
             const int slices = (int)std::min<size_t>(1024, NA_WS_BYTES / g.stride);
@@ -2718,7 +2718,7 @@ int css_compute_forces_noalloc(const css_mesh* mesh, int64_t n, const int32_t* f
             int& bps = D.bps[precision];
             if (!bps) bps = cssi::waves_blocks_per_sm(precision, g.lay, warps, 1, 0);
             if (bps < 1) e = cudaErrorInvalidConfiguration;
-            ctas = c->sm_count * bps;
+            ctas = (int)std::min<size_t>((size_t)c->sm_count * bps, NA_WS_BYTES / (g.stride * warps));
         }
         const cssi::GeoQueue q{nullptr, nullptr, (int32_t)n,
                                pass ? defer + (pass - 1) * NA_MAX_PARTICLES : nullptr, pass ? scal + 1 + 2 * pass : nullptr,

@@ -28,11 +28,10 @@
 // keeps rotations and directions in FP32.  Lengths of results are FP64 in both forms.
 //
 // Measured against windows kept in per-edge lists and trimmed against one another (the same
-// evaluations, default launch shapes): 65536 particles on a noisy level-8 sphere 110.7 -> 21.7 ms
-// (FP64) and 73.1 -> 18.5 ms (FP32), 8192 on a 256 x 256 height field 127 -> 13.9 ms, every pair of
-// 64 on a flat plane 30 -> 2.9 ms.  The windows unfolded per source are the same within 10 %
-// (482 against 440, 3991 against 3950, 5135 against 5151); a window costs a fifth: no list walk,
-// no FP64 split, no local-memory frames.
+// evaluations, default launch shapes): 65536 particles on a noisy level-8 sphere 110.7 -> 12.2 ms
+// (FP64) and 73.1 -> 13.0 ms (FP32), 8192 on a 256 x 256 height field 127 -> 9.4 ms, every pair of
+// 64 on a flat plane 30 -> 2.2 ms.  The windows unfolded per source are the same within 10 %
+// (482 against 440, 3991 against 3950, 5135 against 5151).
 #include <cuda_runtime.h>
 #include <limits.h>
 #include <math.h>
@@ -53,10 +52,44 @@ using cssi::WaveLay;
 using cssi::WaveWs;
 
 constexpr int MAXW = 8;          // warps per CTA
-constexpr int EV = 32;           // queued target tests per warp
+constexpr int EV = 10;           // queued target tests per warp
 constexpr int NONE = -1;
 constexpr int FIRST = 1 << 30;   // ring entry: starts at a vertex of the face behind its edge
 constexpr int FROM_VERTEX = 1 << 29;   // test: straight from a vertex of the target's face
+constexpr unsigned QUEUED = 1u << 31;  // path record: its vertex waits to start windows
+
+template <class R>
+struct Vec2;
+template <>
+struct Vec2<double> {
+    using type = double2;
+};
+template <>
+struct Vec2<float> {
+    using type = float2;
+};
+template <class R>
+using V2 = typename Vec2<R>::type;
+__device__ __forceinline__ double2 vec2(double x, double y) { return make_double2(x, y); }
+__device__ __forceinline__ float2 vec2(float x, float y) { return make_float2(x, y); }
+
+// index of a vertex slot or of a vertex's path record: 16 bits where the tables are in shared memory
+template <int PL>
+struct Index;
+template <>
+struct Index<1> {
+    using type = uint16_t;
+    using pair = ushort2;
+    static constexpr uint16_t none = 0xffffu;
+    static __device__ __forceinline__ ushort2 make(int a, int b) { return make_ushort2((uint16_t)a, (uint16_t)b); }
+};
+template <>
+struct Index<0> {
+    using type = int32_t;
+    using pair = int2;
+    static constexpr int32_t none = -1;
+    static __device__ __forceinline__ int2 make(int a, int b) { return make_int2(a, b); }
+};
 
 // relative tolerance of a point on the rim of a cone
 template <class R>
@@ -69,27 +102,22 @@ template <>
 struct Rim<float> {
     static constexpr float t = 2e-6f;
 };
-// relative excess up to which a window's path is taken over a path from a vertex of the target's face
-template <class R>
-struct Tie;
-template <>
-struct Tie<double> {
-    static constexpr double t = 1e-13;
-};
-template <>
-struct Tie<float> {
-    static constexpr double t = 1e-6;
-};
+// FP32 form: relative excess up to which a window's path is taken over a path from a vertex of the
+// target's face
+constexpr double TIE32 = 1e-6;
 
 // the counters of one source
 struct GroupSm {
-    int head, tail;      // first waiting window, end of the ring (both only grow)
+    int head, tail;      // first waiting window and end of the ring (both only grow)
+    int shead, stail;    // the same of the spill area
     int nem[2], cur;     // vertices waiting to start windows: two lists, the one in use
     unsigned emin;       // a lower bound on their distances (FP32 bits)
-    int nv, nt, nlog;    // table entries: vertices, targets, target improvements
+    int nv, ni, nt, nlog;   // table entries: vertices, their path records, targets, improvements
     int err;
     int item;
-    unsigned nprop;
+};
+// a team's per-warp values
+struct TeamSm {
     float km[MAXW];
     double fx[MAXW], fy[MAXW], en[MAXW];
 };
@@ -99,18 +127,6 @@ template <class T>
 __device__ __forceinline__ T* at(unsigned char* b, int off) { return reinterpret_cast<T*>(b + off); }
 
 __device__ __forceinline__ uint32_t hash_of(int32_t key, int logcap) { return ((uint32_t)key * 2654435761u) >> (32 - logcap); }
-
-__device__ __forceinline__ int tab_find(const int32_t* keys, int logcap, int32_t key) {
-    const uint32_t mask = (1u << logcap) - 1u;
-    uint32_t s = hash_of(key, logcap);
-    for (uint32_t p = 0; p <= mask; ++p) {
-        const int32_t c = *(volatile const int32_t*)(keys + s);
-        if (c == key) return (int)s;
-        if (c == NONE) return NONE;
-        s = (s + 1u) & mask;
-    }
-    return NONE;
-}
 
 // slot of the key, claimed if it is new; NONE when the table holds `most` keys already
 __device__ __forceinline__ int tab_insert(int32_t* keys, int logcap, int32_t key, int* count, int most, bool& claimed) {
@@ -135,6 +151,37 @@ __device__ __forceinline__ int tab_insert(int32_t* keys, int logcap, int32_t key
     return NONE;
 }
 
+// FP64 instructions run at 1/58 of the FP32 rate, conversions among them, and were what bounded the
+// FP64 form with 16 warps on an SM (about 130 a wave; 46 with these conversions, FP32 tests of the
+// rims and the roots below: 4.03 -> 2.95 ms for 16384 sources on a noisy sphere, 0.27 -> 0.14 ms
+// for 1024 on an icosphere).  So values only needed to FP32 precision are converted with integer
+// instructions, rounded toward zero: too small becomes 0, too large the largest number.
+__device__ __forceinline__ float f32(double x) {
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const unsigned mag = min(hi & 0x7fffffffu, 0x47efffffu);
+    const unsigned f = __funnelshift_l(lo, mag - 0x38000000u, 3);
+    return __uint_as_float((mag < 0x38100000u ? 0u : f) | (hi & 0x80000000u));
+}
+__device__ __forceinline__ float f32(float x) { return x; }
+__device__ __forceinline__ double f64(float x) {   // x > 0 and normal
+    const unsigned f = __float_as_uint(x);
+    return __hiloint2double((int)((f >> 3) + 0x38000000u), (int)(f << 29));
+}
+__device__ __forceinline__ bool is_inf(double x) { return __double2hiint(x) == 0x7ff00000; }
+// square root to 2^-22
+__device__ __forceinline__ float root(float x) { return x > 0.0f ? x * rsqrtf(x) : 0.0f; }
+// x^(1/2) and x^(-1/2) in FP64 from the FP32 reciprocal root: Goldschmidt's iteration (it squares the
+// relative error: 2^-22, 2^-43), then a Newton step each on the residual; x normal in FP32
+__device__ __forceinline__ void roots(double x, double& r, double& inv) {
+    const double y = f64(rsqrtf(f32(x)));
+    double g = x * y, h = 0.5 * y;
+    const double e = fma(-g, h, 0.5);
+    g = fma(g, e, g);
+    h = fma(h, e, h);
+    r = fma(fma(-g, g, x), h, g);
+    inv = 2.0 * fma(h, fma(-g, h, 0.5), h);
+}
+
 // Where the path through an edge's start vertex (along the edge) stops being the shorter one:
 // the window (pseudo-source at (sx, sy) with s2 = |s|^2, sx measured from that vertex) beats it
 // for x > x0 only, (x - sx)^2 + sy^2 < (x + a)^2 with a = the vertex's distance minus sigma.
@@ -146,92 +193,121 @@ __device__ __forceinline__ float cut_at(float sx, float s2, float a, float L, fl
     return den * L > num * 0.999f ? __fdividef(num, den) - 1e-5f * L : 2.0f * L;
 }
 
-// Evaluate a warp's queued tests: the target's point in the frame of the entered half-edge, inside
-// the cone or not, its length; every improvement of a target's distance is logged with its
-// direction at the source (the log is read once the source is done).  Paths that end with a
+// Evaluate a warp's queued tests (all lanes; lane k takes entry k < nev): the target's point in the
+// frame of the entered half-edge, inside the cone or not, its length.  Paths that end with a
 // straight piece from a vertex of the target's own face are kept apart from those that come
 // through a window: a window wins over them unless they are shorter by more than the form's
-// precision, so that a direction does not hang on the last bits of two equal lengths.
-template <class R>
+// precision, so that a direction does not hang on the last bits of two equal lengths (FP32 form; in
+// FP64 the shorter one is the one).  One warp writes the direction of an improvement beside the
+// length it lowered; a team's warps, which may lower one length at the same time, log them, and the
+// log is read once the source is done.
+template <class R, int PL, bool TEAM>
 __device__ __noinline__ void eval_tests(const cssi::GeoJob& J, const WaveLay& Y, unsigned char* b, unsigned char* e,
                                         GroupSm& sm, int nev, int lane) {
-    if (lane >= nev) return;
     const DMesh& m = J.m;
-    const int he = at<int>(e, Y.e_he)[lane], j = at<int>(e, Y.e_j)[lane];
-    int vs = at<int>(e, Y.e_vs)[lane];
-    const bool vertex = vs >= 0 && (vs & FROM_VERTEX);
-    if (vertex) vs &= ~FROM_VERTEX;
-    const double sx = at<double>(e, Y.e_sx)[lane], sy = at<double>(e, Y.e_sy)[lane];
-    const R ra = at<R>(e, Y.e_ra)[lane], rb = at<R>(e, Y.e_rb)[lane];
-    const R d0x = at<R>(e, Y.e_d0x)[lane], d0y = at<R>(e, Y.e_d0y)[lane];
-    const R d1x = at<R>(e, Y.e_d1x)[lane], d1y = at<R>(e, Y.e_d1y)[lane];
-    const HeRec& r = m.he[he];
-    const int k = he % 3;
-    const double* bj = J.bary + 3 * (size_t)j;
-    const double bv = bj[k == 2 ? 0 : k + 1], bc = bj[k == 0 ? 2 : k - 1];
-    const double gx = bv * r.L + bc * r.cx - sx, gy = bc * r.cy - sy;
-    const R fx = (R)gx, fy = (R)gy;
-    const R qx = fx * ra + fy * rb, qy = fy * ra - fx * rb;
-    const R tol = Rim<R>::t * (R)r.L;
-    const bool in = d0x * qy - d0y * qx <= tol * (fabs(d0x) + fabs(d0y)) &&
-                    d1x * qy - d1y * qx >= -tol * (fabs(d1x) + fabs(d1y));
-    const double n = sqrt(gx * gx + gy * gy), sig = vs < 0 ? 0.0 : at<double>(b, Y.vdist)[vs];
-    const double d = sig + n;
-    if (!(in && d < J.rc)) return;
-    bool claimed;
-    const int s = tab_insert(at<int32_t>(b, Y.tkey), Y.th_log, j, &sm.nt, Y.t_most, claimed);
-    if (s < 0) {
-        atomicOr(&sm.err, css::ST_HASH_OVERFLOW);
-        return;
-    }
-    const unsigned long long bits = (unsigned long long)__double_as_longlong(d);   // lengths start at infinity
-    if (atomicMin((unsigned long long*)at<double>(b, vertex ? Y.tvert : Y.tdist) + s, bits) <= bits) return;
-    const int l = atomicAdd(&sm.nlog, 1);
-    if (l >= Y.lg_cap) {
-        atomicOr(&sm.err, css::ST_HASH_OVERFLOW);
-        return;
-    }
-    R tx, ty;
-    if (vs < 0) {
-        const R inv = n > 0.0 ? (R)1 / (R)n : (R)0;
-        tx = qx * inv;
-        ty = qy * inv;
-    } else {
-        tx = at<R>(b, Y.vtan)[2 * vs];
-        ty = at<R>(b, Y.vtan)[2 * vs + 1];
-    }
-    // the length that decides between a window and a vertex: in the FP32 form from FP32
-    // coordinates of the target in its face, like every other comparison of that form
-    double w = d;
-    if constexpr (sizeof(R) == 4) {
-        const int f = he / 3;
-        const float L01 = m.lay32[3 * f], x2 = m.lay32[3 * f + 1], y2 = m.lay32[3 * f + 2];
-        const float px = (float)bj[1] * L01 + (float)bj[2] * x2, py = (float)bj[2] * y2;
-        const float ax = k == 0 ? 0.0f : (k == 1 ? L01 : x2), ay = k == 2 ? y2 : 0.0f;
-        if (vertex) w = sig + (double)sqrtf((px - ax) * (px - ax) + (py - ay) * (py - ay));
-        else {
-            const float bx = k == 0 ? L01 : (k == 1 ? x2 : 0.0f), by = k == 1 ? y2 : 0.0f, L = m.he32[he].L;
-            const float ex = (bx - ax) / L, ey = (by - ay) / L;
-            const float hx = (px - ax) * ex + (py - ay) * ey - (float)sx, hy = ex * (py - ay) - ey * (px - ax) - (float)sy;
-            w = (double)((float)sig + sqrtf(hx * hx + hy * hy));
+    bool won = false, apart = false;
+    int s = NONE;
+    double d = 0.0, w = 0.0;
+    V2<R> t = vec2((R)0, (R)0);
+    unsigned long long bits = 0;
+    if (lane < nev) {
+        const int4 w4 = at<int4>(e, Y.e[4])[lane];
+        const int he = w4.x, j = w4.z;
+        int vs = w4.y;
+        const bool vertex = vs >= 0 && (vs & FROM_VERTEX);
+        if (vertex) vs &= ~FROM_VERTEX;
+        const double2 S = at<double2>(e, Y.e[0])[lane];
+        const V2<R> rot = at<V2<R>>(e, Y.e[1])[lane], d0 = at<V2<R>>(e, Y.e[2])[lane], d1 = at<V2<R>>(e, Y.e[3])[lane];
+        const HeRec& r = m.he[he];
+        const int k = he % 3;
+        const double* bj = J.bary + 3 * (size_t)j;
+        const double bv = bj[k == 2 ? 0 : k + 1], bc = bj[k == 0 ? 2 : k - 1];
+        const double gx = bv * r.L + bc * r.cx - S.x, gy = bc * r.cy - S.y;
+        const R fx = (R)gx, fy = (R)gy;
+        const R qx = fx * rot.x + fy * rot.y, qy = fy * rot.x - fx * rot.y;
+        const R tol = Rim<R>::t * (R)r.L;
+        const bool in = d0.x * qy - d0.y * qx <= tol * (fabs(d0.x) + fabs(d0.y)) &&
+                        d1.x * qy - d1.y * qx >= -tol * (fabs(d1.x) + fabs(d1.y));
+        const double n = sqrt(gx * gx + gy * gy), sig = vs < 0 ? 0.0 : at<double>(b, Y.vdist)[vs];
+        d = sig + n;
+        if (in && d < J.rc) {
+            bool claimed;
+            s = tab_insert(at<int32_t>(b, Y.tkey), Y.th_log, j, &sm.nt, Y.t_most, claimed);
+            if (s < 0) atomicOr(&sm.err, css::ST_HASH_OVERFLOW);
+            else {
+                bits = (unsigned long long)__double_as_longlong(d);   // lengths start at infinity
+                apart = sizeof(R) == 4 && vertex;
+                won = atomicMin((unsigned long long*)at<double>(b, apart ? Y.tvert : Y.tdist) + s, bits) > bits;
+            }
+        }
+        if (won) {
+            if (vs < 0) {
+                const R inv = n > 0.0 ? (R)1 / (R)n : (R)0;
+                t = vec2(qx * inv, qy * inv);
+            } else t = at<V2<R>>(b, Y.itan)[at<typename Index<PL>::type>(b, Y.vinfo)[vs]];
+            // the length that decides between a window and a vertex: from FP32 coordinates of the
+            // target in its face, like every other comparison of that form
+            if constexpr (sizeof(R) == 4) {
+                const int f = he / 3;
+                const float L01 = m.lay32[3 * f], x2 = m.lay32[3 * f + 1], y2 = m.lay32[3 * f + 2];
+                const float px = (float)bj[1] * L01 + (float)bj[2] * x2, py = (float)bj[2] * y2;
+                const float ax = k == 0 ? 0.0f : (k == 1 ? L01 : x2), ay = k == 2 ? y2 : 0.0f;
+                if (vertex) w = sig + (double)sqrtf((px - ax) * (px - ax) + (py - ay) * (py - ay));
+                else {
+                    const float bx = k == 0 ? L01 : (k == 1 ? x2 : 0.0f), by = k == 1 ? y2 : 0.0f, L = m.he32[he].L;
+                    const float ex = (bx - ax) / L, ey = (by - ay) / L;
+                    const float hx = (px - ax) * ex + (py - ay) * ey - (float)S.x;
+                    const float hy = ex * (py - ay) - ey * (px - ax) - (float)S.y;
+                    w = (double)((float)sig + sqrtf(hx * hx + hy * hy));
+                }
+            }
         }
     }
-    at<double>(b, Y.ldist)[l] = d;
-    at<double>(b, Y.lcmp)[l] = w;
-    at<R>(b, Y.ltan)[2 * l] = tx;
-    at<R>(b, Y.ltan)[2 * l + 1] = ty;
-    at<int>(b, Y.lslot)[l] = vertex ? s | FROM_VERTEX : s;
+    if constexpr (TEAM) {
+        if (won) {
+            const int l = atomicAdd(&sm.nlog, 1);
+            if (l >= Y.lg_cap) atomicOr(&sm.err, css::ST_HASH_OVERFLOW);
+            else {
+                at<double>(b, Y.ldist)[l] = d;
+                at<V2<R>>(b, Y.ttan)[l] = t;
+                if constexpr (sizeof(R) == 4) at<double>(b, Y.tcmp)[l] = w;
+                at<int>(b, Y.lslot)[l] = apart ? s | FROM_VERTEX : s;
+            }
+        }
+    } else {
+        __syncwarp();
+        // of the lanes that lowered one length only the lowest one's value is there now
+        const int at_ = apart ? s + (1 << Y.th_log) : s;   // records of windows, then of vertices
+        if (won && *((volatile unsigned long long*)at<double>(b, apart ? Y.tvert : Y.tdist) + s) == bits) {
+            at<V2<R>>(b, Y.ttan)[at_] = t;
+            if constexpr (sizeof(R) == 4) at<double>(b, Y.tcmp)[at_] = w;
+        }
+    }
 }
 
 // ------------------------------------------------------------------ one source
+template <class R>
+struct Win {
+    double2 s;          // the pseudo-source in the frame of half-edge he
+    V2<R> rot, d0, d1;  // image of its own frame's x axis; left and right rim of the cone, in its frame
+    float b0, b1, key;
+    int he, vs;
+    int su, sv;         // slots of the edge's end vertices
+};
+
 template <class R, int PL, bool TEAM>
 struct Group {
+    using Idx = typename Index<PL>::type;
     const cssi::GeoJob& J;
     const WaveLay& Y;
-    unsigned char* b;      // tables and ring
-    unsigned char* e;      // this warp's queued tests
+    unsigned char* b;      // tables
+    unsigned char* h;      // ring
+    unsigned char* e;      // this warp's queued tests and task list
+    unsigned char* x;      // spill area
     GroupSm& sm;
+    TeamSm* tm;
     int src, lane, wid, tid, T;
+    float rcf;             // the cutoff, rounded up
     int nev = 0;
 
     __device__ __forceinline__ void bar() const {
@@ -240,26 +316,26 @@ struct Group {
     }
     __device__ __forceinline__ int32_t* vkey() const { return at<int32_t>(b, Y.vkey); }
     __device__ __forceinline__ double* vdist() const { return at<double>(b, Y.vdist); }
-    __device__ __forceinline__ R* vtan() const { return at<R>(b, Y.vtan); }
-    __device__ __forceinline__ unsigned* vflag() const { return at<unsigned>(b, Y.vflag); }
+    __device__ __forceinline__ Idx* vinfo() const { return at<Idx>(b, Y.vinfo); }
+    __device__ __forceinline__ V2<R>* itan() const { return at<V2<R>>(b, Y.itan); }
+    __device__ __forceinline__ float* iback() const { return at<float>(b, Y.iback); }
+    __device__ __forceinline__ unsigned* ihc() const { return at<unsigned>(b, Y.ihc); }
+    __device__ __forceinline__ Idx* waiting(int list) const { return at<Idx>(b, Y.emit) + list * Y.i_cap; }
     __device__ __forceinline__ int32_t* tkey() const { return at<int32_t>(b, Y.tkey); }
     __device__ __forceinline__ double* tdist() const { return at<double>(b, Y.tdist); }
     __device__ __forceinline__ double* tvert() const { return at<double>(b, Y.tvert); }
 
-    __device__ __forceinline__ double dist_of(int32_t v) const {
-        const int s = tab_find(vkey(), Y.vh_log, v);
-        return s < 0 ? CUDART_INF : *(volatile double*)(vdist() + s);
-    }
+    __device__ __forceinline__ double dist_at(int s) const { return s < 0 ? CUDART_INF : *(volatile double*)(vdist() + s); }
 
     __device__ __forceinline__ void eval() {
         __syncwarp();
-        if (nev) eval_tests<R>(J, Y, b, e, sm, nev, lane);
+        if (nev) eval_tests<R, PL, TEAM>(J, Y, b, e, sm, nev, lane);
         __syncwarp();
         nev = 0;
     }
 
-    // queue the particles of face bucket `key` for the lanes that have one; put(entry) writes
-    // the window part of an entry
+    // queue the particles of face bucket `key` for the lanes that have one; put(entry, particle)
+    // writes an entry
     template <class Put>
     __device__ __forceinline__ void tests(bool has, int key, Put put) {
         int st = 0, cnt = 0;
@@ -270,90 +346,132 @@ struct Group {
         for (int r = 0; __any_sync(CSS_FULL, r < cnt); ++r) {
             int j = src;
             if (r < cnt) j = J.fitems[st + r];
-            const unsigned mk = __ballot_sync(CSS_FULL, j != src);
-            const int c = __popc(mk);
-            if (nev + c > EV) eval();
-            if (j != src) {
+            unsigned mk = __ballot_sync(CSS_FULL, j != src);
+            while (mk) {   // as many as there is room for
                 const int k = nev + __popc(mk & css::lanemask_lt());
-                at<int>(e, Y.e_j)[k] = j;
-                put(k);
+                const bool now = j != src && (mk >> lane & 1u) && k < EV;
+                if (now) put(k, j);
+                const unsigned done = __ballot_sync(CSS_FULL, now);
+                nev += __popc(done);
+                mk &= ~done;
+                if (nev == EV) eval();
             }
-            nev += c;
         }
     }
+    __device__ __forceinline__ void put_test(int k, double2 s, V2<R> rot, V2<R> d0, V2<R> d1, int he, int vs, int j) {
+        at<double2>(e, Y.e[0])[k] = s;
+        at<V2<R>>(e, Y.e[1])[k] = rot;
+        at<V2<R>>(e, Y.e[2])[k] = d0;
+        at<V2<R>>(e, Y.e[3])[k] = d1;
+        at<int4>(e, Y.e[4])[k] = make_int4(he, vs, j, 0);
+    }
+    // every particle of the face is seen: a cone of no directions holds all
+    __device__ __forceinline__ void put_open_test(int k, double2 s, V2<R> rot, int he, int vs, int j) {
+        const V2<R> none = vec2((R)0, (R)0);
+        put_test(k, s, rot, none, none, he, vs, j);
+    }
 
-    // append windows to the ring (lanes with has); `head` is where the ring's waiting part starts
-    struct Win {
-        double sx, sy;
-        R ra, rb, d0x, d0y, d1x, d1y;
-        float b0, b1, key;
-        int he, vs;
-    };
-    __device__ __forceinline__ void push(bool has, const Win& w, int head) {
+    // The interval of a ring entry: 16-bit fractions of the edge, rounded outward (0 and 1 are exact).
+    static __device__ __forceinline__ int pack_interval(float b0, float b1, float L) {
+        const float q = __fdividef(65535.0f, L);
+        const int i0 = max(0, (int)floorf(b0 * q * 0.999999f - 0.01f));
+        const int i1 = b1 >= L ? 65535 : min(65535, (int)ceilf(b1 * q * 1.000001f + 0.01f));
+        return i0 | i1 << 16;
+    }
+    static __device__ __forceinline__ void unpack_interval(unsigned p, float L, float& b0, float& b1) {
+        const unsigned i0 = p & 0xffffu, i1 = p >> 16;
+        b0 = (float)i0 * (L * (1.0f / 65535.0f));
+        b1 = i1 == 65535u ? L : (float)i1 * (L * (1.0f / 65535.0f));
+    }
+
+    __device__ __forceinline__ void store(unsigned char* to, const int* o, int k, const Win<R>& w, int b01) {
+        at<double2>(to, o[0])[k] = w.s;
+        at<V2<R>>(to, o[1])[k] = w.rot;
+        at<V2<R>>(to, o[2])[k] = w.d0;
+        at<V2<R>>(to, o[3])[k] = w.d1;
+        at<int4>(to, o[4])[k] = make_int4(w.he, w.vs, __float_as_int(w.key), b01);
+        at<typename Index<PL>::pair>(to, o[5])[k] = Index<PL>::make(w.su, w.sv);
+    }
+    // append windows (lanes with has): to the ring up to position `lim`, then to the spill area
+    __device__ __forceinline__ void push(bool has, const Win<R>& w, float L, int lim) {
         const unsigned mk = __ballot_sync(CSS_FULL, has);
         if (!mk) return;
+        const int n = __popc(mk);
         int base = 0;
         if constexpr (TEAM) {
-            if (lane == 0) base = atomicAdd(&sm.tail, __popc(mk));
+            if (lane == 0) base = atomicAdd(&sm.tail, n);
             base = __shfl_sync(CSS_FULL, base, 0);
         } else {
             base = sm.tail;
             __syncwarp();
-            if (lane == 0) sm.tail = base + __popc(mk);
-            __syncwarp();
+            if (lane == 0) sm.tail = min(base + n, max(lim, base));
         }
-        const int pos = base + __popc(mk & css::lanemask_lt());
-        if (has) {
-            if (pos - head >= (1 << Y.ring_log)) atomicOr(&sm.err, css::ST_WIN_OVERFLOW);
-            else {
-                const int s = pos & ((1 << Y.ring_log) - 1);
-                at<double>(b, Y.sx)[s] = w.sx;
-                at<double>(b, Y.sy)[s] = w.sy;
-                at<R>(b, Y.ra)[s] = w.ra;
-                at<R>(b, Y.rb)[s] = w.rb;
-                at<R>(b, Y.d0x)[s] = w.d0x;
-                at<R>(b, Y.d0y)[s] = w.d0y;
-                at<R>(b, Y.d1x)[s] = w.d1x;
-                at<R>(b, Y.d1y)[s] = w.d1y;
-                at<float>(b, Y.b0)[s] = w.b0;
-                at<float>(b, Y.b1)[s] = w.b1;
-                at<float>(b, Y.key)[s] = w.key;
-                at<int>(b, Y.he)[s] = w.he;
-                at<int>(b, Y.vs)[s] = w.vs;
+        const int rank = __popc(mk & css::lanemask_lt());
+        const int b01 = pack_interval(w.b0, w.b1, L);
+        if (has && base + rank < lim) store(h, Y.r, (base + rank) & Y.r_mask, w, b01);
+        if (base + n > lim) {
+            const int in = max(0, lim - base);   // those that went to the ring
+            int sb = 0;
+            if constexpr (TEAM) {
+                if (lane == 0) sb = atomicAdd(&sm.stail, n - in);
+                sb = __shfl_sync(CSS_FULL, sb, 0);
+            } else {
+                sb = sm.stail;
+                __syncwarp();
+                if (lane == 0) sm.stail = sb + n - in;
+            }
+            const int p = sb + rank - in;
+            if (has && rank >= in) {
+                if (p - sm.shead >= Y.s_cap) atomicOr(&sm.err, css::ST_WIN_OVERFLOW);
+                else store(x, Y.s, p & (Y.s_cap - 1), w, b01);
             }
         }
+        __syncwarp();
     }
 
-    // cut [b0, b1] of an edge of length L by its end vertices' distances du, dv; false if nothing is left
-    __device__ __forceinline__ bool cut(float sx, float sy, double sig, double du, double dv, float L, float& b0,
-                                        float& b1) const {
-        const float sy2 = sy * sy;
-        const float tx = L - sx, eps = 2.4e-7f * (fabsf(sx) + L);
-        if (du < 1e300) b0 = fmaxf(b0, cut_at(sx, sx * sx + sy2, (float)(du - sig), L, eps));
-        if (dv < 1e300) b1 = fminf(b1, L - cut_at(tx, tx * tx + sy2, (float)(dv - sig), L, eps));
+    // a vertex distance less sigma
+    __device__ __forceinline__ float rel(int slot, double sig) const {
+        return slot < 0 ? 3e38f : f32(*(volatile double*)(vdist() + slot) - sig);
+    }
+    // cut [b0, b1] of an edge of length L by its end vertices' distances (less sigma) au, av; false if
+    // nothing is left
+    __device__ __forceinline__ bool cut(float sx, float sy, float au, float av, float L, float& b0, float& b1) const {
+        const float sy2 = sy * sy, tx = L - sx, eps = 2.4e-7f * (fabsf(sx) + L);
+        b0 = fmaxf(b0, cut_at(sx, sx * sx + sy2, au, L, eps));
+        b1 = fminf(b1, L - cut_at(tx, tx * tx + sy2, av, L, eps));
         return b1 > b0;
     }
     // a lower bound on the lengths the window carries
     __device__ __forceinline__ float key_of(float sx, float sy, float sig, float b0, float b1) const {
         const float x = fminf(fmaxf(sx, b0), b1) - sx;
-        return (sig + sqrtf(x * x + sy * sy)) * (1.0f - 2e-6f) - 2.4e-7f * (fabsf(sx) + b1);
+        return (sig + root(x * x + sy * sy)) * (1.0f - 3e-6f) - 4e-7f * (fabsf(sx) + b1);
     }
 
     // a vertex that got a smaller distance: its path's direction at the source and its last leg's
-    // direction back; queued for starting windows if it does that and is not queued yet
-    __device__ __forceinline__ void improved(int slot, double d, R tx, R ty, float back) {
-        vtan()[2 * slot] = tx;
-        vtan()[2 * slot + 1] = ty;
-        const unsigned f = vflag()[slot];
-        vflag()[slot] = (geo::pack_back(back) << 16) | 1u;
-        const unsigned dl = __float_as_uint(__double2float_rd(d));
-        atomicMin(&sm.emin, dl);
-        if (!(f & 1u)) {
+    // direction back; queued for starting windows if it is not queued yet
+    // (angle `back` counter-clockwise from the first edge of corner hc; NaN where it is not known)
+    __device__ __forceinline__ void improved(int slot, double d, V2<R> t, int hc, float back) {
+        int i = vinfo()[slot];
+        bool queued = false;
+        if (i == (int)Index<PL>::none) {
+            i = atomicAdd(&sm.ni, 1);
+            if (i >= Y.i_cap) {
+                atomicOr(&sm.err, css::ST_HASH_OVERFLOW);
+                return;
+            }
+            vinfo()[slot] = (Idx)i;
+        } else queued = ihc()[i] & QUEUED;
+        itan()[i] = t;
+        iback()[i] = hc < 0 ? __int_as_float(0x7fffffff) : back;
+        ihc()[i] = (hc < 0 ? 0u : (unsigned)hc) | QUEUED;
+        atomicMin(&sm.emin, __float_as_uint(f32(d)));
+        if (!queued) {   // a path record is in one of the lists at most once
             const int p = atomicAdd(&sm.nem[sm.cur], 1);
-            if (p < Y.em_cap) at<int>(b, Y.emit)[sm.cur * Y.em_cap + p] = slot;
+            if (p < Y.i_cap) waiting(sm.cur)[p] = (Idx)slot;
             else atomicOr(&sm.err, css::ST_HASH_OVERFLOW);
         }
     }
+    __device__ __forceinline__ V2<R> tangent_of(int slot) const { return itan()[vinfo()[slot]]; }
 
     // slot of a vertex, entered with an infinite distance if it is new (distances are reset
     // when the source starts)
@@ -366,24 +484,11 @@ struct Group {
 
     __device__ __forceinline__ void seed(int f0, double b1, double b2);
     __device__ __forceinline__ void seed_at_vertex(int hc);
-    __device__ __forceinline__ void emit(int ne, int head, float kmin);
+    __device__ __forceinline__ void emit(int ne, int lim, float kmin);
     __device__ __forceinline__ void wave(int head, int n);
-    __device__ __forceinline__ int run(int item, int32_t* defer_list, int* defer_count, int* status,
-                                       unsigned long long* counters);
+    __device__ __forceinline__ void run(int item, int32_t* defer_list, int* defer_count, int* status,
+                                        unsigned long long* counters);
 };
-
-// out-of-line entries of the rarely run parts; the group goes by value so that the caller's copy stays
-// in registers, its count of queued tests comes back
-template <class R, int PL, bool TEAM>
-__device__ __noinline__ int call_seed_at_vertex(Group<R, PL, TEAM> g, int hc) {
-    g.seed_at_vertex(hc);
-    return g.nev;
-}
-template <class R, int PL, bool TEAM>
-__device__ __noinline__ int call_emit(Group<R, PL, TEAM> g, int ne, int head, float kmin) {
-    g.emit(ne, head, kmin);
-    return g.nev;
-}
 
 // Start a source (warp 0): tests for its own face, distances of its corners, one window for
 // each edge of its face.
@@ -391,11 +496,11 @@ template <class R, int PL, bool TEAM>
 __device__ __forceinline__ void Group<R, PL, TEAM>::seed(int f0, double b1, double b2) {
     const DMesh& m = J.m;
     const bool c3 = lane < 3;
-    const int h = 3 * f0 + (c3 ? lane : 0);
-    const HeRec r = m.he[h];
+    const int hh = 3 * f0 + (c3 ? lane : 0);
+    const HeRec r = m.he[hh];
     // the source from the corner's own weights (no cancellation next to a corner): (hx, hy) in the
     // frame of half-edge h, lx from its end; (ex, ey) the frame's x axis in the face's layout
-    const int k0 = h - 3 * f0;
+    const int k0 = hh - 3 * f0;
     const double wt[3] = {1.0 - b1 - b2, b1, b2};
     const double wa = k0 == 0 ? wt[0] : (k0 == 1 ? wt[1] : wt[2]), wb = k0 == 0 ? wt[1] : (k0 == 1 ? wt[2] : wt[0]);
     const double wc = k0 == 0 ? wt[2] : (k0 == 1 ? wt[0] : wt[1]);
@@ -405,47 +510,38 @@ __device__ __forceinline__ void Group<R, PL, TEAM>::seed(int f0, double b1, doub
     css::face_corner(m, f0, k0 + 1, bx, by);
     const double ex = (bx - ax) / r.L, ey = (by - ay) / r.L;
     const double vx = hy * ey - hx * ex, vy = -hy * ex - hx * ey;   // from the source to the corner, in the layout
-    tests(lane == 0, m.frank ? m.frank[f0] : f0, [&](int k) {
-        at<int>(e, Y.e_he)[k] = h;
-        at<int>(e, Y.e_vs)[k] = NONE;
-        at<double>(e, Y.e_sx)[k] = hx;
-        at<double>(e, Y.e_sy)[k] = hy;
-        at<R>(e, Y.e_ra)[k] = (R)1;   // half-edge 0's frame is the layout's
-        at<R>(e, Y.e_rb)[k] = (R)0;
-        at<R>(e, Y.e_d0x)[k] = at<R>(e, Y.e_d0y)[k] = at<R>(e, Y.e_d1x)[k] = at<R>(e, Y.e_d1y)[k] = (R)0;
+    tests(lane == 0, m.frank ? m.frank[f0] : f0, [&](int k, int j) {   // half-edge 0's frame is the layout's
+        put_open_test(k, make_double2(hx, hy), vec2((R)1, (R)0), hh, NONE, j);
     });
     // a source on a corner (to the rounding of its position) has no direction to it: its windows start at the vertex, all around
     const double vd = sqrt(hx * hx + hy * hy);
     const unsigned on = __ballot_sync(CSS_FULL, c3 && vd <= 1e-15 * r.L);
-    if (c3 && vd < J.rc && (on == 0 || (on >> lane & 1u))) {
-        const int s = vertex(m.fv[h]);
-        if (s >= 0) {
-            vdist()[s] = vd;
-            if (!on && (m.htop[h].x & css::EMITS))
-                improved(s, vd, (R)(vx / vd), (R)(vy / vd), geo::back_angle(m, h, ex, ey, -vx, -vy, m.lay[3 * f0]));
-        }
+    const int slot = c3 ? vertex(m.fv[hh]) : NONE;
+    if (slot >= 0 && vd < J.rc && (on == 0 || (on >> lane & 1u))) {
+        vdist()[slot] = vd;
+        if (!on && (m.htop[hh].x & css::EMITS))
+            improved(slot, vd, vec2((R)(vx / vd), (R)(vy / vd)), vd > 1e-6 * r.L ? hh : NONE, atan2f((float)hy, (float)hx));
     }
+    const int next = __shfl_sync(CSS_FULL, slot, lane == 2 ? 0 : lane + 1);
     __syncwarp();
     if (on) {
-        nev = call_seed_at_vertex<R, PL, TEAM>(*this, 3 * f0 + __ffs(on) - 1);
+        seed_at_vertex(3 * f0 + __ffs(on) - 1);
         return;
     }
-    const int tw = m.twin[h];
-    Win w;
+    const int tw = m.twin[hh];
+    Win<R> w;
     w.he = tw;
     w.vs = NONE;
-    w.sx = lx;   // the twin runs from the edge's end to its start
-    w.sy = -hy;
-    w.ra = (R)-ex;
-    w.rb = (R)ey;
-    w.d0x = (R)(lx * ex + hy * ey);
-    w.d0y = (R)(lx * ey - hy * ex);
-    w.d1x = (R)vx;
-    w.d1y = (R)vy;
+    w.s = make_double2(lx, -hy);   // the twin runs from the edge's end to its start
+    w.rot = vec2((R)-ex, (R)ey);
+    w.d0 = vec2((R)(lx * ex + hy * ey), (R)(lx * ey - hy * ex));
+    w.d1 = vec2((R)vx, (R)vy);
     w.b0 = 0.0f;
     w.b1 = (float)r.L;
-    w.key = key_of((float)w.sx, (float)w.sy, 0.0f, w.b0, w.b1);
-    push(c3 && tw >= 0 && w.key < J.rc, w, 0);
+    w.key = key_of((float)lx, (float)-hy, 0.0f, w.b0, w.b1);
+    w.su = next;
+    w.sv = slot;
+    push(c3 && slot >= 0 && next >= 0 && tw >= 0 && w.key < rcf, w, w.b1, Y.r_mask + 1);
 }
 
 // A source on corner hc's vertex: one window opposite each corner of the vertex's ring, tests for
@@ -467,72 +563,65 @@ __device__ __forceinline__ void Group<R, PL, TEAM>::seed_at_vertex(int hc) {
     int left = deg;
 #pragma unroll 1
     for (int dir = 0; dir < 2; ++dir) {
-        int h = hc;
+        int g = hc;
         double phi = phi0;   // direction of corner h's first edge in the source face's layout
         for (int q = 0; q < (dir == 0 ? half : deg) && left > 0; ++q) {
             if (q > 0 || dir == 1) {
                 if (dir == 0) {   // the next corner, across this corner's last edge
-                    const int f = h / 3, k = h - 3 * f;
-                    const HeRec& a = m.he[h];
+                    const int f = g / 3, k = g - 3 * f;
+                    const HeRec& a = m.he[g];
                     phi += atan2(a.cy, a.cx);
-                    h = m.twin[3 * f + (k == 0 ? 2 : k - 1)];
-                    if (h < 0) break;
+                    g = m.twin[3 * f + (k == 0 ? 2 : k - 1)];
+                    if (g < 0) break;
                 } else {          // the corner across this corner's first edge
-                    const int o = m.twin[h];
+                    const int o = m.twin[g];
                     if (o < 0) break;
-                    const int g = o / 3, kg = o - 3 * g;
-                    h = 3 * g + (kg == 2 ? 0 : kg + 1);
-                    const HeRec& a = m.he[h];
+                    const int fo = o / 3, kg = o - 3 * fo;
+                    g = 3 * fo + (kg == 2 ? 0 : kg + 1);
+                    const HeRec& a = m.he[g];
                     phi -= atan2(a.cy, a.cx);
                 }
-                if (h == hc) break;
+                if (g == hc) break;
             }
             --left;
-            const int fh = h / 3, kh = h - 3 * fh;
-            const HeRec r = m.he[h];
+            const int fh = g / 3, kh = g - 3 * fh;
+            const HeRec r = m.he[g];
             const double co = cos(phi), si = sin(phi);
-            tests(lane == 0 && h != hc, m.frank ? m.frank[fh] : fh, [&](int t) {
-                at<int>(e, Y.e_he)[t] = h;
-                at<int>(e, Y.e_vs)[t] = NONE;
-                at<double>(e, Y.e_sx)[t] = at<double>(e, Y.e_sy)[t] = 0.0;
-                at<R>(e, Y.e_ra)[t] = (R)co;
-                at<R>(e, Y.e_rb)[t] = (R)-si;
-                at<R>(e, Y.e_d0x)[t] = at<R>(e, Y.e_d0y)[t] = at<R>(e, Y.e_d1x)[t] = at<R>(e, Y.e_d1y)[t] = (R)0;
+            tests(lane == 0 && g != hc, m.frank ? m.frank[fh] : fh, [&](int t, int j) {
+                put_open_test(t, make_double2(0.0, 0.0), vec2((R)co, (R)-si), g, NONE, j);
             });
             const double ang = atan2(r.cy, r.cx), lc = sqrt(r.cx * r.cx + r.cy * r.cy);
+            int slot = NONE;
             if (lane < 2) {   // the two other corners of the face, along its edges from the vertex
                 const int hn = lane == 0 ? 3 * fh + (kh == 2 ? 0 : kh + 1) : 3 * fh + (kh == 0 ? 2 : kh - 1);
                 const double d = lane == 0 ? r.L : lc, a = lane == 0 ? phi : phi + ang;
-                if (d < J.rc) {
-                    const int s = vertex(m.fv[hn]);
-                    if (s >= 0) {
-                        const unsigned long long bits = (unsigned long long)__double_as_longlong(d);
-                        const unsigned long long old = atomicMin((unsigned long long*)(vdist() + s), bits);
-                        if (old > bits && (m.htop[hn].x & css::EMITS))
-                            improved(s, d, (R)cos(a), (R)sin(a), __int_as_float(0x7fffffff));
-                    }
+                slot = vertex(m.fv[hn]);
+                if (slot >= 0 && d < J.rc) {
+                    const unsigned long long bits = (unsigned long long)__double_as_longlong(d);
+                    const unsigned long long old = atomicMin((unsigned long long*)(vdist() + slot), bits);
+                    if (old > bits && (m.htop[hn].x & css::EMITS))
+                        improved(slot, d, vec2((R)cos(a), (R)sin(a)), NONE, 0.0f);
                 }
             }
+            const int s1 = __shfl_sync(CSS_FULL, slot, 0), s2 = __shfl_sync(CSS_FULL, slot, 1);
             __syncwarp();
             const int hop = 3 * fh + (kh == 2 ? 0 : kh + 1);
-            Win w;
+            Win<R> w;
             w.he = m.twin[hop];
             w.vs = NONE;
             const HeRec o = m.he[hop];
-            w.sx = o.L - o.cx;
-            w.sy = -o.cy;
+            w.s = make_double2(o.L - o.cx, -o.cy);
             // the twin's x axis runs from the face's far corner c to the first edge's end
             const double tx = (r.L - r.cx) / o.L, ty = -r.cy / o.L;
-            w.ra = (R)(tx * co - ty * si);
-            w.rb = (R)-(tx * si + ty * co);
-            w.d0x = (R)(r.cx * co - r.cy * si);
-            w.d0y = (R)(r.cx * si + r.cy * co);
-            w.d1x = (R)(r.L * co);
-            w.d1y = (R)(r.L * si);
+            w.rot = vec2((R)(tx * co - ty * si), (R)-(tx * si + ty * co));
+            w.d0 = vec2((R)(r.cx * co - r.cy * si), (R)(r.cx * si + r.cy * co));
+            w.d1 = vec2((R)(r.L * co), (R)(r.L * si));
             w.b0 = 0.0f;
             w.b1 = (float)o.L;
-            w.key = key_of((float)w.sx, (float)w.sy, 0.0f, w.b0, w.b1);
-            push(lane == 0 && w.he >= 0 && w.key < J.rc, w, 0);
+            w.key = key_of((float)w.s.x, (float)w.s.y, 0.0f, w.b0, w.b1);
+            w.su = s2;
+            w.sv = s1;
+            push(lane == 0 && s1 >= 0 && s2 >= 0 && w.he >= 0 && w.key < rcf, w, w.b1, Y.r_mask + 1);
             __syncwarp();
         }
     }
@@ -547,7 +636,7 @@ __device__ __forceinline__ void Group<R, PL, TEAM>::seed_at_vertex(int hc) {
 // rounding of b and the corner angles.  Vertices without a known b, boundary and non-manifold
 // ones start windows over their whole ring.
 template <class R, int PL, bool TEAM>
-__device__ __forceinline__ void Group<R, PL, TEAM>::emit(int ne, int head, float kmin) {
+__device__ __forceinline__ void Group<R, PL, TEAM>::emit(int ne, int lim, float kmin) {
     const DMesh& m = J.m;
     const int from = sm.cur, to = 1 - from;
     bar();
@@ -563,25 +652,26 @@ __device__ __forceinline__ void Group<R, PL, TEAM>::emit(int ne, int head, float
         bool go = false;
         double dv = 0.0;
         if (it < ne) {
-            vs = at<int>(b, Y.emit)[from * Y.em_cap + it];
+            vs = waiting(from)[it];
             dv = vdist()[vs];
             go = dv <= (double)kmin;
             if (!go) {
-                at<int>(b, Y.emit)[to * Y.em_cap + atomicAdd(&sm.nem[to], 1)] = vs;
+                waiting(to)[atomicAdd(&sm.nem[to], 1)] = (Idx)vs;
                 atomicMin(&sm.emin, __float_as_uint(__double2float_rd(dv)));
             }
         }
         int rs = 0, len = 0;
         float lo = -INFINITY, hi = INFINITY, th = 0.0f;
         if (go) {
-            const unsigned fl = vflag()[vs];
-            vflag()[vs] = fl & ~1u;
+            const int i = vinfo()[vs];
+            const unsigned hb = ihc()[i] & ~QUEUED;
+            const float bk = iback()[i] + m.cang[hb].x;   // NaN where either is not known
+            ihc()[i] = hb;
             const int vid = vkey()[vs];
             rs = m.ring_start[vid];
             len = m.ring_start[vid + 1] - rs;
-            if ((fl >> 16) != 0xffffu) {
+            if (bk == bk) {
                 th = (float)m.theta[vid];
-                const float bk = geo::unpack_back(fl >> 16);
                 lo = bk + 3.14159265f - geo::SHADOW_TOL;
                 lo -= th * floorf(lo / th);
                 hi = lo + (th - 6.28318531f + 2.0f * geo::SHADOW_TOL);
@@ -622,27 +712,21 @@ __device__ __forceinline__ void Group<R, PL, TEAM>::emit(int ne, int head, float
                     }
                 }
             }
-            tests(hit, hit ? m.htop[hc].w : 0, [&](int k) {
-                at<int>(e, Y.e_he)[k] = hc;
-                at<int>(e, Y.e_vs)[k] = o_vs | FROM_VERTEX;
-                at<double>(e, Y.e_sx)[k] = at<double>(e, Y.e_sy)[k] = 0.0;
-                at<R>(e, Y.e_ra)[k] = (R)1;
-                at<R>(e, Y.e_rb)[k] = (R)0;
-                at<R>(e, Y.e_d0x)[k] = at<R>(e, Y.e_d0y)[k] = at<R>(e, Y.e_d1x)[k] = at<R>(e, Y.e_d1y)[k] = (R)0;
+            tests(hit, hit ? m.htop[hc].w : 0, [&](int k, int j) {
+                put_open_test(k, make_double2(0.0, 0.0), vec2((R)1, (R)0), hc, o_vs | FROM_VERTEX, j);
             });
-            Win w;
+            Win<R> w;
             bool ok = false;
+            float L = 0.0f;
             if (hit) {
                 const int k = hc - 3 * f, hop = 3 * f + (k == 2 ? 0 : k + 1);
                 w.he = m.twin[hop];
                 if (w.he >= 0) {
                     const HeRec r = m.he[hop];
-                    const float L = (float)r.L;
+                    L = (float)r.L;
                     w.vs = o_vs | FIRST;
-                    w.sx = r.L - r.cx;
-                    w.sy = -r.cy;
-                    w.ra = (R)1;
-                    w.rb = (R)0;
+                    w.s = make_double2(r.L - r.cx, -r.cy);
+                    w.rot = vec2((R)1, (R)0);
                     w.b0 = 0.0f;
                     w.b1 = L;
                     if (o_th != 0.0f) {
@@ -650,28 +734,28 @@ __device__ __forceinline__ void Group<R, PL, TEAM>::emit(int ne, int head, float
                         const css::HeRec32 q = m.he32[hc];
                         const float ex = q.cx - q.L, ey = q.cy;
                         if (c0 > 1e-5f) {
-                            const float s = sinf(c0), c = cosf(c0);
+                            const float s = __sinf(c0), c = __cosf(c0);
                             const float x = fminf(fmaxf(q.L * s / (ey * c - ex * s), 0.0f), 1.0f);
                             w.b1 = fminf(L, L * (1.0f - x) + 1e-5f * L);
                         }
                         if (c1 < wid_c - 1e-5f) {
-                            const float s = sinf(c1), c = cosf(c1);
+                            const float s = __sinf(c1), c = __cosf(c1);
                             const float x = fminf(fmaxf(q.L * s / (ey * c - ex * s), 0.0f), 1.0f);
                             w.b0 = fmaxf(0.0f, L * (1.0f - x) - 1e-5f * L);
                         }
                     }
-                    w.d0x = (R)((double)w.b0 - w.sx);
-                    w.d0y = (R)-w.sy;
-                    w.d1x = (R)((w.b1 == L ? r.L : (double)w.b1) - w.sx);
-                    w.d1y = (R)-w.sy;
+                    w.d0 = vec2((R)((double)w.b0 - w.s.x), (R)-w.s.y);
+                    w.d1 = vec2((R)((w.b1 == L ? r.L : (double)w.b1) - w.s.x), (R)-w.s.y);
                     const int4 tp = m.htop[w.he];
-                    ok = cut((float)w.sx, (float)w.sy, o_dv, dist_of(tp.x & css::VMASK), dist_of(tp.y & css::VMASK), L,
-                             w.b0, w.b1);
-                    w.key = key_of((float)w.sx, (float)w.sy, (float)o_dv, w.b0, w.b1);
-                    ok = ok && w.key < J.rc;
+                    w.su = vertex(tp.x & css::VMASK);
+                    w.sv = vertex(tp.y & css::VMASK);
+                    const float fx = f32(w.s.x), fy = f32(w.s.y);
+                    ok = cut(fx, fy, rel(w.su, o_dv), rel(w.sv, o_dv), L, w.b0, w.b1) && w.su >= 0 && w.sv >= 0;
+                    w.key = key_of(fx, fy, f32(o_dv), w.b0, w.b1);
+                    ok = ok && w.key < rcf;
                 }
             }
-            push(ok, w, head);
+            push(ok, w, L, lim);
         }
     }
 }
@@ -681,201 +765,273 @@ template <class R, int PL, bool TEAM>
 __device__ __forceinline__ void Group<R, PL, TEAM>::wave(int head, int n) {
     const DMesh& m = J.m;
     const bool on = tid < n;
-    const int s = (head + tid) & ((1 << Y.ring_log) - 1);
-    const int he = on ? at<int>(b, Y.he)[s] : 0;
+    const int s = (head + tid) & Y.r_mask;
+    const int4 w4 = on ? at<int4>(h, Y.r[4])[s] : make_int4(0, NONE, 0, 0);
+    const int he = w4.x;
+    const bool first = w4.y >= 0 && (w4.y & FIRST);
+    const int vs = w4.y < 0 ? NONE : w4.y & ~FIRST;
     const int4 tp = m.htop[he];
-    tests(on, tp.w, [&](int k) {
-        at<int>(e, Y.e_he)[k] = he;
-        const int v = at<int>(b, Y.vs)[s];
-        at<int>(e, Y.e_vs)[k] = v < 0 ? v : v & ~FIRST;
-        at<double>(e, Y.e_sx)[k] = at<double>(b, Y.sx)[s];
-        at<double>(e, Y.e_sy)[k] = at<double>(b, Y.sy)[s];
-        at<R>(e, Y.e_ra)[k] = at<R>(b, Y.ra)[s];
-        at<R>(e, Y.e_rb)[k] = at<R>(b, Y.rb)[s];
-        at<R>(e, Y.e_d0x)[k] = at<R>(b, Y.d0x)[s];
-        at<R>(e, Y.e_d0y)[k] = at<R>(b, Y.d0y)[s];
-        at<R>(e, Y.e_d1x)[k] = at<R>(b, Y.d1x)[s];
-        at<R>(e, Y.e_d1y)[k] = at<R>(b, Y.d1y)[s];
-    });
     const HeRec r = m.he[he];
     const css::HeRec32 q = m.he32[he];
-    const double sx = at<double>(b, Y.sx)[s], sy = at<double>(b, Y.sy)[s];
-    const R ra = at<R>(b, Y.ra)[s], rb = at<R>(b, Y.rb)[s];
-    const R d0x = at<R>(b, Y.d0x)[s], d0y = at<R>(b, Y.d0y)[s], d1x = at<R>(b, Y.d1x)[s], d1y = at<R>(b, Y.d1y)[s];
-    float b0 = at<float>(b, Y.b0)[s], b1 = at<float>(b, Y.b1)[s];
-    int vs = at<int>(b, Y.vs)[s];
-    const bool first = on && vs >= 0 && (vs & FIRST);
-    if (vs >= 0) vs &= ~FIRST;
-    if (!on) vs = NONE;
-    bar();   // the ring's slots up to head + n are free from here on
-    const int head2 = head + n;
+    tests(on, tp.w, [&](int k, int j) {
+        put_test(k, at<double2>(h, Y.r[0])[s], at<V2<R>>(h, Y.r[1])[s], at<V2<R>>(h, Y.r[2])[s], at<V2<R>>(h, Y.r[3])[s],
+                 he, vs, j);
+    });
+    const double2 S = at<double2>(h, Y.r[0])[s];
+    const typename Index<PL>::pair ends = at<typename Index<PL>::pair>(h, Y.r[5])[s];
+    const int su = on ? (int)ends.x : NONE, sv = on ? (int)ends.y : NONE;
+    float b0, b1;
+    unpack_interval((unsigned)w4.w, q.L, b0, b1);
     const double sig = vs < 0 ? 0.0 : vdist()[vs];
-    const float fsx = (float)sx, fsy = (float)sy, fsig = (float)sig;
-    const int32_t vu = tp.x & css::VMASK, vv = tp.y & css::VMASK, vc = tp.z & css::VMASK;
-    const bool act = on && cut(fsx, fsy, sig, dist_of(vu), dist_of(vv), q.L, b0, b1) &&
-                     key_of(fsx, fsy, fsig, b0, b1) < J.rc;
-    // the far corner seen from s: gx, gy in this frame, px, py in the pseudo-source's
-    const double gx = r.cx - sx, gy = r.cy - sy;
-    const R fgx = (R)gx, fgy = (R)gy;
-    const R px = fgx * ra + fgy * rb, py = fgy * ra - fgx * rb;
-    const float em = 4e-6f * (fabsf(fsx) + fabsf(fsy) + q.L);   // bounds the rounding of FP32 crossings
-    const float xc = fsx - (q.cx - fsx) * __fdividef(fsy, q.cy - fsy);
-    const R tolg = Rim<R>::t * (R)(fabsf((float)fgx) + fabsf((float)fgy));
-    const R t0 = tolg * (fabs(d0x) + fabs(d0y)), t1 = tolg * (fabs(d1x) + fabs(d1y));
-    const R cr0 = d0x * py - d0y * px, cr1 = d1x * py - d1y * px;   // < 0: c lies right of the direction
-    const bool left = act && cr0 < -t0 && xc > b0 - em, right = act && cr1 > t1 && xc < b1 + em;
-    const bool cin = act && cr0 <= t0 && cr1 >= -t1 && xc >= b0 - em && xc <= b1 + em;
+    const float fsx = f32(S.x), fsy = f32(S.y), fsig = f32(sig);
+    const bool act = on && cut(fsx, fsy, rel(su, sig), rel(sv, sig), q.L, b0, b1) && key_of(fsx, fsy, fsig, b0, b1) < rcf;
+    // the far corner seen from s, in FP32 (fgx, fgy), and its side of the cone's rims
+    const float fgx = q.cx - fsx, fgy = q.cy - fsy, size = fabsf(fsx) + fabsf(fsy) + q.L;
+    const float em = 4e-6f * size;   // bounds the rounding of FP32 crossings
+    const float xc = fsx - fgx * __fdividef(fsy, fgy);
+    bool in0, in1, beyond0, beyond1;   // c on or right of the left rim, on or left of the right rim; strictly
+    {
+        const V2<R> rot = at<V2<R>>(h, Y.r[1])[s], d0 = at<V2<R>>(h, Y.r[2])[s], d1 = at<V2<R>>(h, Y.r[3])[s];
+        const float rx = f32(rot.x), ry = f32(rot.y), px = fgx * rx + fgy * ry, py = fgy * rx - fgx * ry;
+        const float ax = f32(d0.x), ay = f32(d0.y), bx = f32(d1.x), by = f32(d1.y);
+        const float cr0 = ax * py - ay * px, cr1 = bx * py - by * px;   // < 0: c lies right of the rim
+        const float t = (sizeof(R) == 4 ? Rim<float>::t : 8e-6f) * (fabsf(fgx) + fabsf(fgy) + (sizeof(R) == 4 ? 0.0f : size));
+        const float t0 = t * (fabsf(ax) + fabsf(ay)), t1 = t * (fabsf(bx) + fabsf(by));
+        in0 = cr0 <= t0;
+        beyond0 = cr0 < -t0;
+        in1 = cr1 >= -t1;
+        beyond1 = cr1 > t1;
+        if (sizeof(R) == 8 && on && ((in0 && !beyond0) || (in1 && !beyond1))) {   // too close to a rim for FP32
+            const double gx = r.cx - S.x, gy = r.cy - S.y;
+            const double ex = gx * rot.x + gy * rot.y, ey = gy * rot.x - gx * rot.y;
+            const double tg = Rim<double>::t * (fabs(gx) + fabs(gy));
+            const double e0 = tg * (fabs(d0.x) + fabs(d0.y)), e1 = tg * (fabs(d1.x) + fabs(d1.y));
+            const double c0 = d0.x * ey - d0.y * ex, c1 = d1.x * ey - d1.y * ex;
+            in0 = c0 <= e0;
+            beyond0 = c0 < -e0;
+            in1 = c1 >= -e1;
+            beyond1 = c1 > e1;
+        }
+    }
+    const bool left = act && beyond0 && xc > b0 - em && r.tl >= 0, right = act && beyond1 && xc < b1 + em && r.tr >= 0;
+    const bool cin = act && in0 && in1 && xc >= b0 - em && xc <= b1 + em;
     // distance candidates: the far corner, and the two ends of a window that just started
+    int sc = NONE;
     const int nq = (TEAM ? __syncthreads_or(first) : __any_sync(CSS_FULL, first)) ? 3 : 1;
 #pragma unroll 1
     for (int a = 0; a < nq; ++a) {
-        bool has = a == 0 ? cin : (first && act && (a == 1 ? b0 <= 0.0f : b1 >= q.L));
-        const double vx = a == 0 ? gx : (a == 1 ? -sx : r.L - sx), vy = a == 0 ? gy : -sy;
+        const bool has = a == 0 ? cin : (first && act && (a == 1 ? b0 <= 0.0f : b1 >= q.L));
+        const float fvx = a == 0 ? fgx : (a == 1 ? -fsx : q.L - fsx), fvy = a == 0 ? fgy : -fsy;
         const int vtop = a == 0 ? tp.z : (a == 1 ? tp.x : tp.y);
-        const float fd = fsig + sqrtf((float)vx * (float)vx + (float)vy * (float)vy);
-        int slot = NONE;
+        const float fd = fsig + root(fvx * fvx + fvy * fvy), fe = 1e-6f * (fd + size);   // its rounding
+        int slot = a == 1 ? su : sv;
+        if (a == 0) {
+            slot = left || right || cin ? vertex(vtop & css::VMASK) : NONE;
+            sc = slot;
+            bar();
+        }
         unsigned long long bits = 0, old = 0;
         double d = 0.0;
-        if (has && (double)fd * (1.0 - 1e-6) < J.rc) {
-            slot = vertex(vtop & css::VMASK);
-            if (slot >= 0 && (double)fd * (1.0 - 1e-6) < *(volatile double*)(vdist() + slot)) {
-                // the other vertices' distances only cut windows: an FP32 upper bound will do
-                d = (vtop & css::EMITS) ? sig + sqrt(vx * vx + vy * vy) : (double)(fd * (1.0f + 1e-6f));
-                bits = (unsigned long long)__double_as_longlong(d);
-                if (d < J.rc) old = atomicMin((unsigned long long*)(vdist() + slot), bits);
-            }
+        V2<R> t = vec2((R)0, (R)0);
+        if (has && slot >= 0 && fd - fe < rcf && fd - fe < f32(dist_at(slot)) * (1.0f + 3e-7f)) {
+            // the other vertices' distances only cut windows: an FP32 upper bound will do
+            if (vtop & css::EMITS) {
+                const double vx = a == 0 ? r.cx - S.x : (a == 1 ? -S.x : r.L - S.x), vy = a == 0 ? r.cy - S.y : -S.y;
+                double n, inv;
+                roots(vx * vx + vy * vy, n, inv);
+                d = sig + n;
+                if (vs < 0) {
+                    const V2<R> rot = at<V2<R>>(h, Y.r[1])[s];
+                    const R gx = (R)vx, gy = (R)vy, ri = (R)inv;
+                    t = vec2((gx * rot.x + gy * rot.y) * ri, (gy * rot.x - gx * rot.y) * ri);
+                }
+            } else d = f64(fd + fe);
+            bits = (unsigned long long)__double_as_longlong(d);
+            if (d < J.rc) old = atomicMin((unsigned long long*)(vdist() + slot), bits);
         }
         bar();
-        if (old > bits && (vtop & css::EMITS) &&
-            *(volatile unsigned long long*)(vdist() + slot) == bits) {
-            R tx, ty;
-            if (vs < 0) {
-                const R inv = (R)1 / (R)d;   // sigma is 0
-                tx = px * inv;
-                ty = py * inv;
-            } else {
-                tx = vtan()[2 * vs];
-                ty = vtan()[2 * vs + 1];
-            }
+        if (old > bits && (vtop & css::EMITS) && *(volatile unsigned long long*)(vdist() + slot) == bits) {
+            if (vs >= 0) t = tangent_of(vs);
             const int f = he / 3, k = he - 3 * f;
             const int hc = a == 0 ? 3 * f + (k == 0 ? 2 : k - 1) : (a == 1 ? he : m.twin[he]);
-            improved(slot, d, tx, ty,
-                     geo::back_angle(m, hc, a == 0 ? -r.cx : (a == 1 ? 1.0 : -1.0), a == 0 ? -r.cy : 0.0, -vx, -vy, r.L));
+            // the last leg back, from the corner's first edge: c -> u, u -> v, v -> u
+            const float ex = a == 0 ? -q.cx : (a == 1 ? 1.0f : -1.0f), ey = a == 0 ? -q.cy : 0.0f;
+            improved(slot, d, t, fvx * fvx + fvy * fvy > 1e-6f * size * size ? hc : NONE,
+                     atan2f(ey * fvx - ex * fvy, -ex * fvx - ey * fvy));
         }
         bar();
     }
-    // the children: side 0 the edge u -> c, side 1 the edge c -> v
-    const double du = dist_of(vu), dc = dist_of(vc), dv = dist_of(vv);
+    // The children, side 0 across the edge u -> c, side 1 across c -> v: one lane each, packed densely
+    // (a window has one child on average, at most two).  A child's lane reads its parent's
+    // window from the ring again; the parent's slots are free once the last round has read them.
+    // (the corner bounds a child's cone unless it lies beyond the rim on the child's side)
+    const unsigned lm = __ballot_sync(CSS_FULL, left), rm = __ballot_sync(CSS_FULL, right);
+    const int nleft = __popc(lm), total = nleft + __popc(rm);
+    unsigned char* task = e + Y.e_task;
+    if (left) task[__popc(lm & css::lanemask_lt())] = (unsigned char)(lane | (in1 ? 64 : 0));
+    if (right) task[nleft + __popc(rm & css::lanemask_lt())] = (unsigned char)(lane | 32 | (in0 ? 64 : 0));
+    __syncwarp();
 #pragma unroll 1
-    for (int a = 0; a < 2; ++a) {
-        Win w;
-        w.he = a == 0 ? r.tl : r.tr;
-        bool has = (a == 0 ? left : right) && w.he >= 0;
-        if (has) {
-            const double co = a == 0 ? r.cl : r.cr, si = a == 0 ? r.sl : r.sr;
-            const R fco = sizeof(R) == 4 ? (R)(a == 0 ? q.cl : q.cr) : (R)co, fsi = sizeof(R) == 4 ? (R)(a == 0 ? q.sl : q.sr) : (R)si;
-            const double ux = a == 0 ? sx : -gx, uy = a == 0 ? sy : -gy;   // s from the child edge's start
-            w.sx = ux * co + uy * si;
-            w.sy = uy * co - ux * si;
-            if (w.sy > 0.0) w.sy = 0.0;
-            w.ra = ra * fco + rb * fsi;
-            w.rb = rb * fco - ra * fsi;
-            // the corner bounds the child's cone unless it lies beyond the rim on that side
-            const bool n0 = a == 1 && cr0 <= t0, n1 = a == 0 && cr1 >= -t1;
-            w.d0x = n0 ? px : d0x;
-            w.d0y = n0 ? py : d0y;
-            w.d1x = n1 ? px : d1x;
-            w.d1y = n1 ? py : d1y;
+    for (int base = 0; base < total; base += 32) {
+        const bool is = base + lane < total;
+        const int code = is ? task[base + lane] : 0;
+        const int par = code & 31;
+        const float pb0 = __shfl_sync(CSS_FULL, b0, par), pb1 = __shfl_sync(CSS_FULL, b1, par);
+        const int psu = __shfl_sync(CSS_FULL, su, par), psv = __shfl_sync(CSS_FULL, sv, par);
+        const int psc = __shfl_sync(CSS_FULL, sc, par);
+        const int ps = (head + tid - lane + par) & Y.r_mask;
+        const int4 pw = at<int4>(h, Y.r[4])[ps];
+        const double2 PS = at<double2>(h, Y.r[0])[ps];
+        const V2<R> rot = at<V2<R>>(h, Y.r[1])[ps];
+        Win<R> w;
+        w.d0 = at<V2<R>>(h, Y.r[2])[ps];
+        w.d1 = at<V2<R>>(h, Y.r[3])[ps];
+        __syncwarp();
+        bool has = is;
+        float Lc = 1.0f;
+        if (is) {
+            const bool a = code & 32;
+            const HeRec pr = m.he[pw.x];
+            const css::HeRec32 pq = m.he32[pw.x];
+            w.he = a ? pr.tr : pr.tl;
+            w.vs = pw.y < 0 ? NONE : pw.y & ~FIRST;
+            const double psig = w.vs < 0 ? 0.0 : vdist()[w.vs];
+            const double cx = pr.cx - PS.x, cy = pr.cy - PS.y;
+            w.su = a ? psc : psu;
+            w.sv = a ? psv : psc;
+            if (code & 64) {
+                const R fx = (R)cx, fy = (R)cy;
+                const V2<R> pc = vec2(fx * rot.x + fy * rot.y, fy * rot.x - fx * rot.y);
+                if (a) w.d0 = pc;
+                else w.d1 = pc;
+            }
+            const double co = a ? pr.cr : pr.cl, si = a ? pr.sr : pr.sl;
+            const R fco = sizeof(R) == 4 ? (R)(a ? pq.cr : pq.cl) : (R)co, fsi = sizeof(R) == 4 ? (R)(a ? pq.sr : pq.sl) : (R)si;
+            const double ux = a ? -cx : PS.x, uy = a ? -cy : PS.y;   // s from the child edge's start
+            w.s = make_double2(ux * co + uy * si, uy * co - ux * si);
+            if (__double2hiint(w.s.y) >= 0) w.s.y = 0.0;   // rounding: s never lies above the edge
+            w.rot = vec2(rot.x * fco + rot.y * fsi, rot.y * fco - rot.x * fsi);
             // the interval: where the rays through b0 and b1 meet the child's edge, rounded outward
-            const float ax = a == 0 ? 0.0f : q.cx, ay = a == 0 ? 0.0f : q.cy;
-            const float ex = a == 0 ? q.cx : q.L - q.cx, ey = a == 0 ? q.cy : -q.cy;
-            const float Lc = sqrtf(ex * ex + ey * ey);
-            const float vx = fsx - ax, vy = fsy - ay;
-            const float x0 = b0 - fsx, x1 = b1 - fsx;   // ray directions (x, -sy)
-            const float m0 = -vx * fsy - vy * x0, e0 = -ex * fsy - ey * x0;
-            const float m1 = -vx * fsy - vy * x1, e1 = -ex * fsy - ey * x1;
+            const float sx = f32(PS.x), sy = f32(PS.y), sg = f32(psig);
+            const float pem = 4e-6f * (fabsf(sx) + fabsf(sy) + pq.L);
+            const float pxc = sx - (pq.cx - sx) * __fdividef(sy, pq.cy - sy);
+            const float ax = a ? pq.cx : 0.0f, ay = a ? pq.cy : 0.0f;
+            const float ex = a ? pq.L - pq.cx : pq.cx, ey = a ? -pq.cy : pq.cy;
+            Lc = root(ex * ex + ey * ey);
+            const float vx = sx - ax, vy = sy - ay;
+            const float x0 = pb0 - sx, x1 = pb1 - sx;   // ray directions (x, -sy)
+            const float m0 = -vx * sy - vy * x0, e0 = -ex * sy - ey * x0;
+            const float m1 = -vx * sy - vy * x1, e1 = -ex * sy - ey * x1;
             // rounding of a crossing: that of the coordinates (em), and that of the ray's direction, which
             // grows as s nears the point the ray goes through
-            const float emc = em + 4e-6f * Lc, emd = em * (Lc + q.L);
-            const float p0 = emc + __fdividef(emd, fmaxf(fabsf(x0), -fsy)), p1 = emc + __fdividef(emd, fmaxf(fabsf(x1), -fsy));
-            w.b0 = a == 1 && xc >= b0 ? 0.0f : fmaxf(0.0f, fminf(e0 != 0.0f ? __fdividef(m0, e0) : 0.0f, 1.0f) * Lc - p0);
-            w.b1 = a == 0 && xc <= b1 ? Lc : fminf(Lc, fmaxf(e1 != 0.0f ? __fdividef(m1, e1) : 0.0f, 0.0f) * Lc + p1);
-            const float cx = (float)w.sx, cy = (float)w.sy;
-            has = cut(cx, cy, sig, a == 0 ? du : dc, a == 0 ? dc : dv, Lc, w.b0, w.b1);
-            w.key = key_of(cx, cy, fsig, w.b0, w.b1);
-            has = has && w.key < J.rc;
-            w.vs = vs;
+            const float emc = pem + 4e-6f * Lc, emd = pem * (Lc + pq.L);
+            const float p0 = emc + __fdividef(emd, fmaxf(fabsf(x0), -sy)), p1 = emc + __fdividef(emd, fmaxf(fabsf(x1), -sy));
+            w.b0 = a && pxc >= pb0 ? 0.0f : fmaxf(0.0f, fminf(e0 != 0.0f ? __fdividef(m0, e0) : 0.0f, 1.0f) * Lc - p0);
+            w.b1 = !a && pxc <= pb1 ? Lc : fminf(Lc, fmaxf(e1 != 0.0f ? __fdividef(m1, e1) : 0.0f, 0.0f) * Lc + p1);
+            const float fx = f32(w.s.x), fy = f32(w.s.y);
+            has = cut(fx, fy, rel(w.su, psig), rel(w.sv, psig), Lc, w.b0, w.b1) && psc >= 0;
+            w.key = key_of(fx, fy, sg, w.b0, w.b1);
+            has = has && w.key < rcf;
         }
-        push(has, w, head2);
+        push(has, w, Lc, head + Y.r_mask + 1 + (!TEAM && base + 32 >= total ? n : 0));
     }
 }
 
 template <class R, int PL, bool TEAM>
-__device__ __forceinline__ int Group<R, PL, TEAM>::run(int item, int32_t* defer_list, int* defer_count, int* status,
-                                                       unsigned long long* counters) {
+__device__ __forceinline__ void Group<R, PL, TEAM>::run(int item, int32_t* defer_list, int* defer_count, int* status,
+                                                        unsigned long long* counters) {
     const DMesh& m = J.m;
     const int f0 = J.face[src];
     const double* bs = J.bary + 3 * (size_t)src;
     // empty tables; distances start at infinity
-    for (int k = tid; k < (1 << Y.vh_log); k += T) {
-        vkey()[k] = NONE;
-        vdist()[k] = CUDART_INF;
-        vflag()[k] = 0;
-    }
-    for (int k = tid; k < (1 << Y.th_log); k += T) {
-        tkey()[k] = NONE;
-        tdist()[k] = tvert()[k] = CUDART_INF;
+    {
+        const int4 none = make_int4(-1, -1, -1, -1), inf = make_int4(0, 0x7ff00000, 0, 0x7ff00000);
+        for (int k = tid; k < (1 << Y.vh_log) / 4; k += T) at<int4>(b, Y.vkey)[k] = none;
+        for (int k = tid; k < (1 << Y.vh_log) / 2; k += T) at<int4>(b, Y.vdist)[k] = inf;
+        for (int k = tid; k < (int)sizeof(Idx) * (1 << Y.vh_log) / 16; k += T) at<int4>(b, Y.vinfo)[k] = none;
+        for (int k = tid; k < (1 << Y.th_log) / 4; k += T) at<int4>(b, Y.tkey)[k] = none;
+        for (int k = tid; k < (1 << Y.th_log) / 2; k += T) {
+            at<int4>(b, Y.tdist)[k] = inf;
+            if (sizeof(R) == 4) at<int4>(b, Y.tvert)[k] = inf;
+        }
     }
     if (tid == 0) {
-        sm.head = sm.tail = sm.nem[0] = sm.nem[1] = sm.cur = sm.nv = sm.nt = sm.nlog = sm.err = 0;
+        sm.head = sm.tail = sm.shead = sm.stail = sm.nem[0] = sm.nem[1] = sm.cur = 0;
+        sm.nv = sm.ni = sm.nt = sm.nlog = sm.err = 0;
         sm.emin = 0x7f800000u;
     }
     bar();
     if (wid == 0) seed(f0, bs[1], bs[2]);
     unsigned nprop = 0;
-    int waves = 0;
+    int waves = 0, lim = Y.r_mask + 1;
     for (;;) {
         bar();
-        const int head = sm.head;
-        int tail = sm.tail;
-        const int ne = sm.nem[sm.cur];
-        int err = sm.err;
+        const int head = sm.head, ne = sm.nem[sm.cur], waits = sm.stail - sm.shead;
+        int tail = min(sm.tail, lim), err = sm.err;   // a team's claims may run past the ring's end
         if (++waves > Y.max_waves) err |= css::ST_ITER_LIMIT;
         bar();
-        if (err || (head == tail && ne == 0)) {
+        if (err || (head == tail && ne == 0 && waits == 0)) {
             if (tid == 0) sm.err = err;
             break;
         }
+        // spilled windows come back as the ring empties
+        const int back = waits > 0 && tail - head < T ? min(waits, Y.r_mask + 1 - (tail - head)) : 0;
+        if (back > 0) {
+            const int from = sm.shead;
+            for (int k = tid; k < back; k += T) {
+                const int i = (from + k) & (Y.s_cap - 1), o = (tail + k) & Y.r_mask;
+                at<double2>(h, Y.r[0])[o] = at<double2>(x, Y.s[0])[i];
+                at<V2<R>>(h, Y.r[1])[o] = at<V2<R>>(x, Y.s[1])[i];
+                at<V2<R>>(h, Y.r[2])[o] = at<V2<R>>(x, Y.s[2])[i];
+                at<V2<R>>(h, Y.r[3])[o] = at<V2<R>>(x, Y.s[3])[i];
+                at<int4>(h, Y.r[4])[o] = at<int4>(x, Y.s[4])[i];
+                at<typename Index<PL>::pair>(h, Y.r[5])[o] = at<typename Index<PL>::pair>(x, Y.s[5])[i];
+            }
+            tail += back;
+            bar();
+            if (tid == 0) sm.shead = from + back;
+        }
+        if (tid == 0) sm.tail = tail;
+        lim = head + Y.r_mask + 1;
+        bar();
         if (ne > 0) {
             float km = INFINITY;
-            tail = min(tail, head + (1 << Y.ring_log));
-            for (int k = head + tid; k < tail; k += T) km = fminf(km, at<float>(b, Y.key)[k & ((1 << Y.ring_log) - 1)]);
+            for (int k = head + tid; k < tail; k += T) km = fminf(km, __int_as_float(at<int4>(h, Y.r[4])[k & Y.r_mask].z));
+            for (int k = sm.shead + tid; k < sm.stail; k += T)
+                km = fminf(km, __int_as_float(at<int4>(x, Y.s[4])[k & (Y.s_cap - 1)].z));
             km = __uint_as_float(__reduce_min_sync(CSS_FULL, __float_as_uint(km)));
             if constexpr (TEAM) {
-                if (lane == 0) sm.km[wid] = km;
+                if (lane == 0) tm->km[wid] = km;
                 __syncthreads();
-                for (int w = 0; w < (T >> 5); ++w) km = fminf(km, sm.km[w]);
+                for (int w = 0; w < (T >> 5); ++w) km = fminf(km, tm->km[w]);
             }
             if (head == tail || __uint_as_float(sm.emin) <= km) {
-                nev = call_emit<R, PL, TEAM>(*this, ne, head, km);
+                emit(ne, lim, km);
                 bar();
-                tail = sm.tail;
+                tail = min(sm.tail, lim);
             }
         }
-        const int n = min(min(tail - head, 1 << Y.ring_log), T);   // a full ring dropped the rest (and reports it)
+        const int n = min(tail - head, T);
         wave(head, n);
         nprop += n;
-        if (tid == 0) sm.head = head + n;
+        if (!TEAM) lim += n;   // the popped slots were free for the last children
+        bar();
+        if (tid == 0) {
+            sm.head = head + n;
+            if (TEAM) sm.tail = min(sm.tail, lim);
+        }
     }
     eval();
     bar();
     const int err = sm.err;
-    if (defer_list && err) {   // a patch too large for this pass: the second pass takes the source
+    if (err) {   // a patch too large for this pass: the second pass takes the source, or the host hears of it
         if (tid == 0) {
-            defer_list[atomicAdd(defer_count, 1)] = item;
-            atomicAdd(counters + 4, 1ull);
+            if (defer_list) {
+                defer_list[atomicAdd(defer_count, 1)] = item;
+                atomicAdd(counters + 4, 1ull);
+            } else atomicOr(status, err);
         }
-        return 0;
+        return;
     }
     // the targets in particle order (every sum below runs in that order, so it does not depend on
     // the order of discovery)
@@ -911,27 +1067,38 @@ __device__ __forceinline__ int Group<R, PL, TEAM>::run(int item, int32_t* defer_
             }
     }
     bar();
-    // the log entries that hold each target's distance through a window and from a vertex
+    // a team: the log entries that hold each target's distance (through a window, and from a vertex)
     int* own = list;
     int* ownv = ord + (1 << Y.th_log);
-    for (int l = tid; l < min(sm.nlog, Y.lg_cap); l += T) {
-        const int s = at<int>(b, Y.lslot)[l] & ~FROM_VERTEX;
-        const bool vertex = at<int>(b, Y.lslot)[l] & FROM_VERTEX;
-        if (at<double>(b, Y.ldist)[l] == (vertex ? tvert() : tdist())[s]) (vertex ? ownv : own)[s] = l;
+    if constexpr (TEAM) {
+        for (int l = tid; l < min(sm.nlog, Y.lg_cap); l += T) {
+            const int c = at<int>(b, Y.lslot)[l], s = c & ~FROM_VERTEX;
+            const bool vertex = sizeof(R) == 4 && (c & FROM_VERTEX);
+            if (at<double>(b, Y.ldist)[l] == (vertex ? tvert() : tdist())[s]) (vertex ? ownv : own)[s] = l;
+        }
+        bar();
     }
-    bar();
     double fx = 0.0, fy = 0.0, en = 0.0;
     const double* fr = m.frame + 9 * (size_t)f0;
     for (int k = tid; k < nt; k += T) {
         const int s = ord[k];
-        const double dw = tdist()[s], dv = tvert()[s];
-        int l = dw < CUDART_INF ? own[s] : ownv[s];
-        if (dw < CUDART_INF && dv < dw) {
-            const double cw = at<double>(b, Y.lcmp)[l], cv = at<double>(b, Y.lcmp)[ownv[s]];
-            if (cv < cw - Tie<R>::t * cv) l = ownv[s];
+        int l = TEAM ? own[s] : s;
+        double d = tdist()[s];
+        if constexpr (sizeof(R) == 4) {
+            const double dv = tvert()[s];
+            const int lv = TEAM ? ownv[s] : s + (1 << Y.th_log);
+            bool vertex = !(d < CUDART_INF);
+            if (!vertex && dv < d) {
+                const double cw = at<double>(b, Y.tcmp)[l], cv = at<double>(b, Y.tcmp)[lv];
+                vertex = cv < cw - TIE32 * cv;
+            }
+            if (vertex) {
+                l = lv;
+                d = dv;
+            }
         }
-        const double d = at<double>(b, Y.ldist)[l];
-        const double tx = (double)at<R>(b, Y.ltan)[2 * l], ty = (double)at<R>(b, Y.ltan)[2 * l + 1];
+        const V2<R> t = at<V2<R>>(b, Y.ttan)[l];
+        const double tx = (double)t.x, ty = (double)t.y;
         if (J.want_pairs && k < J.pair_cap) {
             const size_t o = (size_t)src * J.pair_cap + k;
             J.pj[o] = tkey()[s];
@@ -952,16 +1119,16 @@ __device__ __forceinline__ int Group<R, PL, TEAM>::run(int item, int32_t* defer_
     en = css::warp_sum(en);
     if constexpr (TEAM) {
         if (lane == 0) {
-            sm.fx[wid] = fx;
-            sm.fy[wid] = fy;
-            sm.en[wid] = en;
+            tm->fx[wid] = fx;
+            tm->fy[wid] = fy;
+            tm->en[wid] = en;
         }
         __syncthreads();
         if (tid == 0)
             for (int w = 1; w < (T >> 5); ++w) {
-                fx += sm.fx[w];
-                fy += sm.fy[w];
-                en += sm.en[w];
+                fx += tm->fx[w];
+                fy += tm->fy[w];
+                en += tm->en[w];
             }
     }
     if (tid == 0) {
@@ -972,15 +1139,12 @@ __device__ __forceinline__ int Group<R, PL, TEAM>::run(int item, int32_t* defer_
             if (J.epot) atomicAdd(J.epot, en);
         }
         if (J.pcnt) J.pcnt[src] = nt;
-        int st = err;
-        if (J.want_pairs && nt > J.pair_cap) st |= css::ST_PAIR_OVERFLOW;
-        if (st) atomicOr(status, st);
+        if (J.want_pairs && nt > J.pair_cap) atomicOr(status, css::ST_PAIR_OVERFLOW);
         atomicAdd(counters + 0, 1ull);
-        atomicAdd(counters + 1, (unsigned long long)sm.tail);
+        atomicAdd(counters + 1, (unsigned long long)nprop);
         atomicAdd(counters + 2, (unsigned long long)nprop);
         atomicAdd(counters + 3, (unsigned long long)nt);
     }
-    return 0;
 }
 
 // PL 1: tables and ring in shared memory, 0: in the group's slice of global memory.  TEAM: the
@@ -992,13 +1156,21 @@ __global__ void __launch_bounds__(256, 2) k_waves(const __grid_constant__ cssi::
                                                   const __grid_constant__ WaveWs g, int* work, int* status,
                                                   unsigned long long* counters) {
     __shared__ GroupSm sms[TEAM ? 1 : MAXW];
+    TeamSm* tm = nullptr;
+    if constexpr (TEAM) {
+        __shared__ TeamSm team;
+        tm = &team;
+    }
     extern __shared__ __align__(16) unsigned char dsm[];
     const int wpc = blockDim.x >> 5, wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int in_cta = TEAM ? 0 : wid, groups = TEAM ? 1 : wpc;
     GroupSm& sm = sms[in_cta];
     const int gid = blockIdx.x * groups + in_cta;
-    unsigned char* b = PL == 1 ? dsm + (size_t)in_cta * g.lay.bytes : (unsigned char*)g.base + (size_t)gid * g.stride;
-    unsigned char* e = dsm + (PL == 1 ? (size_t)groups * g.lay.bytes : 0) + (size_t)wid * g.lay.e_bytes;
+    // each group's ring and (PL 1) tables, then each warp's queued tests
+    unsigned char* h = dsm + (size_t)in_cta * (g.lay.h_bytes + (PL == 1 ? g.lay.t_bytes : 0));
+    unsigned char* b = PL == 1 ? h + g.lay.h_bytes : (unsigned char*)g.base + (size_t)gid * g.stride;
+    unsigned char* x = (unsigned char*)g.base + (size_t)gid * g.stride + (PL == 1 ? 0 : g.lay.t_bytes);
+    unsigned char* e = dsm + (size_t)groups * (g.lay.h_bytes + (PL == 1 ? g.lay.t_bytes : 0)) + (size_t)wid * g.lay.e_bytes;
     const int nitems = q.item_count ? min(*(volatile const int*)q.item_count, q.nitems) : q.nitems;
     const int tile = TEAM ? 1 : max(1, q.tile);
     for (;;) {
@@ -1019,8 +1191,8 @@ __global__ void __launch_bounds__(256, 2) k_waves(const __grid_constant__ cssi::
             const int jid = q.job_of_item ? q.job_of_item[item] : 0;
             const cssi::GeoJob& J = jobs ? jobs[jid] : job0;
             const int pos = q.src_of_item ? q.src_of_item[item] : item;
-            Group<R, PL, TEAM> G{J, g.lay, b, e, sm, J.order ? J.order[pos] : pos, lane, wid,
-                                 TEAM ? (int)threadIdx.x : lane, TEAM ? (int)blockDim.x : 32};
+            Group<R, PL, TEAM> G{J, g.lay, b, h, e, x, sm, tm, J.order ? J.order[pos] : pos, lane, wid,
+                                 TEAM ? (int)threadIdx.x : lane, TEAM ? (int)blockDim.x : 32, __double2float_ru(J.rc)};
             if constexpr (!TEAM) { G.wid = 0; }
             G.run(item, q.defer_list, q.defer_count, status, counters);
             G.bar();
@@ -1034,41 +1206,50 @@ namespace cssi {
 
 namespace {
 
-// byte offsets of one group's working memory for the given capacities
+// byte offsets of one group's working memory for the given capacities (s_cap 0: no spill area)
 template <class R>
-WaveLay lay_out(int ring_log, int vh_log, int th_log) {
+WaveLay lay_out(int ring_log, int s_cap, int vh_log, int th_log, bool shared, bool team) {
     WaveLay y{};
-    y.ring_log = ring_log;
+    y.r_mask = (1 << ring_log) - 1;
+    y.s_cap = s_cap;
     y.vh_log = vh_log;
     y.th_log = th_log;
-    const int RG = 1 << ring_log, VH = 1 << vh_log, TH = 1 << th_log;
+    const int RG = 1 << ring_log, VH = 1 << vh_log, TH = 1 << th_log, ix = shared ? 2 : 4;
     y.v_most = VH - VH / 8;
     y.t_most = TH - TH / 8;
-    y.em_cap = VH / 2;
-    y.lg_cap = TH + TH / 2;
+    y.i_cap = VH * 5 / 16;
+    y.lg_cap = team ? 2 * TH : 0;
     int o = 0;
     auto take = [&](int n, int size) {
         const int p = o;
         o = (o + n * size + 15) & ~15;
         return p;
     };
-    y.sx = take(RG, 8); y.sy = take(RG, 8);
-    y.ra = take(RG, sizeof(R)); y.rb = take(RG, sizeof(R));
-    y.d0x = take(RG, sizeof(R)); y.d0y = take(RG, sizeof(R));
-    y.d1x = take(RG, sizeof(R)); y.d1y = take(RG, sizeof(R));
-    y.b0 = take(RG, 4); y.b1 = take(RG, 4); y.key = take(RG, 4);
-    y.he = take(RG, 4); y.vs = take(RG, 4);
-    y.vkey = take(VH, 4); y.vdist = take(VH, 8); y.vtan = take(VH, 2 * sizeof(R)); y.vflag = take(VH, 4);
-    y.tkey = take(TH, 4); y.tdist = take(TH, 8); y.tvert = take(TH, 8); y.tlist = take(3 * TH, 4);
-    y.emit = take(2 * y.em_cap, 4);
-    y.ldist = take(y.lg_cap, 8); y.lcmp = take(y.lg_cap, 8); y.ltan = take(y.lg_cap, 2 * sizeof(R)); y.lslot = take(y.lg_cap, 4);
-    y.bytes = o;
+    auto record = [&](int* to, int n) {
+        to[0] = take(n, 16);
+        for (int k = 1; k < 4; ++k) to[k] = take(n, 2 * sizeof(R));
+        to[4] = take(n, 16);
+        to[5] = take(n, 2 * ix);
+    };
+    record(y.r, RG);
+    y.h_bytes = o;
     o = 0;
-    y.e_sx = take(EV, 8); y.e_sy = take(EV, 8);
-    y.e_ra = take(EV, sizeof(R)); y.e_rb = take(EV, sizeof(R));
-    y.e_d0x = take(EV, sizeof(R)); y.e_d0y = take(EV, sizeof(R));
-    y.e_d1x = take(EV, sizeof(R)); y.e_d1y = take(EV, sizeof(R));
-    y.e_he = take(EV, 4); y.e_vs = take(EV, 4); y.e_j = take(EV, 4);
+    y.vkey = take(VH, 4); y.vdist = take(VH, 8); y.vinfo = take(VH, ix);
+    // 3 TH ints, used once the source is done: in the place of the vertex keys where they fit
+    y.tlist = 3 * TH <= VH ? y.vkey : take(3 * TH, 4);
+    y.itan = take(y.i_cap, 2 * sizeof(R)); y.iback = take(y.i_cap, 4); y.ihc = take(y.i_cap, 4);
+    y.emit = take(2 * y.i_cap, ix);
+    y.tkey = take(TH, 4); y.tdist = take(TH, 8); y.tvert = take(sizeof(R) == 4 ? TH : 0, 8);
+    const int recs = team ? y.lg_cap : (sizeof(R) == 4 ? 2 * TH : TH);
+    y.ttan = take(recs, 2 * sizeof(R)); y.tcmp = take(sizeof(R) == 4 ? recs : 0, 8);
+    y.ldist = take(y.lg_cap, 8); y.lslot = take(y.lg_cap, 4);
+    y.t_bytes = o;
+    o = 0;
+    record(y.s, s_cap);
+    y.s_bytes = o;
+    o = 0;
+    record(y.e, EV);
+    y.e_task = take(64, 1);
     y.e_bytes = o;
     return y;
 }
@@ -1101,39 +1282,48 @@ int blocks_of(int warps, size_t dyn) {
 }
 
 size_t dyn_bytes(const WaveLay& y, int warps, bool shared, bool team) {
-    return (shared ? (size_t)(team ? 1 : warps) * y.bytes : 0) + (size_t)warps * y.e_bytes;
+    return (size_t)(team ? 1 : warps) * (y.h_bytes + (shared ? y.t_bytes : 0)) + (size_t)warps * y.e_bytes;
 }
 
 }  // namespace
 
-// Capacities of one source's working memory.  In shared memory: 256 vertices and 64 targets
-// times the scale, and a ring of a sixteenth of the windows (a quarter in the team form, whose
-// waves are wider), at most 128 times the scale (1024 for a team) and halved until the shape
-// fits an SM.  In global memory the tables follow the table capacity (0: the windows).
+// Capacities of one source's working memory.  The ring holds 64 waiting windows in shared memory
+// (a team's 128 a warp), the rest of half the windows waits in a spill area in global memory.
+// Tables in shared memory: 256 vertices (a team's 1024) and 64 targets (256) times the scale; in
+// global memory they follow the table capacity (0: the windows).  A team's tables and ring are
+// halved until the shape fits an SM.
+// 64 slots: a small patch has 60-100 windows waiting (CPU counts: 71 icosphere, 101 noisy sphere at
+// most), a wave takes 32 and makes as many; 14 KB a warp in all then leave room for 16 warps.
 WaveLay wave_layout(int precision, int win_cap, int tab_cap, int shared_scale, int warps, int team) {
-    const int share = team ? win_cap / 4 : win_cap / 16;
     const bool f32 = precision == CSS_FP32;
-    auto lay = [&](int r, int v, int t) { return f32 ? lay_out<float>(r, v, t) : lay_out<double>(r, v, t); };
+    const int tab = tab_cap > 0 ? tab_cap : win_cap;
+    int wait = win_cap / 2;
+    if (!shared_scale) wait = std::min(wait, std::max(32, tab / 4));
+    int rl = std::min(log2_up(wait), team ? log2_up(128 * warps) : 6);
+    int vl = shared_scale ? log2_up((team ? 1024 : 256) * shared_scale) : log2_up(std::max(64, tab / 2));
+    int tl = shared_scale ? log2_up((team ? 256 : 64) * shared_scale) : log2_up(std::max(64, tab / 4));
     WaveLay y;
-    if (shared_scale) {
-        const int most = team ? std::max(1024, 128 * shared_scale) : 128 * shared_scale;
-        int rl = log2_up(std::min(share, most));
-        const int vl = log2_up(256 * shared_scale), tl = log2_up(64 * shared_scale);
-        y = lay(rl, vl, tl);
-        while (rl > 5 && dyn_bytes(y, warps, true, team != 0) > WAVE_SHARED_MAX) y = lay(--rl, vl, tl);
-    } else {
-        const int tab = tab_cap > 0 ? tab_cap : win_cap;
-        y = lay(log2_up(std::min(share, std::max(32, tab / 4))), log2_up(std::max(64, tab / 2)), log2_up(std::max(64, tab / 4)));
+    for (;;) {
+        const int spill = wait > (1 << rl) ? 1 << log2_up(wait) : 0;
+        y = f32 ? lay_out<float>(rl, spill, vl, tl, shared_scale != 0, team != 0)
+                : lay_out<double>(rl, spill, vl, tl, shared_scale != 0, team != 0);
+        if (dyn_bytes(y, warps, shared_scale != 0, team != 0) <= WAVE_SHARED_MAX || !team) break;
+        if (shared_scale && vl > log2_up(256 * shared_scale)) { --vl; --tl; }
+        else if (rl > 6) --rl;
+        else break;
     }
     y.max_waves = 4096 + 8 * win_cap;
     return y;
 }
 
-WaveLay wave_layout_of(int precision, int ring_log, int vh_log, int th_log) {
-    WaveLay y = precision == CSS_FP32 ? lay_out<float>(ring_log, vh_log, th_log) : lay_out<double>(ring_log, vh_log, th_log);
-    y.max_waves = 4096 + (128 << ring_log);
+WaveLay wave_layout_of(int precision, int spill_log, int vh_log, int th_log) {
+    WaveLay y = precision == CSS_FP32 ? lay_out<float>(6, 1 << spill_log, vh_log, th_log, false, false)
+                                      : lay_out<double>(6, 1 << spill_log, vh_log, th_log, false, false);
+    y.max_waves = 4096 + (64 << spill_log);
     return y;
 }
+
+size_t waves_global_bytes(const WaveLay& y, int shared) { return (size_t)y.s_bytes + (shared ? 0 : y.t_bytes); }
 
 int waves_blocks_per_sm(int precision, const WaveLay& y, int warps, int shared, int team) {
     if (warps < 1 || warps > MAXW) return 0;
