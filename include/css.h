@@ -342,10 +342,11 @@ int css_fma_peak(css_ctx* ctx, int precision, double* flops_per_s);
  *                      on one source together -- each wave unfolds up to 32 x warps_per_cta
  *                      windows -- for sets with fewer sources than resident warps
  * css_set_launch fails with CSS_ERR_INVALID_ARG when a value is out of range or the
- * shape's shared memory does not fit an SM.  Until a shape is set or tuned, a context
- * starts from {4, 0, 1, 1, 2048, 16384, 2, 1, 0, 0} and adapts by itself: after an evaluation
- * that deferred more than a quarter of its sources it switches the first pass to global
- * tables with a four times larger pool (up to 2^17 windows). */
+ * shape's shared memory does not fit an SM.  Until a shape is set or tuned, css_get_launch
+ * returns {4, 0, 1, 1, 2048, 16384, 2, 1, 0, 0} and the context picks the shape of each
+ * evaluation by itself, from the number of sources and the share of the mesh the cutoff
+ * reaches (a team for few sources with large patches, larger tables after an evaluation that
+ * deferred more than one source in 25). */
 typedef struct css_launch {
     int32_t warps_per_cta, ctas_per_sm, tile, shared_scale;
     int32_t window_capacity, window_capacity2, warps2_per_sm, occupancy;

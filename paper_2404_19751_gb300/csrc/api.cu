@@ -72,7 +72,7 @@ int next_pow2(int x) {
 // ---- the two passes of the persistent neighbour/force kernel
 struct GeoPlan {
     WaveWs g1, g2;
-    int wpc1 = 0, nctas1 = 0, wpc2 = 0, nctas2 = 0;
+    int wpc1 = 0, nctas1 = 0, wpc2 = 0, nctas2 = 0, tile = 1;
 };
 
 // one pass: layout, grid and (for tables in global memory) its workspace
@@ -109,10 +109,64 @@ int plan_pass(css_ctx* c, cssi::WsBuf& b, int precision, int win_cap, int tab_ca
     return CSS_OK;
 }
 
-// both passes for the context's launch shape and up to `nitems` work items
-int ensure_plan(css_ctx* c, int precision, int64_t nitems, GeoPlan* P) {
-    const cssi::LaunchCfg& L = c->cfg;
+// What one source of a set sees within the cutoff, by its share of the mesh's area.
+struct Reach {
+    double faces = 0.0, verts = 0.0, targets = 0.0;
+    void add(const css_parts* p, double rc) {   // the largest over several sets
+        const css_mesh* m = p->mesh;
+        const double part = std::isinf(rc) ? 1.0 : std::min(1.0, M_PI * rc * rc / m->area);
+        const double f = std::max(3.0, part * (double)m->nf);
+        faces = std::max(faces, f);
+        verts = std::max(verts, std::min((double)m->nv, 0.6 * f + 2.5 * sqrt(f) + 12.0));
+        targets = std::max(targets, part * (double)p->n);
+    }
+};
+
+// The launch shape for a context whose shape nobody set or tuned.  Measured on one GB300, kernel
+// times in ms (sources; windows a source):
+//   - as many sources as fill 16 warps an SM, small patches: tables in shared memory at scale 1
+//     (noisy sphere, 16384; 473: 2.96, scale 2 with its 8 warps an SM 3.95, tables in global memory
+//     3.32).  Where the tables are too small for the patch, global memory (height field, 8192;
+//     3957: 10.2 with 16 warps an SM, shared at scale 8 with 2 warps 27.3)
+//   - fewer sources than 8 warps an SM: scale 2 (icosphere, 1024; 301: 0.107 against 0.138; torus, 999;
+//     407: 0.353 against 0.805, whose scale-1 tables deferred 132 sources)
+//   - few sources, large patches: a team of 8, 4 or 2 warps a source, as many as leave an SM 16
+//     warps or so (flat plane, 64; 5046: one warp 1.60, teams of 2, 4, 8 0.93, 0.65, 0.55; torus,
+//     100; 86000: 23.7 -> 10.0, 6.5, 5.9); on 300 windows a team loses (0.187 against 0.107).  Between
+//     them lies a patch of 350 faces: its waves are about 8 sqrt(6 x 350) windows wide in all.
+cssi::LaunchCfg pick_shape(const css_ctx* c, int64_t nitems, const Reach& R) {
+    cssi::LaunchCfg L = c->cfg;
+    const double grow = (double)(1 << c->auto_level), verts = grow * R.verts, targets = grow * R.targets;
+    const int64_t sms = c->sm_count;
+    const bool big = R.faces >= 350.0;
+    L.warps_per_cta = 4;
+    L.ctas_per_sm = 0;
+    L.tile = 1;
+    L.tab_cap = 0;
+    L.team = 0;
+    if (big && nitems <= 12 * sms) {
+        L.team = 1;
+        L.warps_per_cta = nitems <= 3 * sms ? 8 : (nitems <= 6 * sms ? 4 : 2);
+        L.win_cap = 16384;
+        L.shared_scale = verts <= 800.0 && targets <= 200.0 ? 1 : (verts <= 1600.0 && targets <= 400.0 ? 2 : 0);
+    } else if (verts <= 200.0 && targets <= 48.0) L.shared_scale = nitems <= 8 * sms ? 2 : 1;
+    else if (verts <= 400.0 && targets <= 96.0 && nitems <= 8 * sms) L.shared_scale = 2;
+    else if (verts <= 800.0 && targets <= 192.0 && nitems <= 4 * sms) L.shared_scale = 4;
+    else L.shared_scale = 0;
+    if (!L.team) L.win_cap = 2048 * std::max(1, L.shared_scale);
+    if (!L.shared_scale) {   // vertices at half load, targets, and the windows waiting at a time
+        const double need = std::max({3.2 * verts, 5.2 * targets, 32.0 * sqrt(6.0 * R.faces) * grow, 512.0});
+        L.tab_cap = next_pow2((int)std::min(need, 1048576.0));
+        L.win_cap = std::max(8192, L.tab_cap);
+    }
+    return L;
+}
+
+// both passes for the launch shape and up to `nitems` work items
+int ensure_plan(css_ctx* c, int precision, int64_t nitems, const Reach& R, GeoPlan* P) {
+    const cssi::LaunchCfg L = c->cfg_explicit ? c->cfg : pick_shape(c, nitems, R);
     P->wpc1 = L.warps_per_cta;
+    P->tile = L.tile;
     int rc = plan_pass(c, c->ws1, precision, L.win_cap, L.tab_cap, L.shared_scale, L.warps_per_cta, L.team,
                        L.ctas_per_sm, &P->g1, &P->nctas1);
     if (rc) return rc;
@@ -133,7 +187,7 @@ int ensure_plan(css_ctx* c, int precision, int64_t nitems, GeoPlan* P) {
 std::string plan_key(const css_ctx* c, const GeoPlan& P) {
     std::string k((const char*)&P.g1, sizeof(P.g1));
     k.append((const char*)&P.g2, sizeof(P.g2));
-    const int64_t v[6] = {(int64_t)(uintptr_t)c->defer, P.wpc1, P.nctas1, P.wpc2, P.nctas2, c->cfg.tile};
+    const int64_t v[6] = {(int64_t)(uintptr_t)c->defer, P.wpc1, P.nctas1, P.wpc2, P.nctas2, P.tile};
     k.append((const char*)v, sizeof(v));
     return k;
 }
@@ -190,7 +244,7 @@ int enqueue_passes(css_ctx* c, const GeoJob& j0, const GeoJob* djobs, const int3
     TRY(c, "reset", cudaMemsetAsync(c->dscal, 0, sizeof(int), st));
     TRY(c, "reset", cudaMemsetAsync(c->dscal + 2, 0, 2 * sizeof(int), st));
     TRY(c, "event", record_ev(c, c->ev_geo0));
-    cssi::GeoQueue q1{job_of_item, src_of_item, nitems, nullptr, nullptr, c->defer, c->dscal + 2, c->cfg.tile};
+    cssi::GeoQueue q1{job_of_item, src_of_item, nitems, nullptr, nullptr, c->defer, c->dscal + 2, P.tile};
     TRY(c, "geodesic", cssi::launch_waves(j0, djobs, q1, prec, P.g1, P.wpc1, P.nctas1, c->dscal, c->dscal + 1,
                                           c->dcount, st));
     cssi::GeoQueue q2{job_of_item, src_of_item, nitems, c->defer, c->dscal + 2, nullptr, nullptr, 1};
@@ -247,16 +301,12 @@ int status_error(css_ctx* c, int status) {
     return CSS_ERR_CUDA;
 }
 
-// A context whose launch shape nobody set or tuned adapts its first pass: when more than a
-// quarter of the evaluated sources were deferred (patches too large for the shared tables
-// or the pool), later evaluations use global tables and a four times larger pool.
+// A context whose launch shape nobody set or tuned doubles its first pass's tables when more than one
+// source in 25 was deferred (patches larger than the estimate).
 void adapt_default(css_ctx* c) {
     if (c->cfg_explicit) return;
     const int64_t done = c->last_counters[0], deferred = c->last_counters[4];
-    if (done > 0 && deferred * 4 > done && c->cfg.win_cap < (1 << 17)) {
-        c->cfg.shared_scale = 0;
-        c->cfg.win_cap = std::max(c->cfg.win_cap * 4, 8192);
-    }
+    if (done > 0 && deferred * 25 > done && c->auto_level < 8) ++c->auto_level;
 }
 
 // synchronous neighbour / force evaluation with overflow retries
@@ -267,7 +317,9 @@ int run_geo(css_parts* p, double rc, int prec, int want_pairs, int want_forces, 
     for (;;) {
         if (want_pairs) { int rc2 = ensure_pairs(p, c->pair_cap); if (rc2) return rc2; }
         GeoPlan P;
-        int rc1 = ensure_plan(c, prec, p->n, &P);
+        Reach R;
+        R.add(p, rc);
+        int rc1 = ensure_plan(c, prec, p->n, R, &P);
         if (rc1) return rc1;
         TRY(c, "reset", cudaMemsetAsync(c->dcount, 0, 8 * sizeof(unsigned long long), c->stream));
         TRY(c, "reset", cudaMemsetAsync(c->dscal + 1, 0, sizeof(int), c->stream));
@@ -800,7 +852,9 @@ int css_integrate_step(css_parts* p, const css_potential* pot, const css_integra
     for (;;) {
         TRY(c, "snapshot", snap_take(p));
         GeoPlan P;
-        rc = ensure_plan(c, precision, p->n, &P);
+        Reach R;
+        R.add(p, r_c);
+        rc = ensure_plan(c, precision, p->n, R, &P);
         if (rc) break;
         TRY(c, "reset", cudaMemsetAsync(c->dscal + 1, 0, sizeof(int), st));
         TRY(c, "reset", cudaMemsetAsync(c->dcount, 0, 8 * sizeof(unsigned long long), st));
@@ -959,7 +1013,9 @@ int css_batch_step(css_batch* b, const css_potential* pot, const css_integrator*
     for (;;) {
         for (css_parts* p : b->sets) TRY(c, "snapshot", snap_take(p));
         GeoPlan P;
-        int rc = ensure_plan(c, precision, b->nitems, &P);
+        Reach R;
+        for (const css_parts* p : b->sets) R.add(p, r_c);
+        int rc = ensure_plan(c, precision, b->nitems, R, &P);
         if (rc) return rc;
         TRY(c, "reset", cudaMemsetAsync(c->dscal + 1, 0, sizeof(int), st));
         TRY(c, "reset", cudaMemsetAsync(c->dcount, 0, 8 * sizeof(unsigned long long), st));
@@ -1020,7 +1076,7 @@ int tune_run(css_ctx* c, const GeoJob* djobs, const GeoJob& j0, const int32_t* j
     int retries = 0;
     for (;;) {
         GeoPlan P;
-        int rc = ensure_plan(c, prec, nitems, &P);
+        int rc = ensure_plan(c, prec, nitems, Reach(), &P);
         if (rc) return rc;
         TRY(c, "reset", cudaMemsetAsync(c->dscal + 1, 0, sizeof(int), c->stream));
         TRY(c, "reset", cudaMemsetAsync(c->dcount, 0, 8 * sizeof(unsigned long long), c->stream));
@@ -1080,6 +1136,8 @@ int css_autotune(css_ctx* c, css_parts* const* sets, int32_t n_sets, const css_p
     if (e != cudaSuccess) { cleanup(); return cuda_fail(c, "autotune", e); }
     const int32_t nitems = (int32_t)hj.size();
     const cssi::LaunchCfg base = c->cfg;
+    const int was_explicit = c->cfg_explicit;
+    c->cfg_explicit = 1;   // the candidates are run as they are
     constexpr int POOL_UNIT = 2048;   // first-pass windows per warp at table scale 1
     constexpr int TAB_UNIT = 4096;    // global-table slots tried besides tables tied to the pool
     cssi::LaunchCfg pick = base;
@@ -1212,7 +1270,7 @@ int css_autotune(css_ctx* c, css_parts* const* sets, int32_t n_sets, const css_p
     }
     cleanup();
     c->cfg = rc == CSS_OK ? pick : base;
-    if (rc == CSS_OK) c->cfg_explicit = 1;
+    if (rc != CSS_OK) c->cfg_explicit = was_explicit;
     for (int k = 0; k < n_sets; ++k) sets[k]->force_valid = 0;   // forces of the sample only
     if (rc) return rc;
     if (best) css_get_launch(c, best);

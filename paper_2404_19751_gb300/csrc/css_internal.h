@@ -44,7 +44,8 @@ struct css_ctx {
     cssi::WsBuf ws1, ws2;
     cssi::LaunchCfg cfg;
     std::map<int64_t, int> bps_cache;   // resident CTAs per SM by (precision, shape)
-    int cfg_explicit = 0;               // the shape was set or tuned (no automatic adaptation)
+    int cfg_explicit = 0;               // the shape was set or tuned (else one is picked for each evaluation)
+    int auto_level = 0;                 // doublings of the picked shape's tables after deferrals
     int pair_cap = 64;               // pairs per source slab
     // deferral list of the first pass (one entry per work item at most)
     int32_t* defer = nullptr;
@@ -72,6 +73,7 @@ void vhm_free(css_mesh* m);
 struct css_mesh {
     css_ctx* ctx = nullptr;
     int64_t nv = 0, nf = 0, ne = 0, npseudo = 0;
+    double area = 0.0;
     int periodic = 0;
     double per[2] = {0, 0};
     // device arrays

@@ -217,25 +217,31 @@ __global__ void k_vertices(int64_t nv, const int32_t* ring_start, int32_t* ring,
     }
     if (!closed)
         for (int i = s; i < e; ++i) cang[ring[i]] = make_float2(NAN, NAN);
+    // bit 1: shortest paths may bend here.  An interior vertex of angle sum 2 pi (within 1e-12, a
+    // flat one) needs no windows of its own: the straight lines on its two sides meet behind it
+    if (p && !(closed && th <= TWO_PI + 1e-12)) pseudo[v] = 3;
 }
 
-// Topology records of the half-edges.  A shortest path bends only at a boundary, non-manifold or
-// saddle vertex.  An interior vertex of angle sum 2 pi (within 1e-12, a flat one) needs no windows
-// of its own: the straight lines on its two sides meet behind it.
-__global__ void k_htop(int64_t nf, const int32_t* fv, const uint8_t* pseudo, const double* theta,
-                       const float2* cang, const int32_t* ring_start, const int32_t* ring, const int32_t* frank,
-                       int4* htop) {
-    const int64_t h = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (h >= 3 * nf) return;
-    const int64_t f = h / 3;
-    const int k = (int)(h - 3 * f);
+// total area (what share of the faces a cutoff reaches)
+__global__ void k_area(const double* lay, int64_t nf, double* area) {
+    const int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const double a = css::warp_sum(f < nf ? 0.5 * lay[3 * f] * lay[3 * f + 2] : 0.0);
+    if ((threadIdx.x & 31) == 0) atomicAdd(area, a);
+}
+
+// Topology records of the half-edges
+__global__ void k_htop(int64_t nf, const int32_t* fv, const uint8_t* pseudo, const int32_t* frank, int4* htop) {
+    const int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (f >= nf) return;
     int32_t o[3];
     for (int q = 0; q < 3; ++q) {
-        const int32_t v = fv[3 * f + (k + q) % 3];
-        const bool fan = !isnan(cang[ring[ring_start[v]]].x);   // one closed fan of faces
-        o[q] = v | (pseudo[v] && !(fan && theta[v] <= TWO_PI + 1e-12) ? css::EMITS : 0);
+        const int32_t v = fv[3 * f + q];
+        o[q] = v | (pseudo[v] & 2 ? css::EMITS : 0);
     }
-    htop[h] = make_int4(o[0], o[1], o[2], frank[f]);
+    const int32_t r = frank[f];
+    htop[3 * f] = make_int4(o[0], o[1], o[2], r);
+    htop[3 * f + 1] = make_int4(o[1], o[2], o[0], r);
+    htop[3 * f + 2] = make_int4(o[2], o[0], o[1], r);
 }
 
 inline unsigned nblk(int64_t n, int b = 256) { return (unsigned)((n + b - 1) / b); }
@@ -315,7 +321,7 @@ int build_mesh(css_ctx* ctx, const double* dX, int64_t nv, const int32_t* dF, in
     int32_t* ring_cnt = nullptr;
     int32_t* tmp = nullptr;
     int hflag = 0;
-    unsigned long long hcnt[2] = {0, 0};
+    unsigned long long hcnt[3] = {0, 0, 0};   // edges, pseudo-source vertices, area (a double's bits)
     m->nv = nv;
     m->nf = nf;
     if (period) { m->periodic = 1; m->per[0] = period[0]; m->per[1] = period[1]; }
@@ -324,7 +330,7 @@ int build_mesh(css_ctx* ctx, const double* dX, int64_t nv, const int32_t* dF, in
     CK(cudaMalloc(&t.h0, cap * sizeof(int32_t)));
     CK(cudaMalloc(&t.h1, cap * sizeof(int32_t)));
     CK(cudaMalloc(&dflag, sizeof(int)));
-    CK(cudaMalloc(&dcnt, 2 * sizeof(unsigned long long)));
+    CK(cudaMalloc(&dcnt, 3 * sizeof(unsigned long long)));
     CK(cudaMalloc(&m->he, nh * sizeof(HeRec)));
     CK(cudaMalloc(&m->twin, nh * sizeof(int32_t)));
     CK(cudaMalloc(&m->edge, nh * sizeof(int32_t)));
@@ -349,7 +355,7 @@ int build_mesh(css_ctx* ctx, const double* dX, int64_t nv, const int32_t* dF, in
     CK(cudaMemsetAsync(t.key, 0xff, cap * sizeof(unsigned long long), st));
     CK(cudaMemsetAsync(t.cnt, 0, cap * sizeof(int32_t), st));
     CK(cudaMemsetAsync(dflag, 0, sizeof(int), st));
-    CK(cudaMemsetAsync(dcnt, 0, 2 * sizeof(unsigned long long), st));
+    CK(cudaMemsetAsync(dcnt, 0, 3 * sizeof(unsigned long long), st));
     CK(cudaMemsetAsync(m->bnd, 0, nv, st));
     CK(cudaMemsetAsync(ring_cnt, 0, (nv + 1) * sizeof(int32_t), st));
     k_check_faces<<<nblk(nf), 256, 0, st>>>(dF, nf, nv, dflag);
@@ -374,10 +380,13 @@ int build_mesh(css_ctx* ctx, const double* dX, int64_t nv, const int32_t* dF, in
     k_vertices<<<nblk(nv), 256, 0, st>>>(nv, m->ring_start, m->ring, m->he, m->twin, m->theta, m->bnd, m->pseudo,
                                          m->cang, dcnt + 1);
     CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(hcnt, dcnt, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
+    k_area<<<nblk(nf), 256, 0, st>>>(m->lay, nf, (double*)(dcnt + 2));
+    CK(cudaGetLastError());
+    CK(cudaMemcpyAsync(hcnt, dcnt, 3 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     m->ne = (int64_t)hcnt[0];
     m->npseudo = (int64_t)hcnt[1];
+    memcpy(&m->area, hcnt + 2, sizeof(double));
     {   // Morton rank of every face (host sort, once per mesh)
         float* dorg = nullptr;
         CK(cudaMalloc(&dorg, 3 * nf * sizeof(float)));
@@ -404,8 +413,7 @@ int build_mesh(css_ctx* ctx, const double* dX, int64_t nv, const int32_t* dF, in
         std::vector<int32_t> rank(nf);
         for (int64_t r = 0; r < nf; ++r) rank[(int64_t)(key[r] & 0xffffffffu)] = (int32_t)r;
         CK(cudaMemcpyAsync(m->frank, rank.data(), nf * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-        k_htop<<<nblk(nh), 256, 0, st>>>(nf, m->fv, m->pseudo, m->theta, m->cang, m->ring_start, m->ring,
-                                         m->frank, m->htop);
+        k_htop<<<nblk(nf), 256, 0, st>>>(nf, m->fv, m->pseudo, m->frank, m->htop);
         CK(cudaGetLastError());
         CK(cudaStreamSynchronize(st));
     }
