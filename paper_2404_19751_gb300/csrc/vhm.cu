@@ -19,8 +19,10 @@
 //
 // GPU organisation: K sources at a time (K a power of two <= 256), fields vertex-major
 // with the K sources contiguous, thread (v, s) at v K + s, so the K threads of a row share
-// the row's operator entries.  The heat systems are solved by Gauss-Seidel sweeps over a
-// colouring of the vertex graph (one launch per colour): the matrices are symmetric positive
+// the row's operator entries.  Where the fields of one column fit in a CTA's shared memory
+// (about 14300 vertices), a cluster of CTAs solves one column in one kernel (Rows below);
+// larger meshes take one launch per colour of a sweep and six per iteration.  The heat
+// systems are solved by Gauss-Seidel sweeps over a colouring of the vertex graph: the matrices are symmetric positive
 // definite, so the sweeps converge on any mesh; where the scalar matrix is an M-matrix every
 // sweep adds non-negative terms, and the solution keeps its relative accuracy where it is
 // tiny far from the source (a Krylov solver's residual norm would not); the sweeps stop when
@@ -28,6 +30,7 @@
 // Poisson system is solved by Jacobi-preconditioned conjugate gradients, one column per
 // source, with per-source reductions in a fixed order (the result does not depend on
 // thread timing).
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -424,6 +427,320 @@ __global__ void k_cg_dir(Op o, int K, const int* active, const double* beta, con
     if (active[s]) p[g] = z[g] + beta[s] * p[g];
 }
 
+// ------------------------------------------------------------------ solves of one column
+// Where a column's fields fit in shared memory, a whole solve of one column runs in one
+// kernel: every sweep and every iteration between two block barriers instead of two
+// launches, the fields in shared memory instead of L2.  Rows are the vertices in the order
+// of the colouring, each colour padded to full slices of 32 rows; a slice's entries lie
+// [entry][row of the slice], so a warp reads them in one line, and the two half weights of
+// an edge (one per face at it) are one entry, half the FP64 operations of the general form.
+// Bound by the FP64 pipe (two FMA a clock and SM): 4 FMA an entry for the transported
+// vector, 1 for the scalar.  Whole calls on one GB300, all pairs, general form -> this one:
+// 3916 vertices with 100 sources 59.4 -> 11.3 ms (heat 5.4, conjugate gradients 5.1; their
+// FP64 operations alone take 3.3 and 3.8 on the 100 SMs in use), with 20 sources 27.0 -> 5.8,
+// with 256 91.0 -> 19.9; 800 vertices with 100 sources 12.7 -> 2.3; 12800 vertices with 3
+// sources 35.4 -> 11.0.  CTAs of 1024 threads take 10.8 ms in the first case and 22.6 with 256
+// sources, where two CTAs of 512 share an SM.
+struct Rows {
+    int32_t np = 0;          // rows, a multiple of 32
+    int32_t ncol = 0;
+    const int32_t* cslice;   // first slice of each colour, ncol + 1
+    const int32_t* soff;     // first entry line of each slice, np / 32 + 1
+    const int32_t* vert;     // vertex of a row, -1 for padding
+    const int32_t* rowof;    // row of a vertex
+    const int32_t* j;        // neighbour's row (padding: the row itself with weight 0)
+    const double* w;         // cotan weight
+    const double2* cs;       // weight times the turn of the connection
+    const double* mass;
+    const double* diag;
+};
+
+constexpr int CT = 512;       // threads of a CTA of the column kernels
+constexpr int CHECK_EVERY = 8;
+constexpr int CL_MAX = 8;     // CTAs of a cluster
+
+struct ColumnShared {
+    double wsum[CT / 32];
+    double csum[2][CL_MAX];
+    double res;
+    int stop;
+    int moved[CL_MAX];
+    int row[3];
+    double2 rhs[3];
+};
+
+struct Cluster {
+    cooperative_groups::cluster_group g;
+    int rank, size;
+    __device__ __forceinline__ void sync() const {
+        if (size == 1) __syncthreads();
+        else g.sync();
+    }
+    template <class T>
+    __device__ __forceinline__ void store_all(T* p, T v) const {   // every CTA's copy of *p
+        *p = v;
+        for (int k = 1; k < size; ++k) {
+            const int r = rank + k < size ? rank + k : rank + k - size;
+            *g.map_shared_rank(p, r) = v;
+        }
+    }
+};
+
+__device__ __forceinline__ Cluster this_cluster_of_column() {
+    Cluster c{cooperative_groups::this_cluster(), 0, 1};
+    c.rank = (int)c.g.block_rank();
+    c.size = (int)c.g.num_blocks();
+    return c;
+}
+
+// inverse diagonals of the heat systems divided by t and of the Poisson system
+__global__ void k_row_scale(Rows o, double t, double* inv_heat, double* inv_diag) {
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= o.np) return;
+    inv_heat[p] = o.vert[p] >= 0 ? 1.0 / (o.mass[p] / t + o.diag[p]) : 0.0;
+    inv_diag[p] = o.vert[p] >= 0 ? 1.0 / o.diag[p] : 0.0;
+}
+
+__device__ __forceinline__ void row_terms(const Rows& o, int e, const double* x, double& acc) {
+    acc = fma(o.w[e], x[o.j[e]], acc);
+}
+__device__ __forceinline__ void row_terms(const Rows& o, int e, const double2* x, double2& acc) {
+    const double2 c = o.cs[e], y = x[o.j[e]];
+    acc.x = fma(c.x, y.x, fma(-c.y, y.y, acc.x));
+    acc.y = fma(c.y, y.x, fma(c.x, y.y, acc.y));
+}
+__device__ __forceinline__ double largest(double a) { return fabs(a); }
+__device__ __forceinline__ double largest(double2 a) { return fmax(fabs(a.x), fabs(a.y)); }
+__device__ __forceinline__ double scaled(double a, double k) { return a * k; }
+__device__ __forceinline__ double2 scaled(double2 a, double k) { return {a.x * k, a.y * k}; }
+__device__ __forceinline__ double less(double a, double b) { return a - b; }
+__device__ __forceinline__ double2 less(double2 a, double2 b) { return {a.x - b.x, a.y - b.y}; }
+__device__ __forceinline__ double relaxed(double x, double a, double om, double k) { return fma(a, k, (1.0 - om) * x); }
+__device__ __forceinline__ double2 relaxed(double2 x, double2 a, double om, double k) {
+    return {fma(a.x, k, (1.0 - om) * x.x), fma(a.y, k, (1.0 - om) * x.y)};
+}
+__device__ __forceinline__ void first(double2 v, double& o) { o = v.x; }
+__device__ __forceinline__ void first(double2 v, double2& o) { o = v; }
+
+// Sweeps of one heat system (divided by t) over one column until a sweep changes no entry
+// by more than 1e-14 of the terms it is summed from (in the largest component).  The sweeps
+// are over-relaxed with the factor of Young's theory, 2 / (1 + sqrt(1 - rho^2)), rho the
+// ratio of the off-diagonal sum to the diagonal: it both minimises the number of sweeps and is
+// the largest factor at which rounding errors do not grow with distance from the source
+// relative to the solution's own decay (with rho = 0.8, t = h^2: 252 plain sweeps, 120 relaxed
+// ones on a torus of 4005 vertices; at t = 0.1 h^2 a factor of 1.35 instead of 1.04 loses the far
+// field).  Every eighth sweep is a plain one and is the one that checks.  After plain_after
+// sweeps all are plain.
+template <class T>
+__device__ __forceinline__ void heat_column(const Rows& o, const Cluster& cl, ColumnShared& sh, T* x,
+                                            const double* inv_d, double omega, int plain_after, int max_sweeps,
+                                            int* sweeps_out, int* status) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = CT / 32;
+    for (int p = threadIdx.x; p < o.np; p += CT) x[p] = T{};
+    cl.sync();
+    T b0, b1, b2;
+    first(sh.rhs[0], b0);
+    first(sh.rhs[1], b1);
+    first(sh.rhs[2], b2);
+    const int r0 = sh.row[0], r1 = sh.row[1], r2 = sh.row[2];
+    int sweep = 0;
+    for (;;) {
+        const bool check = (sweep & (CHECK_EVERY - 1)) == CHECK_EVERY - 1;
+        const double om = check || sweep >= plain_after ? 1.0 : omega;
+        bool moved = false;
+        for (int c = 0; c < o.ncol; ++c) {
+            const int s1 = o.cslice[c + 1];
+            for (int sl = o.cslice[c] + warp * cl.size + cl.rank; sl < s1; sl += nw * cl.size) {
+                const int p = sl * 32 + lane;
+                T acc = T{};
+                if (p == r0) acc = b0;
+                if (p == r1) acc = b1;
+                if (p == r2) acc = b2;
+                const int e1 = o.soff[sl + 1] * 32 + lane;
+                const double iD = inv_d[p];
+                if (!check) {
+#pragma unroll 6
+                    for (int e = o.soff[sl] * 32 + lane; e < e1; e += 32) row_terms(o, e, x, acc);
+                    cl.store_all(x + p, relaxed(x[p], acc, om, om * iD));
+                } else {
+                    double mag = largest(acc);
+                    for (int e = o.soff[sl] * 32 + lane; e < e1; e += 32) {
+                        row_terms(o, e, x, acc);
+                        mag = fma(fabs(o.w[e]), largest(x[o.j[e]]), mag);
+                    }
+                    const T y = scaled(acc, iD);
+                    mag *= iD;
+                    moved |= mag > 1e-290 && largest(less(y, x[p])) > 1e-14 * mag;
+                    cl.store_all(x + p, y);
+                }
+            }
+            cl.sync();
+        }
+        ++sweep;
+        if (!check) continue;
+        int any = __syncthreads_or(moved);
+        if (cl.size > 1) {
+            if (threadIdx.x == 0) cl.store_all(&sh.moved[cl.rank], any);
+            cl.sync();
+            any = 0;
+            for (int k = 0; k < cl.size; ++k) any |= sh.moved[k];
+        }
+        if (!any) break;
+        if (sweep >= max_sweeps) {
+            if (threadIdx.x == 0) atomicOr(status, 1);
+            break;
+        }
+    }
+    if (threadIdx.x == 0) atomicMax(sweeps_out, sweep);
+}
+
+// Both heat systems of every column: clusters [0, ns) solve the vector system, the longer one,
+// and [ns, 2 ns) the scalar one.
+__global__ void __launch_bounds__(CT, 2) k_heat_columns(Op m, Rows o, int K, int ns, double t, double omega,
+                                                        int plain_after, int max_sweeps, const int32_t* src,
+                                                        const int32_t* face, const double* bary, const double* inv_d,
+                                                        double* u, double* Y, int* sweeps_out, int* status) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ ColumnShared sh;
+    const Cluster cl = this_cluster_of_column();
+    const int id = blockIdx.x / cl.size;
+    const bool vec = id < ns;
+    const int s = vec ? id : id - ns;
+    if (threadIdx.x < 3) {
+        const int k = threadIdx.x, i = src[s], f0 = face[i], v = m.fv[3 * f0 + k];
+        const double b = bary[3 * (size_t)i + k] / t;
+        const double psi = m.phi[3 * f0 + k] + m.scale[v] * wrap_pi(0.0 - m.gam[3 * f0 + k]);
+        sh.row[k] = o.rowof[v];
+        sh.rhs[k] = vec ? make_double2(b * cos(psi), b * sin(psi)) : make_double2(b, 0.0);
+    }
+    if (vec) {
+        double2* x = (double2*)smem;
+        heat_column(o, cl, sh, x, inv_d, omega, plain_after, max_sweeps, sweeps_out, status);
+        for (int p = threadIdx.x * cl.size + cl.rank; p < o.np; p += CT * cl.size)
+            if (o.vert[p] >= 0) ((double2*)Y)[(size_t)o.vert[p] * K + s] = x[p];
+    } else {
+        double* x = (double*)smem;
+        heat_column(o, cl, sh, x, inv_d, omega, plain_after, max_sweeps, sweeps_out, status);
+        for (int p = threadIdx.x * cl.size + cl.rank; p < o.np; p += CT * cl.size)
+            if (o.vert[p] >= 0) u[(size_t)o.vert[p] * K + s] = x[p];
+    }
+}
+
+// The sum of v over the cluster's threads, in a fixed order, for thread 0; the caller's
+// next barrier is a block barrier.
+__device__ __forceinline__ double column_sum(double v, const Cluster& cl, ColumnShared& sh, int parity) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int d = 16; d; d >>= 1) v += __shfl_xor_sync(CSS_FULL, v, d);
+    if (lane == 0) sh.wsum[warp] = v;
+    __syncthreads();
+    if (warp == 0) {
+        v = lane < CT / 32 ? sh.wsum[lane] : 0.0;
+        for (int d = 16; d; d >>= 1) v += __shfl_xor_sync(CSS_FULL, v, d);
+        if (cl.size > 1 && lane == 0) cl.store_all(&sh.csum[parity][cl.rank], v);
+    }
+    if (cl.size > 1) {
+        cl.sync();
+        if (threadIdx.x == 0) {
+            v = 0.0;
+            for (int k = 0; k < cl.size; ++k) v += sh.csum[parity][k];
+        }
+    }
+    return v;
+}
+
+// The Poisson system of one column by conjugate gradients with the diagonal as preconditioner:
+// the direction p in shared memory (every CTA of the cluster holds all of it), L p of a CTA's
+// own rows beside it, solution and residual of its own rows in global memory, where only
+// the thread that owns a row touches them.
+__global__ void __launch_bounds__(CT, 2) k_cg_columns(Rows o, int nv, int K, double tol2, int max_iters,
+                                                      const double* b, double* x, double* r, const double* inv_diag,
+                                                      int* iters_out, int* status) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ ColumnShared sh;
+    const Cluster cl = this_cluster_of_column();
+    const int s = blockIdx.x / cl.size;
+    double* p = (double*)smem;
+    double* q = p + o.np;
+    double* rc = r + (size_t)s * o.np;
+    double* xc = r + ((size_t)K + s) * o.np;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int first_slice = warp * cl.size + cl.rank, step = CT / 32 * cl.size, nsl = o.np / 32;
+    if (cl.size > 1) cl.sync();   // every CTA of the cluster runs before its shared memory is written
+    double rz = 0.0, rz0 = 0.0;   // thread 0's
+    double acc = 0.0;
+    for (int sl = first_slice; sl < nsl; sl += step) {
+        const int v = o.vert[sl * 32 + lane];
+        if (v >= 0) acc += b[(size_t)v * K + s];
+    }
+    acc = column_sum(acc, cl, sh, 0);
+    if (threadIdx.x == 0) sh.res = acc / nv;
+    __syncthreads();
+    const double mean = sh.res;
+    acc = 0.0;
+    for (int sl = first_slice; sl < nsl; sl += step) {
+        const int i = sl * 32 + lane, v = o.vert[i];
+        const double bb = v >= 0 ? b[(size_t)v * K + s] - mean : 0.0;
+        const double z = bb * inv_diag[i];
+        rc[i] = bb;
+        xc[i] = 0.0;
+        cl.store_all(p + i, z);
+        acc = fma(bb, z, acc);
+    }
+    acc = column_sum(acc, cl, sh, 1);
+    if (threadIdx.x == 0) rz = rz0 = acc;
+    cl.sync();
+    int it = 0;
+    for (;;) {
+        acc = 0.0;
+        for (int sl = first_slice; sl < nsl; sl += step) {
+            const int i = sl * 32 + lane, e1 = o.soff[sl + 1] * 32 + lane;
+            const double pi = p[i];
+            double a = o.diag[i] * pi;
+#pragma unroll 6
+            for (int e = o.soff[sl] * 32 + lane; e < e1; e += 32) a = fma(-o.w[e], p[o.j[e]], a);
+            q[i] = a;
+            acc = fma(pi, a, acc);
+        }
+        acc = column_sum(acc, cl, sh, 0);
+        if (threadIdx.x == 0) sh.res = acc != 0.0 ? rz / acc : 0.0;
+        __syncthreads();
+        const double alpha = sh.res;
+        acc = 0.0;
+        for (int sl = first_slice; sl < nsl; sl += step) {
+            const int i = sl * 32 + lane;
+            xc[i] = fma(alpha, p[i], xc[i]);
+            const double rr = fma(-alpha, q[i], rc[i]);
+            rc[i] = rr;
+            const double z = rr * inv_diag[i];
+            q[i] = z;
+            acc = fma(rr, z, acc);
+        }
+        acc = column_sum(acc, cl, sh, 1);
+        ++it;
+        if (threadIdx.x == 0) {
+            sh.res = rz != 0.0 ? acc / rz : 0.0;
+            rz = acc;
+            sh.stop = !(acc > tol2 * rz0) ? 1 : it >= max_iters ? 2 : 0;
+        }
+        __syncthreads();
+        if (sh.stop) break;
+        const double beta = sh.res;
+        for (int sl = first_slice; sl < nsl; sl += step) {
+            const int i = sl * 32 + lane;
+            cl.store_all(p + i, fma(beta, p[i], q[i]));
+        }
+        cl.sync();
+    }
+    for (int sl = first_slice; sl < nsl; sl += step) {
+        const int i = sl * 32 + lane, v = o.vert[i];
+        if (v >= 0) x[(size_t)v * K + s] = xc[i];
+    }
+    if (threadIdx.x == 0) {
+        if (sh.stop == 2) atomicOr(status, 2);
+        atomicMax(iters_out, it);
+    }
+}
+
 // distance and world tangent of target j from source column s; keep = (j != i, d < r_c)
 __global__ void k_evaluate(Op o, int K, int nsrc, int n, const int32_t* src, const int32_t* face, const double* bary,
                            const double* phi, const double* Y, double rc, double* od, double* ot, int32_t* keep) {
@@ -536,6 +853,9 @@ struct VhmOp {
     int32_t *pos = nullptr, *ej = nullptr;
     int32_t* cverts = nullptr;        // vertices grouped by colour (no two neighbours share one)
     std::vector<int32_t> cstart;      // colour c is cverts[cstart[c] .. cstart[c + 1])
+    double sum_mass = 0.0, sum_diag = 0.0;
+    Rows rows;                        // np = 0: too many vertices for the column kernels
+    void* rows_mem = nullptr;
 };
 
 void vhm_free(css_mesh* m) {
@@ -544,6 +864,7 @@ void vhm_free(css_mesh* m) {
     cudaFree(o->ang); cudaFree(o->cot); cudaFree(o->gam); cudaFree(o->area); cudaFree(o->mass);
     cudaFree(o->diag); cudaFree(o->scale); cudaFree(o->phi); cudaFree(o->ew); cudaFree(o->ec); cudaFree(o->es);
     cudaFree(o->pos); cudaFree(o->ej); cudaFree(o->cverts);
+    cudaFree(o->rows_mem);
     delete o;
     m->vhm = nullptr;
 }
@@ -560,6 +881,118 @@ namespace {
             return e__ == cudaErrorMemoryAllocation ? CSS_ERR_OOM : CSS_ERR_CUDA;                \
         }                                                                                        \
     } while (0)
+
+// Rows of the column kernels, for meshes whose fields of one column fit in a CTA's shared
+// memory (two doubles a row: about 14300 vertices)
+constexpr size_t COLUMN_SHARED_MAX = cssi::WAVE_SHARED_MAX;
+
+cudaError_t build_rows(cssi::VhmOp* o, const std::vector<int32_t>& rs, const std::vector<int32_t>& ej,
+                       const std::vector<int32_t>& order, cudaStream_t st) {
+    const int32_t nv = o->nv;
+    const int ncol = (int)o->cstart.size() - 1;
+    std::vector<int32_t> cslice(1, 0);
+    for (int c = 0; c < ncol; ++c) cslice.push_back(cslice.back() + (o->cstart[c + 1] - o->cstart[c] + 31) / 32);
+    const int nsl = cslice[ncol];
+    if ((size_t)nsl * 32 * 2 * sizeof(double) > COLUMN_SHARED_MAX) return cudaSuccess;
+    const int32_t np = nsl * 32;
+    const size_t ne = ej.size();
+    std::vector<double> ew(ne), ec(ne), es(ne), mass(nv), diag(nv);
+    cudaError_t e = cudaMemcpyAsync(ew.data(), o->ew, ne * sizeof(double), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(ec.data(), o->ec, ne * sizeof(double), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(es.data(), o->es, ne * sizeof(double), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(mass.data(), o->mass, nv * sizeof(double), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(diag.data(), o->diag, nv * sizeof(double), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return e;
+    for (int32_t v = 0; v < nv; ++v) {
+        o->sum_mass += mass[v];
+        o->sum_diag += diag[v];
+    }
+    struct Entry { int32_t j; double w, c, s; };
+    std::vector<std::vector<Entry>> row(nv);   // one entry per neighbour
+    for (int32_t v = 0; v < nv; ++v)
+        for (int32_t k = 2 * rs[v]; k < 2 * rs[v + 1]; ++k) {
+            const Entry n{ej[k], ew[k], ew[k] * ec[k], ew[k] * es[k]};
+            auto f = std::find_if(row[v].begin(), row[v].end(), [&](const Entry& q) { return q.j == n.j; });
+            if (f == row[v].end()) row[v].push_back(n);
+            else { f->w += n.w; f->c += n.c; f->s += n.s; }
+        }
+    std::vector<int32_t> vert(np, -1), rowof(nv), soff(1, 0);
+    for (int c = 0; c < ncol; ++c) {   // rows of like length share a slice
+        std::vector<int32_t> vs(order.begin() + o->cstart[c], order.begin() + o->cstart[c + 1]);
+        std::stable_sort(vs.begin(), vs.end(), [&](int32_t a, int32_t b) { return row[a].size() > row[b].size(); });
+        for (size_t k = 0; k < vs.size(); ++k) {
+            vert[cslice[c] * 32 + k] = vs[k];
+            rowof[vs[k]] = cslice[c] * 32 + (int32_t)k;
+        }
+    }
+    for (int sl = 0; sl < nsl; ++sl) {
+        size_t w = 0;
+        for (int l = 0; l < 32; ++l)
+            if (vert[sl * 32 + l] >= 0) w = std::max(w, row[vert[sl * 32 + l]].size());
+        soff.push_back(soff.back() + (int32_t)w);
+    }
+    const size_t nent = (size_t)soff[nsl] * 32;
+    std::vector<int32_t> j(nent);
+    std::vector<double> w(nent, 0.0), cs(2 * nent, 0.0), pm(np, 0.0), pd(np, 0.0);
+    for (int p = 0; p < np; ++p) {
+        const int sl = p / 32, v = vert[p];
+        for (int32_t k = 0; k < soff[sl + 1] - soff[sl]; ++k) {
+            const size_t a = (size_t)(soff[sl] + k) * 32 + p % 32;
+            j[a] = p;
+            if (v < 0 || (size_t)k >= row[v].size()) continue;
+            j[a] = rowof[row[v][k].j];
+            w[a] = row[v][k].w;
+            cs[2 * a] = row[v][k].c;
+            cs[2 * a + 1] = row[v][k].s;
+        }
+        if (v >= 0) { pm[p] = mass[v]; pd[p] = diag[v]; }
+    }
+    // one allocation, the widest items first
+    size_t off = 0;
+    auto place = [&](size_t bytes) { const size_t a = off; off += (bytes + 15) / 16 * 16; return a; };
+    const size_t a_cs = place(2 * nent * 8), a_w = place(nent * 8), a_m = place(pm.size() * 8), a_d = place(pd.size() * 8),
+                 a_j = place(nent * 4), a_v = place(vert.size() * 4), a_r = place(rowof.size() * 4),
+                 a_so = place(soff.size() * 4), a_c = place(cslice.size() * 4);
+    std::vector<unsigned char> host(off);
+    auto put = [&](size_t at, const void* src, size_t bytes) { memcpy(host.data() + at, src, bytes); };
+    put(a_cs, cs.data(), 2 * nent * 8); put(a_w, w.data(), nent * 8); put(a_m, pm.data(), pm.size() * 8);
+    put(a_d, pd.data(), pd.size() * 8); put(a_j, j.data(), nent * 4); put(a_v, vert.data(), vert.size() * 4);
+    put(a_r, rowof.data(), rowof.size() * 4); put(a_so, soff.data(), soff.size() * 4);
+    put(a_c, cslice.data(), cslice.size() * 4);
+    e = cudaMalloc(&o->rows_mem, off);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(o->rows_mem, host.data(), off, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_heat_columns, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)COLUMN_SHARED_MAX);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_cg_columns, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)COLUMN_SHARED_MAX);
+    if (e != cudaSuccess) return e;
+    const unsigned char* d = (const unsigned char*)o->rows_mem;
+    o->rows = Rows{np, ncol, (const int32_t*)(d + a_c), (const int32_t*)(d + a_so), (const int32_t*)(d + a_v),
+                   (const int32_t*)(d + a_r), (const int32_t*)(d + a_j), (const double*)(d + a_w),
+                   (const double2*)(d + a_cs), (const double*)(d + a_m), (const double*)(d + a_d)};
+    return cudaSuccess;
+}
+
+// one cluster per column: as many CTAs (1, 2, 4 or 8) as keep the vector systems within one
+// CTA per SM
+template <class... A>
+cudaError_t launch_columns(void (*kernel)(A...), int clusters, int size, size_t smem, cudaStream_t st,
+                           std::common_type_t<A>... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(clusters * size));
+    cfg.blockDim = dim3(CT);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)size;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
 
 int build_op(css_mesh* m) {
     css_ctx* c = m->ctx;
@@ -647,6 +1080,7 @@ int build_op(css_mesh* m) {
     e = cudaMalloc(&o->cverts, std::max<size_t>(nv, 1) * sizeof(int32_t));
     if (e == cudaSuccess) e = cudaMemcpyAsync(o->cverts, order.data(), (size_t)nv * sizeof(int32_t), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e == cudaSuccess) e = build_rows(o, rs, ej, order, st);
     if (e != cudaSuccess) {
         cssi::vhm_free(m);
         c->err = std::string("vhm operators: ") + cudaGetErrorString(e);
@@ -716,20 +1150,29 @@ int css_vhm_neighbors(css_parts* parts, double r_c, double t_factor, int64_t cap
     Batch B;
     const size_t VK = (size_t)nv * K;
     const int nbv = (int)vblk((int64_t)VK);
+    const Rows& R = O.rows;
+    const bool columns = R.np > 0;
     VTRY("vhm", B.get(&B.u, VK)); VTRY("vhm", B.get(&B.Y, 2 * VK));
-    VTRY("vhm", B.get(&B.bu, VK)); VTRY("vhm", B.get(&B.bY, 2 * VK));
     VTRY("vhm", B.get(&B.X, 2 * (size_t)nf * K)); VTRY("vhm", B.get(&B.b, VK)); VTRY("vhm", B.get(&B.x, VK));
-    VTRY("vhm", B.get(&B.r, VK)); VTRY("vhm", B.get(&B.z, VK)); VTRY("vhm", B.get(&B.p, VK));
-    VTRY("vhm", B.get(&B.q, VK)); VTRY("vhm", B.get(&B.partial, (size_t)nbv * K));
-    VTRY("vhm", B.get(&B.sc, 8 * (size_t)K)); VTRY("vhm", B.get(&B.src, (size_t)K));
-    VTRY("vhm", B.get(&B.ints, 2 + (size_t)K)); VTRY("vhm", B.get(&B.cnt, (size_t)K));
-    VTRY("vhm", B.get(&B.roff, (size_t)K));
+    VTRY("vhm", B.get(&B.src, (size_t)K)); VTRY("vhm", B.get(&B.ints, 3 + (size_t)K));
+    VTRY("vhm", B.get(&B.cnt, (size_t)K)); VTRY("vhm", B.get(&B.roff, (size_t)K));
     VTRY("vhm", B.get(&B.od, (size_t)K * n)); VTRY("vhm", B.get(&B.ot, 3 * (size_t)K * n));
     VTRY("vhm", B.get(&B.keep, (size_t)K * n));
-    VTRY("vhm", B.get(&B.wt, 6 * (size_t)nf)); VTRY("vhm", B.get(&B.wc, 6 * (size_t)nf));
-    VTRY("vhm", B.get(&B.wsn, 6 * (size_t)nf)); VTRY("vhm", B.get(&B.invd, (size_t)nv));
-    k_heat_entries<<<vblk(std::max<int64_t>(6 * (int64_t)nf, nv)), VT, 0, st>>>(op, t, B.wt, B.wc, B.wsn, B.invd);
+    if (columns) {
+        VTRY("vhm", B.get(&B.r, 2 * (size_t)R.np * K)); VTRY("vhm", B.get(&B.invd, 2 * (size_t)R.np));
+        k_row_scale<<<vblk(R.np), VT, 0, st>>>(R, t, B.invd, B.invd + R.np);
+    } else {
+        VTRY("vhm", B.get(&B.bu, VK)); VTRY("vhm", B.get(&B.bY, 2 * VK));
+        VTRY("vhm", B.get(&B.r, VK)); VTRY("vhm", B.get(&B.z, VK)); VTRY("vhm", B.get(&B.p, VK));
+        VTRY("vhm", B.get(&B.q, VK)); VTRY("vhm", B.get(&B.partial, (size_t)nbv * K));
+        VTRY("vhm", B.get(&B.sc, 8 * (size_t)K));
+        VTRY("vhm", B.get(&B.wt, 6 * (size_t)nf)); VTRY("vhm", B.get(&B.wc, 6 * (size_t)nf));
+        VTRY("vhm", B.get(&B.wsn, 6 * (size_t)nf)); VTRY("vhm", B.get(&B.invd, (size_t)nv));
+        k_heat_entries<<<vblk(std::max<int64_t>(6 * (int64_t)nf, nv)), VT, 0, st>>>(op, t, B.wt, B.wc, B.wsn, B.invd);
+    }
     VTRY("vhm", cudaGetLastError());
+    const double rho = t * O.sum_diag / (O.sum_mass + t * O.sum_diag);
+    const double omega = rho > 0.0 && rho < 1.0 ? 2.0 / (1.0 + std::sqrt(1.0 - rho * rho)) : 1.0;
     double* bsum = B.sc;          // K
     double* rz = B.sc + K;        // K
     double* rz0 = B.sc + 2 * K;   // K
@@ -745,7 +1188,7 @@ int css_vhm_neighbors(css_parts* parts, double r_c, double t_factor, int64_t cap
     std::vector<int64_t> rows((size_t)n + 1, 0);
     int64_t total = 0;
     int64_t iters_heat = 0, iters_cg = 0;
-    const int MAX_SWEEPS = 50000, MAX_CG = 50000, CHUNK = 16;
+    const int MAX_SWEEPS = 50000, MAX_CG = 50000, CHUNK = 16, PLAIN_AFTER = 4096;
     GraphExec chunk;
     int chunk_ns = -1;
     for (int s0 = 0; s0 < n; s0 += K) {
@@ -753,85 +1196,101 @@ int css_vhm_neighbors(css_parts* parts, double r_c, double t_factor, int64_t cap
         std::vector<int32_t> hsrc(K);
         for (int s = 0; s < K; ++s) hsrc[s] = s0 + std::min(s, ns - 1);
         VTRY("vhm", cudaMemcpyAsync(B.src, hsrc.data(), K * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-        // ---- heat steps (Gauss-Seidel sweeps from zero, colour by colour)
-        VTRY("vhm", cudaMemsetAsync(B.bu, 0, VK * sizeof(double), st));
-        VTRY("vhm", cudaMemsetAsync(B.bY, 0, 2 * VK * sizeof(double), st));
-        VTRY("vhm", cudaMemsetAsync(B.u, 0, VK * sizeof(double), st));
-        VTRY("vhm", cudaMemsetAsync(B.Y, 0, 2 * VK * sizeof(double), st));
-        k_heat_rhs<<<vblk(3 * ns), VT, 0, st>>>(op, K, ns, B.src, parts->face, parts->bary, B.bu, B.bY);
-        VTRY("vhm heat", cudaGetLastError());
         double *u = B.u, *Y = B.Y;
-        int sweeps = 0;
-        // a chunk of sweeps (one launch per colour and sweep) is captured once as a graph and
-        // replayed: on small meshes the launches, not the sweeps, would set the time
-        if (!chunk.exec || chunk_ns != ns) {
-            chunk.reset();
-            cudaGraph_t graph = nullptr;
-            VTRY("vhm capture", cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-            cudaError_t e = cudaMemsetAsync(flag, 0, sizeof(int), st);
-            const int ncol = (int)O.cstart.size() - 1;
-            for (int k = 0; k < CHUNK && e == cudaSuccess; ++k)
-                for (int cc = 0; cc < ncol; ++cc) {
-                    const int nvc = O.cstart[cc + 1] - O.cstart[cc];
-                    k_heat_gs<<<vblk((int64_t)nvc * K), VT, 0, st>>>(op, K, ns, B.wt, B.wc, B.wsn, B.invd,
-                                                                      O.cverts + O.cstart[cc], nvc, B.bu, B.bY, u, Y,
-                                                                      k == CHUNK - 1, flag);
-                }
-            if (e == cudaSuccess) e = cudaGetLastError();
-            const cudaError_t e2 = cudaStreamEndCapture(st, &graph);
-            if (e == cudaSuccess) e = e2;
-            if (e == cudaSuccess) e = cudaGraphInstantiate(&chunk.exec, graph, 0);
-            if (graph) cudaGraphDestroy(graph);
-            VTRY("vhm capture", e);
-            chunk_ns = ns;
-        }
-        for (;;) {
-            VTRY("vhm heat", cudaGraphLaunch(chunk.exec, st));
-            sweeps += CHUNK;
-            int hf = 0;
-            VTRY("vhm heat", cudaMemcpyAsync(&hf, flag, sizeof(int), cudaMemcpyDeviceToHost, st));
-            VTRY("vhm heat", cudaStreamSynchronize(st));
-            if (!hf) break;
-            if (sweeps >= MAX_SWEEPS) { c->err = "vhm: heat sweeps did not converge"; return CSS_ERR_ITER_LIMIT; }
-        }
-        iters_heat = std::max<int64_t>(iters_heat, sweeps);
-        // ---- unit field, Poisson right-hand side (mean-free), conjugate gradients
         const int nbf = (int)vblk((int64_t)nf * K);
-        k_unit_field<<<nbf, VT, 0, st>>>(op, K, u, B.X);
-        k_neg_div<<<nbv, VT, 0, st>>>(op, K, ns, B.X, B.b);
-        k_partial_of<<<nbv, VT, 0, st>>>(op, K, B.b, B.partial);
-        k_col_sum<<<K, VT, 0, st>>>(K, nbv, B.partial, bsum);
-        k_cg_start<<<nbv, VT, 0, st>>>(op, K, bsum, B.b, B.x, B.r, B.z, B.p, B.partial);
-        k_col_sum<<<K, VT, 0, st>>>(K, nbv, B.partial, rz);
-        VTRY("vhm poisson", cudaGetLastError());
-        VTRY("vhm poisson", cudaMemcpyAsync(rz0, rz, K * sizeof(double), cudaMemcpyDeviceToDevice, st));
-        {
-            std::vector<int> ha(K);
-            for (int s = 0; s < K; ++s) ha[s] = s < ns ? 1 : 0;
-            VTRY("vhm poisson", cudaMemcpyAsync(active, ha.data(), K * sizeof(int), cudaMemcpyHostToDevice, st));
-        }
-        int cg = 0;
-        for (;;) {
-            VTRY("vhm poisson", cudaMemsetAsync(nact, 0, sizeof(int), st));
-            for (int k = 0; k < CHUNK; ++k) {
-                k_cg_apply<<<nbv, VT, 0, st>>>(op, K, B.p, B.q, B.partial);
-                k_col_sum<<<K, VT, 0, st>>>(K, nbv, B.partial, pq);
-                k_cg_alpha<<<vblk(K), VT, 0, st>>>(K, rz, pq, active, alpha);
-                k_cg_step<<<nbv, VT, 0, st>>>(op, K, alpha, B.p, B.q, B.x, B.r, B.z, B.partial);
-                k_col_sum<<<K, VT, 0, st>>>(K, nbv, B.partial, rzn);
-                if (k == CHUNK - 1) VTRY("vhm poisson", cudaMemsetAsync(nact, 0, sizeof(int), st));
-                k_cg_beta<<<vblk(K), VT, 0, st>>>(K, 1e-28, rz0, rz, rzn, active, beta, nact);
-                k_cg_dir<<<nbv, VT, 0, st>>>(op, K, active, beta, B.z, B.p);
-            }
+        int hs[3] = {0, 0, 0};   // the column kernels' status, most sweeps, most iterations
+        if (columns) {
+            int size = 1;
+            while (size < CL_MAX && ns * size * 2 <= c->sm_count) size *= 2;
+            const size_t smem = 2 * sizeof(double) * (size_t)R.np;
+            VTRY("vhm", cudaMemsetAsync(B.ints, 0, sizeof(hs), st));
+            VTRY("vhm heat", launch_columns(k_heat_columns, 2 * ns, size, smem, st, op, R, K, ns, t, omega, PLAIN_AFTER,
+                                            MAX_SWEEPS, B.src, parts->face, parts->bary, B.invd, u, Y, B.ints + 1,
+                                            B.ints));
+            k_unit_field<<<nbf, VT, 0, st>>>(op, K, u, B.X);
+            k_neg_div<<<nbv, VT, 0, st>>>(op, K, ns, B.X, B.b);
             VTRY("vhm poisson", cudaGetLastError());
-            cg += CHUNK;
-            int ha = 0;
-            VTRY("vhm poisson", cudaMemcpyAsync(&ha, nact, sizeof(int), cudaMemcpyDeviceToHost, st));
-            VTRY("vhm poisson", cudaStreamSynchronize(st));
-            if (!ha) break;
-            if (cg >= MAX_CG) { c->err = "vhm: Poisson solve did not converge"; return CSS_ERR_ITER_LIMIT; }
+            VTRY("vhm poisson", launch_columns(k_cg_columns, ns, size, smem, st, R, nv, K, 1e-28, MAX_CG, B.b, B.x, B.r,
+                                               B.invd + R.np, B.ints + 2, B.ints));
+        } else {
+            // ---- heat steps (Gauss-Seidel sweeps from zero, colour by colour)
+            VTRY("vhm", cudaMemsetAsync(B.bu, 0, VK * sizeof(double), st));
+            VTRY("vhm", cudaMemsetAsync(B.bY, 0, 2 * VK * sizeof(double), st));
+            VTRY("vhm", cudaMemsetAsync(B.u, 0, VK * sizeof(double), st));
+            VTRY("vhm", cudaMemsetAsync(B.Y, 0, 2 * VK * sizeof(double), st));
+            k_heat_rhs<<<vblk(3 * ns), VT, 0, st>>>(op, K, ns, B.src, parts->face, parts->bary, B.bu, B.bY);
+            VTRY("vhm heat", cudaGetLastError());
+            int sweeps = 0;
+            // a chunk of sweeps (one launch per colour and sweep) is captured once as a graph and
+            // replayed: on small meshes the launches, not the sweeps, would set the time
+            if (!chunk.exec || chunk_ns != ns) {
+                chunk.reset();
+                cudaGraph_t graph = nullptr;
+                VTRY("vhm capture", cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
+                cudaError_t e = cudaMemsetAsync(flag, 0, sizeof(int), st);
+                const int ncol = (int)O.cstart.size() - 1;
+                for (int k = 0; k < CHUNK && e == cudaSuccess; ++k)
+                    for (int cc = 0; cc < ncol; ++cc) {
+                        const int nvc = O.cstart[cc + 1] - O.cstart[cc];
+                        k_heat_gs<<<vblk((int64_t)nvc * K), VT, 0, st>>>(op, K, ns, B.wt, B.wc, B.wsn, B.invd,
+                                                                          O.cverts + O.cstart[cc], nvc, B.bu, B.bY, u, Y,
+                                                                          k == CHUNK - 1, flag);
+                    }
+                if (e == cudaSuccess) e = cudaGetLastError();
+                const cudaError_t e2 = cudaStreamEndCapture(st, &graph);
+                if (e == cudaSuccess) e = e2;
+                if (e == cudaSuccess) e = cudaGraphInstantiate(&chunk.exec, graph, 0);
+                if (graph) cudaGraphDestroy(graph);
+                VTRY("vhm capture", e);
+                chunk_ns = ns;
+            }
+            for (;;) {
+                VTRY("vhm heat", cudaGraphLaunch(chunk.exec, st));
+                sweeps += CHUNK;
+                int hf = 0;
+                VTRY("vhm heat", cudaMemcpyAsync(&hf, flag, sizeof(int), cudaMemcpyDeviceToHost, st));
+                VTRY("vhm heat", cudaStreamSynchronize(st));
+                if (!hf) break;
+                if (sweeps >= MAX_SWEEPS) { c->err = "vhm: heat sweeps did not converge"; return CSS_ERR_ITER_LIMIT; }
+            }
+            iters_heat = std::max<int64_t>(iters_heat, sweeps);
+            // ---- unit field, Poisson right-hand side (mean-free), conjugate gradients
+            k_unit_field<<<nbf, VT, 0, st>>>(op, K, u, B.X);
+            k_neg_div<<<nbv, VT, 0, st>>>(op, K, ns, B.X, B.b);
+            k_partial_of<<<nbv, VT, 0, st>>>(op, K, B.b, B.partial);
+            k_col_sum<<<K, VT, 0, st>>>(K, nbv, B.partial, bsum);
+            k_cg_start<<<nbv, VT, 0, st>>>(op, K, bsum, B.b, B.x, B.r, B.z, B.p, B.partial);
+            k_col_sum<<<K, VT, 0, st>>>(K, nbv, B.partial, rz);
+            VTRY("vhm poisson", cudaGetLastError());
+            VTRY("vhm poisson", cudaMemcpyAsync(rz0, rz, K * sizeof(double), cudaMemcpyDeviceToDevice, st));
+            {
+                std::vector<int> ha(K);
+                for (int s = 0; s < K; ++s) ha[s] = s < ns ? 1 : 0;
+                VTRY("vhm poisson", cudaMemcpyAsync(active, ha.data(), K * sizeof(int), cudaMemcpyHostToDevice, st));
+            }
+            int cg = 0;
+            for (;;) {
+                VTRY("vhm poisson", cudaMemsetAsync(nact, 0, sizeof(int), st));
+                for (int k = 0; k < CHUNK; ++k) {
+                    k_cg_apply<<<nbv, VT, 0, st>>>(op, K, B.p, B.q, B.partial);
+                    k_col_sum<<<K, VT, 0, st>>>(K, nbv, B.partial, pq);
+                    k_cg_alpha<<<vblk(K), VT, 0, st>>>(K, rz, pq, active, alpha);
+                    k_cg_step<<<nbv, VT, 0, st>>>(op, K, alpha, B.p, B.q, B.x, B.r, B.z, B.partial);
+                    k_col_sum<<<K, VT, 0, st>>>(K, nbv, B.partial, rzn);
+                    if (k == CHUNK - 1) VTRY("vhm poisson", cudaMemsetAsync(nact, 0, sizeof(int), st));
+                    k_cg_beta<<<vblk(K), VT, 0, st>>>(K, 1e-28, rz0, rz, rzn, active, beta, nact);
+                    k_cg_dir<<<nbv, VT, 0, st>>>(op, K, active, beta, B.z, B.p);
+                }
+                VTRY("vhm poisson", cudaGetLastError());
+                cg += CHUNK;
+                int ha = 0;
+                VTRY("vhm poisson", cudaMemcpyAsync(&ha, nact, sizeof(int), cudaMemcpyDeviceToHost, st));
+                VTRY("vhm poisson", cudaStreamSynchronize(st));
+                if (!ha) break;
+                if (cg >= MAX_CG) { c->err = "vhm: Poisson solve did not converge"; return CSS_ERR_ITER_LIMIT; }
+            }
+            iters_cg += cg;
         }
-        iters_cg += cg;
         // ---- targets: distance, tangent, kept pairs in j order
         k_evaluate<<<vblk((int64_t)ns * n), VT, 0, st>>>(op, K, ns, n, B.src, parts->face, parts->bary, B.x, Y, r_c,
                                                          B.od, B.ot, B.keep);
@@ -839,7 +1298,14 @@ int css_vhm_neighbors(css_parts* parts, double r_c, double t_factor, int64_t cap
         VTRY("vhm evaluate", cudaGetLastError());
         std::vector<int64_t> hc(ns);
         VTRY("vhm evaluate", cudaMemcpyAsync(hc.data(), B.cnt, ns * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+        if (columns) VTRY("vhm evaluate", cudaMemcpyAsync(hs, B.ints, sizeof(hs), cudaMemcpyDeviceToHost, st));
         VTRY("vhm evaluate", cudaStreamSynchronize(st));
+        if (hs[0]) {
+            c->err = hs[0] & 1 ? "vhm: heat sweeps did not converge" : "vhm: Poisson solve did not converge";
+            return CSS_ERR_ITER_LIMIT;
+        }
+        iters_heat = std::max<int64_t>(iters_heat, hs[1]);
+        iters_cg += hs[2];
         int64_t bt = 0;
         std::vector<int64_t> off(ns);
         for (int s = 0; s < ns; ++s) {
