@@ -237,20 +237,40 @@ cudaError_t record_ev(css_ctx* c, cudaEvent_t ev) {
     return cudaEventRecord(ev, c->stream);
 }
 
-// the two passes over a work queue, timed by the context's events (no synchronisation)
-int enqueue_passes(css_ctx* c, const GeoJob& j0, const GeoJob* djobs, const int32_t* job_of_item,
-                   const int32_t* src_of_item, int32_t nitems, int prec, const GeoPlan& P) {
+// The two passes over a work queue whose counters are zero, timed by the context's events (no
+// synchronisation).
+int enqueue_pass1(css_ctx* c, const GeoJob& j0, const GeoJob* djobs, const int32_t* job_of_item,
+                  const int32_t* src_of_item, int32_t nitems, int prec, const GeoPlan& P) {
     cudaStream_t st = c->stream;
-    TRY(c, "reset", cudaMemsetAsync(c->dscal, 0, sizeof(int), st));
-    TRY(c, "reset", cudaMemsetAsync(c->dscal + 2, 0, 2 * sizeof(int), st));
     TRY(c, "event", record_ev(c, c->ev_geo0));
     cssi::GeoQueue q1{job_of_item, src_of_item, nitems, nullptr, nullptr, c->defer, c->dscal + 2, P.tile};
     TRY(c, "geodesic", cssi::launch_waves(j0, djobs, q1, prec, P.g1, P.wpc1, P.nctas1, c->dscal, c->dscal + 1,
                                           c->dcount, st));
+    return CSS_OK;
+}
+
+int enqueue_pass2(css_ctx* c, const GeoJob& j0, const GeoJob* djobs, const int32_t* job_of_item,
+                  const int32_t* src_of_item, int32_t nitems, int prec, const GeoPlan& P) {
+    cudaStream_t st = c->stream;
     cssi::GeoQueue q2{job_of_item, src_of_item, nitems, c->defer, c->dscal + 2, nullptr, nullptr, 1};
     TRY(c, "geodesic", cssi::launch_waves(j0, djobs, q2, prec, P.g2, P.wpc2, P.nctas2, c->dscal + 3, c->dscal + 1,
                                           c->dcount, st));
+    return CSS_OK;
+}
+
+int enqueue_passes(css_ctx* c, const GeoJob& j0, const GeoJob* djobs, const int32_t* job_of_item,
+                   const int32_t* src_of_item, int32_t nitems, int prec, const GeoPlan& P) {
+    int rc = enqueue_pass1(c, j0, djobs, job_of_item, src_of_item, nitems, prec, P);
+    if (rc == CSS_OK) rc = enqueue_pass2(c, j0, djobs, job_of_item, src_of_item, nitems, prec, P);
+    if (rc) return rc;
     TRY(c, "event", record_ev(c, c->ev_geo1));
+    return CSS_OK;
+}
+
+int enqueue_bucket(css_parts* p, int* queue, double* epot) {
+    css_ctx* c = p->ctx;
+    TRY(c, "bucket", cssi::launch_bucket((int32_t)p->n, (int32_t)p->mesh->nf, p->face, p->mesh->frank, p->fcnt, p->fstart,
+                                         p->fitems, p->ftmp, p->scan_tmp, queue, epot, c->stream));
     return CSS_OK;
 }
 
@@ -258,18 +278,27 @@ int enqueue_passes(css_ctx* c, const GeoJob& j0, const GeoJob* djobs, const int3
 int enqueue_geo(css_parts* p, double rc, int prec, int want_pairs, int want_forces, const css_potential* pot,
                 const GeoPlan& P) {
     css_ctx* c = p->ctx;
-    TRY(c, "bucket", cssi::launch_bucket((int32_t)p->n, (int32_t)p->mesh->nf, p->face, p->mesh->frank, p->fcnt, p->fstart, p->fitems, p->ftmp,
-                                         p->scan_tmp, c->stream));
+    int r = enqueue_bucket(p, c->dscal, c->depot);
+    if (r) return r;
     GeoJob j = make_job(p, rc, want_pairs, want_forces, pot);
     return enqueue_passes(c, j, nullptr, nullptr, nullptr, (int32_t)p->n, prec, P);
 }
 
+// status and counters to zero, before an evaluation or a run of steps
+int reset_status(css_ctx* c) {
+    TRY(c, "reset", cudaMemsetAsync(c->dscal, 0, 4 * sizeof(int) + 8 * sizeof(unsigned long long), c->stream));
+    return CSS_OK;
+}
+
+const double* host_epot(const css_ctx* c) { return (const double*)((const char*)c->hstat + ((char*)c->depot - (char*)c->dscal)); }
+const int64_t* host_total(const css_ctx* c) { return (const int64_t*)((const char*)c->hstat + ((char*)c->dtotal - (char*)c->dscal)); }
+
 int read_status(css_ctx* c, int* status) {
-    TRY(c, "status", cudaMemcpyAsync(c->hstat, c->dscal + 1, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-    TRY(c, "status", cudaMemcpyAsync(c->hcount, c->dcount, 8 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream));
+    TRY(c, "status", cudaMemcpyAsync(c->hstat, c->dscal, cssi::SCALAR_BYTES, cudaMemcpyDeviceToHost, c->stream));
     TRY(c, "sync", cudaStreamSynchronize(c->stream));
-    *status = *c->hstat;
-    for (int k = 0; k < 5; ++k) c->last_counters[k] = (int64_t)c->hcount[k];
+    *status = c->hstat[1];
+    const unsigned long long* count = (const unsigned long long*)(c->hstat + 4);
+    for (int k = 0; k < 5; ++k) c->last_counters[k] = (int64_t)count[k];
     return CSS_OK;
 }
 
@@ -309,8 +338,12 @@ void adapt_default(css_ctx* c) {
     if (done > 0 && deferred * 25 > done && c->auto_level < 8) ++c->auto_level;
 }
 
-// synchronous neighbour / force evaluation with overflow retries
-int run_geo(css_parts* p, double rc, int prec, int want_pairs, int want_forces, const css_potential* pot) {
+// Synchronous neighbour / force evaluation with overflow retries.  after() enqueues what the
+// caller reads with the status.  The second pass is launched only if the first deferred
+// a source, which costs a second synchronisation then; a context whose last evaluation deferred
+// some launches both at once.
+template <class Fn>
+int run_geo(css_parts* p, double rc, int prec, int want_pairs, int want_forces, const css_potential* pot, Fn after) {
     css_ctx* c = p->ctx;
     int retries = 0;
     c->last_counters[5] = 0;
@@ -321,14 +354,29 @@ int run_geo(css_parts* p, double rc, int prec, int want_pairs, int want_forces, 
         R.add(p, rc);
         int rc1 = ensure_plan(c, prec, p->n, R, &P);
         if (rc1) return rc1;
-        TRY(c, "reset", cudaMemsetAsync(c->dcount, 0, 8 * sizeof(unsigned long long), c->stream));
-        TRY(c, "reset", cudaMemsetAsync(c->dscal + 1, 0, sizeof(int), c->stream));
-        TRY(c, "reset", cudaMemsetAsync(c->depot, 0, sizeof(double), c->stream));
-        rc1 = enqueue_geo(p, rc, prec, want_pairs, want_forces, pot, P);
+        const bool both = c->last_counters[4] > 0;
+        rc1 = reset_status(c);
+        if (rc1 == CSS_OK) rc1 = enqueue_bucket(p, c->dscal, c->depot);
+        if (rc1) return rc1;
+        GeoJob j = make_job(p, rc, want_pairs, want_forces, pot);
+        const int32_t n = (int32_t)p->n;
+        rc1 = enqueue_pass1(c, j, nullptr, nullptr, nullptr, n, prec, P);
+        if (rc1 == CSS_OK && both) rc1 = enqueue_pass2(c, j, nullptr, nullptr, nullptr, n, prec, P);
+        if (rc1) return rc1;
+        TRY(c, "event", record_ev(c, c->ev_geo1));
+        rc1 = after();
         if (rc1) return rc1;
         int status = 0;
         rc1 = read_status(c, &status);
         if (rc1) return rc1;
+        if (!both && status == 0 && c->hstat[2] > 0) {
+            rc1 = enqueue_pass2(c, j, nullptr, nullptr, nullptr, n, prec, P);
+            if (rc1) return rc1;
+            TRY(c, "event", record_ev(c, c->ev_geo1));
+            rc1 = after();
+            if (rc1 == CSS_OK) rc1 = read_status(c, &status);
+            if (rc1) return rc1;
+        }
         if (status == 0) { adapt_default(c); return CSS_OK; }
         if (!grow_for(c, status, &retries)) return status_error(c, status);
     }
@@ -373,11 +421,8 @@ int css_create(css_ctx** out, int device, void* stream) {
         c->own_stream = 1;
     }
     c->sm_count = prop.multiProcessorCount;
-    if (cudaMalloc(&c->dscal, 4 * sizeof(int)) != cudaSuccess ||
-        cudaMalloc(&c->dcount, 8 * sizeof(unsigned long long)) != cudaSuccess ||
-        cudaMalloc(&c->depot, sizeof(double)) != cudaSuccess ||
-        cudaMallocHost(&c->hstat, 4 * sizeof(int)) != cudaSuccess ||
-        cudaMallocHost(&c->hcount, 8 * sizeof(unsigned long long)) != cudaSuccess) {
+    if (cudaMalloc(&c->dscal, cssi::SCALAR_BYTES) != cudaSuccess ||
+        cudaMallocHost(&c->hstat, 128 + cssi::BOUNCE_BYTES) != cudaSuccess) {
         css_destroy(c);
         return CSS_ERR_OOM;
     }
@@ -386,8 +431,14 @@ int css_create(css_ctx** out, int device, void* stream) {
         css_destroy(c);
         return CSS_ERR_CUDA;
     }
-    cudaMemset(c->dscal, 0, 4 * sizeof(int));
-    cudaMemset(c->dcount, 0, 8 * sizeof(unsigned long long));
+    c->bounce = (unsigned char*)c->hstat + 128;
+    c->dcount = (unsigned long long*)(c->dscal + 4);
+    c->depot = (double*)(c->dcount + 8);
+    c->dtotal = (int64_t*)(c->depot + 1);
+    if (cudaMemset(c->dscal, 0, cssi::SCALAR_BYTES) != cudaSuccess || cssi::dynamics_setup() != cudaSuccess) {
+        css_destroy(c);
+        return CSS_ERR_CUDA;
+    }
     *out = c;
     return CSS_OK;
 }
@@ -398,10 +449,7 @@ int css_destroy(css_ctx* c) {
     cudaFree(c->ws2.ws);
     cudaFree(c->defer);
     cudaFree(c->dscal);
-    cudaFree(c->dcount);
-    cudaFree(c->depot);
     cudaFreeHost(c->hstat);
-    cudaFreeHost(c->hcount);
     if (c->ev_geo0) cudaEventDestroy(c->ev_geo0);
     if (c->ev_geo1) cudaEventDestroy(c->ev_geo1);
     if (c->ev_order) cudaEventDestroy(c->ev_order);
@@ -573,6 +621,7 @@ int css_particles_set(css_ctx* c, css_mesh* m, int64_t n, const int32_t* face, c
     if (e == cudaSuccess) e = cudaMalloc(&p->ftmp, n * sizeof(int32_t));
     if (e == cudaSuccess) e = cudaMalloc(&p->scan_tmp, cssi::scan_tmp_ints(nf + 1) * sizeof(int32_t));
     if (e == cudaSuccess) e = cudaMalloc(&p->pcnt, n * sizeof(int32_t));
+    if (e == cudaSuccess) e = cudaMalloc(&p->rows, (n + 1 + cssi::scan_tmp_ints(n + 1)) * sizeof(int64_t));
     if (e == cudaSuccess) e = cudaMalloc(&p->dstep, sizeof(int64_t));
     if (e == cudaSuccess) e = cudaMalloc(&p->dfire, 16 * sizeof(double));
     if (e == cudaSuccess) e = cudaMemsetAsync(p->dstep, 0, sizeof(int64_t), st);
@@ -668,50 +717,80 @@ int css_particles_free(css_parts* p) {
     cudaFree(p->state); cudaFree(p->snap);
     cudaFree(p->fcnt); cudaFree(p->fstart); cudaFree(p->fitems); cudaFree(p->ftmp); cudaFree(p->scan_tmp); cudaFree(p->order);
     cudaFree(p->pcnt); cudaFree(p->pj); cudaFree(p->pd); cudaFree(p->pt); cudaFree(p->dstep); cudaFree(p->dfire);
+    cudaFree(p->rows); cudaFree(p->stage);
     delete p;
     return CSS_OK;
 }
 
+
+constexpr size_t STAGE_KEEP = 64u << 20;
 
 int css_geodesic_neighbors(css_parts* p, double r_c, int precision, int64_t capacity, int64_t* n_pairs,
                            int64_t* row_start, int32_t* nbr_j, double* dist, double* tangent) {
     Range range_("css_geodesic_neighbors");
     if (!p || !n_pairs || bad_prec(precision) || bad_rc(r_c) || capacity < 0) return CSS_ERR_INVALID_ARG;
     css_ctx* c = p->ctx;
-    int rc = run_geo(p, r_c, precision, 1, 0, nullptr);
-    if (rc) return rc;
     cudaStream_t st = c->stream;
     const int32_t n = (int32_t)p->n;
-    int64_t* drows = nullptr;
-    TRY(c, "neighbors", cudaMalloc(&drows, (n + 1 + cssi::scan_tmp_ints(n + 1)) * sizeof(int64_t)));
-    cudaError_t e = cssi::launch_scan_rows(p->pcnt, drows, n, st);
-    int64_t total = 0;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&total, drows + n, sizeof(int64_t), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) { cudaFree(drows); return cuda_fail(c, "neighbors", e); }
+    int rc = run_geo(p, r_c, precision, 1, 0, nullptr, [&]() -> int {
+        TRY(c, "neighbors", cssi::launch_scan_rows(p->pcnt, p->rows, c->dtotal, n, st));
+        return CSS_OK;
+    });
+    if (rc) return rc;
+    const int64_t total = *host_total(c);
     *n_pairs = total;
-    if (total > capacity) { cudaFree(drows); c->err = "neighbors: capacity too small"; return CSS_ERR_CAPACITY; }
-    if (!row_start || (total > 0 && (!nbr_j || !dist || !tangent))) { cudaFree(drows); return CSS_ERR_INVALID_ARG; }
-    const bool dev_out = is_device_ptr(nbr_j) && is_device_ptr(dist) && is_device_ptr(tangent);
+    if (total > capacity) { c->err = "neighbors: capacity too small"; return CSS_ERR_CAPACITY; }
+    if (!row_start || (total > 0 && (!nbr_j || !dist || !tangent))) return CSS_ERR_INVALID_ARG;
+    const int ndev = (int)is_device_ptr(nbr_j) + (int)is_device_ptr(dist) + (int)is_device_ptr(tangent);
+    const bool dev_out = ndev == 3;
     int32_t* oj = nbr_j;
     double* od = dist;
     double* ot = tangent;
-    if (!dev_out && total > 0) {
-        e = cudaMalloc(&oj, total * sizeof(int32_t));
-        if (e == cudaSuccess) e = cudaMalloc(&od, total * sizeof(double));
-        if (e == cudaSuccess) e = cudaMalloc(&ot, 3 * total * sizeof(double));
-        if (e != cudaSuccess) { cudaFree(drows); return cuda_fail(c, "neighbors", e); }
+    const size_t bytes = (size_t)total * (4 * sizeof(double) + sizeof(int32_t)), row_bytes = ((size_t)n + 1) * sizeof(int64_t);
+    if (!dev_out && total > 0) {   // packed rows, kept with the set up to STAGE_KEEP bytes
+        if (p->stage_bytes < bytes) {
+            cudaFree(p->stage);
+            p->stage = nullptr;
+            p->stage_bytes = 0;
+            TRY(c, "neighbors", cudaMalloc(&p->stage, bytes + bytes / 4));
+            p->stage_bytes = bytes + bytes / 4;
+        }
+        ot = (double*)p->stage;
+        od = ot + 3 * total;
+        oj = (int32_t*)(od + total);
     }
-    if (total > 0) e = cssi::launch_pairs_compact(n, p->pcnt, p->pj, p->pd, p->pt, p->pair_cap_alloc, drows, oj, od, ot, st);
-    if (e == cudaSuccess) e = copy_out(row_start, drows, (size_t)n + 1, st);
-    if (!dev_out && total > 0) {
-        if (e == cudaSuccess) e = cudaMemcpyAsync(nbr_j, oj, total * sizeof(int32_t), cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(dist, od, total * sizeof(double), cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(tangent, ot, 3 * total * sizeof(double), cudaMemcpyDeviceToHost, st);
+    cudaError_t e = cudaSuccess;
+    if (total > 0) e = cssi::launch_pairs_compact(n, p->pcnt, p->pj, p->pd, p->pt, p->pair_cap_alloc, p->rows, oj, od, ot, st);
+    // small results cross in one pinned piece, larger ones by themselves
+    const bool small = ndev == 0 && bytes + row_bytes <= cssi::BOUNCE_BYTES && !is_device_ptr(row_start);
+    if (small) {
+        unsigned char* h = c->bounce;
+        if (e == cudaSuccess) e = cudaMemcpyAsync(h, p->rows, row_bytes, cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess && total > 0) e = cudaMemcpyAsync(h + row_bytes, p->stage, bytes, cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (e == cudaSuccess) {
+            memcpy(row_start, h, row_bytes);
+            h += row_bytes;
+            if (total > 0) {
+                memcpy(tangent, h, 3 * total * sizeof(double));
+                memcpy(dist, h + 3 * total * sizeof(double), total * sizeof(double));
+                memcpy(nbr_j, h + 4 * total * sizeof(double), total * sizeof(int32_t));
+            }
+        }
+    } else {
+        if (e == cudaSuccess) e = copy_out(row_start, p->rows, (size_t)n + 1, st);
+        if (!dev_out && total > 0) {
+            if (e == cudaSuccess) e = cudaMemcpyAsync(nbr_j, oj, total * sizeof(int32_t), cudaMemcpyDeviceToHost, st);
+            if (e == cudaSuccess) e = cudaMemcpyAsync(dist, od, total * sizeof(double), cudaMemcpyDeviceToHost, st);
+            if (e == cudaSuccess) e = cudaMemcpyAsync(tangent, ot, 3 * total * sizeof(double), cudaMemcpyDeviceToHost, st);
+        }
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (!dev_out && total > 0) { cudaFree(oj); cudaFree(od); cudaFree(ot); }
-    cudaFree(drows);
+    if (p->stage_bytes > STAGE_KEEP) {
+        cudaFree(p->stage);
+        p->stage = nullptr;
+        p->stage_bytes = 0;
+    }
     if (e != cudaSuccess) return cuda_fail(c, "neighbors", e);
     return CSS_OK;
 }
@@ -720,15 +799,23 @@ int css_compute_forces(css_parts* p, const css_potential* pot, double r_c, int p
     Range range_("css_compute_forces");
     if (!p || !pot || bad_prec(precision) || bad_rc(r_c) || pot->kind < 0 || pot->kind > 2) return CSS_ERR_INVALID_ARG;
     css_ctx* c = p->ctx;
-    int rc = run_geo(p, r_c, precision, 0, 1, pot);
+    const size_t bytes = 3 * (size_t)p->n * sizeof(double);
+    const bool small = forces && bytes <= cssi::BOUNCE_BYTES && !is_device_ptr(forces);
+    int rc = run_geo(p, r_c, precision, 0, 1, pot, [&]() -> int {   // small results come with the status
+        if (small) TRY(c, "forces", cudaMemcpyAsync(c->bounce, p->force, bytes, cudaMemcpyDeviceToHost, c->stream));
+        return CSS_OK;
+    });
     if (rc) return rc;
     p->force_valid = 1;
     p->force_rc = r_c;
     p->force_prec = precision;
     p->force_pot = *pot;
-    TRY(c, "forces", copy_out(forces, p->force, 3 * p->n, c->stream));
-    if (e_pot) TRY(c, "forces", cudaMemcpyAsync(e_pot, c->depot, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    TRY(c, "forces", cudaStreamSynchronize(c->stream));
+    if (small) memcpy(forces, c->bounce, bytes);
+    else if (forces) {
+        TRY(c, "forces", copy_out(forces, p->force, 3 * p->n, c->stream));
+        TRY(c, "forces", cudaStreamSynchronize(c->stream));
+    }
+    if (e_pot) *e_pot = *host_epot(c);
     return CSS_OK;
 }
 
@@ -783,7 +870,6 @@ int enqueue_step(css_parts* p, const css_potential* pot, const css_integrator* i
     css_ctx* c = p->ctx;
     int r = enqueue_move(p, it, noise, 0);
     if (r) return r;
-    TRY(c, "reset", cudaMemsetAsync(c->depot, 0, sizeof(double), c->stream));
     r = enqueue_geo(p, rc, prec, 0, 1, pot, P);
     if (r) return r;
     return enqueue_move(p, it, noise, 1);
@@ -856,8 +942,8 @@ int css_integrate_step(css_parts* p, const css_potential* pot, const css_integra
         R.add(p, r_c);
         rc = ensure_plan(c, precision, p->n, R, &P);
         if (rc) break;
-        TRY(c, "reset", cudaMemsetAsync(c->dscal + 1, 0, sizeof(int), st));
-        TRY(c, "reset", cudaMemsetAsync(c->dcount, 0, 8 * sizeof(unsigned long long), st));
+        rc = reset_status(c);
+        if (rc) break;
         if (!dnoise) {
             // one captured step, kept with the parameters it was captured for, replayed
             std::string key((const char*)pot, sizeof(*pot));
@@ -892,10 +978,7 @@ int css_integrate_step(css_parts* p, const css_potential* pot, const css_integra
     p->force_rc = r_c;
     p->force_prec = precision;
     p->force_pot = *pot;
-    if (e_pot) {
-        TRY(c, "e_pot", cudaMemcpyAsync(e_pot, c->depot, sizeof(double), cudaMemcpyDeviceToHost, st));
-        TRY(c, "e_pot", cudaStreamSynchronize(st));
-    }
+    if (e_pot) *e_pot = *host_epot(c);
     return CSS_OK;
 }
 
@@ -976,8 +1059,8 @@ namespace {
 int batch_enqueue_forces(css_batch* b, const css_potential* pot, double rc, int prec, const GeoPlan& P) {
     css_ctx* c = b->ctx;
     cudaStream_t st = c->stream;
-    TRY(c, "bucket", cssi::launch_batch_bucket(b->dviews, b->doffs, (int)b->sets.size(), b->nitems, st));
-    TRY(c, "reset", cudaMemsetAsync(c->depot, 0, sizeof(double), st));
+    TRY(c, "bucket", cssi::launch_batch_bucket(b->dviews, b->doffs, (int)b->sets.size(), b->nitems,
+                                                     c->dscal, c->depot, st));
     GeoJob j0 = make_job(b->sets[0], rc, 0, 1, pot);
     return enqueue_passes(c, j0, b->djobs, b->job_of_item, b->src_of_item, b->nitems, prec, P);
 }
@@ -1017,8 +1100,8 @@ int css_batch_step(css_batch* b, const css_potential* pot, const css_integrator*
         for (const css_parts* p : b->sets) R.add(p, r_c);
         int rc = ensure_plan(c, precision, b->nitems, R, &P);
         if (rc) return rc;
-        TRY(c, "reset", cudaMemsetAsync(c->dscal + 1, 0, sizeof(int), st));
-        TRY(c, "reset", cudaMemsetAsync(c->dcount, 0, 8 * sizeof(unsigned long long), st));
+        rc = reset_status(c);
+        if (rc) return rc;
         if (nve) {   // forces at the starting positions
             rc = batch_enqueue_forces(b, pot, r_c, precision, P);
             if (rc) return rc;
@@ -1078,8 +1161,8 @@ int tune_run(css_ctx* c, const GeoJob* djobs, const GeoJob& j0, const int32_t* j
         GeoPlan P;
         int rc = ensure_plan(c, prec, nitems, Reach(), &P);
         if (rc) return rc;
-        TRY(c, "reset", cudaMemsetAsync(c->dscal + 1, 0, sizeof(int), c->stream));
-        TRY(c, "reset", cudaMemsetAsync(c->dcount, 0, 8 * sizeof(unsigned long long), c->stream));
+        rc = reset_status(c);
+        if (rc) return rc;
         TRY(c, "reset", cudaMemsetAsync(c->depot, 0, sizeof(double), c->stream));
         rc = enqueue_passes(c, j0, djobs, job_of_item, src_of_item, nitems, prec, P);
         if (rc) return rc;
@@ -1130,7 +1213,7 @@ int css_autotune(css_ctx* c, css_parts* const* sets, int32_t n_sets, const css_p
     for (int k = 0; k < n_sets && e == cudaSuccess; ++k) {
         css_parts* p = sets[k];
         e = cssi::launch_bucket((int32_t)p->n, (int32_t)p->mesh->nf, p->face, p->mesh->frank, p->fcnt, p->fstart, p->fitems, p->ftmp,
-                                p->scan_tmp, st);
+                                p->scan_tmp, nullptr, nullptr, st);
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) { cleanup(); return cuda_fail(c, "autotune", e); }
@@ -1378,15 +1461,15 @@ int run_path_kernel(css_parts* p, double rc, const std::vector<int32_t>& us, con
     g.occupancy = 1;
     g.lbase = lbase;
     g.lstride = lstride;
-    TRY(c, "bucket", cssi::launch_bucket((int32_t)p->n, (int32_t)p->mesh->nf, p->face, p->mesh->frank, p->fcnt,
-                                         p->fstart, p->fitems, p->ftmp, p->scan_tmp, st));
+    int rc1 = enqueue_bucket(p, nullptr, nullptr);
+    if (rc1) return rc1;
     GeoJob j = make_job(p, rc, 1, 0, nullptr);
     j.order = dus;
     j.lmax = PATH_MAX_LEGS;
     j.lnum = dlnum; j.lfk = dlfk; j.ldir = dldir; j.llen = dllen;
     cssi::GeoQueue q{nullptr, nullptr, nus, nullptr, nullptr, nullptr, nullptr, 1};
-    TRY(c, "reset", cudaMemsetAsync(c->dscal, 0, 2 * sizeof(int), st));
-    TRY(c, "reset", cudaMemsetAsync(c->dcount, 0, 8 * sizeof(unsigned long long), st));
+    rc1 = reset_status(c);
+    if (rc1) return rc1;
     TRY(c, "paths", cssi::launch_geodesic_links(j, q, g, wpc, nwarps / wpc, c->dscal, c->dscal + 1, c->dcount, st));
     return read_status(c, status);
 }

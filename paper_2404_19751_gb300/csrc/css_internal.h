@@ -50,13 +50,14 @@ struct css_ctx {
     // deferral list of the first pass (one entry per work item at most)
     int32_t* defer = nullptr;
     int64_t defer_cap = 0;
-    // small device scalars: [0] first-pass work counter, [1] status, [2] deferred count,
-    // [3] second-pass work counter
+    // one block of small device scalars and its pinned mirror, read in one copy: dscal [0] first-pass
+    // work counter, [1] status, [2] deferred count, [3] second-pass work counter
     int* dscal = nullptr;
-    unsigned long long* dcount = nullptr;   // 8 counters
-    double* depot = nullptr;
-    int* hstat = nullptr;                   // pinned mirror of status
-    unsigned long long* hcount = nullptr;   // pinned mirror of counters
+    unsigned long long* dcount = nullptr;   // 8 counters, behind dscal
+    double* depot = nullptr;                // potential energy, behind dcount
+    int64_t* dtotal = nullptr;              // pairs of a neighbour call, behind depot
+    int* hstat = nullptr;                   // the mirror, 128 bytes, and
+    unsigned char* bounce = nullptr;        // BOUNCE_BYTES for small results on their way to the host, behind it
     int64_t last_counters[6] = {0, 0, 0, 0, 0, 0};
     cudaEvent_t ev_geo0 = nullptr, ev_geo1 = nullptr;   // around the neighbour/force kernel
     int ev_valid = 0;
@@ -66,6 +67,8 @@ struct css_ctx {
 };
 
 namespace cssi {
+constexpr size_t SCALAR_BYTES = 4 * sizeof(int) + 8 * sizeof(unsigned long long) + sizeof(double) + sizeof(int64_t);
+constexpr size_t BOUNCE_BYTES = 512u << 10;
 struct VhmOp;   // operators of the approximate solver (vhm.cu), built on first use
 void vhm_free(css_mesh* m);
 }  // namespace cssi
@@ -133,6 +136,9 @@ struct css_parts {
     double* pd = nullptr;
     double* pt = nullptr;
     int pair_cap_alloc = 0;
+    int64_t* rows = nullptr;    // row starts of a neighbour call, n + 1 and the scan's scratch
+    void* stage = nullptr;      // packed rows on their way to the host (STAGE_KEEP bytes at most are kept)
+    size_t stage_bytes = 0;
     // captured single-step graph and the launch parameters it was captured for
     cudaGraphExec_t graph = nullptr;
     std::string graph_key;
@@ -277,12 +283,15 @@ cudaError_t launch_pairs_compact(int32_t n, const int32_t* pcnt, const int32_t* 
 // face), fitems lists the particles in rank order
 // face buckets of n particles: counts, offsets, then the particles of each face in index
 // order (ftmp: n ints of scratch for the unordered scatter)
+cudaError_t dynamics_setup();   // once per device, before the launches below
+// queue (of GeoQueue counters: [0], [2], [3]) and epot, where given, are set to zero on the way
 cudaError_t launch_bucket(int32_t n, int32_t nf, const int32_t* face, const int32_t* frank, int32_t* fcnt,
-                          int32_t* fstart, int32_t* fitems, int32_t* ftmp, int32_t* scan_tmp, cudaStream_t st);
+                          int32_t* fstart, int32_t* fitems, int32_t* ftmp, int32_t* scan_tmp, int* queue, double* epot,
+                          cudaStream_t st);
 size_t scan_tmp_ints(int64_t count);
 cudaError_t launch_scan_i32(const int32_t* in, int32_t* out_excl, int64_t count, int32_t* tmp,
                             cudaStream_t st);
-cudaError_t launch_scan_rows(const int32_t* cnt, int64_t* row_start, int32_t n, cudaStream_t st);
+cudaError_t launch_scan_rows(const int32_t* cnt, int64_t* row_start, int64_t* total, int32_t n, cudaStream_t st);
 cudaError_t launch_nve_kick_drift(const css::DMesh& m, int32_t n, int32_t* face, double* bary,
                                   double* vel, const double* force, css_integrator it, int* status,
                                   cudaStream_t st);
@@ -312,7 +321,8 @@ cudaError_t launch_state_diff(int32_t n, const int32_t* nf, const int32_t* of, c
                               const double* nv, const double* ov, int* flag, cudaStream_t st);
 // batched forms over the sets of a batch: item k belongs to set s with offs[s] <= k < offs[s+1]
 // (offs has nsets + 1 entries on the device; total = offs[nsets])
-cudaError_t launch_batch_bucket(const SetView* sv, const int32_t* offs, int nsets, int64_t total, cudaStream_t st);
+cudaError_t launch_batch_bucket(const SetView* sv, const int32_t* offs, int nsets, int64_t total, int* queue, double* epot,
+                                cudaStream_t st);
 cudaError_t launch_batch_move(const SetView* sv, const int32_t* offs, int nsets, int64_t total, css_integrator it,
                               int half, int* status, cudaStream_t st);
 

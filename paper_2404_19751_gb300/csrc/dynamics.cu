@@ -97,8 +97,14 @@ __global__ void k_tile_apply(const Ti* in, int64_t n_in, int64_t n, const To* su
 }
 
 // ------------------------------------------------------------------ bucketing (face CSR)
-__global__ void k_count(int32_t n, const int32_t* face, const int32_t* frank, int32_t* cnt) {
+__device__ __forceinline__ void reset_queue(int* queue, double* epot) {
+    if (queue) queue[0] = queue[2] = queue[3] = 0;
+    if (epot) *epot = 0.0;
+}
+
+__global__ void k_count(int32_t n, const int32_t* face, const int32_t* frank, int32_t* cnt, int* queue, double* epot) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0) reset_queue(queue, epot);
     if (i < n) atomicAdd(cnt + (frank ? frank[face[i]] : face[i]), 1);
 }
 
@@ -134,8 +140,7 @@ __device__ __forceinline__ void heap_sift(int32_t* a, int root, int end) {
     a[root] = v;
 }
 
-__device__ __forceinline__ void rank_in_bucket(int i, int key, const int32_t* start, const int32_t* tmp, int32_t* items) {
-    const int st = start[key], cnt = start[key + 1] - st;
+__device__ __forceinline__ void rank_in_bucket(int i, int st, int cnt, const int32_t* tmp, int32_t* items) {
     if (cnt <= RANK_SCAN) {
         int r = 0;
         for (int q = 0; q < cnt; ++q) r += tmp[st + q] < i;
@@ -158,7 +163,112 @@ __global__ void k_rank(int32_t n, const int32_t* face, const int32_t* frank, con
                        int32_t* items) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    rank_in_bucket(i, frank ? frank[face[i]] : face[i], start, tmp, items);
+    const int key = frank ? frank[face[i]] : face[i];
+    rank_in_bucket(i, start[key], start[key + 1] - start[key], tmp, items);
+}
+
+// The whole bucketing of a small set in one CTA: counts, unranked buckets and the scan in its
+// shared memory, each thread's particles and their faces' ranks in registers.  The six
+// launches above take about 3 us each whatever they do.  Bound by latency: two dependent
+// loads a particle, one pass over the counts for the sums of each thread's run of quads (an
+// odd number of them, so that a warp's reads meet no bank twice) and one for the prefix.
+constexpr int CTA_BUCKET_FACES = 32768;
+constexpr int CTA_BUCKET_ITEMS = 4096;
+__host__ __device__ inline int cta_bucket_quads(int nf) { return (nf + 1 + 4 * SCAN_THREADS - 1) / (4 * SCAN_THREADS) | 1; }
+
+__global__ void __launch_bounds__(SCAN_THREADS) k_bucket_cta(int32_t n, int32_t nf, const int32_t* face,
+                                                             const int32_t* frank, int32_t* start, int32_t* items,
+                                                             int* queue, double* epot) {
+    extern __shared__ __align__(16) int32_t cnt[];   // the counts, then the buckets before they are ranked
+    __shared__ int32_t sh[SCAN_THREADS / 32];
+    constexpr int PER = CTA_BUCKET_ITEMS / SCAN_THREADS;
+    const int t = threadIdx.x, quads = cta_bucket_quads(nf);
+    int32_t* tmp = cnt + 4 * SCAN_THREADS * quads;
+    if (t == 0) reset_queue(queue, epot);
+    int key[PER];
+#pragma unroll
+    for (int k = 0; k < PER; ++k) key[k] = t + k * SCAN_THREADS < n ? face[t + k * SCAN_THREADS] : -1;
+    int4* cnt4 = (int4*)cnt;
+    for (int b = t; b < quads * SCAN_THREADS; b += SCAN_THREADS) cnt4[b] = make_int4(0, 0, 0, 0);
+    if (frank) {
+#pragma unroll
+        for (int k = 0; k < PER; ++k)
+            if (key[k] >= 0) key[k] = frank[key[k]];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < PER; ++k)
+        if (key[k] >= 0) atomicAdd(cnt + key[k], 1);
+    __syncthreads();
+    int4* mine = cnt4 + t * quads;
+    int32_t sum = 0;
+    for (int q = 0; q < quads; ++q) {
+        const int4 c = mine[q];
+        sum += c.x + c.y + c.z + c.w;
+    }
+    int32_t total;
+    int32_t ex = block_excl_scan<int32_t, int32_t>(sum, sh, total);
+    for (int q = 0; q < quads; ++q) {
+        const int4 c = mine[q];
+        mine[q] = make_int4(ex, ex + c.x, ex + c.x + c.y, ex + c.x + c.y + c.z);
+        ex += c.x + c.y + c.z + c.w;
+    }
+    __syncthreads();
+    for (int b = t; b <= nf; b += SCAN_THREADS) start[b] = cnt[b];
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < PER; ++k)
+        if (key[k] >= 0) tmp[atomicAdd(cnt + key[k], 1)] = t + k * SCAN_THREADS;
+    __syncthreads();   // a count is now the end of its bucket and the start of the next
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        if (key[k] < 0) continue;
+        const int st = key[k] ? cnt[key[k] - 1] : 0;
+        rank_in_bucket(t + k * SCAN_THREADS, st, cnt[key[k]] - st, tmp, items);
+    }
+}
+
+// row_start[0 .. n] from the n counts of a small set in one CTA: about 2.2 us for each tile of
+// 2048 rows, where the three launches and the copy of the total take 11 us
+constexpr int CTA_SCAN_ROWS = 8192;
+__global__ void __launch_bounds__(SCAN_THREADS) k_scan_rows_cta(int32_t n, const int32_t* cnt, int64_t* row_start,
+                                                                int64_t* total_out) {
+    __shared__ int64_t sh[SCAN_THREADS / 32];
+    int64_t carry = 0;
+    for (int base = 0; base < n; base += SCAN_TILE) {
+        const int b = base + threadIdx.x * SCAN_ITEMS;
+        int32_t c[SCAN_ITEMS];
+        int64_t s = 0;
+        for (int k = 0; k < SCAN_ITEMS; ++k) { c[k] = b + k < n ? cnt[b + k] : 0; s += c[k]; }
+        int64_t total;
+        int64_t ex = block_excl_scan<int64_t, int64_t>(s, sh, total) + carry;
+        for (int k = 0; k < SCAN_ITEMS; ++k) {
+            if (b + k < n) row_start[b + k] = ex;
+            ex += c[k];
+        }
+        carry += total;
+    }
+    if (threadIdx.x == 0) {
+        row_start[n] = carry;
+        *total_out = carry;
+    }
+}
+
+// CSR rows from the pair slab (a row lies there in increasing j), one warp per row so that a
+// row is read and written in whole lines (1024 rows of about 20 pairs: 4.5 us, 18.6 with a
+// thread per row)
+__global__ void k_compact(int32_t n, const int32_t* pcnt, const int32_t* pj, const double* pd, const double* pt,
+                          int pair_cap, const int64_t* row_start, int32_t* oj, double* od, double* ot) {
+    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (i >= n) return;
+    const int c = min(pcnt[i], pair_cap);
+    const int64_t o = row_start[i];
+    const size_t s = (size_t)i * pair_cap;
+    for (int a = lane; a < c; a += 32) {
+        oj[o + a] = pj[s + a];
+        od[o + a] = pd[s + a];
+    }
+    for (int a = lane; a < 3 * c; a += 32) ot[3 * o + a] = pt[3 * s + a];
 }
 
 // ------------------------------------------------------------------ face walk
@@ -601,8 +711,9 @@ __global__ void k_batch_step_inc(const cssi::SetView* sv, int nsets) {
     if (s < nsets) *sv[s].dstep += 1;
 }
 
-__global__ void k_batch_count(const cssi::SetView* sv, const int32_t* offs, int nsets) {
+__global__ void k_batch_count(const cssi::SetView* sv, const int32_t* offs, int nsets, int* queue, double* epot) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k == 0) reset_queue(queue, epot);
     if (k >= offs[nsets]) return;
     const int s = set_of(offs, nsets, k);
     const cssi::SetView& V = sv[s];
@@ -644,9 +755,15 @@ __global__ void k_batch_rank(const cssi::SetView* sv, const int32_t* offs, int n
     const cssi::SetView& V = sv[s];
     const int i = k - offs[s];
     const int f = V.face[i];
-    rank_in_bucket(i, V.m.frank ? V.m.frank[f] : f, V.fstart, V.ftmp, V.fitems);
+    const int key = V.m.frank ? V.m.frank[f] : f;
+    rank_in_bucket(i, V.fstart[key], V.fstart[key + 1] - V.fstart[key], V.ftmp, V.fitems);
 }
 
+
+// A walk is a chain of dependent FP64 operations: one warp per CTA spreads the chains over the SMs,
+// so that fewer of them share an SM's FP64 pipe (1024 particles' kick and drift: 19-24 us, 22-26
+// with four warps per CTA; no difference for 65536).
+constexpr int MOVE_THREADS = 32;
 
 inline unsigned nb(int64_t n, int b = 256) { return (unsigned)((n + b - 1) / b); }
 
@@ -666,19 +783,42 @@ cudaError_t launch_scan_i32(const int32_t* in, int32_t* out_excl, int64_t count,
 
 // row_start[0..n] (int64) from n counts: the tile sums live at the end of row_start's
 // scratch tail, so the caller passes row_start with n + 1 + scan_tmp_ints(n + 1) slots
-cudaError_t launch_scan_rows(const int32_t* cnt, int64_t* row_start, int32_t n, cudaStream_t st) {
+cudaError_t launch_scan_rows(const int32_t* cnt, int64_t* row_start, int64_t* total, int32_t n, cudaStream_t st) {
+    if (n <= CTA_SCAN_ROWS) {
+        k_scan_rows_cta<<<1, SCAN_THREADS, 0, st>>>(n, cnt, row_start, total);
+        return cudaGetLastError();
+    }
     const int64_t count = (int64_t)n + 1;
     const int nt = (int)((count + SCAN_TILE - 1) / SCAN_TILE);
     int64_t* tmp = row_start + count;
     k_tile_sums<int32_t, int64_t><<<nt, SCAN_THREADS, 0, st>>>(cnt, n, tmp);
     k_scan_sums<int64_t><<<1, SCAN_THREADS, 0, st>>>(tmp, nt);
     k_tile_apply<int32_t, int64_t><<<nt, SCAN_THREADS, 0, st>>>(cnt, n, count, tmp, row_start);
-    return cudaGetLastError();
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    return cudaMemcpyAsync(total, row_start + n, sizeof(int64_t), cudaMemcpyDeviceToDevice, st);
 }
 
+inline size_t cta_bucket_bytes(int32_t nf) {
+    return (4 * (size_t)SCAN_THREADS * cta_bucket_quads(nf) + CTA_BUCKET_ITEMS) * sizeof(int32_t);
+}
+
+cudaError_t dynamics_setup() {
+    return cudaFuncSetAttribute(k_bucket_cta, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)cta_bucket_bytes(CTA_BUCKET_FACES));
+}
+
+// The one-CTA form while the counts fit in its shared memory and eight particles a thread are
+// enough: 9.5 us against 22 us of the six launches at 1024 particles and 32768 faces, 13.3
+// against 23 at 4096.
 cudaError_t launch_bucket(int32_t n, int32_t nf, const int32_t* face, const int32_t* frank, int32_t* fcnt,
-                          int32_t* fstart, int32_t* fitems, int32_t* ftmp, int32_t* scan_tmp, cudaStream_t st) {
-    k_count<<<nb(n), 256, 0, st>>>(n, face, frank, fcnt);
+                          int32_t* fstart, int32_t* fitems, int32_t* ftmp, int32_t* scan_tmp, int* queue, double* epot,
+                          cudaStream_t st) {
+    if (n <= CTA_BUCKET_ITEMS && nf <= CTA_BUCKET_FACES) {
+        k_bucket_cta<<<1, SCAN_THREADS, cta_bucket_bytes(nf), st>>>(n, nf, face, frank, fstart, fitems, queue, epot);
+        return cudaGetLastError();
+    }
+    k_count<<<nb(n), 256, 0, st>>>(n, face, frank, fcnt, queue, epot);
     cudaError_t e = launch_scan_i32(fcnt, fstart, (int64_t)nf + 1, scan_tmp, st);
     if (e != cudaSuccess) return e;
     k_scatter<<<nb(n), 256, 0, st>>>(n, face, frank, fcnt, fstart, ftmp);
@@ -686,9 +826,16 @@ cudaError_t launch_bucket(int32_t n, int32_t nf, const int32_t* face, const int3
     return cudaGetLastError();
 }
 
+cudaError_t launch_pairs_compact(int32_t n, const int32_t* pcnt, const int32_t* pj, const double* pd,
+                                 const double* pt, int pair_cap, const int64_t* row_start, int32_t* out_j,
+                                 double* out_d, double* out_t, cudaStream_t st) {
+    k_compact<<<nb((int64_t)n * 32), 256, 0, st>>>(n, pcnt, pj, pd, pt, pair_cap, row_start, out_j, out_d, out_t);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_nve_kick_drift(const DMesh& m, int32_t n, int32_t* face, double* bary, double* vel,
                                   const double* force, css_integrator it, int* status, cudaStream_t st) {
-    k_nve_kick_drift<<<nb(n, 128), 128, 0, st>>>(m, n, face, bary, vel, force, it, status);
+    k_nve_kick_drift<<<nb(n, MOVE_THREADS), MOVE_THREADS, 0, st>>>(m, n, face, bary, vel, force, it, status);
     return cudaGetLastError();
 }
 
@@ -700,7 +847,7 @@ cudaError_t launch_nve_kick(int32_t n, double* vel, const double* force, css_int
 cudaError_t launch_overdamped_move(const DMesh& m, int32_t n, int32_t* face, double* bary, double* orient,
                                    const double* force, css_integrator it, uint64_t seed, const int64_t* dstep,
                                    const double* noise, int* status, cudaStream_t st) {
-    k_overdamped<<<nb(n, 128), 128, 0, st>>>(m, n, face, bary, orient, force, it, seed, dstep, noise, status);
+    k_overdamped<<<nb(n, MOVE_THREADS), MOVE_THREADS, 0, st>>>(m, n, face, bary, orient, force, it, seed, dstep, noise, status);
     return cudaGetLastError();
 }
 
@@ -716,7 +863,7 @@ cudaError_t launch_fire_move(const DMesh& m, int32_t n, int32_t* face, double* b
         const int64_t n3 = 3 * (int64_t)n;
         k_fire_reduce<<<(unsigned)std::min<int64_t>(nb(n3), 1024), 256, 0, st>>>(n3, vel, force, fire_state);
         k_fire_control<<<1, 1, 0, st>>>(fire_state, 10.0 * it.dt);
-        k_fire_mix_kick_drift<<<nb(n, 128), 128, 0, st>>>(m, n, face, bary, vel, force, fire_state, it, status);
+        k_fire_mix_kick_drift<<<nb(n, MOVE_THREADS), MOVE_THREADS, 0, st>>>(m, n, face, bary, vel, force, fire_state, it, status);
     } else {
         k_fire_kick<<<nb(3 * (int64_t)n), 256, 0, st>>>(3 * (int64_t)n, vel, force, fire_state, it.mass);
     }
@@ -955,7 +1102,7 @@ cudaError_t launch_trace(const DMesh& m, int64_t npaths, const int32_t* pface, c
                          const int32_t* src, const double* tan, const double* len, int cap, double* pts,
                          int32_t* npts, int32_t* end_face, double* end_bary, int* status, cudaStream_t st) {
     if (npaths < 1) return cudaSuccess;
-    k_trace<<<nb(npaths, 128), 128, 0, st>>>(m, npaths, pface, pbary, src, tan, len, cap, pts, npts, end_face,
+    k_trace<<<nb(npaths, MOVE_THREADS), MOVE_THREADS, 0, st>>>(m, npaths, pface, pbary, src, tan, len, cap, pts, npts, end_face,
                                               end_bary, status);
     return cudaGetLastError();
 }
@@ -965,7 +1112,7 @@ cudaError_t launch_legs(const DMesh& m, int64_t nleg, const int32_t* pface, cons
                         const int32_t* next_fk, const int32_t* next_pi, int cap, double* rec, int32_t* nrec,
                         double* start_w, double* next_w, double* gap, cudaStream_t st) {
     if (nleg < 1) return cudaSuccess;
-    k_legs<<<nb(nleg, 128), 128, 0, st>>>(m, nleg, pface, pbary, start_fk, start_pi, dir, len, next_fk, next_pi, cap,
+    k_legs<<<nb(nleg, MOVE_THREADS), MOVE_THREADS, 0, st>>>(m, nleg, pface, pbary, start_fk, start_pi, dir, len, next_fk, next_pi, cap,
                                           rec, nrec, start_w, next_w, gap);
     return cudaGetLastError();
 }
@@ -976,9 +1123,10 @@ cudaError_t launch_state_diff(int32_t n, const int32_t* new_f, const int32_t* ol
     return cudaGetLastError();
 }
 
-cudaError_t launch_batch_bucket(const SetView* sv, const int32_t* offs, int nsets, int64_t total, cudaStream_t st) {
+cudaError_t launch_batch_bucket(const SetView* sv, const int32_t* offs, int nsets, int64_t total, int* queue, double* epot,
+                                cudaStream_t st) {
     if (total < 1) return cudaSuccess;
-    k_batch_count<<<nb(total), 256, 0, st>>>(sv, offs, nsets);
+    k_batch_count<<<nb(total), 256, 0, st>>>(sv, offs, nsets, queue, epot);
     k_batch_scan<<<nsets, SCAN_THREADS, 0, st>>>(sv);
     k_batch_scatter<<<nb(total), 256, 0, st>>>(sv, offs, nsets);
     k_batch_rank<<<nb(total), 256, 0, st>>>(sv, offs, nsets);
@@ -989,10 +1137,10 @@ cudaError_t launch_batch_move(const SetView* sv, const int32_t* offs, int nsets,
                               int half, int* status, cudaStream_t st) {
     if (total < 1) return cudaSuccess;
     if (it.kind == CSS_INT_NVE) {
-        if (half == 0) k_batch_kick_drift<<<nb(total, 128), 128, 0, st>>>(sv, offs, nsets, it, status);
+        if (half == 0) k_batch_kick_drift<<<nb(total, MOVE_THREADS), MOVE_THREADS, 0, st>>>(sv, offs, nsets, it, status);
         else k_batch_kick<<<nb(total), 256, 0, st>>>(sv, offs, nsets, 0.5 * it.dt / it.mass);
     } else if (half == 1) {
-        k_batch_overdamped<<<nb(total, 128), 128, 0, st>>>(sv, offs, nsets, it, status);
+        k_batch_overdamped<<<nb(total, MOVE_THREADS), MOVE_THREADS, 0, st>>>(sv, offs, nsets, it, status);
         k_batch_step_inc<<<nb(nsets), 256, 0, st>>>(sv, nsets);
     }
     return cudaGetLastError();

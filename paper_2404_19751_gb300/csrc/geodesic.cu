@@ -2340,29 +2340,6 @@ __global__ void __launch_bounds__(256, OCC) k_geodesic(const __grid_constant__ c
     if (lane == 0) g.gen[gw] = gen;
 }
 
-// CSR compaction: rows sorted by neighbour index
-__global__ void k_compact(int32_t n, const int32_t* pcnt, const int32_t* pj, const double* pd, const double* pt,
-                          int pair_cap, const int64_t* row_start, int32_t* oj, double* od, double* ot) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int c = min(pcnt[i], pair_cap);
-    const int64_t o = row_start[i];
-    const size_t s = (size_t)i * pair_cap;
-    for (int a = 0; a < c; ++a) { oj[o + a] = pj[s + a]; od[o + a] = pd[s + a];
-        ot[3 * (o + a)] = pt[3 * (s + a)]; ot[3 * (o + a) + 1] = pt[3 * (s + a) + 1]; ot[3 * (o + a) + 2] = pt[3 * (s + a) + 2]; }
-    for (int a = 1; a < c; ++a) {           // insertion sort by j (rows are short)
-        const int32_t kj = oj[o + a];
-        const double kd = od[o + a], k0 = ot[3 * (o + a)], k1 = ot[3 * (o + a) + 1], k2 = ot[3 * (o + a) + 2];
-        int b = a - 1;
-        while (b >= 0 && oj[o + b] > kj) {
-            oj[o + b + 1] = oj[o + b]; od[o + b + 1] = od[o + b];
-            ot[3 * (o + b + 1)] = ot[3 * (o + b)]; ot[3 * (o + b + 1) + 1] = ot[3 * (o + b) + 1]; ot[3 * (o + b + 1) + 2] = ot[3 * (o + b) + 2];
-            --b;
-        }
-        oj[o + b + 1] = kj; od[o + b + 1] = kd; ot[3 * (o + b + 1)] = k0; ot[3 * (o + b + 1) + 1] = k1; ot[3 * (o + b + 1) + 2] = k2;
-    }
-}
-
 }  // namespace
 
 namespace cssi {
@@ -2520,13 +2497,6 @@ int geodesic_team_blocks_per_sm(int precision, int warps_per_cta, int shared_sca
     return f32 ? team_blocks_per_sm<float, 1, 0>(warps_per_cta, dyn) : team_blocks_per_sm<double, 1, 0>(warps_per_cta, dyn);
 }
 
-cudaError_t launch_pairs_compact(int32_t n, const int32_t* pcnt, const int32_t* pj, const double* pd,
-                                 const double* pt, int pair_cap, const int64_t* row_start, int32_t* out_j,
-                                 double* out_d, double* out_t, cudaStream_t st) {
-    k_compact<<<(n + 127) / 128, 128, 0, st>>>(n, pcnt, pj, pd, pt, pair_cap, row_start, out_j, out_d, out_t);
-    return cudaGetLastError();
-}
-
 }  // namespace cssi
 
 // =====================================================================================
@@ -2681,7 +2651,8 @@ int css_compute_forces_noalloc(const css_mesh* mesh, int64_t n, const int32_t* f
     if (e_pot) e = cudaMemsetAsync(e_pot, 0, sizeof(double), st);
     if (e == cudaSuccess)
         // the pair-count region doubles as the scatter scratch: the kernel below rewrites it
-        e = cssi::launch_bucket((int32_t)n, (int32_t)mesh->nf, face, mesh->frank, fcnt, fstart, fitems, pcnt, scan, st);
+        e = cssi::launch_bucket((int32_t)n, (int32_t)mesh->nf, face, mesh->frank, fcnt, fstart, fitems, pcnt, scan, nullptr, nullptr,
+                                st);
     cssi::GeoJob j{};
     j.m = mesh->view();
     j.n = (int32_t)n;
