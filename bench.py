@@ -56,8 +56,8 @@ TRAFFIC = {
     # 2.419 GB written in 8.72 ms (one ncu pass, dram__bytes_read.sum + dram__bytes_write.sum)
     "noisy_ico8_n65536": {"bytes": 5828550400 + 2418572544, "sources": 8192, "kernel": "0c622ec7855f2012"},
 }
-KERNEL_SOURCES = ("paper_2404_19751_gb300/csrc/geodesic.cu", "paper_2404_19751_gb300/csrc/css_dev.cuh",
-                  "paper_2404_19751_gb300/csrc/css_internal.h")
+KERNEL_SOURCES = ("paper_2404_19751_gb300/csrc/waves.cu", "paper_2404_19751_gb300/csrc/geo_common.cuh",
+                  "paper_2404_19751_gb300/csrc/css_dev.cuh")
 
 
 def kernel_digest() -> str:

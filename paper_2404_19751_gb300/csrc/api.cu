@@ -75,6 +75,16 @@ struct GeoPlan {
     int wpc1 = 0, nctas1 = 0, wpc2 = 0, nctas2 = 0, tile = 1;
 };
 
+int grow_ws(css_ctx* c, cssi::WsBuf& b, size_t need) {
+    if (need <= b.bytes) return CSS_OK;
+    cudaFree(b.ws);
+    b.ws = nullptr;
+    b.bytes = 0;
+    TRY(c, "workspace", cudaMalloc(&b.ws, need));
+    b.bytes = need;
+    return CSS_OK;
+}
+
 // one pass: layout, grid and (for tables in global memory) its workspace
 int plan_pass(css_ctx* c, cssi::WsBuf& b, int precision, int win_cap, int tab_cap, int shared, int warps, int team,
               int max_ctas, WaveWs* out, int* nctas) {
@@ -96,17 +106,10 @@ int plan_pass(css_ctx* c, cssi::WsBuf& b, int precision, int win_cap, int tab_ca
     if (max_ctas > 0) bps = std::min(bps, max_ctas);
     *nctas = c->sm_count * bps;
     g.stride = cssi::waves_global_bytes(g.lay, g.shared);
-    const size_t need = g.stride * (size_t)*nctas * (team ? 1 : warps);
-    if (need > b.bytes) {
-        cudaFree(b.ws);
-        b.ws = nullptr;
-        b.bytes = 0;
-        TRY(c, "workspace", cudaMalloc(&b.ws, need));
-        b.bytes = need;
-    }
+    int rc = grow_ws(c, b, g.stride * (size_t)*nctas * (team ? 1 : warps));
     g.base = (char*)b.ws;
     *out = g;
-    return CSS_OK;
+    return rc;
 }
 
 // What one source of a set sees within the cutoff, by its share of the mesh's area.
@@ -1430,48 +1433,50 @@ struct PathBufs {
     ~PathBufs() { for (void* q : ptrs) cudaFree(q); }
 };
 
-// One launch of the path instantiation of the neighbour kernel over the distinct sources
-// (us, on the device as dus): rows in the set's pair slab, legs per (rank in us, row slot).
+// The path form of the neighbour kernel over the distinct sources (us, on the device as dus): rows in
+// the set's pair slab, legs per (rank in us, row slot).  Sources whose patch should fit take
+// tables in shared memory first; those that do not fit, and all of large patches, tables in global
+// memory for win_cap windows.  The table sizes at which a shape is taken are those of pick_shape
+// for few sources (40 sources of 480 windows each: 0.25 ms, 1.41 ms in the window-list kernel).
 int run_path_kernel(css_parts* p, double rc, const std::vector<int32_t>& us, const int32_t* dus, int win_cap,
                     int32_t* dlnum, int32_t* dlfk, double* dldir, double* dllen, int* status) {
     css_ctx* c = p->ctx;
     cudaStream_t st = c->stream;
-    const int nus = (int)us.size();
-    int le, lv, lf, fcap, emcap;
-    const size_t stride = cssi::geo_ws_bytes_per_warp(CSS_FP64, win_cap, 0, &le, &lv, &lf, &fcap, &emcap);
-    const size_t lstride = cssi::geo_link_bytes_per_warp(lv);
-    const int wpc = 8;
-    const int nwarps = std::min(c->sm_count * wpc, ((nus + wpc - 1) / wpc) * wpc);
-    PathBufs B;
-    char *base = nullptr, *lbase = nullptr;
-    uint32_t* gen = nullptr;
-    TRY(c, "paths workspace", B.alloc(&base, (size_t)nwarps * stride));
-    TRY(c, "paths workspace", B.alloc(&lbase, (size_t)nwarps * lstride));
-    TRY(c, "paths workspace", B.alloc(&gen, (size_t)nwarps));
-    TRY(c, "paths workspace", cudaMemsetAsync(base, 0, (size_t)nwarps * stride, st));
-    TRY(c, "paths workspace", cudaMemsetAsync(gen, 0, (size_t)nwarps * sizeof(uint32_t), st));
-    cssi::GeoWs g{};
-    g.shared = 0;
-    g.base = base;
-    g.stride = stride;
-    g.log_eh = le; g.log_vh = lv; g.log_fh = lf;
-    g.wcap = win_cap; g.fcap = fcap; g.emcap = emcap;
-    g.gen = gen;
-    g.nwarps = nwarps;
-    g.occupancy = 1;
-    g.lbase = lbase;
-    g.lstride = lstride;
-    int rc1 = enqueue_bucket(p, nullptr, nullptr);
+    Reach R;
+    R.add(p, rc);
+    const int scale = R.verts <= 200.0 && R.targets <= 48.0 ? 2 : (R.verts <= 800.0 && R.targets <= 192.0 ? 4 : 0);
+    int rc1 = enqueue_bucket(p, c->dscal, nullptr);
+    if (rc1 == CSS_OK) rc1 = reset_status(c);
     if (rc1) return rc1;
     GeoJob j = make_job(p, rc, 1, 0, nullptr);
     j.order = dus;
     j.lmax = PATH_MAX_LEGS;
     j.lnum = dlnum; j.lfk = dlfk; j.ldir = dldir; j.llen = dllen;
-    cssi::GeoQueue q{nullptr, nullptr, nus, nullptr, nullptr, nullptr, nullptr, 1};
-    rc1 = reset_status(c);
-    if (rc1) return rc1;
-    TRY(c, "paths", cssi::launch_geodesic_links(j, q, g, wpc, nwarps / wpc, c->dscal, c->dscal + 1, c->dcount, st));
-    return read_status(c, status);
+    PathBufs B;
+    int32_t* defer = nullptr;
+    const int nus = (int)us.size();
+    TRY(c, "paths", B.alloc(&defer, us.size()));
+    int left = nus;
+    for (int pass = scale ? 0 : 1; pass < 2 && left > 0; ++pass) {
+        cssi::WaveWs g{};
+        g.shared = pass == 0;
+        g.lay = cssi::wave_layout(CSS_FP64, pass == 0 ? 2048 * scale : win_cap, 0, pass == 0 ? scale : 0, 1, 0);
+        g.stride = cssi::waves_global_bytes(g.lay, g.shared) + cssi::waves_link_bytes(g.lay);
+        const int ctas = std::min(left, c->sm_count * (pass == 0 ? 4 : 2));
+        cssi::WsBuf& b = pass == 0 ? c->ws1 : c->ws2;
+        rc1 = grow_ws(c, b, g.stride * (size_t)ctas);
+        if (rc1) return rc1;
+        g.base = (char*)b.ws;
+        const bool list = pass == 1 && scale;
+        const cssi::GeoQueue q{nullptr, nullptr, nus, list ? defer : nullptr, list ? c->dscal + 2 : nullptr,
+                               pass == 0 ? defer : nullptr, pass == 0 ? c->dscal + 2 : nullptr, 1};
+        TRY(c, "paths", cssi::launch_waves_links(j, q, g, 1, ctas, pass == 0 ? c->dscal : c->dscal + 3, c->dscal + 1,
+                                                 c->dcount, st));
+        rc1 = read_status(c, status);
+        if (rc1 || *status) return rc1;
+        left = pass == 0 ? c->hstat[2] : 0;
+    }
+    return CSS_OK;
 }
 
 }  // namespace
@@ -1537,52 +1542,34 @@ int css_geodesic_paths(css_parts* p, double r_c, int64_t n_pairs, const int32_t*
             return status_error(c, status);
         }
     }
-    // rows and legs of the distinct sources
-    const size_t slots = (size_t)nus * cap;
-    std::vector<int32_t> pcnt(p->n), pj((size_t)p->n * cap), lnum(slots), lfk(slots * PATH_MAX_LEGS);
-    std::vector<double> pd((size_t)p->n * cap), ldir(2 * slots * PATH_MAX_LEGS), llen(slots * PATH_MAX_LEGS);
-    TRY(c, "paths", cudaMemcpyAsync(pcnt.data(), p->pcnt, pcnt.size() * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-    TRY(c, "paths", cudaMemcpyAsync(pj.data(), p->pj, pj.size() * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-    TRY(c, "paths", cudaMemcpyAsync(pd.data(), p->pd, pd.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
-    TRY(c, "paths", cudaMemcpyAsync(lnum.data(), dlnum, lnum.size() * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-    TRY(c, "paths", cudaMemcpyAsync(lfk.data(), dlfk, lfk.size() * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-    TRY(c, "paths", cudaMemcpyAsync(ldir.data(), dldir, ldir.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
-    TRY(c, "paths", cudaMemcpyAsync(llen.data(), dllen, llen.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
+    // distances and numbers of legs of the requested pairs, then the legs, from the target back to the source
+    std::vector<int32_t> hr(np), lnum(np);
+    std::vector<double> hdist(np);
+    for (size_t k = 0; k < np; ++k) hr[k] = (int32_t)(std::lower_bound(us.begin(), us.end(), hs[k]) - us.begin());
+    int32_t *d_src, *d_dst, *d_rank, *d_legs, *d_slot;
+    double* d_dist;
+    int64_t* d_first;
+    TRY(c, "paths", B.alloc(&d_src, 5 * np));
+    d_dst = d_src + np; d_rank = d_dst + np; d_legs = d_rank + np; d_slot = d_legs + np;
+    TRY(c, "paths", B.alloc(&d_dist, np));
+    TRY(c, "paths", B.alloc(&d_first, np + 1));
+    TRY(c, "paths", cudaMemcpyAsync(d_src, hs.data(), np * sizeof(int32_t), cudaMemcpyHostToDevice, st));
+    TRY(c, "paths", cudaMemcpyAsync(d_dst, hd.data(), np * sizeof(int32_t), cudaMemcpyHostToDevice, st));
+    TRY(c, "paths", cudaMemcpyAsync(d_rank, hr.data(), np * sizeof(int32_t), cudaMemcpyHostToDevice, st));
+    TRY(c, "paths", cssi::launch_path_find((int64_t)np, d_src, d_dst, d_rank, p->pcnt, p->pj, p->pd, cap, dlnum, d_dist,
+                                           d_legs, d_slot, st));
+    TRY(c, "paths", cudaMemcpyAsync(lnum.data(), d_legs, np * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+    TRY(c, "paths", cudaMemcpyAsync(hdist.data(), d_dist, np * sizeof(double), cudaMemcpyDeviceToHost, st));
     TRY(c, "paths", cudaStreamSynchronize(st));
-    // the legs of every requested pair, from the target back to the source
     std::vector<int64_t> first(np + 1, 0);
-    std::vector<int32_t> s_fk, s_pi, n_fk, n_pi;
-    std::vector<double> l_dir, l_len;
-    std::vector<double> hdist(np, INFINITY);
     for (size_t k = 0; k < np; ++k) {
-        first[k] = (int64_t)s_fk.size();
-        const int i = hs[k], jj = hd[k];
-        const int r = (int)(std::lower_bound(us.begin(), us.end(), i) - us.begin());
-        const int cnt = std::min(pcnt[i], cap);
-        int pos = -1;
-        for (int a = 0; a < cnt; ++a)
-            if (pj[(size_t)i * cap + a] == jj) { pos = a; break; }
-        if (pos < 0) continue;   // not within the cutoff
-        hdist[k] = pd[(size_t)i * cap + pos];
-        const size_t o = (size_t)r * cap + pos;
-        const int nl = lnum[o];
-        if (nl <= 0) {
+        if (std::isfinite(hdist[k]) && lnum[k] <= 0) {
             c->err = "geodesic_paths: the path of pair " + std::to_string(k) +
-                     (nl == -1 ? " has more legs than the limit" : " lost a vertex link");
+                     (lnum[k] == -1 ? " has more legs than the limit" : " lost a vertex link");
             return CSS_ERR_ITER_LIMIT;
         }
-        for (int l = 0; l < nl; ++l) {
-            const size_t a = o * PATH_MAX_LEGS + l;
-            s_fk.push_back(lfk[a]);
-            s_pi.push_back(l == 0 ? jj : -1);
-            l_dir.push_back(ldir[2 * a]);
-            l_dir.push_back(ldir[2 * a + 1]);
-            l_len.push_back(llen[a]);
-            if (l + 1 < nl) { n_fk.push_back(lfk[a + 1]); n_pi.push_back(-1); }
-            else { n_fk.push_back(-1); n_pi.push_back(i); }
-        }
+        first[k + 1] = first[k] + lnum[k];
     }
-    first[np] = (int64_t)s_fk.size();
     const int64_t nleg = first[np];
     std::vector<int32_t> nrec(nleg);
     std::vector<double> rec((size_t)nleg * max_points * 3), sw(3 * (size_t)nleg), nw(3 * (size_t)nleg), lg(nleg);
@@ -1600,12 +1587,9 @@ int css_geodesic_paths(css_parts* p, double r_c, int64_t n_pairs, const int32_t*
         TRY(c, "paths", B.alloc(&d_sw, sw.size()));
         TRY(c, "paths", B.alloc(&d_nw, nw.size()));
         TRY(c, "paths", B.alloc(&d_gap, lg.size()));
-        TRY(c, "paths", cudaMemcpyAsync(d_sfk, s_fk.data(), nleg * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-        TRY(c, "paths", cudaMemcpyAsync(d_spi, s_pi.data(), nleg * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-        TRY(c, "paths", cudaMemcpyAsync(d_nfk, n_fk.data(), nleg * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-        TRY(c, "paths", cudaMemcpyAsync(d_npi, n_pi.data(), nleg * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-        TRY(c, "paths", cudaMemcpyAsync(d_dir, l_dir.data(), 2 * nleg * sizeof(double), cudaMemcpyHostToDevice, st));
-        TRY(c, "paths", cudaMemcpyAsync(d_len, l_len.data(), nleg * sizeof(double), cudaMemcpyHostToDevice, st));
+        TRY(c, "paths", cudaMemcpyAsync(d_first, first.data(), (np + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, st));
+        TRY(c, "paths", cssi::launch_path_gather((int64_t)np, d_src, d_dst, d_slot, d_first, PATH_MAX_LEGS, dlfk, dldir,
+                                                 dllen, d_sfk, d_spi, d_dir, d_len, d_nfk, d_npi, st));
         TRY(c, "paths", cssi::launch_legs(p->mesh->view(), nleg, p->face, p->bary, d_sfk, d_spi, d_dir, d_len, d_nfk,
                                           d_npi, max_points, d_rec, d_nrec, d_sw, d_nw, d_gap, st));
         TRY(c, "paths", cudaMemcpyAsync(nrec.data(), d_nrec, nleg * sizeof(int32_t), cudaMemcpyDeviceToHost, st));

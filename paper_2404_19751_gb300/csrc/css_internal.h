@@ -205,19 +205,6 @@ struct GeoQueue {
     int tile;
 };
 
-struct GeoWs {
-    int shared;              // scale of the keyed tables in shared memory, 0: global slice
-    char* base;
-    size_t stride;           // bytes per warp
-    int log_eh, log_vh, log_fh;
-    int wcap, fcap, emcap;
-    uint32_t* gen;
-    int nwarps;
-    int occupancy;           // kernel variant: 1 (255 registers a thread) or 2 (128)
-    char* lbase = nullptr;   // path launches: per-warp vertex link arrays (lstride bytes a warp)
-    size_t lstride = 0;
-};
-
 // One source's working memory in k_waves: capacities (powers of two of the vertex and target tables
 // and of the spill area, the fills at which they count as full) and byte offsets of its arrays.
 // A window record is six arrays: pseudo-source, rotation, two rims, (half-edge, vertex, key,
@@ -255,30 +242,16 @@ cudaError_t launch_waves(const GeoJob& job0, const GeoJob* djobs, const GeoQueue
                          int warps, int nctas, int* work_counter, int* status, unsigned long long* counters,
                          cudaStream_t st);
 
-// geodesic.cu
-size_t geo_ws_bytes_per_warp(int precision, int win_cap, int tab_cap, int* log_eh, int* log_vh, int* log_fh,
-                             int* fcap, int* emcap);
-cudaError_t launch_geodesic(const GeoJob& job0, const GeoJob* djobs, const GeoQueue& q, int precision,
-                            const GeoWs& ws, int warps_per_cta, int nctas, int* work_counter,
-                            int* status, unsigned long long* counters, cudaStream_t st);
-// the FP64, global-table kernel that also records the legs of every pair's path
-size_t geo_link_bytes_per_warp(int log_vh);
-cudaError_t launch_geodesic_links(const GeoJob& job, const GeoQueue& q, const GeoWs& ws, int warps_per_cta,
-                                  int nctas, int* work_counter, int* status, unsigned long long* counters,
-                                  cudaStream_t st);
-int geodesic_blocks_per_sm(int precision, int warps_per_cta, int shared_scale, int occupancy);
-// team form of the first pass: all warps of a CTA (2..8) on one source; ws counts teams
-cudaError_t launch_geodesic_team(const GeoJob& job0, const GeoJob* djobs, const GeoQueue& q, int precision,
-                                 const GeoWs& ws, int warps_per_cta, int nctas, int* work_counter, int* status,
-                                 unsigned long long* counters, cudaStream_t st);
-int geodesic_team_blocks_per_sm(int precision, int warps_per_cta, int shared_scale, int occupancy);
-size_t geodesic_team_shared_bytes(int precision, int warps_per_cta, int shared_scale);
-size_t geodesic_shared_bytes(int precision, int warps_per_cta, int shared_scale);
+// the FP64 form with one warp per source that also records the legs of every pair's path (behind each
+// group's spill area)
+size_t waves_link_bytes(const WaveLay& y);
+cudaError_t launch_waves_links(const GeoJob& job, const GeoQueue& q, const WaveWs& g, int warps, int nctas,
+                               int* work_counter, int* status, unsigned long long* counters, cudaStream_t st);
+
+// dynamics.cu
 cudaError_t launch_pairs_compact(int32_t n, const int32_t* pcnt, const int32_t* pj, const double* pd,
                                  const double* pt, int pair_cap, const int64_t* row_start,
                                  int32_t* out_j, double* out_d, double* out_t, cudaStream_t st);
-
-// dynamics.cu
 // particles bucketed by face rank: fstart (nf + 1) is indexed by frank[face] (NULL: by
 // face), fitems lists the particles in rank order
 // face buckets of n particles: counts, offsets, then the particles of each face in index
@@ -309,6 +282,16 @@ cudaError_t launch_fire_move(const css::DMesh& m, int32_t n, int32_t* face, doub
                              cudaStream_t st);
 // straightest-walk polylines of npaths paths (see css_trace_geodesics)
 // walks the legs of shortest paths (see k_legs in dynamics.cu)
+// the legs of requested pairs: k_path_find gives each pair's distance (infinity: not in the row of its
+// source, rank in the list of distinct sources) and number of legs, k_path_gather their legs from
+// first[pair] on in the form launch_legs takes
+cudaError_t launch_path_find(int64_t np, const int32_t* src, const int32_t* dst, const int32_t* rank,
+                             const int32_t* pcnt, const int32_t* pj, const double* pd, int pair_cap, const int32_t* lnum,
+                             double* dist, int32_t* legs, int32_t* slot, cudaStream_t st);
+cudaError_t launch_path_gather(int64_t np, const int32_t* src, const int32_t* dst, const int32_t* slot,
+                               const int64_t* first, int lmax, const int32_t* lfk, const double* ldir,
+                               const double* llen, int32_t* start_fk, int32_t* start_pi, double* dir, double* len,
+                               int32_t* next_fk, int32_t* next_pi, cudaStream_t st);
 cudaError_t launch_legs(const css::DMesh& m, int64_t nleg, const int32_t* pface, const double* pbary,
                         const int32_t* start_fk, const int32_t* start_pi, const double* dir, const double* len,
                         const int32_t* next_fk, const int32_t* next_pi, int cap, double* rec, int32_t* nrec,

@@ -1107,6 +1107,60 @@ cudaError_t launch_trace(const DMesh& m, int64_t npaths, const int32_t* pface, c
     return cudaGetLastError();
 }
 
+// one warp per pair looks the target up in its source's row
+__global__ void k_path_find(int64_t np, const int32_t* src, const int32_t* dst, const int32_t* rank, const int32_t* pcnt,
+                            const int32_t* pj, const double* pd, int pair_cap, const int32_t* lnum, double* dist,
+                            int32_t* legs, int32_t* slot) {
+    const int64_t k = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (k >= np) return;
+    const int i = src[k], j = dst[k], c = min(pcnt[i], pair_cap);
+    int pos = -1;
+    for (int a = lane; a < c; a += 32)
+        if (pj[(size_t)i * pair_cap + a] == j) pos = a;
+    pos = __reduce_max_sync(CSS_FULL, pos);
+    if (lane) return;
+    const int64_t o = (int64_t)rank[k] * pair_cap + pos;
+    dist[k] = pos < 0 ? __longlong_as_double(0x7ff0000000000000ll) : pd[(size_t)i * pair_cap + pos];
+    legs[k] = pos < 0 ? 0 : lnum[o];
+    slot[k] = pos < 0 ? -1 : (int32_t)o;
+}
+
+__global__ void k_path_gather(int64_t np, const int32_t* src, const int32_t* dst, const int32_t* slot, const int64_t* first,
+                              int lmax, const int32_t* lfk, const double* ldir, const double* llen, int32_t* start_fk,
+                              int32_t* start_pi, double* dir, double* len, int32_t* next_fk, int32_t* next_pi) {
+    const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (k >= np) return;
+    const int64_t f = first[k];
+    const int nl = (int)(first[k + 1] - f);
+    for (int l = 0; l < nl; ++l) {
+        const size_t a = (size_t)slot[k] * lmax + l;
+        start_fk[f + l] = lfk[a];
+        start_pi[f + l] = l == 0 ? dst[k] : -1;
+        dir[2 * (f + l)] = ldir[2 * a];
+        dir[2 * (f + l) + 1] = ldir[2 * a + 1];
+        len[f + l] = llen[a];
+        next_fk[f + l] = l + 1 < nl ? lfk[a + 1] : -1;
+        next_pi[f + l] = l + 1 < nl ? -1 : src[k];
+    }
+}
+
+cudaError_t launch_path_find(int64_t np, const int32_t* src, const int32_t* dst, const int32_t* rank,
+                             const int32_t* pcnt, const int32_t* pj, const double* pd, int pair_cap, const int32_t* lnum,
+                             double* dist, int32_t* legs, int32_t* slot, cudaStream_t st) {
+    k_path_find<<<nb(np * 32), 256, 0, st>>>(np, src, dst, rank, pcnt, pj, pd, pair_cap, lnum, dist, legs, slot);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_path_gather(int64_t np, const int32_t* src, const int32_t* dst, const int32_t* slot,
+                               const int64_t* first, int lmax, const int32_t* lfk, const double* ldir,
+                               const double* llen, int32_t* start_fk, int32_t* start_pi, double* dir, double* len,
+                               int32_t* next_fk, int32_t* next_pi, cudaStream_t st) {
+    k_path_gather<<<nb(np), 256, 0, st>>>(np, src, dst, slot, first, lmax, lfk, ldir, llen, start_fk, start_pi, dir, len,
+                                          next_fk, next_pi);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_legs(const DMesh& m, int64_t nleg, const int32_t* pface, const double* pbary,
                         const int32_t* start_fk, const int32_t* start_pi, const double* dir, const double* len,
                         const int32_t* next_fk, const int32_t* next_pi, int cap, double* rec, int32_t* nrec,

@@ -14,24 +14,6 @@ using css::DMesh;
 // Widening (rad) of the range in which a shortest path can leave a vertex it passes through.
 constexpr float SHADOW_TOL = 1e-3f;
 
-// Cumulative angle at a vertex of the direction g, given the vertex's corner hc whose first
-// edge runs along e (both in one face layout); NaN when g is too short to have a reliable
-// direction or the corner has no cumulative angle.
-__device__ __forceinline__ float back_angle(const DMesh& m, int hc, double ex, double ey, double gx, double gy,
-                                            double scale) {
-    if (hc < 0 || !(gx * gx + gy * gy > 1e-12 * scale * scale)) return __int_as_float(0x7fffffff);
-    return m.cang[hc].x + atan2f((float)(ex * gy - ey * gx), (float)(ex * gx + ey * gy));
-}
-
-// A back direction in 16 bits: steps of 1/4096 rad offset by 4 rad; 0xffff where it is unknown or
-// out of range.
-constexpr float BACK_STEP = 4096.0f, BACK_OFF = 4.0f;
-__device__ __forceinline__ unsigned pack_back(float b) {
-    const float t = (b + BACK_OFF) * BACK_STEP;
-    return (t >= 0.0f && t < 65535.0f) ? (unsigned)__float2int_rn(t) : 0xffffu;   // NaN -> unknown
-}
-__device__ __forceinline__ float unpack_back(unsigned q) { return (float)q * (1.0f / BACK_STEP) - BACK_OFF; }
-
 __device__ __forceinline__ double pot_dudl(const css_potential& p, double l) {
     if (!(l < p.r_cut)) return 0.0;
     if (p.kind == CSS_POT_HARMONIC) return -2.0 * p.eps * (1.0 - l / p.sigma) / p.sigma;

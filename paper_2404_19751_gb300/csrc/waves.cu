@@ -122,6 +122,50 @@ struct TeamSm {
     double fx[MAXW], fy[MAXW], en[MAXW];
 };
 
+// ------------------------------------------------------------------ links of paths
+// How a vertex or a target was reached (LK instantiations, FP64, one warp per source): the slot of
+// the vertex its last straight leg comes from (NONE: the source), and the leg back, as a unit
+// direction and a length, in the layout of face fk / 4 from its corner fk % 4 (3: from the target).
+// In global memory behind the group's spill area, the vertices' links, then the targets': they are
+// written on improvements only and read once per leg.
+struct Link {
+    int par, fk;
+    double len;
+    double2 dir;
+};
+template <bool LK>
+struct Links {};
+template <>
+struct Links<true> {
+    Link* p;
+};
+
+// the link of the point (X, Y) of half-edge he's frame straight back to the pseudo-source S: which
+// 2 the far corner of the face the window enters, 3 a point in that face; 0, 1 the start and the end of
+// the edge, whose leg points into the face on the other side and is written in that face
+__device__ __forceinline__ void link_back(const DMesh& m, int he, double2 S, double X, double Y, int which, int par, Link& l) {
+    const double a = S.x - X, b = S.y - Y, n = sqrt(a * a + b * b);
+    double va = n > 0.0 ? a / n : 1.0, vb = n > 0.0 ? b / n : 0.0;
+    int g = he / 3, kg = he - 3 * g, kc = which == 2 ? (kg == 0 ? 2 : kg - 1) : 3;
+    if (which < 2 && m.twin[he] >= 0) {
+        const int tw = m.twin[he];   // runs from the edge's end to its start
+        g = tw / 3;
+        kg = tw - 3 * g;
+        kc = which == 0 ? (kg == 2 ? 0 : kg + 1) : kg;
+        va = -va;
+        vb = -vb;
+    }
+    double ax, ay, bx, by;
+    css::face_corner(m, g, kg, ax, ay);
+    css::face_corner(m, g, kg + 1, bx, by);
+    const double L = sqrt((bx - ax) * (bx - ax) + (by - ay) * (by - ay));
+    const double ex = (bx - ax) / L, ey = (by - ay) / L;
+    l.par = par;
+    l.fk = 4 * g + kc;
+    l.len = n;
+    l.dir = make_double2(va * ex - vb * ey, va * ey + vb * ex);
+}
+
 // ------------------------------------------------------------------ working memory
 template <class T>
 __device__ __forceinline__ T* at(unsigned char* b, int off) { return reinterpret_cast<T*>(b + off); }
@@ -201,9 +245,9 @@ __device__ __forceinline__ float cut_at(float sx, float s2, float a, float L, fl
 // FP64 the shorter one is the one).  One warp writes the direction of an improvement beside the
 // length it lowered; a team's warps, which may lower one length at the same time, log them, and the
 // log is read once the source is done.
-template <class R, int PL, bool TEAM>
+template <class R, int PL, bool TEAM, bool LK>
 __device__ __noinline__ void eval_tests(const cssi::GeoJob& J, const WaveLay& Y, unsigned char* b, unsigned char* e,
-                                        GroupSm& sm, int nev, int lane) {
+                                        GroupSm& sm, int nev, int lane, Links<LK> lk) {
     const DMesh& m = J.m;
     bool won = false, apart = false;
     int s = NONE;
@@ -281,6 +325,16 @@ __device__ __noinline__ void eval_tests(const cssi::GeoJob& J, const WaveLay& Y,
         if (won && *((volatile unsigned long long*)at<double>(b, apart ? Y.tvert : Y.tdist) + s) == bits) {
             at<V2<R>>(b, Y.ttan)[at_] = t;
             if constexpr (sizeof(R) == 4) at<double>(b, Y.tcmp)[at_] = w;
+            if constexpr (LK) {
+                const int4 w4 = at<int4>(e, Y.e[4])[lane];
+                const double2 S = at<double2>(e, Y.e[0])[lane];
+                const HeRec& r = m.he[w4.x];
+                const int k = w4.x % 3;
+                const double* bj = J.bary + 3 * (size_t)w4.z;
+                const double bv = bj[k == 2 ? 0 : k + 1], bc = bj[k == 0 ? 2 : k - 1];
+                link_back(m, w4.x, S, bv * r.L + bc * r.cx, bc * r.cy, 3, w4.y < 0 ? NONE : w4.y & ~FROM_VERTEX,
+                          lk.p[(1 << Y.vh_log) + s]);
+            }
         }
     }
 }
@@ -295,7 +349,7 @@ struct Win {
     int su, sv;         // slots of the edge's end vertices
 };
 
-template <class R, int PL, bool TEAM>
+template <class R, int PL, bool TEAM, bool LK>
 struct Group {
     using Idx = typename Index<PL>::type;
     const cssi::GeoJob& J;
@@ -308,6 +362,7 @@ struct Group {
     TeamSm* tm;
     int src, lane, wid, tid, T;
     float rcf;             // the cutoff, rounded up
+    Links<LK> lk;
     int nev = 0;
 
     __device__ __forceinline__ void bar() const {
@@ -329,7 +384,7 @@ struct Group {
 
     __device__ __forceinline__ void eval() {
         __syncwarp();
-        if (nev) eval_tests<R, PL, TEAM>(J, Y, b, e, sm, nev, lane);
+        if (nev) eval_tests<R, PL, TEAM, LK>(J, Y, b, e, sm, nev, lane, lk);
         __syncwarp();
         nev = 0;
     }
@@ -492,8 +547,8 @@ struct Group {
 
 // Start a source (warp 0): tests for its own face, distances of its corners, one window for
 // each edge of its face.
-template <class R, int PL, bool TEAM>
-__device__ __forceinline__ void Group<R, PL, TEAM>::seed(int f0, double b1, double b2) {
+template <class R, int PL, bool TEAM, bool LK>
+__device__ __forceinline__ void Group<R, PL, TEAM, LK>::seed(int f0, double b1, double b2) {
     const DMesh& m = J.m;
     const bool c3 = lane < 3;
     const int hh = 3 * f0 + (c3 ? lane : 0);
@@ -519,6 +574,7 @@ __device__ __forceinline__ void Group<R, PL, TEAM>::seed(int f0, double b1, doub
     const int slot = c3 ? vertex(m.fv[hh]) : NONE;
     if (slot >= 0 && vd < J.rc && (on == 0 || (on >> lane & 1u))) {
         vdist()[slot] = vd;
+        if constexpr (LK) lk.p[slot] = {NONE, 4 * f0 + k0, vd, make_double2(vd > 0.0 ? -vx / vd : 1.0, vd > 0.0 ? -vy / vd : 0.0)};
         if (!on && (m.htop[hh].x & css::EMITS))
             improved(slot, vd, vec2((R)(vx / vd), (R)(vy / vd)), vd > 1e-6 * r.L ? hh : NONE, atan2f((float)hy, (float)hx));
     }
@@ -549,8 +605,8 @@ __device__ __forceinline__ void Group<R, PL, TEAM>::seed(int f0, double b1, doub
 // the ring from the source's face, counter-clockwise for the first half and clockwise for the
 // rest (at a vertex the direction in the source face's plane depends on that choice).  Serial:
 // this is rare.
-template <class R, int PL, bool TEAM>
-__device__ __forceinline__ void Group<R, PL, TEAM>::seed_at_vertex(int hc) {
+template <class R, int PL, bool TEAM, bool LK>
+__device__ __forceinline__ void Group<R, PL, TEAM, LK>::seed_at_vertex(int hc) {
     const DMesh& m = J.m;
     const int32_t v = m.fv[hc];
     const int deg = m.ring_start[v + 1] - m.ring_start[v];
@@ -599,8 +655,15 @@ __device__ __forceinline__ void Group<R, PL, TEAM>::seed_at_vertex(int hc) {
                 if (slot >= 0 && d < J.rc) {
                     const unsigned long long bits = (unsigned long long)__double_as_longlong(d);
                     const unsigned long long old = atomicMin((unsigned long long*)(vdist() + slot), bits);
-                    if (old > bits && (m.htop[hn].x & css::EMITS))
+                    if (old > bits && (m.htop[hn].x & css::EMITS)) {
                         improved(slot, d, vec2((R)cos(a), (R)sin(a)), NONE, 0.0f);
+                        if constexpr (LK) {   // along the edge, back to the source's corner
+                            double px, py, sx, sy;
+                            css::face_corner(m, fh, hn - 3 * fh, px, py);
+                            css::face_corner(m, fh, kh, sx, sy);
+                            lk.p[slot] = {NONE, 4 * fh + (hn - 3 * fh), d, make_double2((sx - px) / d, (sy - py) / d)};
+                        }
+                    }
                 }
             }
             const int s1 = __shfl_sync(CSS_FULL, slot, 0), s2 = __shfl_sync(CSS_FULL, slot, 1);
@@ -635,8 +698,8 @@ __device__ __forceinline__ void Group<R, PL, TEAM>::seed_at_vertex(int hc) {
 // any shortest path to it.  The window is clipped to that range, widened by SHADOW_TOL for the
 // rounding of b and the corner angles.  Vertices without a known b, boundary and non-manifold
 // ones start windows over their whole ring.
-template <class R, int PL, bool TEAM>
-__device__ __forceinline__ void Group<R, PL, TEAM>::emit(int ne, int lim, float kmin) {
+template <class R, int PL, bool TEAM, bool LK>
+__device__ __forceinline__ void Group<R, PL, TEAM, LK>::emit(int ne, int lim, float kmin) {
     const DMesh& m = J.m;
     const int from = sm.cur, to = 1 - from;
     bar();
@@ -761,8 +824,8 @@ __device__ __forceinline__ void Group<R, PL, TEAM>::emit(int ne, int lim, float 
 }
 
 // Unfold the windows head .. head + n of the ring (at most one per thread).
-template <class R, int PL, bool TEAM>
-__device__ __forceinline__ void Group<R, PL, TEAM>::wave(int head, int n) {
+template <class R, int PL, bool TEAM, bool LK>
+__device__ __forceinline__ void Group<R, PL, TEAM, LK>::wave(int head, int n) {
     const DMesh& m = J.m;
     const bool on = tid < n;
     const int s = (head + tid) & Y.r_mask;
@@ -858,6 +921,9 @@ __device__ __forceinline__ void Group<R, PL, TEAM>::wave(int head, int n) {
             const float ex = a == 0 ? -q.cx : (a == 1 ? 1.0f : -1.0f), ey = a == 0 ? -q.cy : 0.0f;
             improved(slot, d, t, fvx * fvx + fvy * fvy > 1e-6f * size * size ? hc : NONE,
                      atan2f(ey * fvx - ex * fvy, -ex * fvx - ey * fvy));
+            if constexpr (LK)
+                link_back(m, he, S, a == 0 ? r.cx : (a == 1 ? 0.0 : r.L), a == 0 ? r.cy : 0.0, a == 0 ? 2 : a - 1, vs,
+                          lk.p[slot]);
         }
         bar();
     }
@@ -937,8 +1003,8 @@ __device__ __forceinline__ void Group<R, PL, TEAM>::wave(int head, int n) {
     }
 }
 
-template <class R, int PL, bool TEAM>
-__device__ __forceinline__ void Group<R, PL, TEAM>::run(int item, int32_t* defer_list, int* defer_count, int* status,
+template <class R, int PL, bool TEAM, bool LK>
+__device__ __forceinline__ void Group<R, PL, TEAM, LK>::run(int item, int32_t* defer_list, int* defer_count, int* status,
                                                         unsigned long long* counters) {
     const DMesh& m = J.m;
     const int f0 = J.face[src];
@@ -1107,6 +1173,25 @@ __device__ __forceinline__ void Group<R, PL, TEAM>::run(int item, int32_t* defer
             J.pt[3 * o + 1] = tx * fr[4] + ty * fr[7];
             J.pt[3 * o + 2] = tx * fr[5] + ty * fr[8];
         }
+        if constexpr (LK) {   // the pair's legs, from the target back to the source
+            if (k < J.pair_cap) {
+                const size_t o = (size_t)item * J.pair_cap + k;
+                Link l = lk.p[(1 << Y.vh_log) + s];
+                int nl = 0;
+                for (;;) {
+                    if (nl >= J.lmax) { nl = -1; break; }
+                    const size_t a = o * J.lmax + nl;
+                    J.lfk[a] = l.fk;
+                    J.ldir[2 * a] = l.dir.x;
+                    J.ldir[2 * a + 1] = l.dir.y;
+                    J.llen[a] = l.len;
+                    ++nl;
+                    if (l.par < 0) break;
+                    l = lk.p[l.par];
+                }
+                J.lnum[o] = nl;
+            }
+        }
         if (J.want_forces) {
             const double du = geo::pot_dudl(J.pot, d);
             fx += du * tx;
@@ -1150,8 +1235,8 @@ __device__ __forceinline__ void Group<R, PL, TEAM>::run(int item, int32_t* defer
 // PL 1: tables and ring in shared memory, 0: in the group's slice of global memory.  TEAM: the
 // warps of a CTA work on one source, else each warp on its own.  Persistent: groups pull work
 // items from a counter.
-template <class R, int PL, bool TEAM>
-__global__ void __launch_bounds__(256, 2) k_waves(const __grid_constant__ cssi::GeoJob job0, const cssi::GeoJob* jobs,
+template <class R, int PL, bool TEAM, bool LK>
+__global__ void __launch_bounds__(256, LK ? 1 : 2) k_waves(const __grid_constant__ cssi::GeoJob job0, const cssi::GeoJob* jobs,
                                                   const __grid_constant__ cssi::GeoQueue q,
                                                   const __grid_constant__ WaveWs g, int* work, int* status,
                                                   unsigned long long* counters) {
@@ -1191,8 +1276,9 @@ __global__ void __launch_bounds__(256, 2) k_waves(const __grid_constant__ cssi::
             const int jid = q.job_of_item ? q.job_of_item[item] : 0;
             const cssi::GeoJob& J = jobs ? jobs[jid] : job0;
             const int pos = q.src_of_item ? q.src_of_item[item] : item;
-            Group<R, PL, TEAM> G{J, g.lay, b, h, e, x, sm, tm, J.order ? J.order[pos] : pos, lane, wid,
-                                 TEAM ? (int)threadIdx.x : lane, TEAM ? (int)blockDim.x : 32, __double2float_ru(J.rc)};
+            Group<R, PL, TEAM, LK> G{J, g.lay, b, h, e, x, sm, tm, J.order ? J.order[pos] : pos, lane, wid,
+                                 TEAM ? (int)threadIdx.x : lane, TEAM ? (int)blockDim.x : 32, __double2float_ru(J.rc), {}};
+            if constexpr (LK) G.lk.p = reinterpret_cast<Link*>(x + g.lay.s_bytes);
             if constexpr (!TEAM) { G.wid = 0; }
             G.run(item, q.defer_list, q.defer_count, status, counters);
             G.bar();
@@ -1260,21 +1346,21 @@ int log2_up(int x) {
     return l;
 }
 
-template <class R, int PL, bool TEAM>
+template <class R, int PL, bool TEAM, bool LK>
 int blocks_of(int warps, size_t dyn) {
     int dev = 0, optin = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     cudaFuncAttributes fa;
-    if (cudaFuncGetAttributes(&fa, k_waves<R, PL, TEAM>) != cudaSuccess) { cudaGetLastError(); return 0; }
+    if (cudaFuncGetAttributes(&fa, k_waves<R, PL, TEAM, LK>) != cudaSuccess) { cudaGetLastError(); return 0; }
     const int room = optin - (int)fa.sharedSizeBytes;
     if (dyn > (size_t)room) return 0;
-    if (cudaFuncSetAttribute(k_waves<R, PL, TEAM>, cudaFuncAttributeMaxDynamicSharedMemorySize, room) != cudaSuccess) {
+    if (cudaFuncSetAttribute(k_waves<R, PL, TEAM, LK>, cudaFuncAttributeMaxDynamicSharedMemorySize, room) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_waves<R, PL, TEAM>, 32 * warps, dyn) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_waves<R, PL, TEAM, LK>, 32 * warps, dyn) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
@@ -1329,10 +1415,10 @@ int waves_blocks_per_sm(int precision, const WaveLay& y, int warps, int shared, 
     if (warps < 1 || warps > MAXW) return 0;
     const size_t dyn = dyn_bytes(y, warps, shared != 0, team != 0);
 #define CSS_PICK(F)                                                                                        \
-    (precision == CSS_FP32 ? (shared ? (team ? F<float, 1, true>(warps, dyn) : F<float, 1, false>(warps, dyn))     \
-                                     : (team ? F<float, 0, true>(warps, dyn) : F<float, 0, false>(warps, dyn)))    \
-                           : (shared ? (team ? F<double, 1, true>(warps, dyn) : F<double, 1, false>(warps, dyn))   \
-                                     : (team ? F<double, 0, true>(warps, dyn) : F<double, 0, false>(warps, dyn))))
+    (precision == CSS_FP32 ? (shared ? (team ? F<float, 1, true, false>(warps, dyn) : F<float, 1, false, false>(warps, dyn))     \
+                                     : (team ? F<float, 0, true, false>(warps, dyn) : F<float, 0, false, false>(warps, dyn)))    \
+                           : (shared ? (team ? F<double, 1, true, false>(warps, dyn) : F<double, 1, false, false>(warps, dyn))   \
+                                     : (team ? F<double, 0, true, false>(warps, dyn) : F<double, 0, false, false>(warps, dyn))))
     return CSS_PICK(blocks_of);
 #undef CSS_PICK
 }
@@ -1342,7 +1428,7 @@ cudaError_t launch_waves(const GeoJob& job0, const GeoJob* djobs, const GeoQueue
                          cudaStream_t st) {
     const size_t dyn = dyn_bytes(g.lay, warps, g.shared != 0, g.team != 0);
 #define CSS_LAUNCH(RT, P, T) \
-    k_waves<RT, P, T><<<nctas, 32 * warps, dyn, st>>>(job0, djobs, q, g, work_counter, status, counters)
+    k_waves<RT, P, T, false><<<nctas, 32 * warps, dyn, st>>>(job0, djobs, q, g, work_counter, status, counters)
     if (precision == CSS_FP32) {
         if (g.shared) { if (g.team) CSS_LAUNCH(float, 1, true); else CSS_LAUNCH(float, 1, false); }
         else { if (g.team) CSS_LAUNCH(float, 0, true); else CSS_LAUNCH(float, 0, false); }
@@ -1351,6 +1437,18 @@ cudaError_t launch_waves(const GeoJob& job0, const GeoJob* djobs, const GeoQueue
         else { if (g.team) CSS_LAUNCH(double, 0, true); else CSS_LAUNCH(double, 0, false); }
     }
 #undef CSS_LAUNCH
+    return cudaGetLastError();
+}
+
+size_t waves_link_bytes(const WaveLay& y) { return sizeof(Link) * (((size_t)1 << y.vh_log) + ((size_t)1 << y.th_log)); }
+
+cudaError_t launch_waves_links(const GeoJob& job, const GeoQueue& q, const WaveWs& g, int warps, int nctas,
+                               int* work_counter, int* status, unsigned long long* counters, cudaStream_t st) {
+    const size_t dyn = dyn_bytes(g.lay, warps, g.shared != 0, false);
+    if ((g.shared ? blocks_of<double, 1, false, true>(warps, dyn) : blocks_of<double, 0, false, true>(warps, dyn)) < 1)
+        return cudaErrorInvalidConfiguration;
+    if (g.shared) k_waves<double, 1, false, true><<<nctas, 32 * warps, dyn, st>>>(job, nullptr, q, g, work_counter, status, counters);
+    else k_waves<double, 0, false, true><<<nctas, 32 * warps, dyn, st>>>(job, nullptr, q, g, work_counter, status, counters);
     return cudaGetLastError();
 }
 
