@@ -51,6 +51,11 @@ using css::HeRec;
 using cssi::WaveLay;
 using cssi::WaveWs;
 
+// Where sources fill the chip, instruction fetch sets the pace: a wave is about 2000 instructions of
+// mostly straight code, 16 warps sit at different places of it, and 43 % of stall cycles waited for
+// instructions.  So loops are not unrolled, rare branches are marked and divisions in FP32 are the
+// short ones (16384 sources on a noisy sphere: 2.96 -> 2.45 ms in FP64, 3.10 -> 2.63 in FP32; 8192 on
+// a height field 3.55 -> 3.23; small sets and teams unchanged within 2 %).
 constexpr int MAXW = 8;          // warps per CTA
 constexpr int EV = 10;           // queued target tests per warp
 constexpr int NONE = -1;
@@ -177,6 +182,7 @@ __device__ __forceinline__ int tab_insert(int32_t* keys, int logcap, int32_t key
     const uint32_t mask = (1u << logcap) - 1u;
     uint32_t s = hash_of(key, logcap);
     claimed = false;
+#pragma unroll 1
     for (uint32_t p = 0; p <= mask; ++p) {
         const int32_t c = *(volatile int32_t*)(keys + s);
         if (c == key) return (int)s;
@@ -398,10 +404,12 @@ struct Group {
             st = J.fstart[key];
             cnt = J.fstart[key + 1] - st;
         }
+#pragma unroll 1
         for (int r = 0; __any_sync(CSS_FULL, r < cnt); ++r) {
             int j = src;
             if (r < cnt) j = J.fitems[st + r];
             unsigned mk = __ballot_sync(CSS_FULL, j != src);
+#pragma unroll 1
             while (mk) {   // as many as there is room for
                 const int k = nev + __popc(mk & css::lanemask_lt());
                 const bool now = j != src && (mk >> lane & 1u) && k < EV;
@@ -409,7 +417,7 @@ struct Group {
                 const unsigned done = __ballot_sync(CSS_FULL, now);
                 nev += __popc(done);
                 mk &= ~done;
-                if (nev == EV) eval();
+                if (TEAM ? nev == EV : __builtin_expect(nev == EV, 0)) eval();
             }
         }
     }
@@ -464,7 +472,7 @@ struct Group {
         const int rank = __popc(mk & css::lanemask_lt());
         const int b01 = pack_interval(w.b0, w.b1, L);
         if (has && base + rank < lim) store(h, Y.r, (base + rank) & Y.r_mask, w, b01);
-        if (base + n > lim) {
+        if (TEAM ? base + n > lim : __builtin_expect(base + n > lim, 0)) {
             const int in = max(0, lim - base);   // those that went to the ring
             int sb = 0;
             if constexpr (TEAM) {
@@ -510,7 +518,7 @@ struct Group {
         bool queued = false;
         if (i == (int)Index<PL>::none) {
             i = atomicAdd(&sm.ni, 1);
-            if (i >= Y.i_cap) {
+            if (TEAM ? i >= Y.i_cap : __builtin_expect(i >= Y.i_cap, 0)) {
                 atomicOr(&sm.err, css::ST_HASH_OVERFLOW);
                 return;
             }
@@ -621,6 +629,7 @@ __device__ __forceinline__ void Group<R, PL, TEAM, LK>::seed_at_vertex(int hc) {
     for (int dir = 0; dir < 2; ++dir) {
         int g = hc;
         double phi = phi0;   // direction of corner h's first edge in the source face's layout
+#pragma unroll 1
         for (int q = 0; q < (dir == 0 ? half : deg) && left > 0; ++q) {
             if (q > 0 || dir == 1) {
                 if (dir == 0) {   // the next corner, across this corner's last edge
@@ -709,6 +718,7 @@ __device__ __forceinline__ void Group<R, PL, TEAM, LK>::emit(int ne, int lim, fl
         sm.emin = 0x7f800000u;
     }
     bar();
+#pragma unroll 1
     for (int base = tid - lane; base < ne; base += T) {
         const int it = base + lane;
         int vs = 0;
@@ -736,13 +746,14 @@ __device__ __forceinline__ void Group<R, PL, TEAM, LK>::emit(int ne, int lim, fl
             if (bk == bk) {
                 th = (float)m.theta[vid];
                 lo = bk + 3.14159265f - geo::SHADOW_TOL;
-                lo -= th * floorf(lo / th);
+                lo -= th * floorf(__fdividef(lo, th));
                 hi = lo + (th - 6.28318531f + 2.0f * geo::SHADOW_TOL);
             }
         }
         // one lane per (vertex, corner)
         const int incl = geo::warp_incl_scan(len, lane);
         const int total = __shfl_sync(CSS_FULL, incl, 31);
+#pragma unroll 1
         for (int tb = 0; tb < total; tb += 32) {
             const int t = tb + lane;
             const int owner = geo::scan_owner(incl, t);
@@ -798,12 +809,12 @@ __device__ __forceinline__ void Group<R, PL, TEAM, LK>::emit(int ne, int lim, fl
                         const float ex = q.cx - q.L, ey = q.cy;
                         if (c0 > 1e-5f) {
                             const float s = __sinf(c0), c = __cosf(c0);
-                            const float x = fminf(fmaxf(q.L * s / (ey * c - ex * s), 0.0f), 1.0f);
+                            const float x = fminf(fmaxf(__fdividef(q.L * s, ey * c - ex * s), 0.0f), 1.0f);
                             w.b1 = fminf(L, L * (1.0f - x) + 1e-5f * L);
                         }
                         if (c1 < wid_c - 1e-5f) {
                             const float s = __sinf(c1), c = __cosf(c1);
-                            const float x = fminf(fmaxf(q.L * s / (ey * c - ex * s), 0.0f), 1.0f);
+                            const float x = fminf(fmaxf(__fdividef(q.L * s, ey * c - ex * s), 0.0f), 1.0f);
                             w.b0 = fmaxf(0.0f, L * (1.0f - x) - 1e-5f * L);
                         }
                     }
@@ -864,7 +875,7 @@ __device__ __forceinline__ void Group<R, PL, TEAM, LK>::wave(int head, int n) {
         beyond0 = cr0 < -t0;
         in1 = cr1 >= -t1;
         beyond1 = cr1 > t1;
-        if (sizeof(R) == 8 && on && ((in0 && !beyond0) || (in1 && !beyond1))) {   // too close to a rim for FP32
+        if (sizeof(R) == 8 && (TEAM ? on && ((in0 && !beyond0) || (in1 && !beyond1)) : __builtin_expect(on && ((in0 && !beyond0) || (in1 && !beyond1)), 0))) {   // too close to a rim for FP32
             const double gx = r.cx - S.x, gy = r.cy - S.y;
             const double ex = gx * rot.x + gy * rot.y, ey = gy * rot.x - gx * rot.y;
             const double tg = Rim<double>::t * (fabs(gx) + fabs(gy));
@@ -1012,10 +1023,15 @@ __device__ __forceinline__ void Group<R, PL, TEAM, LK>::run(int item, int32_t* d
     // empty tables; distances start at infinity
     {
         const int4 none = make_int4(-1, -1, -1, -1), inf = make_int4(0, 0x7ff00000, 0, 0x7ff00000);
+#pragma unroll 1
         for (int k = tid; k < (1 << Y.vh_log) / 4; k += T) at<int4>(b, Y.vkey)[k] = none;
+#pragma unroll 1
         for (int k = tid; k < (1 << Y.vh_log) / 2; k += T) at<int4>(b, Y.vdist)[k] = inf;
+#pragma unroll 1
         for (int k = tid; k < (int)sizeof(Idx) * (1 << Y.vh_log) / 16; k += T) at<int4>(b, Y.vinfo)[k] = none;
+#pragma unroll 1
         for (int k = tid; k < (1 << Y.th_log) / 4; k += T) at<int4>(b, Y.tkey)[k] = none;
+#pragma unroll 1
         for (int k = tid; k < (1 << Y.th_log) / 2; k += T) {
             at<int4>(b, Y.tdist)[k] = inf;
             if (sizeof(R) == 4) at<int4>(b, Y.tvert)[k] = inf;
@@ -1036,14 +1052,16 @@ __device__ __forceinline__ void Group<R, PL, TEAM, LK>::run(int item, int32_t* d
         int tail = min(sm.tail, lim), err = sm.err;   // a team's claims may run past the ring's end
         if (++waves > Y.max_waves) err |= css::ST_ITER_LIMIT;
         bar();
-        if (err || (head == tail && ne == 0 && waits == 0)) {
+        const bool done = err || (head == tail && ne == 0 && waits == 0);
+        if (TEAM ? done : __builtin_expect(done, 0)) {
             if (tid == 0) sm.err = err;
             break;
         }
         // spilled windows come back as the ring empties
         const int back = waits > 0 && tail - head < T ? min(waits, Y.r_mask + 1 - (tail - head)) : 0;
-        if (back > 0) {
+        if (TEAM ? back > 0 : __builtin_expect(back > 0, 0)) {
             const int from = sm.shead;
+#pragma unroll 1
             for (int k = tid; k < back; k += T) {
                 const int i = (from + k) & (Y.s_cap - 1), o = (tail + k) & Y.r_mask;
                 at<double2>(h, Y.r[0])[o] = at<double2>(x, Y.s[0])[i];
@@ -1062,7 +1080,9 @@ __device__ __forceinline__ void Group<R, PL, TEAM, LK>::run(int item, int32_t* d
         bar();
         if (ne > 0) {
             float km = INFINITY;
+#pragma unroll 1
             for (int k = head + tid; k < tail; k += T) km = fminf(km, __int_as_float(at<int4>(h, Y.r[4])[k & Y.r_mask].z));
+#pragma unroll 1
             for (int k = sm.shead + tid; k < sm.stail; k += T)
                 km = fminf(km, __int_as_float(at<int4>(x, Y.s[4])[k & (Y.s_cap - 1)].z));
             km = __uint_as_float(__reduce_min_sync(CSS_FULL, __float_as_uint(km)));
@@ -1106,23 +1126,30 @@ __device__ __forceinline__ void Group<R, PL, TEAM, LK>::run(int item, int32_t* d
     int* ord = list + (1 << Y.th_log);
     if (tid == 0) sm.head = 0;
     bar();
+#pragma unroll 1
     for (int k = tid; k < (1 << Y.th_log); k += T)
         if (tkey()[k] != NONE) list[atomicAdd(&sm.head, 1)] = k;
     bar();
     if (nt <= 128) {
+#pragma unroll 1
         for (int k = tid; k < nt; k += T) {
             const int s = list[k], j = tkey()[s];
             int rank = 0;
+#pragma unroll 1
             for (int q = 0; q < nt; ++q) rank += tkey()[list[q]] < j;
             ord[rank] = s;
         }
     } else {   // bitonic sort
         int n2 = 128;
         while (n2 < nt) n2 <<= 1;
+#pragma unroll 1
         for (int k = tid; k < n2; k += T) ord[k] = k < nt ? list[k] : NONE;
         bar();
+#pragma unroll 1
         for (int size = 2; size <= n2; size <<= 1)
+#pragma unroll 1
             for (int step = size >> 1; step > 0; step >>= 1) {
+#pragma unroll 1
                 for (int k = tid; k < n2 / 2; k += T) {
                     const int lo = 2 * k - (k & (step - 1)), hi = lo + step;
                     const int a = ord[lo], c = ord[hi];
@@ -1146,6 +1173,7 @@ __device__ __forceinline__ void Group<R, PL, TEAM, LK>::run(int item, int32_t* d
     }
     double fx = 0.0, fy = 0.0, en = 0.0;
     const double* fr = m.frame + 9 * (size_t)f0;
+#pragma unroll 1
     for (int k = tid; k < nt; k += T) {
         const int s = ord[k];
         int l = TEAM ? own[s] : s;
