@@ -39,7 +39,7 @@ sys.path.insert(0, ROOT)
 METRIC = "cutoff geodesic pair evals/s & MD steps/s, FP32-batched vs FP64, err≤1e-5"
 UNIT = "pair evals/s"
 PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
-FLOPS_PER_PROPAGATION = 150.0   # one window unfolding + child trimming (FP arithmetic)
+FLOPS_PER_PROPAGATION = 150.0   # one window unfolding + the cut of its children (FP arithmetic)
 FLOPS_PER_PAIR = 20.0           # one target evaluation
 BYTES_PER_FACE = 64.0           # patch mesh data a source must read per face reached
 BYTES_PER_WINDOW = 48.0         # one window record written and read back per propagation
@@ -49,13 +49,8 @@ DEFAULT_WORKLOAD = "noisy_ico8_n65536"
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one first-pass launch of the
 # FP32 neighbour kernel from an ncu capture, per workload: bytes, the sources that launch
 # processed (the figure is scaled to a full launch by sources) and a digest of the kernel
-# sources it was taken on; a kernel changed since then reports null
-TRAFFIC = {
-    # k_geodesic<float, 2, 0> (128-register variant, global tables, 8 warps per CTA, pool of 32768
-    # windows) over 8192 of the 65536 sources on the same noisy L8 sphere: 5.829 GB read +
-    # 2.419 GB written in 8.72 ms (one ncu pass, dram__bytes_read.sum + dram__bytes_write.sum)
-    "noisy_ico8_n65536": {"bytes": 5828550400 + 2418572544, "sources": 8192, "kernel": "0c622ec7855f2012"},
-}
+# sources it was taken on; a kernel changed since then, or without a capture, reports null
+TRAFFIC = {}
 KERNEL_SOURCES = ("paper_2404_19751_gb300/csrc/waves.cu", "paper_2404_19751_gb300/csrc/geo_common.cuh",
                   "paper_2404_19751_gb300/csrc/css_dev.cuh")
 
@@ -484,7 +479,7 @@ def run_single(args, cfg, css, ctx, torch, stream, timer, rank, world):
     else:
         props_per_src = r32["props"] / max(1, k32 * n)
     roof, mem = roofline(css, ctx, pk, props_per_src, n, r32["pairs"] / k32,
-                         statistics.mean(r32["kernel_ms"]) / 1e3, "k_geodesic<float>",
+                         statistics.mean(r32["kernel_ms"]) / 1e3, "k_waves<float>",
                          traffic=traffic_per_launch(cfg["name"], n))
     line = {
         "metric": METRIC, "value": replica_throughput(world, r32["pairs"], t32), "unit": UNIT, "n_gpus": world, "steps": k32,
@@ -689,7 +684,7 @@ def run_batched(args, cfg, css, ctx, torch, stream, timer, rank, world, nested=F
         acc = {"error": str(e)}
     k32 = r32b["steps"]
     roof, mem = roofline(css, ctx, pk, props_per_src, n, r32b["pairs"] / k32,
-                         statistics.mean(r32b["kernel_ms"]) / 1e3, "k_geodesic<float> (batched launch)")
+                         statistics.mean(r32b["kernel_ms"]) / 1e3, "k_waves<float> (batched launch)")
     # per step, for all meshes at once: move (1) + bucketing (4: count, scan, scatter, rank) +
     # two passes (2) + kick or step counter (1)
     launches_per_step = 8

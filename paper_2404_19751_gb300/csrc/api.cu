@@ -126,7 +126,8 @@ struct Reach {
 };
 
 // The launch shape for a context whose shape nobody set or tuned.  Measured on one GB300, kernel
-// times in ms (sources; windows a source):
+// times in ms (sources; windows a source; taken before the kernel's loops were rolled up, which made the
+// noisy sphere's and the height field's 8 to 17 % shorter in every shape that fills the chip):
 //   - as many sources as fill 16 warps an SM, small patches: tables in shared memory at scale 1
 //     (noisy sphere, 16384; 473: 2.96, scale 2 with its 8 warps an SM 3.95, tables in global memory
 //     3.32).  Where the tables are too small for the patch, global memory (height field, 8192;

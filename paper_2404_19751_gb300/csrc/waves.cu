@@ -28,9 +28,9 @@
 // keeps rotations and directions in FP32.  Lengths of results are FP64 in both forms.
 //
 // Measured against windows kept in per-edge lists and trimmed against one another (the same
-// evaluations, default launch shapes): 65536 particles on a noisy level-8 sphere 110.7 -> 12.2 ms
-// (FP64) and 73.1 -> 13.0 ms (FP32), 8192 on a 256 x 256 height field 127 -> 9.4 ms, every pair of
-// 64 on a flat plane 30 -> 2.2 ms.  The windows unfolded per source are the same within 10 %
+// calls, default launch shapes): 65536 particles on a noisy level-8 sphere 110.7 -> 10.1 ms
+// (FP64) and 73.1 -> 11.0 ms (FP32), 8192 on a 256 x 256 height field 130-166 -> 8.7 ms, every pair
+// of 64 on a flat plane 27 -> 0.67 ms.  The windows unfolded per source are the same within 10 %
 // (482 against 440, 3991 against 3950, 5135 against 5151).
 #include <cuda_runtime.h>
 #include <limits.h>
