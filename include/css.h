@@ -52,8 +52,8 @@ extern "C" {
 
 /* ---------------------------------------------------------------- enums */
 #define CSS_FP64 0   /* every window, distance and walk operation in FP64            */
-#define CSS_FP32 1   /* FP32 window arithmetic; FP64 kept for unfolded source
-                        coordinates, near-degenerate predicates and the face walk  */
+#define CSS_FP32 1   /* FP32 target tests, path directions and tie rule; FP64 kept for
+                        windows, lengths, near-degenerate predicates and the face walk */
 
 #define CSS_POT_HARMONIC 0   /* U = eps (1 - l/sigma)^2            for l < r_cut     */
 #define CSS_POT_WCA      1   /* U = 4 eps ((s/l)^12 - (s/l)^6) + eps for l < r_cut   */

@@ -564,7 +564,7 @@ int css_mesh_free(css_mesh* m) {
     if (!m) return CSS_ERR_INVALID_ARG;
     cudaFree(m->he); cudaFree(m->twin); cudaFree(m->edge); cudaFree(m->fv); cudaFree(m->lay);
     cudaFree(m->frame); cudaFree(m->theta); cudaFree(m->pseudo); cudaFree(m->bnd);
-    cudaFree(m->ring_start); cudaFree(m->ring); cudaFree(m->X); cudaFree(m->he32); cudaFree(m->lay32);
+    cudaFree(m->ring_start); cudaFree(m->ring); cudaFree(m->X); cudaFree(m->he32);
     cudaFree(m->frank);
     cudaFree(m->cang);
     cudaFree(m->htop);

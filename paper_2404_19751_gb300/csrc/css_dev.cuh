@@ -48,7 +48,6 @@ struct DMesh {
     const int32_t* ring_start;    // nv + 1
     const int32_t* ring;          // 3 nf corners h with fv[h] == v, grouped by vertex
     const HeRec32* he32;          // 3 nf, FP32 copies of he
-    const float* lay32;           // 3 nf, FP32 copies of lay
     const int32_t* frank;         // nf: rank of each face along a Morton curve (bucket order)
     const float2* cang;           // 3 nf: (start, width) of corner h around its vertex, angles
                                   // counted counter-clockwise from one fixed edge; NaN on boundary

@@ -93,7 +93,6 @@ struct css_mesh {
     int32_t* ring = nullptr;
     double* X = nullptr;
     css::HeRec32* he32 = nullptr;
-    float* lay32 = nullptr;
     int32_t* frank = nullptr;   // nf: Morton rank of each face
     float2* cang = nullptr;     // 3 nf: corner (start, width) around its vertex
     int4* htop = nullptr;       // 3 nf: half-edge topology (css::DMesh::htop)
@@ -217,7 +216,7 @@ struct WaveLay {
     int itan, iback, ihc;                              // path records of vertices that start windows
     int emit;                                          // vertices waiting to start windows
     int tkey, tdist, tvert, tlist;                     // targets
-    int ttan, tcmp;                                    // their directions and compared lengths (a team: its log's)
+    int ttan;                                          // their directions (a team: its log's)
     int ldist, lslot;                                  // a team's log of improvements
     int t_bytes;                                       // tables
     int s[6], s_bytes;                                 // spill area (global memory)

@@ -24,8 +24,12 @@
 // A window's cone is two directions in the frame of its pseudo-source, where they stay what
 // they are through every unfolding (the direction to the vertex that bounds the cone), so no
 // error builds up and no ray has to be cut with an edge in FP64: the interval on the edge is
-// FP32 and rounded outward.  The pseudo-source's image s is FP64 in both forms; the FP32 form
-// keeps rotations and directions in FP32.  Lengths of results are FP64 in both forms.
+// FP32 and rounded outward.  Windows are the same in both forms, FP64 images, rotations and rims:
+// with a rotation of its own in FP32, each of the two children of a corner drifts by 6e-8 of a turn
+// an unfolding, and behind a flat vertex nothing covers the gap between them (100 of 6 M pairs of a
+// flat sheet of 80 x 80 vertices were lost, 1270 of 4 M at 200 x 200; with FP32 rims alone 1 of 6 M).
+// The FP32 form tests its targets and keeps the directions of paths in FP32; lengths of results are
+// FP64 in both forms.
 //
 // Measured against windows kept in per-edge lists and trimmed against one another (the same
 // calls, default launch shapes): 65536 particles on a noisy level-8 sphere 110.7 -> 10.1 ms
@@ -96,7 +100,8 @@ struct Index<0> {
     static __device__ __forceinline__ int2 make(int a, int b) { return make_int2(a, b); }
 };
 
-// relative tolerance of a point on the rim of a cone
+// tolerance of a point on the rim of a cone, relative to its distance (FP32: the roundings of the
+// target's point, the rotation and the rim add up to 6.5e-7 at most)
 template <class R>
 struct Rim;
 template <>
@@ -217,6 +222,11 @@ __device__ __forceinline__ double f64(float x) {   // x > 0 and normal
     const unsigned f = __float_as_uint(x);
     return __hiloint2double((int)((f >> 3) + 0x38000000u), (int)(f << 29));
 }
+template <class R>
+__device__ __forceinline__ V2<R> narrow(double2 v) {
+    if constexpr (sizeof(R) == 8) return v;
+    else return make_float2(f32(v.x), f32(v.y));
+}
 __device__ __forceinline__ bool is_inf(double x) { return __double2hiint(x) == 0x7ff00000; }
 // square root to 2^-22
 __device__ __forceinline__ float root(float x) { return x > 0.0f ? x * rsqrtf(x) : 0.0f; }
@@ -248,7 +258,9 @@ __device__ __forceinline__ float cut_at(float sx, float s2, float a, float L, fl
 // straight piece from a vertex of the target's own face are kept apart from those that come
 // through a window: a window wins over them unless they are shorter by more than the form's
 // precision, so that a direction does not hang on the last bits of two equal lengths (FP32 form; in
-// FP64 the shorter one is the one).  One warp writes the direction of an improvement beside the
+// FP64 the shorter one is the one).  The lengths compared are the FP64 ones: FP32 lengths of their
+// own cost two loads, a root and a record a target and 16 % of the kernel (16384 sources on a noisy
+// sphere 2.86 against 2.45 ms).  One warp writes the direction of an improvement beside the
 // length it lowered; a team's warps, which may lower one length at the same time, log them, and the
 // log is read once the source is done.
 template <class R, int PL, bool TEAM, bool LK>
@@ -257,7 +269,7 @@ __device__ __noinline__ void eval_tests(const cssi::GeoJob& J, const WaveLay& Y,
     const DMesh& m = J.m;
     bool won = false, apart = false;
     int s = NONE;
-    double d = 0.0, w = 0.0;
+    double d = 0.0;
     V2<R> t = vec2((R)0, (R)0);
     unsigned long long bits = 0;
     if (lane < nev) {
@@ -267,7 +279,8 @@ __device__ __noinline__ void eval_tests(const cssi::GeoJob& J, const WaveLay& Y,
         const bool vertex = vs >= 0 && (vs & FROM_VERTEX);
         if (vertex) vs &= ~FROM_VERTEX;
         const double2 S = at<double2>(e, Y.e[0])[lane];
-        const V2<R> rot = at<V2<R>>(e, Y.e[1])[lane], d0 = at<V2<R>>(e, Y.e[2])[lane], d1 = at<V2<R>>(e, Y.e[3])[lane];
+        const V2<R> rot = narrow<R>(at<double2>(e, Y.e[1])[lane]);
+        const V2<R> d0 = narrow<R>(at<double2>(e, Y.e[2])[lane]), d1 = narrow<R>(at<double2>(e, Y.e[3])[lane]);
         const HeRec& r = m.he[he];
         const int k = he % 3;
         const double* bj = J.bary + 3 * (size_t)j;
@@ -275,7 +288,8 @@ __device__ __noinline__ void eval_tests(const cssi::GeoJob& J, const WaveLay& Y,
         const double gx = bv * r.L + bc * r.cx - S.x, gy = bc * r.cy - S.y;
         const R fx = (R)gx, fy = (R)gy;
         const R qx = fx * rot.x + fy * rot.y, qy = fy * rot.x - fx * rot.y;
-        const R tol = Rim<R>::t * (R)r.L;
+        // the cross products round with the distance, not with the edge
+        const R tol = Rim<R>::t * (fabs(fx) + fabs(fy) + (R)r.L);
         const bool in = d0.x * qy - d0.y * qx <= tol * (fabs(d0.x) + fabs(d0.y)) &&
                         d1.x * qy - d1.y * qx >= -tol * (fabs(d1.x) + fabs(d1.y));
         const double n = sqrt(gx * gx + gy * gy), sig = vs < 0 ? 0.0 : at<double>(b, Y.vdist)[vs];
@@ -295,22 +309,6 @@ __device__ __noinline__ void eval_tests(const cssi::GeoJob& J, const WaveLay& Y,
                 const R inv = n > 0.0 ? (R)1 / (R)n : (R)0;
                 t = vec2(qx * inv, qy * inv);
             } else t = at<V2<R>>(b, Y.itan)[at<typename Index<PL>::type>(b, Y.vinfo)[vs]];
-            // the length that decides between a window and a vertex: from FP32 coordinates of the
-            // target in its face, like every other comparison of that form
-            if constexpr (sizeof(R) == 4) {
-                const int f = he / 3;
-                const float L01 = m.lay32[3 * f], x2 = m.lay32[3 * f + 1], y2 = m.lay32[3 * f + 2];
-                const float px = (float)bj[1] * L01 + (float)bj[2] * x2, py = (float)bj[2] * y2;
-                const float ax = k == 0 ? 0.0f : (k == 1 ? L01 : x2), ay = k == 2 ? y2 : 0.0f;
-                if (vertex) w = sig + (double)sqrtf((px - ax) * (px - ax) + (py - ay) * (py - ay));
-                else {
-                    const float bx = k == 0 ? L01 : (k == 1 ? x2 : 0.0f), by = k == 1 ? y2 : 0.0f, L = m.he32[he].L;
-                    const float ex = (bx - ax) / L, ey = (by - ay) / L;
-                    const float hx = (px - ax) * ex + (py - ay) * ey - (float)S.x;
-                    const float hy = ex * (py - ay) - ey * (px - ax) - (float)S.y;
-                    w = (double)((float)sig + sqrtf(hx * hx + hy * hy));
-                }
-            }
         }
     }
     if constexpr (TEAM) {
@@ -320,7 +318,6 @@ __device__ __noinline__ void eval_tests(const cssi::GeoJob& J, const WaveLay& Y,
             else {
                 at<double>(b, Y.ldist)[l] = d;
                 at<V2<R>>(b, Y.ttan)[l] = t;
-                if constexpr (sizeof(R) == 4) at<double>(b, Y.tcmp)[l] = w;
                 at<int>(b, Y.lslot)[l] = apart ? s | FROM_VERTEX : s;
             }
         }
@@ -330,7 +327,6 @@ __device__ __noinline__ void eval_tests(const cssi::GeoJob& J, const WaveLay& Y,
         const int at_ = apart ? s + (1 << Y.th_log) : s;   // records of windows, then of vertices
         if (won && *((volatile unsigned long long*)at<double>(b, apart ? Y.tvert : Y.tdist) + s) == bits) {
             at<V2<R>>(b, Y.ttan)[at_] = t;
-            if constexpr (sizeof(R) == 4) at<double>(b, Y.tcmp)[at_] = w;
             if constexpr (LK) {
                 const int4 w4 = at<int4>(e, Y.e[4])[lane];
                 const double2 S = at<double2>(e, Y.e[0])[lane];
@@ -346,10 +342,9 @@ __device__ __noinline__ void eval_tests(const cssi::GeoJob& J, const WaveLay& Y,
 }
 
 // ------------------------------------------------------------------ one source
-template <class R>
 struct Win {
-    double2 s;          // the pseudo-source in the frame of half-edge he
-    V2<R> rot, d0, d1;  // image of its own frame's x axis; left and right rim of the cone, in its frame
+    double2 s, rot;     // the pseudo-source in the frame of half-edge he; image of its own frame's x axis
+    double2 d0, d1;     // left and right rim of the cone, in its frame
     float b0, b1, key;
     int he, vs;
     int su, sv;         // slots of the edge's end vertices
@@ -421,16 +416,16 @@ struct Group {
             }
         }
     }
-    __device__ __forceinline__ void put_test(int k, double2 s, V2<R> rot, V2<R> d0, V2<R> d1, int he, int vs, int j) {
+    __device__ __forceinline__ void put_test(int k, double2 s, double2 rot, double2 d0, double2 d1, int he, int vs, int j) {
         at<double2>(e, Y.e[0])[k] = s;
-        at<V2<R>>(e, Y.e[1])[k] = rot;
-        at<V2<R>>(e, Y.e[2])[k] = d0;
-        at<V2<R>>(e, Y.e[3])[k] = d1;
+        at<double2>(e, Y.e[1])[k] = rot;
+        at<double2>(e, Y.e[2])[k] = d0;
+        at<double2>(e, Y.e[3])[k] = d1;
         at<int4>(e, Y.e[4])[k] = make_int4(he, vs, j, 0);
     }
     // every particle of the face is seen: a cone of no directions holds all
-    __device__ __forceinline__ void put_open_test(int k, double2 s, V2<R> rot, int he, int vs, int j) {
-        const V2<R> none = vec2((R)0, (R)0);
+    __device__ __forceinline__ void put_open_test(int k, double2 s, double2 rot, int he, int vs, int j) {
+        const double2 none = make_double2(0.0, 0.0);
         put_test(k, s, rot, none, none, he, vs, j);
     }
 
@@ -447,16 +442,16 @@ struct Group {
         b1 = i1 == 65535u ? L : (float)i1 * (L * (1.0f / 65535.0f));
     }
 
-    __device__ __forceinline__ void store(unsigned char* to, const int* o, int k, const Win<R>& w, int b01) {
+    __device__ __forceinline__ void store(unsigned char* to, const int* o, int k, const Win& w, int b01) {
         at<double2>(to, o[0])[k] = w.s;
-        at<V2<R>>(to, o[1])[k] = w.rot;
-        at<V2<R>>(to, o[2])[k] = w.d0;
-        at<V2<R>>(to, o[3])[k] = w.d1;
+        at<double2>(to, o[1])[k] = w.rot;
+        at<double2>(to, o[2])[k] = w.d0;
+        at<double2>(to, o[3])[k] = w.d1;
         at<int4>(to, o[4])[k] = make_int4(w.he, w.vs, __float_as_int(w.key), b01);
         at<typename Index<PL>::pair>(to, o[5])[k] = Index<PL>::make(w.su, w.sv);
     }
     // append windows (lanes with has): to the ring up to position `lim`, then to the spill area
-    __device__ __forceinline__ void push(bool has, const Win<R>& w, float L, int lim) {
+    __device__ __forceinline__ void push(bool has, const Win& w, float L, int lim) {
         const unsigned mk = __ballot_sync(CSS_FULL, has);
         if (!mk) return;
         const int n = __popc(mk);
@@ -574,7 +569,7 @@ __device__ __forceinline__ void Group<R, PL, TEAM, LK>::seed(int f0, double b1, 
     const double ex = (bx - ax) / r.L, ey = (by - ay) / r.L;
     const double vx = hy * ey - hx * ex, vy = -hy * ex - hx * ey;   // from the source to the corner, in the layout
     tests(lane == 0, m.frank ? m.frank[f0] : f0, [&](int k, int j) {   // half-edge 0's frame is the layout's
-        put_open_test(k, make_double2(hx, hy), vec2((R)1, (R)0), hh, NONE, j);
+        put_open_test(k, make_double2(hx, hy), make_double2(1.0, 0.0), hh, NONE, j);
     });
     // a source on a corner (to the rounding of its position) has no direction to it: its windows start at the vertex, all around
     const double vd = sqrt(hx * hx + hy * hy);
@@ -593,13 +588,13 @@ __device__ __forceinline__ void Group<R, PL, TEAM, LK>::seed(int f0, double b1, 
         return;
     }
     const int tw = m.twin[hh];
-    Win<R> w;
+    Win w;
     w.he = tw;
     w.vs = NONE;
     w.s = make_double2(lx, -hy);   // the twin runs from the edge's end to its start
-    w.rot = vec2((R)-ex, (R)ey);
-    w.d0 = vec2((R)(lx * ex + hy * ey), (R)(lx * ey - hy * ex));
-    w.d1 = vec2((R)vx, (R)vy);
+    w.rot = make_double2(-ex, ey);
+    w.d0 = make_double2(lx * ex + hy * ey, lx * ey - hy * ex);
+    w.d1 = make_double2(vx, vy);
     w.b0 = 0.0f;
     w.b1 = (float)r.L;
     w.key = key_of((float)lx, (float)-hy, 0.0f, w.b0, w.b1);
@@ -653,7 +648,7 @@ __device__ __forceinline__ void Group<R, PL, TEAM, LK>::seed_at_vertex(int hc) {
             const HeRec r = m.he[g];
             const double co = cos(phi), si = sin(phi);
             tests(lane == 0 && g != hc, m.frank ? m.frank[fh] : fh, [&](int t, int j) {
-                put_open_test(t, make_double2(0.0, 0.0), vec2((R)co, (R)-si), g, NONE, j);
+                put_open_test(t, make_double2(0.0, 0.0), make_double2(co, -si), g, NONE, j);
             });
             const double ang = atan2(r.cy, r.cx), lc = sqrt(r.cx * r.cx + r.cy * r.cy);
             int slot = NONE;
@@ -678,16 +673,16 @@ __device__ __forceinline__ void Group<R, PL, TEAM, LK>::seed_at_vertex(int hc) {
             const int s1 = __shfl_sync(CSS_FULL, slot, 0), s2 = __shfl_sync(CSS_FULL, slot, 1);
             __syncwarp();
             const int hop = 3 * fh + (kh == 2 ? 0 : kh + 1);
-            Win<R> w;
+            Win w;
             w.he = m.twin[hop];
             w.vs = NONE;
             const HeRec o = m.he[hop];
             w.s = make_double2(o.L - o.cx, -o.cy);
             // the twin's x axis runs from the face's far corner c to the first edge's end
             const double tx = (r.L - r.cx) / o.L, ty = -r.cy / o.L;
-            w.rot = vec2((R)(tx * co - ty * si), (R)-(tx * si + ty * co));
-            w.d0 = vec2((R)(r.cx * co - r.cy * si), (R)(r.cx * si + r.cy * co));
-            w.d1 = vec2((R)(r.L * co), (R)(r.L * si));
+            w.rot = make_double2(tx * co - ty * si, -(tx * si + ty * co));
+            w.d0 = make_double2(r.cx * co - r.cy * si, r.cx * si + r.cy * co);
+            w.d1 = make_double2(r.L * co, r.L * si);
             w.b0 = 0.0f;
             w.b1 = (float)o.L;
             w.key = key_of((float)w.s.x, (float)w.s.y, 0.0f, w.b0, w.b1);
@@ -787,9 +782,9 @@ __device__ __forceinline__ void Group<R, PL, TEAM, LK>::emit(int ne, int lim, fl
                 }
             }
             tests(hit, hit ? m.htop[hc].w : 0, [&](int k, int j) {
-                put_open_test(k, make_double2(0.0, 0.0), vec2((R)1, (R)0), hc, o_vs | FROM_VERTEX, j);
+                put_open_test(k, make_double2(0.0, 0.0), make_double2(1.0, 0.0), hc, o_vs | FROM_VERTEX, j);
             });
-            Win<R> w;
+            Win w;
             bool ok = false;
             float L = 0.0f;
             if (hit) {
@@ -800,7 +795,7 @@ __device__ __forceinline__ void Group<R, PL, TEAM, LK>::emit(int ne, int lim, fl
                     L = (float)r.L;
                     w.vs = o_vs | FIRST;
                     w.s = make_double2(r.L - r.cx, -r.cy);
-                    w.rot = vec2((R)1, (R)0);
+                    w.rot = make_double2(1.0, 0.0);
                     w.b0 = 0.0f;
                     w.b1 = L;
                     if (o_th != 0.0f) {
@@ -818,8 +813,8 @@ __device__ __forceinline__ void Group<R, PL, TEAM, LK>::emit(int ne, int lim, fl
                             w.b0 = fmaxf(0.0f, L * (1.0f - x) - 1e-5f * L);
                         }
                     }
-                    w.d0 = vec2((R)((double)w.b0 - w.s.x), (R)-w.s.y);
-                    w.d1 = vec2((R)((w.b1 == L ? r.L : (double)w.b1) - w.s.x), (R)-w.s.y);
+                    w.d0 = make_double2((double)w.b0 - w.s.x, -w.s.y);
+                    w.d1 = make_double2((w.b1 == L ? r.L : (double)w.b1) - w.s.x, -w.s.y);
                     const int4 tp = m.htop[w.he];
                     w.su = vertex(tp.x & css::VMASK);
                     w.sv = vertex(tp.y & css::VMASK);
@@ -848,7 +843,7 @@ __device__ __forceinline__ void Group<R, PL, TEAM, LK>::wave(int head, int n) {
     const HeRec r = m.he[he];
     const css::HeRec32 q = m.he32[he];
     tests(on, tp.w, [&](int k, int j) {
-        put_test(k, at<double2>(h, Y.r[0])[s], at<V2<R>>(h, Y.r[1])[s], at<V2<R>>(h, Y.r[2])[s], at<V2<R>>(h, Y.r[3])[s],
+        put_test(k, at<double2>(h, Y.r[0])[s], at<double2>(h, Y.r[1])[s], at<double2>(h, Y.r[2])[s], at<double2>(h, Y.r[3])[s],
                  he, vs, j);
     });
     const double2 S = at<double2>(h, Y.r[0])[s];
@@ -865,17 +860,18 @@ __device__ __forceinline__ void Group<R, PL, TEAM, LK>::wave(int head, int n) {
     const float xc = fsx - fgx * __fdividef(fsy, fgy);
     bool in0, in1, beyond0, beyond1;   // c on or right of the left rim, on or left of the right rim; strictly
     {
-        const V2<R> rot = at<V2<R>>(h, Y.r[1])[s], d0 = at<V2<R>>(h, Y.r[2])[s], d1 = at<V2<R>>(h, Y.r[3])[s];
+        const double2 rot = at<double2>(h, Y.r[1])[s], d0 = at<double2>(h, Y.r[2])[s], d1 = at<double2>(h, Y.r[3])[s];
         const float rx = f32(rot.x), ry = f32(rot.y), px = fgx * rx + fgy * ry, py = fgy * rx - fgx * ry;
         const float ax = f32(d0.x), ay = f32(d0.y), bx = f32(d1.x), by = f32(d1.y);
         const float cr0 = ax * py - ay * px, cr1 = bx * py - by * px;   // < 0: c lies right of the rim
-        const float t = (sizeof(R) == 4 ? Rim<float>::t : 8e-6f) * (fabsf(fgx) + fabsf(fgy) + (sizeof(R) == 4 ? 0.0f : size));
+        const float t = 8e-6f * (fabsf(fgx) + fabsf(fgy) + size);
         const float t0 = t * (fabsf(ax) + fabsf(ay)), t1 = t * (fabsf(bx) + fabsf(by));
         in0 = cr0 <= t0;
         beyond0 = cr0 < -t0;
         in1 = cr1 >= -t1;
         beyond1 = cr1 > t1;
-        if (sizeof(R) == 8 && (TEAM ? on && ((in0 && !beyond0) || (in1 && !beyond1)) : __builtin_expect(on && ((in0 && !beyond0) || (in1 && !beyond1)), 0))) {   // too close to a rim for FP32
+        const bool near = on && ((in0 && !beyond0) || (in1 && !beyond1));
+        if (TEAM ? near : __builtin_expect(near, 0)) {   // too close to a rim for FP32
             const double gx = r.cx - S.x, gy = r.cy - S.y;
             const double ex = gx * rot.x + gy * rot.y, ey = gy * rot.x - gx * rot.y;
             const double tg = Rim<double>::t * (fabs(gx) + fabs(gy));
@@ -915,7 +911,7 @@ __device__ __forceinline__ void Group<R, PL, TEAM, LK>::wave(int head, int n) {
                 roots(vx * vx + vy * vy, n, inv);
                 d = sig + n;
                 if (vs < 0) {
-                    const V2<R> rot = at<V2<R>>(h, Y.r[1])[s];
+                    const V2<R> rot = narrow<R>(at<double2>(h, Y.r[1])[s]);
                     const R gx = (R)vx, gy = (R)vy, ri = (R)inv;
                     t = vec2((gx * rot.x + gy * rot.y) * ri, (gy * rot.x - gx * rot.y) * ri);
                 }
@@ -959,10 +955,10 @@ __device__ __forceinline__ void Group<R, PL, TEAM, LK>::wave(int head, int n) {
         const int ps = (head + tid - lane + par) & Y.r_mask;
         const int4 pw = at<int4>(h, Y.r[4])[ps];
         const double2 PS = at<double2>(h, Y.r[0])[ps];
-        const V2<R> rot = at<V2<R>>(h, Y.r[1])[ps];
-        Win<R> w;
-        w.d0 = at<V2<R>>(h, Y.r[2])[ps];
-        w.d1 = at<V2<R>>(h, Y.r[3])[ps];
+        const double2 rot = at<double2>(h, Y.r[1])[ps];
+        Win w;
+        w.d0 = at<double2>(h, Y.r[2])[ps];
+        w.d1 = at<double2>(h, Y.r[3])[ps];
         __syncwarp();
         bool has = is;
         float Lc = 1.0f;
@@ -977,17 +973,15 @@ __device__ __forceinline__ void Group<R, PL, TEAM, LK>::wave(int head, int n) {
             w.su = a ? psc : psu;
             w.sv = a ? psv : psc;
             if (code & 64) {
-                const R fx = (R)cx, fy = (R)cy;
-                const V2<R> pc = vec2(fx * rot.x + fy * rot.y, fy * rot.x - fx * rot.y);
+                const double2 pc = make_double2(cx * rot.x + cy * rot.y, cy * rot.x - cx * rot.y);
                 if (a) w.d0 = pc;
                 else w.d1 = pc;
             }
             const double co = a ? pr.cr : pr.cl, si = a ? pr.sr : pr.sl;
-            const R fco = sizeof(R) == 4 ? (R)(a ? pq.cr : pq.cl) : (R)co, fsi = sizeof(R) == 4 ? (R)(a ? pq.sr : pq.sl) : (R)si;
             const double ux = a ? -cx : PS.x, uy = a ? -cy : PS.y;   // s from the child edge's start
             w.s = make_double2(ux * co + uy * si, uy * co - ux * si);
             if (__double2hiint(w.s.y) >= 0) w.s.y = 0.0;   // rounding: s never lies above the edge
-            w.rot = vec2(rot.x * fco + rot.y * fsi, rot.y * fco - rot.x * fsi);
+            w.rot = make_double2(rot.x * co + rot.y * si, rot.y * co - rot.x * si);
             // the interval: where the rays through b0 and b1 meet the child's edge, rounded outward
             const float sx = f32(PS.x), sy = f32(PS.y), sg = f32(psig);
             const float pem = 4e-6f * (fabsf(sx) + fabsf(sy) + pq.L);
@@ -1065,9 +1059,9 @@ __device__ __forceinline__ void Group<R, PL, TEAM, LK>::run(int item, int32_t* d
             for (int k = tid; k < back; k += T) {
                 const int i = (from + k) & (Y.s_cap - 1), o = (tail + k) & Y.r_mask;
                 at<double2>(h, Y.r[0])[o] = at<double2>(x, Y.s[0])[i];
-                at<V2<R>>(h, Y.r[1])[o] = at<V2<R>>(x, Y.s[1])[i];
-                at<V2<R>>(h, Y.r[2])[o] = at<V2<R>>(x, Y.s[2])[i];
-                at<V2<R>>(h, Y.r[3])[o] = at<V2<R>>(x, Y.s[3])[i];
+                at<double2>(h, Y.r[1])[o] = at<double2>(x, Y.s[1])[i];
+                at<double2>(h, Y.r[2])[o] = at<double2>(x, Y.s[2])[i];
+                at<double2>(h, Y.r[3])[o] = at<double2>(x, Y.s[3])[i];
                 at<int4>(h, Y.r[4])[o] = at<int4>(x, Y.s[4])[i];
                 at<typename Index<PL>::pair>(h, Y.r[5])[o] = at<typename Index<PL>::pair>(x, Y.s[5])[i];
             }
@@ -1181,12 +1175,7 @@ __device__ __forceinline__ void Group<R, PL, TEAM, LK>::run(int item, int32_t* d
         if constexpr (sizeof(R) == 4) {
             const double dv = tvert()[s];
             const int lv = TEAM ? ownv[s] : s + (1 << Y.th_log);
-            bool vertex = !(d < CUDART_INF);
-            if (!vertex && dv < d) {
-                const double cw = at<double>(b, Y.tcmp)[l], cv = at<double>(b, Y.tcmp)[lv];
-                vertex = cv < cw - TIE32 * cv;
-            }
-            if (vertex) {
+            if (dv < d - TIE32 * dv) {
                 l = lv;
                 d = dv;
             }
@@ -1340,9 +1329,7 @@ WaveLay lay_out(int ring_log, int s_cap, int vh_log, int th_log, bool shared, bo
         return p;
     };
     auto record = [&](int* to, int n) {
-        to[0] = take(n, 16);
-        for (int k = 1; k < 4; ++k) to[k] = take(n, 2 * sizeof(R));
-        to[4] = take(n, 16);
+        for (int k = 0; k < 5; ++k) to[k] = take(n, 16);
         to[5] = take(n, 2 * ix);
     };
     record(y.r, RG);
@@ -1355,7 +1342,7 @@ WaveLay lay_out(int ring_log, int s_cap, int vh_log, int th_log, bool shared, bo
     y.emit = take(2 * y.i_cap, ix);
     y.tkey = take(TH, 4); y.tdist = take(TH, 8); y.tvert = take(sizeof(R) == 4 ? TH : 0, 8);
     const int recs = team ? y.lg_cap : (sizeof(R) == 4 ? 2 * TH : TH);
-    y.ttan = take(recs, 2 * sizeof(R)); y.tcmp = take(sizeof(R) == 4 ? recs : 0, 8);
+    y.ttan = take(recs, 2 * sizeof(R));
     y.ldist = take(y.lg_cap, 8); y.lslot = take(y.lg_cap, 4);
     y.t_bytes = o;
     o = 0;
