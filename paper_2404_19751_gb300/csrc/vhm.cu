@@ -493,12 +493,15 @@ __device__ __forceinline__ Cluster this_cluster_of_column() {
     return c;
 }
 
-// inverse diagonals of the heat systems divided by t and of the Poisson system
-__global__ void k_row_scale(Rows o, double t, double* inv_heat, double* inv_diag) {
+// inverse diagonals of the heat systems divided by t and of the Poisson system; the heat systems'
+// relaxation factor of each row (see heat_column)
+__global__ void k_row_scale(Rows o, double t, double* inv_heat, double* inv_diag, double* relax) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= o.np) return;
-    inv_heat[p] = o.vert[p] >= 0 ? 1.0 / (o.mass[p] / t + o.diag[p]) : 0.0;
+    const double d = o.mass[p] / t + o.diag[p], rho = o.diag[p] / d;
+    inv_heat[p] = o.vert[p] >= 0 ? 1.0 / d : 0.0;
     inv_diag[p] = o.vert[p] >= 0 ? 1.0 / o.diag[p] : 0.0;
+    relax[p] = rho > 0.0 && rho < 1.0 ? 2.0 / (1.0 + sqrt(1.0 - rho * rho)) : 1.0;
 }
 
 __device__ __forceinline__ void row_terms(const Rows& o, int e, const double* x, double& acc) {
@@ -524,16 +527,18 @@ __device__ __forceinline__ void first(double2 v, double2& o) { o = v; }
 
 // Sweeps of one heat system (divided by t) over one column until a sweep changes no entry
 // by more than 1e-14 of the terms it is summed from (in the largest component).  The sweeps
-// are over-relaxed with the factor of Young's theory, 2 / (1 + sqrt(1 - rho^2)), rho the
-// ratio of the off-diagonal sum to the diagonal: it both minimises the number of sweeps and is
-// the largest factor at which rounding errors do not grow with distance from the source
-// relative to the solution's own decay (with rho = 0.8, t = h^2: 252 plain sweeps, 120 relaxed
-// ones on a torus of 4005 vertices; at t = 0.1 h^2 a factor of 1.35 instead of 1.04 loses the far
-// field).  Every eighth sweep is a plain one and is the one that checks.  After plain_after
-// sweeps all are plain.
+// are over-relaxed, each row with its own factor of Young's theory, 2 / (1 + sqrt(1 - rho^2)), rho
+// the ratio of the row's off-diagonal sum to its diagonal: it both minimises the number of sweeps
+// and is the largest factor at which rounding errors do not grow with distance from the source
+// relative to the solution's own decay (at t = 0.1 h^2 a factor of 1.35 instead of 1.04 loses the far
+// field).  All factors lie in [1, 2), so the sweeps converge whatever they are.  One factor from
+// the mesh's mean rho is too large where a graded mesh is coarse: such sweeps went on to
+// plain_after (a 64 x 64 grid graded 1 : 10 along both axes: 4104 of them, 976 plain ones, 264 with a
+// factor a row; a torus of 3996 vertices: 128, 256, 112).  Every eighth sweep is a plain one and is
+// the one that checks.  After plain_after sweeps all are plain.
 template <class T>
 __device__ __forceinline__ void heat_column(const Rows& o, const Cluster& cl, ColumnShared& sh, T* x,
-                                            const double* inv_d, double omega, int plain_after, int max_sweeps,
+                                            const double* inv_d, const double* relax, int plain_after, int max_sweeps,
                                             int* sweeps_out, int* status) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = CT / 32;
     for (int p = threadIdx.x; p < o.np; p += CT) x[p] = T{};
@@ -546,7 +551,7 @@ __device__ __forceinline__ void heat_column(const Rows& o, const Cluster& cl, Co
     int sweep = 0;
     for (;;) {
         const bool check = (sweep & (CHECK_EVERY - 1)) == CHECK_EVERY - 1;
-        const double om = check || sweep >= plain_after ? 1.0 : omega;
+        const bool plain = sweep >= plain_after;
         bool moved = false;
         for (int c = 0; c < o.ncol; ++c) {
             const int s1 = o.cslice[c + 1];
@@ -559,6 +564,7 @@ __device__ __forceinline__ void heat_column(const Rows& o, const Cluster& cl, Co
                 const int e1 = o.soff[sl + 1] * 32 + lane;
                 const double iD = inv_d[p];
                 if (!check) {
+                    const double om = plain ? 1.0 : relax[p];
 #pragma unroll 6
                     for (int e = o.soff[sl] * 32 + lane; e < e1; e += 32) row_terms(o, e, x, acc);
                     cl.store_all(x + p, relaxed(x[p], acc, om, om * iD));
@@ -596,10 +602,10 @@ __device__ __forceinline__ void heat_column(const Rows& o, const Cluster& cl, Co
 
 // Both heat systems of every column: clusters [0, ns) solve the vector system, the longer one,
 // and [ns, 2 ns) the scalar one.
-__global__ void __launch_bounds__(CT, 2) k_heat_columns(Op m, Rows o, int K, int ns, double t, double omega,
-                                                        int plain_after, int max_sweeps, const int32_t* src,
+__global__ void __launch_bounds__(CT, 2) k_heat_columns(Op m, Rows o, int K, int ns, double t, int plain_after,
+                                                        int max_sweeps, const int32_t* src,
                                                         const int32_t* face, const double* bary, const double* inv_d,
-                                                        double* u, double* Y, int* sweeps_out, int* status) {
+                                                        const double* relax, double* u, double* Y, int* sweeps_out, int* status) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ ColumnShared sh;
     const Cluster cl = this_cluster_of_column();
@@ -615,12 +621,12 @@ __global__ void __launch_bounds__(CT, 2) k_heat_columns(Op m, Rows o, int K, int
     }
     if (vec) {
         double2* x = (double2*)smem;
-        heat_column(o, cl, sh, x, inv_d, omega, plain_after, max_sweeps, sweeps_out, status);
+        heat_column(o, cl, sh, x, inv_d, relax, plain_after, max_sweeps, sweeps_out, status);
         for (int p = threadIdx.x * cl.size + cl.rank; p < o.np; p += CT * cl.size)
             if (o.vert[p] >= 0) ((double2*)Y)[(size_t)o.vert[p] * K + s] = x[p];
     } else {
         double* x = (double*)smem;
-        heat_column(o, cl, sh, x, inv_d, omega, plain_after, max_sweeps, sweeps_out, status);
+        heat_column(o, cl, sh, x, inv_d, relax, plain_after, max_sweeps, sweeps_out, status);
         for (int p = threadIdx.x * cl.size + cl.rank; p < o.np; p += CT * cl.size)
             if (o.vert[p] >= 0) u[(size_t)o.vert[p] * K + s] = x[p];
     }
@@ -853,7 +859,6 @@ struct VhmOp {
     int32_t *pos = nullptr, *ej = nullptr;
     int32_t* cverts = nullptr;        // vertices grouped by colour (no two neighbours share one)
     std::vector<int32_t> cstart;      // colour c is cverts[cstart[c] .. cstart[c + 1])
-    double sum_mass = 0.0, sum_diag = 0.0;
     Rows rows;                        // np = 0: too many vertices for the column kernels
     void* rows_mem = nullptr;
 };
@@ -904,10 +909,6 @@ cudaError_t build_rows(cssi::VhmOp* o, const std::vector<int32_t>& rs, const std
     if (e == cudaSuccess) e = cudaMemcpyAsync(diag.data(), o->diag, nv * sizeof(double), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return e;
-    for (int32_t v = 0; v < nv; ++v) {
-        o->sum_mass += mass[v];
-        o->sum_diag += diag[v];
-    }
     struct Entry { int32_t j; double w, c, s; };
     std::vector<std::vector<Entry>> row(nv);   // one entry per neighbour
     for (int32_t v = 0; v < nv; ++v)
@@ -1159,8 +1160,8 @@ int css_vhm_neighbors(css_parts* parts, double r_c, double t_factor, int64_t cap
     VTRY("vhm", B.get(&B.od, (size_t)K * n)); VTRY("vhm", B.get(&B.ot, 3 * (size_t)K * n));
     VTRY("vhm", B.get(&B.keep, (size_t)K * n));
     if (columns) {
-        VTRY("vhm", B.get(&B.r, 2 * (size_t)R.np * K)); VTRY("vhm", B.get(&B.invd, 2 * (size_t)R.np));
-        k_row_scale<<<vblk(R.np), VT, 0, st>>>(R, t, B.invd, B.invd + R.np);
+        VTRY("vhm", B.get(&B.r, 2 * (size_t)R.np * K)); VTRY("vhm", B.get(&B.invd, 3 * (size_t)R.np));
+        k_row_scale<<<vblk(R.np), VT, 0, st>>>(R, t, B.invd, B.invd + R.np, B.invd + 2 * (size_t)R.np);
     } else {
         VTRY("vhm", B.get(&B.bu, VK)); VTRY("vhm", B.get(&B.bY, 2 * VK));
         VTRY("vhm", B.get(&B.r, VK)); VTRY("vhm", B.get(&B.z, VK)); VTRY("vhm", B.get(&B.p, VK));
@@ -1171,8 +1172,6 @@ int css_vhm_neighbors(css_parts* parts, double r_c, double t_factor, int64_t cap
         k_heat_entries<<<vblk(std::max<int64_t>(6 * (int64_t)nf, nv)), VT, 0, st>>>(op, t, B.wt, B.wc, B.wsn, B.invd);
     }
     VTRY("vhm", cudaGetLastError());
-    const double rho = t * O.sum_diag / (O.sum_mass + t * O.sum_diag);
-    const double omega = rho > 0.0 && rho < 1.0 ? 2.0 / (1.0 + std::sqrt(1.0 - rho * rho)) : 1.0;
     double* bsum = B.sc;          // K
     double* rz = B.sc + K;        // K
     double* rz0 = B.sc + 2 * K;   // K
@@ -1204,9 +1203,9 @@ int css_vhm_neighbors(css_parts* parts, double r_c, double t_factor, int64_t cap
             while (size < CL_MAX && ns * size * 2 <= c->sm_count) size *= 2;
             const size_t smem = 2 * sizeof(double) * (size_t)R.np;
             VTRY("vhm", cudaMemsetAsync(B.ints, 0, sizeof(hs), st));
-            VTRY("vhm heat", launch_columns(k_heat_columns, 2 * ns, size, smem, st, op, R, K, ns, t, omega, PLAIN_AFTER,
-                                            MAX_SWEEPS, B.src, parts->face, parts->bary, B.invd, u, Y, B.ints + 1,
-                                            B.ints));
+            VTRY("vhm heat", launch_columns(k_heat_columns, 2 * ns, size, smem, st, op, R, K, ns, t, PLAIN_AFTER,
+                                            MAX_SWEEPS, B.src, parts->face, parts->bary, B.invd,
+                                            B.invd + 2 * (size_t)R.np, u, Y, B.ints + 1, B.ints));
             k_unit_field<<<nbf, VT, 0, st>>>(op, K, u, B.X);
             k_neg_div<<<nbv, VT, 0, st>>>(op, K, ns, B.X, B.b);
             VTRY("vhm poisson", cudaGetLastError());
