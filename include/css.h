@@ -107,6 +107,8 @@ int css_last_counters(const css_ctx* ctx, int64_t out[6]);
  * the rigid maps between neighbouring faces, vertex angle sums, and the
  * pseudo-source vertices (boundary, flat or saddle: angle sum >= 2 pi - 1e-9).
  *   verts  nv x 3 doubles, faces nf x 3 int32 (row major), host or device.
+ *          Lengths may be in any unit (edges of about 1e-75 to 1e75): the neighbour kernel works in
+ *          units of a typical edge, so its results at another power of two are the same bits, scaled.
  *   period NULL, or host pointer to {Lx, Ly}: x and y wrap with these periods
  *          and edge vectors use the minimum image.
  * Errors: CSS_ERR_INVALID_ARG (sizes, indices out of range, NaN),

@@ -218,7 +218,7 @@ GeoJob make_job(css_parts* p, double rc, int want_pairs, int want_forces, const 
     j.fstart = p->fstart;
     j.fitems = p->fitems;
     j.order = p->fitems;   // sources in face-rank (Morton) order
-    j.rc = rc;
+    j.rc = p->mesh->in_units(rc);
     j.want_pairs = want_pairs;
     j.pair_cap = p->pair_cap_alloc;
     j.pcnt = p->pcnt;

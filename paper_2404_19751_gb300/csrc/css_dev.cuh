@@ -13,7 +13,8 @@
 
 namespace css {
 
-// Per half-edge record (64 B): everything one unfolding step needs.
+// Per half-edge record (64 B): everything one unfolding step needs.  Lengths are in units of the mesh
+// (DMesh::unit).
 struct __align__(16) HeRec {
     double L;        // edge length
     double cx, cy;   // opposite corner c in this half-edge frame (cy > 0)
@@ -36,6 +37,10 @@ struct DMesh {
     int32_t nv, nf;
     int32_t periodic;
     double per[2];
+    // The power of two next below a typical edge length.  he and he32 hold lengths divided by it, which
+    // is exact, so that squares of lengths stay in FP32's range whatever the mesh's scale; all other
+    // arrays are in the caller's units.
+    double unit, inv_unit;
     const HeRec* he;              // 3 nf
     const int32_t* twin;          // 3 nf
     const int32_t* edge;          // 3 nf, undirected edge id = min(h, twin(h))

@@ -77,6 +77,7 @@ struct css_mesh {
     css_ctx* ctx = nullptr;
     int64_t nv = 0, nf = 0, ne = 0, npseudo = 0;
     double area = 0.0;
+    double unit = 1.0;          // css::DMesh::unit
     int periodic = 0;
     double per[2] = {0, 0};
     // device arrays
@@ -98,6 +99,7 @@ struct css_mesh {
     int4* htop = nullptr;       // 3 nf: half-edge topology (css::DMesh::htop)
     cssi::VhmOp* vhm = nullptr;
     css::DMesh view() const;
+    double in_units(double cutoff) const;   // of the neighbour kernel; > 0 stays > 0
 };
 
 struct css_parts {

@@ -380,7 +380,7 @@ __device__ bool face_walk(const DMesh& m, int& f, double& px, double& py, double
         double ax, ay, bx, by;
         corner(m, f, k, ax, ay);
         corner(m, f, k1, bx, by);
-        const double L = m.he[h].L;
+        const double L = m.he[h].L * m.unit;
         const double ux = (bx - ax) / L, uy = (by - ay) / L;
         if (tw < 0) {
             const double pr = rx * ux + ry * uy;

@@ -13,6 +13,8 @@
 #include <math.h>
 
 #include <algorithm>
+#include <cmath>
+#include <limits>
 #include <vector>
 
 #include "css_internal.h"
@@ -122,13 +124,14 @@ __global__ void k_faces(const double* X, const int32_t* F, int64_t nf, int perio
     }
 }
 
-__global__ void k_halfedges(const double* lay, const int32_t* F, const int32_t* twin, int64_t nf, HeRec* he,
+__global__ void k_halfedges(const double* lay, double inv_unit, const int32_t* F, const int32_t* twin, int64_t nf, HeRec* he,
                             css::HeRec32* he32, uint8_t* bnd, int32_t* ring_cnt) {
     int64_t h = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (h >= 3 * nf) return;
     int64_t f = h / 3;
     int k = (int)(h % 3);
-    double P[3][2] = {{0.0, 0.0}, {lay[3 * f], 0.0}, {lay[3 * f + 1], lay[3 * f + 2]}};
+    const double x1 = lay[3 * f] * inv_unit, x2 = lay[3 * f + 1] * inv_unit, y2 = lay[3 * f + 2] * inv_unit;
+    double P[3][2] = {{0.0, 0.0}, {x1, 0.0}, {x2, y2}};
     const double* A = P[k];
     const double* B = P[(k + 1) % 3];
     const double* C = P[(k + 2) % 3];
@@ -249,12 +252,10 @@ inline unsigned nblk(int64_t n, int b = 256) { return (unsigned)((n + b - 1) / b
 
 namespace {
 // first corner of every face (world), for the face ranking
-__global__ void k_origin(const double* frame, int64_t nf, float* out) {
+__global__ void k_origin(const double* frame, double inv_unit, int64_t nf, float* out) {
     const int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (f >= nf) return;
-    out[3 * f] = (float)frame[9 * f];
-    out[3 * f + 1] = (float)frame[9 * f + 1];
-    out[3 * f + 2] = (float)frame[9 * f + 2];
+    for (int a = 0; a < 3; ++a) out[3 * f + a] = (float)(frame[9 * f + a] * inv_unit);
 }
 
 uint32_t spread10(uint32_t v) {   // 10 bits to every third of 30
@@ -272,6 +273,8 @@ css::DMesh css_mesh::view() const {
     d.nv = (int32_t)nv;
     d.nf = (int32_t)nf;
     d.periodic = periodic;
+    d.unit = unit;
+    d.inv_unit = 1.0 / unit;
     d.per[0] = per[0];
     d.per[1] = per[1];
     d.he = he;
@@ -291,6 +294,8 @@ css::DMesh css_mesh::view() const {
     d.htop = htop;
     return d;
 }
+
+double css_mesh::in_units(double cutoff) const { return std::max(cutoff / unit, std::numeric_limits<double>::min()); }
 
 namespace cssi {
 
@@ -319,7 +324,7 @@ int build_mesh(css_ctx* ctx, const double* dX, int64_t nv, const int32_t* dF, in
     int32_t* ring_cnt = nullptr;
     int32_t* tmp = nullptr;
     int hflag = 0;
-    unsigned long long hcnt[3] = {0, 0, 0};   // edges, pseudo-source vertices, area (a double's bits)
+    unsigned long long hcnt[2] = {0, 0};   // edges, pseudo-source vertices (behind them on the device: the area)
     m->nv = nv;
     m->nf = nf;
     if (period) { m->periodic = 1; m->per[0] = period[0]; m->per[1] = period[1]; }
@@ -364,30 +369,31 @@ int build_mesh(css_ctx* ctx, const double* dX, int64_t nv, const int32_t* dF, in
     k_topo_insert<<<nblk(nh), 256, 0, st>>>(dF, nf, t, dflag);
     k_topo_link<<<nblk(cap), 256, 0, st>>>(dF, t, m->twin, m->edge, dflag, dcnt);
     k_faces<<<nblk(nf), 256, 0, st>>>(dX, dF, nf, m->periodic, m->per[0], m->per[1], m->lay, m->frame, dflag);
+    k_area<<<nblk(nf), 256, 0, st>>>(m->lay, nf, (double*)(dcnt + 2));
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(&hflag, dflag, sizeof(int), cudaMemcpyDeviceToHost, st));
+    CK(cudaMemcpyAsync(&m->area, dcnt + 2, sizeof(double), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     if (hflag & (4 | 8)) { ctx->err = "mesh_upload: an edge is shared by more than two faces"; rc = CSS_ERR_NONMANIFOLD; goto done; }
     if (hflag & 16) { ctx->err = "mesh_upload: inconsistent face orientation"; rc = CSS_ERR_NONMANIFOLD; goto done; }
     if (hflag & 32) { ctx->err = "mesh_upload: degenerate (zero-area) face"; rc = CSS_ERR_NONMANIFOLD; goto done; }
-    k_halfedges<<<nblk(nh), 256, 0, st>>>(m->lay, dF, m->twin, nf, m->he, m->he32, m->bnd, ring_cnt);
+    if (m->area > 0.0 && std::isfinite(m->area))   // the square root of a face's mean area, rounded down
+        m->unit = std::ldexp(1.0, std::ilogb(m->area / (double)nf) >> 1);
+    k_halfedges<<<nblk(nh), 256, 0, st>>>(m->lay, 1.0 / m->unit, dF, m->twin, nf, m->he, m->he32, m->bnd, ring_cnt);
     CK(launch_scan_i32(ring_cnt, m->ring_start, nv + 1, tmp, st));
     CK(cudaMemsetAsync(ring_cnt, 0, (nv + 1) * sizeof(int32_t), st));
     k_ring_scatter<<<nblk(nh), 256, 0, st>>>(dF, nf, m->ring_start, ring_cnt, m->ring);
     k_vertices<<<nblk(nv), 256, 0, st>>>(nv, m->ring_start, m->ring, m->he, m->twin, m->theta, m->bnd, m->pseudo,
                                          m->cang, dcnt + 1);
     CK(cudaGetLastError());
-    k_area<<<nblk(nf), 256, 0, st>>>(m->lay, nf, (double*)(dcnt + 2));
-    CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(hcnt, dcnt, 3 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
+    CK(cudaMemcpyAsync(hcnt, dcnt, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     m->ne = (int64_t)hcnt[0];
     m->npseudo = (int64_t)hcnt[1];
-    memcpy(&m->area, hcnt + 2, sizeof(double));
     {   // Morton rank of every face (host sort, once per mesh)
         float* dorg = nullptr;
         CK(cudaMalloc(&dorg, 3 * nf * sizeof(float)));
-        k_origin<<<nblk(nf), 256, 0, st>>>(m->frame, nf, dorg);
+        k_origin<<<nblk(nf), 256, 0, st>>>(m->frame, 1.0 / m->unit, nf, dorg);
         std::vector<float> org(3 * nf);
         cudaError_t e = cudaMemcpyAsync(org.data(), dorg, 3 * nf * sizeof(float), cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);

@@ -168,7 +168,7 @@ int css_compute_forces_noalloc(const css_mesh* mesh, int64_t n, const int32_t* f
     j.fstart = fstart;
     j.order = fitems;
     j.fitems = fitems;
-    j.rc = r_c;
+    j.rc = mesh->in_units(r_c);
     j.pcnt = pcnt;
     j.want_forces = 1;
     j.pot = *pot;

@@ -29,7 +29,8 @@
 // an unfolding, and behind a flat vertex nothing covers the gap between them (100 of 6 M pairs of a
 // flat sheet of 80 x 80 vertices were lost, 1270 of 4 M at 200 x 200; with FP32 rims alone 1 of 6 M).
 // The FP32 form tests its targets and keeps the directions of paths in FP32; lengths of results are
-// FP64 in both forms.
+// FP64 in both forms.  All lengths in this file are in units of the mesh (DMesh::unit), so the FP32
+// filters and roots see the same numbers at every scale; results are multiplied back, exactly.
 //
 // Measured against windows kept in per-edge lists and trimmed against one another (the same
 // calls, default launch shapes): 65536 particles on a noisy level-8 sphere 110.7 -> 10.1 ms
@@ -150,6 +151,13 @@ struct Links<true> {
     Link* p;
 };
 
+// corner k of face f in its layout, in units of the mesh
+__device__ __forceinline__ void unit_corner(const DMesh& m, int f, int k, double& x, double& y) {
+    css::face_corner(m, f, k, x, y);
+    x *= m.inv_unit;
+    y *= m.inv_unit;
+}
+
 // the link of the point (X, Y) of half-edge he's frame straight back to the pseudo-source S: which
 // 2 the far corner of the face the window enters, 3 a point in that face; 0, 1 the start and the end of
 // the edge, whose leg points into the face on the other side and is written in that face
@@ -166,8 +174,8 @@ __device__ __forceinline__ void link_back(const DMesh& m, int he, double2 S, dou
         vb = -vb;
     }
     double ax, ay, bx, by;
-    css::face_corner(m, g, kg, ax, ay);
-    css::face_corner(m, g, kg + 1, bx, by);
+    unit_corner(m, g, kg, ax, ay);
+    unit_corner(m, g, kg + 1, bx, by);
     const double L = sqrt((bx - ax) * (bx - ax) + (by - ay) * (by - ay));
     const double ex = (bx - ax) / L, ey = (by - ay) / L;
     l.par = par;
@@ -564,8 +572,8 @@ __device__ __forceinline__ void Group<R, PL, TEAM, LK>::seed(int f0, double b1, 
     const double wc = k0 == 0 ? wt[2] : (k0 == 1 ? wt[0] : wt[1]);
     const double hx = wb * r.L + wc * r.cx, lx = wa * r.L + wc * (r.L - r.cx), hy = fmax(wc * r.cy, 0.0);
     double ax, ay, bx, by;
-    css::face_corner(m, f0, k0, ax, ay);
-    css::face_corner(m, f0, k0 + 1, bx, by);
+    unit_corner(m, f0, k0, ax, ay);
+    unit_corner(m, f0, k0 + 1, bx, by);
     const double ex = (bx - ax) / r.L, ey = (by - ay) / r.L;
     const double vx = hy * ey - hx * ex, vy = -hy * ex - hx * ey;   // from the source to the corner, in the layout
     tests(lane == 0, m.frank ? m.frank[f0] : f0, [&](int k, int j) {   // half-edge 0's frame is the layout's
@@ -615,8 +623,8 @@ __device__ __forceinline__ void Group<R, PL, TEAM, LK>::seed_at_vertex(int hc) {
     const int deg = m.ring_start[v + 1] - m.ring_start[v];
     const int f0 = hc / 3;
     double ax, ay, bx, by;
-    css::face_corner(m, f0, hc - 3 * f0, ax, ay);
-    css::face_corner(m, f0, hc - 3 * f0 + 1, bx, by);
+    unit_corner(m, f0, hc - 3 * f0, ax, ay);
+    unit_corner(m, f0, hc - 3 * f0 + 1, bx, by);
     const double phi0 = atan2(by - ay, bx - ax);
     const int half = m.bnd[v] ? deg : (deg + 1) / 2;
     int left = deg;
@@ -663,8 +671,8 @@ __device__ __forceinline__ void Group<R, PL, TEAM, LK>::seed_at_vertex(int hc) {
                         improved(slot, d, vec2((R)cos(a), (R)sin(a)), NONE, 0.0f);
                         if constexpr (LK) {   // along the edge, back to the source's corner
                             double px, py, sx, sy;
-                            css::face_corner(m, fh, hn - 3 * fh, px, py);
-                            css::face_corner(m, fh, kh, sx, sy);
+                            unit_corner(m, fh, hn - 3 * fh, px, py);
+                            unit_corner(m, fh, kh, sx, sy);
                             lk.p[slot] = {NONE, 4 * fh + (hn - 3 * fh), d, make_double2((sx - px) / d, (sy - py) / d)};
                         }
                     }
@@ -1171,7 +1179,7 @@ __device__ __forceinline__ void Group<R, PL, TEAM, LK>::run(int item, int32_t* d
     for (int k = tid; k < nt; k += T) {
         const int s = ord[k];
         int l = TEAM ? own[s] : s;
-        double d = tdist()[s];
+        double d = tdist()[s];   // in units of the mesh until the form's choice is made
         if constexpr (sizeof(R) == 4) {
             const double dv = tvert()[s];
             const int lv = TEAM ? ownv[s] : s + (1 << Y.th_log);
@@ -1180,6 +1188,7 @@ __device__ __forceinline__ void Group<R, PL, TEAM, LK>::run(int item, int32_t* d
                 d = dv;
             }
         }
+        d *= m.unit;
         const V2<R> t = at<V2<R>>(b, Y.ttan)[l];
         const double tx = (double)t.x, ty = (double)t.y;
         if (J.want_pairs && k < J.pair_cap) {
@@ -1201,7 +1210,7 @@ __device__ __forceinline__ void Group<R, PL, TEAM, LK>::run(int item, int32_t* d
                     J.lfk[a] = l.fk;
                     J.ldir[2 * a] = l.dir.x;
                     J.ldir[2 * a + 1] = l.dir.y;
-                    J.llen[a] = l.len;
+                    J.llen[a] = l.len * m.unit;
                     ++nl;
                     if (l.par < 0) break;
                     l = lk.p[l.par];
