@@ -253,10 +253,10 @@ __device__ __forceinline__ void roots(double x, double& r, double& inv) {
 // Where the path through an edge's start vertex (along the edge) stops being the shorter one:
 // the window (pseudo-source at (sx, sy) with s2 = |s|^2, sx measured from that vertex) beats it
 // for x > x0 only, (x - sx)^2 + sy^2 < (x + a)^2 with a = the vertex's distance minus sigma.
-// Rounded so that too little is cut, never too much (eps bounds the rounding of sx); beyond L:
-// nothing of the window is left.
+// Rounded so that too little is cut, never too much (eps bounds that of 2 (a + sx), which nearly cancel
+// where s lies near the edge's line beyond the vertex); beyond L: nothing of the window is left.
 __device__ __forceinline__ float cut_at(float sx, float s2, float a, float L, float eps) {
-    const float num = s2 - a * a - 2e-6f * (s2 + a * a) - 2.0f * eps * fabsf(sx), den = 2.0f * (a + sx);
+    const float num = s2 - a * a - 2e-6f * (s2 + a * a) - eps * fabsf(sx), den = fmaf(2.0f, a + sx, eps);
     if (!(num > 0.0f)) return 0.0f;
     return den * L > num * 0.999f ? __fdividef(num, den) - 1e-5f * L : 2.0f * L;
 }
@@ -502,7 +502,7 @@ struct Group {
     // cut [b0, b1] of an edge of length L by its end vertices' distances (less sigma) au, av; false if
     // nothing is left
     __device__ __forceinline__ bool cut(float sx, float sy, float au, float av, float L, float& b0, float& b1) const {
-        const float sy2 = sy * sy, tx = L - sx, eps = 2.4e-7f * (fabsf(sx) + L);
+        const float sy2 = sy * sy, tx = L - sx, eps = 4.8e-7f * (fabsf(sx) + L);
         b0 = fmaxf(b0, cut_at(sx, sx * sx + sy2, au, L, eps));
         b1 = fminf(b1, L - cut_at(tx, tx * tx + sy2, av, L, eps));
         return b1 > b0;
