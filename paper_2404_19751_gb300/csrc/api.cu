@@ -75,19 +75,45 @@ struct GeoPlan {
     int wpc1 = 0, nctas1 = 0, wpc2 = 0, nctas2 = 0, tile = 1;
 };
 
-int grow_ws(css_ctx* c, cssi::WsBuf& b, size_t need) {
-    if (need <= b.bytes) return CSS_OK;
+// The workspace of a pass: a slice for each group of *nctas CTAs.  One that does not fit what is kept
+// already takes at most an eighth of the free memory (all pairs of 4096 particles on 327680 faces
+// would take 115 GB for as many groups as can be resident), and fewer CTAs where it does not get
+// that; the groups take their sources from a queue, so fewer of them give the same rows.
+constexpr size_t WS_SMALL = 256u << 20;   // asked for as it is
+int grow_ws(css_ctx* c, cssi::WsBuf& b, size_t per_cta, int* nctas) {
+    const size_t want = per_cta * (size_t)*nctas;
+    if (want <= b.bytes) return CSS_OK;
+    if (want <= b.wanted && per_cta <= b.bytes) {   // it was cut before: what there is, not another try on every call
+        *nctas = (int)(b.bytes / per_cta);
+        return CSS_OK;
+    }
     cudaFree(b.ws);
     b.ws = nullptr;
-    b.bytes = 0;
-    TRY(c, "workspace", cudaMalloc(&b.ws, need));
-    b.bytes = need;
-    return CSS_OK;
+    b.bytes = b.wanted = 0;
+    if (want > WS_SMALL) {
+        size_t free_bytes = 0, total = 0;
+        TRY(c, "workspace", cudaMemGetInfo(&free_bytes, &total));
+        const size_t most = std::max(WS_SMALL, free_bytes / 8) / per_cta;
+        *nctas = (int)std::min<size_t>((size_t)*nctas, std::max<size_t>(1, most));
+    }
+    for (;;) {
+        const size_t need = per_cta * (size_t)*nctas;
+        const cudaError_t e = cudaMalloc(&b.ws, need);
+        if (e == cudaSuccess) {
+            b.bytes = need;
+            b.wanted = want;
+            return CSS_OK;
+        }
+        b.ws = nullptr;
+        if (e != cudaErrorMemoryAllocation || *nctas == 1) return cuda_fail(c, "workspace", e);
+        cudaGetLastError();
+        *nctas = (*nctas + 1) / 2;
+    }
 }
 
 // one pass: layout, grid and (for tables in global memory) its workspace
 int plan_pass(css_ctx* c, cssi::WsBuf& b, int precision, int win_cap, int tab_cap, int shared, int warps, int team,
-              int max_ctas, WaveWs* out, int* nctas) {
+              int max_ctas, int64_t nitems, WaveWs* out, int* nctas) {
     WaveWs g{};
     g.lay = cssi::wave_layout(precision, win_cap, tab_cap, shared, warps, team);
     g.shared = shared != 0;
@@ -104,9 +130,9 @@ int plan_pass(css_ctx* c, cssi::WsBuf& b, int precision, int win_cap, int tab_ca
         return CSS_ERR_INVALID_ARG;
     }
     if (max_ctas > 0) bps = std::min(bps, max_ctas);
-    *nctas = c->sm_count * bps;
+    *nctas = (int)std::min<int64_t>((int64_t)c->sm_count * bps, std::max<int64_t>(nitems, 1));
     g.stride = cssi::waves_global_bytes(g.lay, g.shared);
-    int rc = grow_ws(c, b, g.stride * (size_t)*nctas * (team ? 1 : warps));
+    int rc = g.stride ? grow_ws(c, b, g.stride * (size_t)(team ? 1 : warps), nctas) : CSS_OK;
     g.base = (char*)b.ws;
     *out = g;
     return rc;
@@ -172,10 +198,10 @@ int ensure_plan(css_ctx* c, int precision, int64_t nitems, const Reach& R, GeoPl
     P->wpc1 = L.warps_per_cta;
     P->tile = L.tile;
     int rc = plan_pass(c, c->ws1, precision, L.win_cap, L.tab_cap, L.shared_scale, L.warps_per_cta, L.team,
-                       L.ctas_per_sm, &P->g1, &P->nctas1);
+                       L.ctas_per_sm, nitems, &P->g1, &P->nctas1);
     if (rc) return rc;
     P->wpc2 = L.warps2_per_sm;
-    rc = plan_pass(c, c->ws2, precision, L.win_cap2, 0, 0, L.warps2_per_sm, 0, 1, &P->g2, &P->nctas2);
+    rc = plan_pass(c, c->ws2, precision, L.win_cap2, 0, 0, L.warps2_per_sm, 0, 1, nitems, &P->g2, &P->nctas2);
     if (rc) return rc;
     if (c->defer_cap < nitems) {
         cudaFree(c->defer);
@@ -1463,9 +1489,9 @@ int run_path_kernel(css_parts* p, double rc, const std::vector<int32_t>& us, con
         g.shared = pass == 0;
         g.lay = cssi::wave_layout(CSS_FP64, pass == 0 ? 2048 * scale : win_cap, 0, pass == 0 ? scale : 0, 1, 0);
         g.stride = cssi::waves_global_bytes(g.lay, g.shared) + cssi::waves_link_bytes(g.lay);
-        const int ctas = std::min(left, c->sm_count * (pass == 0 ? 4 : 2));
+        int ctas = std::min(left, c->sm_count * (pass == 0 ? 4 : 2));
         cssi::WsBuf& b = pass == 0 ? c->ws1 : c->ws2;
-        rc1 = grow_ws(c, b, g.stride * (size_t)ctas);
+        rc1 = grow_ws(c, b, g.stride, &ctas);
         if (rc1) return rc1;
         g.base = (char*)b.ws;
         const bool list = pass == 1 && scale;

@@ -31,6 +31,7 @@ struct LaunchCfg {
 struct WsBuf {
     void* ws = nullptr;
     size_t bytes = 0;
+    size_t wanted = 0;   // what was asked for when it was allocated (it may have got less)
 };
 }  // namespace cssi
 
