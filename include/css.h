@@ -348,7 +348,7 @@ int css_fma_peak(css_ctx* ctx, int precision, double* flops_per_s);
  * returns {4, 0, 1, 1, 2048, 16384, 2, 1, 0, 0} and the context picks the shape of each
  * evaluation by itself, from the number of sources and the share of the mesh the cutoff
  * reaches (a team for few sources with large patches, larger tables after an evaluation that
- * deferred more than one source in 25). */
+ * deferred more than one source in 25, for that mesh at cutoffs that reach about as far). */
 typedef struct css_launch {
     int32_t warps_per_cta, ctas_per_sm, tile, shared_scale;
     int32_t window_capacity, window_capacity2, warps2_per_sm, occupancy;

@@ -11,6 +11,7 @@
 
 #include <algorithm>
 #include <numeric>
+#include <set>
 #include <string>
 #include <vector>
 
@@ -141,13 +142,18 @@ int plan_pass(css_ctx* c, cssi::WsBuf& b, int precision, int win_cap, int tab_ca
 // What one source of a set sees within the cutoff, by its share of the mesh's area.
 struct Reach {
     double faces = 0.0, verts = 0.0, targets = 0.0;
+    int level = 0;   // doublings of the tables after deferrals (css_mesh::auto_level)
+    static double part_of(const css_mesh* m, double rc) {
+        return std::isinf(rc) ? 1.0 : std::min(1.0, M_PI * rc * rc / m->area);
+    }
+    static double faces_of(const css_mesh* m, double rc) { return std::max(3.0, part_of(m, rc) * (double)m->nf); }
     void add(const css_parts* p, double rc) {   // the largest over several sets
         const css_mesh* m = p->mesh;
-        const double part = std::isinf(rc) ? 1.0 : std::min(1.0, M_PI * rc * rc / m->area);
-        const double f = std::max(3.0, part * (double)m->nf);
+        const double f = faces_of(m, rc), part = part_of(m, rc);
         faces = std::max(faces, f);
         verts = std::max(verts, std::min((double)m->nv, 0.6 * f + 2.5 * sqrt(f) + 12.0));
         targets = std::max(targets, part * (double)p->n);
+        if (f > 0.5 * m->auto_faces && f < 2.0 * m->auto_faces) level = std::max(level, m->auto_level);
     }
 };
 
@@ -166,7 +172,7 @@ struct Reach {
 //     them lies a patch of 350 faces: its waves are about 8 sqrt(6 x 350) windows wide in all.
 cssi::LaunchCfg pick_shape(const css_ctx* c, int64_t nitems, const Reach& R) {
     cssi::LaunchCfg L = c->cfg;
-    const double grow = (double)(1 << c->auto_level), verts = grow * R.verts, targets = grow * R.targets;
+    const double grow = (double)(1 << R.level), verts = grow * R.verts, targets = grow * R.targets;
     const int64_t sms = c->sm_count;
     const bool big = R.faces >= 350.0;
     L.warps_per_cta = 4;
@@ -360,12 +366,19 @@ int status_error(css_ctx* c, int status) {
     return CSS_ERR_CUDA;
 }
 
-// A context whose launch shape nobody set or tuned doubles its first pass's tables when more than one
-// source in 25 was deferred (patches larger than the estimate).
-void adapt_default(css_ctx* c) {
+// Where the launch shape is picked, the first pass's tables are doubled when more than one source in
+// 25 was deferred (patches larger than the estimate): for the mesh evaluated, at cutoffs that reach
+// about as far.
+void adapt_default(const css_ctx* c, css_mesh* m, double rc) {
     if (c->cfg_explicit) return;
     const int64_t done = c->last_counters[0], deferred = c->last_counters[4];
-    if (done > 0 && deferred * 25 > done && c->auto_level < 8) ++c->auto_level;
+    if (!(done > 0 && deferred * 25 > done)) return;
+    const double f = Reach::faces_of(m, rc);
+    if (!(f > 0.5 * m->auto_faces && f < 2.0 * m->auto_faces)) {
+        m->auto_faces = f;
+        m->auto_level = 0;
+    }
+    if (m->auto_level < 8) ++m->auto_level;
 }
 
 // Synchronous neighbour / force evaluation with overflow retries.  after() enqueues what the
@@ -407,7 +420,7 @@ int run_geo(css_parts* p, double rc, int prec, int want_pairs, int want_forces, 
             if (rc1 == CSS_OK) rc1 = read_status(c, &status);
             if (rc1) return rc1;
         }
-        if (status == 0) { adapt_default(c); return CSS_OK; }
+        if (status == 0) { adapt_default(c, p->mesh, rc); return CSS_OK; }
         if (!grow_for(c, status, &retries)) return status_error(c, status);
     }
 }
@@ -998,7 +1011,7 @@ int css_integrate_step(css_parts* p, const css_potential* pot, const css_integra
         int status = 0;
         rc = read_status(c, &status);
         if (rc) break;
-        if (status == 0) { adapt_default(c); break; }
+        if (status == 0) { adapt_default(c, p->mesh, r_c); break; }
         if (!grow_for(c, status, &retries)) { rc = status_error(c, status); break; }
         TRY(c, "restore", snap_restore(p));
     }
@@ -1164,7 +1177,12 @@ int css_batch_step(css_batch* b, const css_potential* pot, const css_integrator*
         int status = 0;
         rc = read_status(c, &status);
         if (rc) return rc;
-        if (status == 0) { adapt_default(c); break; }
+        if (status == 0) {
+            std::set<css_mesh*> meshes;
+            for (const css_parts* p : b->sets) meshes.insert(p->mesh);
+            for (css_mesh* m : meshes) adapt_default(c, m, r_c);
+            break;
+        }
         if (!grow_for(c, status, &retries)) return status_error(c, status);
         for (css_parts* p : b->sets) TRY(c, "restore", snap_restore(p));
     }

@@ -46,7 +46,6 @@ struct css_ctx {
     cssi::LaunchCfg cfg;
     std::map<int64_t, int> bps_cache;   // resident CTAs per SM by (precision, shape)
     int cfg_explicit = 0;               // the shape was set or tuned (else one is picked for each evaluation)
-    int auto_level = 0;                 // doublings of the picked shape's tables after deferrals
     int pair_cap = 64;               // pairs per source slab
     // deferral list of the first pass (one entry per work item at most)
     int32_t* defer = nullptr;
@@ -79,6 +78,8 @@ struct css_mesh {
     int64_t nv = 0, nf = 0, ne = 0, npseudo = 0;
     double area = 0.0;
     double unit = 1.0;          // css::DMesh::unit
+    int auto_level = 0;         // doublings of a picked shape's tables after deferrals, for cutoffs that
+    double auto_faces = 0.0;    // reach between half and twice as many faces as this
     int periodic = 0;
     double per[2] = {0, 0};
     // device arrays

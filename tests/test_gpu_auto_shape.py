@@ -1,0 +1,52 @@
+"""Shapes that a context picks by itself (needs a GB300): what one mesh or cutoff taught them does not carry
+over to others, and the counters of other calls do not steer them."""
+import numpy as np
+import pytest
+
+import synth
+
+css = pytest.importorskip("paper_2404_19751_gb300")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def graded():
+    """The unit square, spacings growing twentyfold along both axes; as many particles in a small face as in
+    a large one, so that patches in the fine corner hold far more faces than their share of the area."""
+    n = 64
+    x = np.concatenate([[0.0], np.cumsum(20.0 ** (np.arange(n - 1) / (n - 2.0)))])
+    m = synth.grid_plane(n, n)
+    k = np.arange(n * n)
+    v = np.stack([x[k % n], x[k // n], 0.0 * k], 1) / x[-1]
+    m = synth.Mesh(v, m.faces, None)
+    return (m,) + synth.place_uniform(m, 3000, 6, area_weighted=False)
+
+
+def _deferred(ctx, parts, r_c):
+    css.geodesic_neighbors(parts, r_c, css.FP64)
+    return ctx.last_counters()["deferred"]
+
+
+def test_larger_tables_stay_with_the_mesh_and_the_reach(graded):
+    m, face, bary = graded
+    near, far = 0.03, 0.05   # 22 and 62 faces by share of the area
+    first = {}
+    for r_c in (near, far):
+        ctx = css.create(0)
+        mesh = css.mesh_upload(ctx, m.verts, m.faces)
+        parts = css.particles_set(ctx, mesh, face, bary)
+        first[r_c] = _deferred(ctx, parts, r_c)
+        assert first[r_c] * 25 > len(face)
+        if r_c == near:   # tables grow until few sources are deferred
+            later = [_deferred(ctx, parts, r_c) for _ in range(6)]
+            assert later[-1] * 25 <= len(face), later
+            mesh2 = css.mesh_upload(ctx, m.verts, m.faces)
+            parts2 = css.particles_set(ctx, mesh2, face, bary)
+            assert _deferred(ctx, parts2, r_c) == first[r_c]
+            other = _deferred(ctx, parts, far)
+            parts2.free()
+            mesh2.free()
+        parts.free()
+        mesh.free()
+        ctx.close()
+    assert other == first[far]
