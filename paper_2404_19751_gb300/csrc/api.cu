@@ -383,7 +383,7 @@ void adapt_default(const css_ctx* c, css_mesh* m, double rc) {
 
 // Synchronous neighbour / force evaluation with overflow retries.  after() enqueues what the
 // caller reads with the status.  The second pass is launched only if the first deferred
-// a source, which costs a second synchronisation then; a context whose last evaluation deferred
+// a source, which costs a second synchronisation then; a set whose last evaluation deferred
 // some launches both at once.
 template <class Fn>
 int run_geo(css_parts* p, double rc, int prec, int want_pairs, int want_forces, const css_potential* pot, Fn after) {
@@ -397,7 +397,7 @@ int run_geo(css_parts* p, double rc, int prec, int want_pairs, int want_forces, 
         R.add(p, rc);
         int rc1 = ensure_plan(c, prec, p->n, R, &P);
         if (rc1) return rc1;
-        const bool both = c->last_counters[4] > 0;
+        const bool both = p->deferred;
         rc1 = reset_status(c);
         if (rc1 == CSS_OK) rc1 = enqueue_bucket(p, c->dscal, c->depot);
         if (rc1) return rc1;
@@ -420,6 +420,7 @@ int run_geo(css_parts* p, double rc, int prec, int want_pairs, int want_forces, 
             if (rc1 == CSS_OK) rc1 = read_status(c, &status);
             if (rc1) return rc1;
         }
+        p->deferred = c->last_counters[4] > 0;
         if (status == 0) { adapt_default(c, p->mesh, rc); return CSS_OK; }
         if (!grow_for(c, status, &retries)) return status_error(c, status);
     }
@@ -1011,6 +1012,7 @@ int css_integrate_step(css_parts* p, const css_potential* pot, const css_integra
         int status = 0;
         rc = read_status(c, &status);
         if (rc) break;
+        p->deferred = c->last_counters[4] > 0;
         if (status == 0) { adapt_default(c, p->mesh, r_c); break; }
         if (!grow_for(c, status, &retries)) { rc = status_error(c, status); break; }
         TRY(c, "restore", snap_restore(p));

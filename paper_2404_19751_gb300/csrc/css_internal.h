@@ -139,6 +139,7 @@ struct css_parts {
     double* pd = nullptr;
     double* pt = nullptr;
     int pair_cap_alloc = 0;
+    int deferred = 0;           // the last neighbour / force evaluation left sources to its second pass
     int64_t* rows = nullptr;    // row starts of a neighbour call, n + 1 and the scan's scratch
     void* stage = nullptr;      // packed rows on their way to the host (STAGE_KEEP bytes at most are kept)
     size_t stage_bytes = 0;

@@ -50,3 +50,31 @@ def test_larger_tables_stay_with_the_mesh_and_the_reach(graded):
         mesh.free()
         ctx.close()
     assert other == first[far]
+
+
+def _kernel_us(ctx, parts, before, reps=30):
+    """Median device time of an evaluation that defers nothing, after before()."""
+    us = []
+    for _ in range(reps):
+        before()
+        assert _deferred(ctx, parts, 0.1) == 0
+        us.append(1e3 * ctx.last_kernel_ms())
+    return float(np.median(us))
+
+
+def test_only_deferrals_bring_the_second_pass():
+    """A second pass adds 5 us to an evaluation of 28, empty or not.  A call of the approximate solver, whose
+    batches are counted where deferrals are, does not bring it."""
+    ctx = css.create(0)
+    ico = synth.icosphere(3, 1.0)
+    mesh = css.mesh_upload(ctx, ico.verts, ico.faces)
+    parts = css.particles_set(ctx, mesh, *synth.place_uniform(ico, 60, 3))
+    alone = _kernel_us(ctx, parts, lambda: _deferred(ctx, parts, 0.1))
+
+    def solver():
+        css.vhm_neighbors(parts, 0.3, 1.0)
+        assert ctx.last_counters()["deferred"] > 0
+    assert _kernel_us(ctx, parts, solver) < alone + 2.5
+    parts.free()
+    mesh.free()
+    ctx.close()
