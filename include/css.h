@@ -310,8 +310,9 @@ int css_compute_forces_noalloc(const css_mesh* mesh, int64_t n, const int32_t* f
 /* ---------------------------------------------------------------- measurement
  * css_last_kernel_ms: device time (ms) between CUDA events recorded on the context
  * stream immediately before the first and after the second pass of the last
- * neighbour/force evaluation (inside captured graphs too).  CSS_ERR_INVALID_ARG before
- * any launch.
+ * neighbour/force evaluation (inside captured graphs too), without the time between the two
+ * where the second pass was launched only once the host had seen deferrals.
+ * CSS_ERR_INVALID_ARG before any launch.
  * css_fma_peak: measured dense FMA throughput (flop/s, 2 per FMA) of this GPU's
  * FP32 or FP64 pipes, from an FMA-chain kernel filling every SM; it has no
  * counterpart in the paper and serves as the ALU roofline denominator. */

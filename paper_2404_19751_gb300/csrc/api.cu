@@ -322,6 +322,7 @@ int enqueue_geo(css_parts* p, double rc, int prec, int want_pairs, int want_forc
 
 // status and counters to zero, before an evaluation or a run of steps
 int reset_status(css_ctx* c) {
+    c->ev_late_valid = 0;
     TRY(c, "reset", cudaMemsetAsync(c->dscal, 0, 4 * sizeof(int) + 8 * sizeof(unsigned long long), c->stream));
     return CSS_OK;
 }
@@ -413,9 +414,11 @@ int run_geo(css_parts* p, double rc, int prec, int want_pairs, int want_forces, 
         rc1 = read_status(c, &status);
         if (rc1) return rc1;
         if (!both && status == 0 && c->hstat[2] > 0) {
+            TRY(c, "event", record_ev(c, c->ev_late0));   // the host's round trip is not device time
             rc1 = enqueue_pass2(c, j, nullptr, nullptr, nullptr, n, prec, P);
             if (rc1) return rc1;
-            TRY(c, "event", record_ev(c, c->ev_geo1));
+            TRY(c, "event", record_ev(c, c->ev_late1));
+            c->ev_late_valid = 1;
             rc1 = after();
             if (rc1 == CSS_OK) rc1 = read_status(c, &status);
             if (rc1) return rc1;
@@ -471,6 +474,7 @@ int css_create(css_ctx** out, int device, void* stream) {
         return CSS_ERR_OOM;
     }
     if (cudaEventCreate(&c->ev_geo0) != cudaSuccess || cudaEventCreate(&c->ev_geo1) != cudaSuccess ||
+        cudaEventCreate(&c->ev_late0) != cudaSuccess || cudaEventCreate(&c->ev_late1) != cudaSuccess ||
         cudaEventCreateWithFlags(&c->ev_order, cudaEventDisableTiming) != cudaSuccess) {
         css_destroy(c);
         return CSS_ERR_CUDA;
@@ -496,6 +500,8 @@ int css_destroy(css_ctx* c) {
     cudaFreeHost(c->hstat);
     if (c->ev_geo0) cudaEventDestroy(c->ev_geo0);
     if (c->ev_geo1) cudaEventDestroy(c->ev_geo1);
+    if (c->ev_late0) cudaEventDestroy(c->ev_late0);
+    if (c->ev_late1) cudaEventDestroy(c->ev_late1);
     if (c->ev_order) cudaEventDestroy(c->ev_order);
     if (c->own_stream) cudaStreamDestroy(c->stream);
     delete c;
@@ -516,6 +522,11 @@ int css_last_kernel_ms(css_ctx* c, double* ms) {
     TRY(c, "kernel timing", cudaEventSynchronize(c->ev_geo1));
     TRY(c, "kernel timing", cudaEventElapsedTime(&f, c->ev_geo0, c->ev_geo1));
     *ms = (double)f;
+    if (c->ev_late_valid) {
+        TRY(c, "kernel timing", cudaEventSynchronize(c->ev_late1));
+        TRY(c, "kernel timing", cudaEventElapsedTime(&f, c->ev_late0, c->ev_late1));
+        *ms += (double)f;
+    }
     return CSS_OK;
 }
 

@@ -61,6 +61,8 @@ struct css_ctx {
     int64_t last_counters[6] = {0, 0, 0, 0, 0, 0};
     cudaEvent_t ev_geo0 = nullptr, ev_geo1 = nullptr;   // around the neighbour/force kernel
     int ev_valid = 0;
+    cudaEvent_t ev_late0 = nullptr, ev_late1 = nullptr;   // around a second pass launched after the host saw the deferrals
+    int ev_late_valid = 0;
     // orders work on another stream after what is queued on `stream` (made at creation so
     // that the allocation-free entry point creates nothing)
     cudaEvent_t ev_order = nullptr;

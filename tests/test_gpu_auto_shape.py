@@ -78,3 +78,24 @@ def test_only_deferrals_bring_the_second_pass():
     parts.free()
     mesh.free()
     ctx.close()
+
+
+def test_kernel_time_holds_no_round_trip():
+    """The first evaluation of a set that defers sources launches the second pass once the host has seen them,
+    later ones with the first: css_last_kernel_ms is the same device time, 870 us here, where the round
+    trip between the passes takes 20 us."""
+    ctx = css.create(0)
+    ctx.set_launch(**dict(ctx.get_launch(), window_capacity=64))
+    m = synth.icosphere(5, 1.0, noise=0.01, seed=1)
+    face, bary = synth.place_uniform(m, 1024, 3)
+    mesh = css.mesh_upload(ctx, m.verts, m.faces)
+    late, once = [], []
+    for _ in range(15):
+        parts = css.particles_set(ctx, mesh, face, bary)
+        for us in (late, once):
+            assert _deferred(ctx, parts, 0.15) > 0
+            us.append(1e3 * ctx.last_kernel_ms())
+        parts.free()
+    mesh.free()
+    ctx.close()
+    assert np.median(late) < np.median(once) + 10.0, (np.median(late), np.median(once))
