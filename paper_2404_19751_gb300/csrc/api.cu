@@ -361,7 +361,6 @@ int status_error(css_ctx* c, int status) {
         return CSS_ERR_QUEUE_OVERFLOW;
     }
     if (status & (css::ST_ITER_LIMIT | css::ST_WALK_LIMIT)) { c->err = "device loop reached its iteration cap"; return CSS_ERR_ITER_LIMIT; }
-    if (status & css::ST_PIECES) { c->err = "window trimming produced too many pieces"; return CSS_ERR_QUEUE_OVERFLOW; }
     if (status & css::ST_PAIR_OVERFLOW) { c->err = "pair slab overflow"; return CSS_ERR_QUEUE_OVERFLOW; }
     c->err = "device status " + std::to_string(status);
     return CSS_ERR_CUDA;
@@ -613,7 +612,7 @@ int css_mesh_upload(css_ctx* c, const double* verts, int64_t nv, const int32_t* 
 
 int css_mesh_free(css_mesh* m) {
     if (!m) return CSS_ERR_INVALID_ARG;
-    cudaFree(m->he); cudaFree(m->twin); cudaFree(m->edge); cudaFree(m->fv); cudaFree(m->lay);
+    cudaFree(m->he); cudaFree(m->twin); cudaFree(m->fv); cudaFree(m->lay);
     cudaFree(m->frame); cudaFree(m->theta); cudaFree(m->pseudo); cudaFree(m->bnd);
     cudaFree(m->ring_start); cudaFree(m->ring); cudaFree(m->X); cudaFree(m->he32);
     cudaFree(m->frank);
@@ -770,7 +769,7 @@ int css_particles_free(css_parts* p) {
     if (!p) return CSS_ERR_INVALID_ARG;
     if (p->graph) cudaGraphExecDestroy(p->graph);
     cudaFree(p->state); cudaFree(p->snap);
-    cudaFree(p->fcnt); cudaFree(p->fstart); cudaFree(p->fitems); cudaFree(p->ftmp); cudaFree(p->scan_tmp); cudaFree(p->order);
+    cudaFree(p->fcnt); cudaFree(p->fstart); cudaFree(p->fitems); cudaFree(p->ftmp); cudaFree(p->scan_tmp);
     cudaFree(p->pcnt); cudaFree(p->pj); cudaFree(p->pd); cudaFree(p->pt); cudaFree(p->dstep); cudaFree(p->dfire);
     cudaFree(p->rows); cudaFree(p->stage);
     delete p;
@@ -1341,63 +1340,33 @@ int css_autotune(css_ctx* c, css_parts* const* sets, int32_t n_sets, const css_p
         }
         if (rc) break;
     }
-    // the register-light variant (twice the resident warps, some spills): with global tables
-    // (shared tables leave no room for 16 warps per SM) and with the best pick's tables
-    for (int variant = 0; variant < 3 && rc == CSS_OK; ++variant) {
-        cssi::LaunchCfg T = pick;
-        if (variant < 2) {
-            T.shared_scale = 0;
-            T.win_cap = POOL_UNIT * 4 * (variant == 1 ? 4 : 1);
-            if (variant == 1 && T.win_cap <= pick.win_cap && pick.shared_scale == 0) continue;
-        } else if (pick.shared_scale == 0) continue;
-        for (int wpc : {4, 8}) {
-            for (int tab : {0, TAB_UNIT}) {
-                if (tab && T.shared_scale) continue;
-                cssi::LaunchCfg L = T;
-                L.occupancy = 2;
-                L.warps_per_cta = wpc;
-                L.ctas_per_sm = 0;
-                L.tile = 1;
-                L.tab_cap = T.shared_scale ? 0 : tab;
-                if (!shape_fits(precision, L.win_cap, L.tab_cap, L.shared_scale, wpc, 0)) continue;
-                double t = 0.0;
-                rc = measure(L, &t);
-                if (rc) break;
-                if (t < pick_ms) { pick_ms = t; pick = c->cfg; }
-            }
-            if (rc) break;
-        }
-    }
     // the team form (all warps of a CTA on one source) where the sampled sources are too few to
     // fill the resident warps one warp each
     if (rc == CSS_OK && (int64_t)nitems < 4 * (int64_t)c->sm_count * 8) {
         for (int s : {1, 4, 0}) {
             for (int wpc : {2, 4, 8}) {
-                for (int occ : {1, 2}) {
-                    if (!shape_fits(precision, POOL_UNIT * (s ? s : 4), 0, s, wpc, 1)) continue;
-                    cssi::LaunchCfg L = base;
-                    L.team = 1;
-                    L.occupancy = occ;
-                    L.shared_scale = s;
-                    L.win_cap = POOL_UNIT * (s ? s : 4);
-                    L.tab_cap = 0;
-                    L.warps_per_cta = wpc;
-                    L.ctas_per_sm = 0;
-                    L.tile = 1;
-                    double t = 0.0;
+                if (!shape_fits(precision, POOL_UNIT * (s ? s : 4), 0, s, wpc, 1)) continue;
+                cssi::LaunchCfg L = base;
+                L.team = 1;
+                L.occupancy = 1;
+                L.shared_scale = s;
+                L.win_cap = POOL_UNIT * (s ? s : 4);
+                L.tab_cap = 0;
+                L.warps_per_cta = wpc;
+                L.ctas_per_sm = 0;
+                L.tile = 1;
+                double t = 0.0;
+                rc = measure(L, &t);
+                if (rc) break;
+                if (t < pick_ms) { pick_ms = t; pick = c->cfg; }
+                // a team's wider waves unfold more windows: sources deferred for want of
+                // pool run twice, so try pools four and sixteen times larger
+                for (int grow = 0; grow < 2 && c->last_counters[4] * 100 > nitems && L.win_cap * 4 <= (1 << 20);
+                     ++grow) {
+                    L.win_cap *= 4;
                     rc = measure(L, &t);
                     if (rc) break;
                     if (t < pick_ms) { pick_ms = t; pick = c->cfg; }
-                    // a team's wider waves unfold more windows: sources deferred for want of
-                    // pool run twice, so try pools four and sixteen times larger
-                    for (int grow = 0; grow < 2 && c->last_counters[4] * 100 > nitems && L.win_cap * 4 <= (1 << 20);
-                         ++grow) {
-                        L.win_cap *= 4;
-                        rc = measure(L, &t);
-                        if (rc) break;
-                        if (t < pick_ms) { pick_ms = t; pick = c->cfg; }
-                    }
-                    if (rc) break;
                 }
                 if (rc) break;
             }

@@ -43,12 +43,10 @@ struct DMesh {
     double unit, inv_unit;
     const HeRec* he;              // 3 nf
     const int32_t* twin;          // 3 nf
-    const int32_t* edge;          // 3 nf, undirected edge id = min(h, twin(h))
     const int32_t* fv;            // 3 nf, vertex at each corner
     const double* lay;            // 3 nf: L01, x2, y2 per face
     const double* frame;          // 9 nf: origin, e1, e2 per face (world)
     const double* theta;          // nv angle sums
-    const uint8_t* pseudo;        // nv: boundary, flat or saddle vertex
     const uint8_t* bnd;           // nv: boundary vertex
     const int32_t* ring_start;    // nv + 1
     const int32_t* ring;          // 3 nf corners h with fv[h] == v, grouped by vertex
@@ -61,52 +59,11 @@ struct DMesh {
                                   // boundary, non-manifold or of an angle sum above 2 pi carry EMITS
 };
 
-__device__ __forceinline__ double cross2(double ax, double ay, double bx, double by) { return ax * by - ay * bx; }
-
 __device__ __forceinline__ void face_corner(const DMesh& m, int f, int k, double& x, double& y) {
     k = (k >= 3) ? k - 3 : k;
     if (k == 0) { x = 0.0; y = 0.0; }
     else if (k == 1) { x = m.lay[3 * f]; y = 0.0; }
     else { x = m.lay[3 * f + 1]; y = m.lay[3 * f + 2]; }
-}
-
-// ------------------------------------------------------------------ generation-tagged hash
-// Entry = (gen << 32) | key.  An entry whose gen differs from the current one is
-// empty, so tables never need clearing between sources.  Reads bypass L1
-// (ld.global.cg) because claims are made with L2 atomics.
-__device__ __forceinline__ unsigned long long ld_cg_u64(const unsigned long long* p) { return __ldcg(p); }
-
-__device__ __forceinline__ int ht_insert(unsigned long long* keys, int logcap, uint32_t gen, int32_t key,
-                                         bool& claimed) {
-    const unsigned long long want = ((unsigned long long)gen << 32) | (uint32_t)key;
-    const uint32_t mask = (1u << logcap) - 1u;
-    uint32_t slot = ((uint32_t)key * 2654435761u) >> (32 - logcap);
-    claimed = false;
-    for (uint32_t probe = 0; probe <= mask; ++probe) {
-        unsigned long long cur = ld_cg_u64(keys + slot);
-        for (;;) {
-            if (cur == want) return (int)slot;
-            if ((uint32_t)(cur >> 32) == gen) break;          // occupied by another key
-            unsigned long long prev = atomicCAS(keys + slot, cur, want);
-            if (prev == cur) { claimed = true; return (int)slot; }
-            cur = prev;                                        // re-examine what won
-        }
-        slot = (slot + 1u) & mask;
-    }
-    return -1;
-}
-
-__device__ __forceinline__ int ht_find(const unsigned long long* keys, int logcap, uint32_t gen, int32_t key) {
-    const unsigned long long want = ((unsigned long long)gen << 32) | (uint32_t)key;
-    const uint32_t mask = (1u << logcap) - 1u;
-    uint32_t slot = ((uint32_t)key * 2654435761u) >> (32 - logcap);
-    for (uint32_t probe = 0; probe <= mask; ++probe) {
-        unsigned long long cur = ld_cg_u64(keys + slot);
-        if (cur == want) return (int)slot;
-        if ((uint32_t)(cur >> 32) != gen) return -1;
-        slot = (slot + 1u) & mask;
-    }
-    return -1;
 }
 
 __device__ __forceinline__ unsigned lanemask_lt() {
@@ -127,7 +84,6 @@ enum : int {
     ST_HASH_OVERFLOW = 2,    // a hash table full
     ST_PAIR_OVERFLOW = 4,    // per-source pair slab full
     ST_ITER_LIMIT = 8,       // loop cap reached
-    ST_PIECES = 16,          // too many interval pieces in one trim
     ST_WALK_LIMIT = 32,      // face walk iteration cap
     ST_BAD_INPUT = 64,
 };

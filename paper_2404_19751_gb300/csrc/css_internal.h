@@ -23,7 +23,7 @@ struct LaunchCfg {
     int win_cap = 2048;
     int win_cap2 = 16384;
     int warps2_per_sm = 2;   // second pass: warps per SM (one CTA each)
-    int occupancy = 1;       // register budget of the first pass: 1 (255 regs) or 2 (128 regs)
+    int occupancy = 1;       // kept for css_get_launch only
     int tab_cap = 0;         // first pass with global tables: table slots (0: tied to win_cap)
     int team = 0;            // 1: the warps of a CTA work on one source together (team form)
 };
@@ -87,7 +87,6 @@ struct css_mesh {
     // device arrays
     css::HeRec* he = nullptr;
     int32_t* twin = nullptr;
-    int32_t* edge = nullptr;
     int32_t* fv = nullptr;
     double* lay = nullptr;
     double* frame = nullptr;
@@ -130,7 +129,6 @@ struct css_parts {
     int32_t* fitems = nullptr;  // n
     int32_t* ftmp = nullptr;    // n, scratch of the bucket scatter
     int32_t* scan_tmp = nullptr;
-    int32_t* order = nullptr;   // source processing order (n)
     int64_t* dstep = nullptr;   // device copy of the step counter (Philox counter word)
     double* dfire = nullptr;    // FIRE state: 8 live doubles, then their snapshot
     int fire_valid = 0;         // the FIRE state belongs to fire_it and the current particles

@@ -73,7 +73,7 @@ __global__ void k_topo_insert(const int32_t* F, int64_t nf, TopoTab t, int* flag
     atomicOr(flag, 8);
 }
 
-__global__ void k_topo_link(const int32_t* F, TopoTab t, int32_t* twin, int32_t* edge, int* flag,
+__global__ void k_topo_link(const int32_t* F, TopoTab t, int32_t* twin, int* flag,
                             unsigned long long* n_edges) {
     int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (s >= (1ll << t.logcap)) return;
@@ -81,13 +81,11 @@ __global__ void k_topo_link(const int32_t* F, TopoTab t, int32_t* twin, int32_t*
     if (c == 0) return;
     atomicAdd(n_edges, 1ull);
     int32_t h0 = t.h0[s];
-    if (c == 1) { twin[h0] = -1; edge[h0] = h0; return; }
+    if (c == 1) { twin[h0] = -1; return; }
     if (c > 2) return;
     int32_t h1 = t.h1[s];
     if (F[h0] == F[h1]) atomicOr(flag, 16);   // both run a->b: inconsistent orientation
     twin[h0] = h1; twin[h1] = h0;
-    int32_t e = h0 < h1 ? h0 : h1;
-    edge[h0] = e; edge[h1] = e;
 }
 
 __device__ void min_image(double* d, int periodic, double px, double py) {
@@ -279,12 +277,10 @@ css::DMesh css_mesh::view() const {
     d.per[1] = per[1];
     d.he = he;
     d.twin = twin;
-    d.edge = edge;
     d.fv = fv;
     d.lay = lay;
     d.frame = frame;
     d.theta = theta;
-    d.pseudo = pseudo;
     d.bnd = bnd;
     d.ring_start = ring_start;
     d.ring = ring;
@@ -336,7 +332,6 @@ int build_mesh(css_ctx* ctx, const double* dX, int64_t nv, const int32_t* dF, in
     CK(cudaMalloc(&dcnt, 3 * sizeof(unsigned long long)));
     CK(cudaMalloc(&m->he, nh * sizeof(HeRec)));
     CK(cudaMalloc(&m->twin, nh * sizeof(int32_t)));
-    CK(cudaMalloc(&m->edge, nh * sizeof(int32_t)));
     CK(cudaMalloc(&m->fv, nh * sizeof(int32_t)));
     CK(cudaMalloc(&m->lay, 3 * nf * sizeof(double)));
     CK(cudaMalloc(&m->frame, 9 * nf * sizeof(double)));
@@ -367,7 +362,7 @@ int build_mesh(css_ctx* ctx, const double* dX, int64_t nv, const int32_t* dF, in
     if (hflag & 1) { ctx->err = "mesh_upload: vertex index out of range or non-finite coordinate"; rc = CSS_ERR_INVALID_ARG; goto done; }
     if (hflag & 2) { ctx->err = "mesh_upload: face with a repeated vertex"; rc = CSS_ERR_NONMANIFOLD; goto done; }
     k_topo_insert<<<nblk(nh), 256, 0, st>>>(dF, nf, t, dflag);
-    k_topo_link<<<nblk(cap), 256, 0, st>>>(dF, t, m->twin, m->edge, dflag, dcnt);
+    k_topo_link<<<nblk(cap), 256, 0, st>>>(dF, t, m->twin, dflag, dcnt);
     k_faces<<<nblk(nf), 256, 0, st>>>(dX, dF, nf, m->periodic, m->per[0], m->per[1], m->lay, m->frame, dflag);
     k_area<<<nblk(nf), 256, 0, st>>>(m->lay, nf, (double*)(dcnt + 2));
     CK(cudaGetLastError());

@@ -85,10 +85,6 @@ int na_status_error(css_ctx* c, int status) {
         c->err = "compute_forces_noalloc: a device loop reached its iteration cap";
         return CSS_ERR_ITER_LIMIT;
     }
-    if (status & css::ST_PIECES) {
-        c->err = "compute_forces_noalloc: window trimming produced too many pieces";
-        return CSS_ERR_QUEUE_OVERFLOW;
-    }
     c->err = "compute_forces_noalloc: device status " + std::to_string(status);
     return CSS_ERR_CUDA;
 }

@@ -235,7 +235,6 @@ __device__ __forceinline__ V2<R> narrow(double2 v) {
     if constexpr (sizeof(R) == 8) return v;
     else return make_float2(f32(v.x), f32(v.y));
 }
-__device__ __forceinline__ bool is_inf(double x) { return __double2hiint(x) == 0x7ff00000; }
 // square root to 2^-22
 __device__ __forceinline__ float root(float x) { return x > 0.0f ? x * rsqrtf(x) : 0.0f; }
 // x^(1/2) and x^(-1/2) in FP64 from the FP32 reciprocal root: Goldschmidt's iteration (it squares the

@@ -99,3 +99,17 @@ def test_kernel_time_holds_no_round_trip():
     mesh.free()
     ctx.close()
     assert np.median(late) < np.median(once) + 10.0, (np.median(late), np.median(once))
+
+
+def test_tuner_times_each_kernel_once():
+    """Occupancy 1 and 2 are the same kernel: the tuner does not let noise choose between them."""
+    m = synth.icosphere(4, 1.0, noise=0.01, seed=1)
+    ctx = css.create(0)
+    mesh = css.mesh_upload(ctx, m.verts, m.faces)
+    parts = css.particles_set(ctx, mesh, *synth.place_uniform(m, 300, 3))
+    pot = dict(kind=css.POT_HARMONIC, eps=1.0, sigma=0.2, r_cut=0.2, A=1.0)
+    for _ in range(3):
+        assert ctx.autotune([parts], pot, 0.2, css.FP64, reps=1)[0]["occupancy"] == 1
+    parts.free()
+    mesh.free()
+    ctx.close()
