@@ -158,18 +158,24 @@ struct Reach {
 };
 
 // The launch shape for a context whose shape nobody set or tuned.  Measured on one GB300, kernel
-// times in ms (sources; windows a source; taken before the kernel's loops were rolled up, which made the
-// noisy sphere's and the height field's 8 to 17 % shorter in every shape that fills the chip):
+// times in ms (sources; windows a source):
 //   - as many sources as fill 16 warps an SM, small patches: tables in shared memory at scale 1
 //     (noisy sphere, 16384; 473: 2.96, scale 2 with its 8 warps an SM 3.95, tables in global memory
 //     3.32).  Where the tables are too small for the patch, global memory (height field, 8192;
-//     3957: 10.2 with 16 warps an SM, shared at scale 8 with 2 warps 27.3)
+//     3957: 10.2 with 16 warps an SM, shared at scale 8 with 2 warps 27.3).  These two were taken before the
+//     kernel's loops were rolled up, which made every shape that fills the chip 8 to 17 % shorter.
 //   - fewer sources than 8 warps an SM: scale 2 (icosphere, 1024; 301: 0.107 against 0.138; torus, 999;
 //     407: 0.353 against 0.805, whose scale-1 tables deferred 132 sources)
-//   - few sources, large patches: a team of 8, 4 or 2 warps a source, as many as leave an SM 16
-//     warps or so (flat plane, 64; 5046: one warp 1.60, teams of 2, 4, 8 0.93, 0.65, 0.55; torus,
-//     100; 86000: 23.7 -> 10.0, 6.5, 5.9); on 300 windows a team loses (0.187 against 0.107).  Between
-//     them lies a patch of 350 faces: its waves are about 8 sqrt(6 x 350) windows wide in all.
+//   - few sources, large patches: a team of 8, 4 or 2 warps a source, as many as leave an SM 16 warps or so
+//     (flat plane, 64; 5046: one warp 1.60, teams of 2, 4, 8 0.93, 0.65, 0.55; torus, 100; 86000:
+//     23.7 -> 10.0, 6.5, 5.9).  Where the two cross on a smooth level-5 sphere, one warp | team:
+//       64 sources, teams of 8    100 faces .073 | .062   350 .263 | .111   1000 1.01 | .235
+//       400, teams of 8           200 .157 | .225   350 .298 | .301   500 .482 | .372   1000 1.06 | .691
+//       800, teams of 4           350 .322 | .350   500 .527 | .487   700 .971 | .702   1000 1.60 | 1.14
+//     at 350 faces or so, on a rough sphere too (400 sources: .702 | .759 at 350, 2.36 | .982 at 500).
+//     With teams of 2 (6 to 12 sources an SM) it depends on how uneven the patches are: 1300 sources with
+//     1200 faces each take 2.20 | 3.67 on the sphere and 8.29 | 5.75 on a torus, whose inner side has
+//     more faces in reach than its share of the area, and teams share out what is uneven.
 cssi::LaunchCfg pick_shape(const css_ctx* c, int64_t nitems, const Reach& R) {
     cssi::LaunchCfg L = c->cfg;
     const double grow = (double)(1 << R.level), verts = grow * R.verts, targets = grow * R.targets;
