@@ -281,7 +281,7 @@ int css_batch_free(css_batch* batch);
  * must stay fixed after start-up).  It computes the same forces and energy as
  * css_compute_forces, for particles given directly as device arrays, and calls no
  * cudaMalloc, cudaFree or allocating library routine: its scratch is one fixed device
- * array of about 59 MB that every GPU loading this library holds until exit.
+ * array of 63 MB that every GPU loading this library holds until exit.
  *   mesh     uploaded beforehand with css_mesh_upload (that call allocates); the call runs
  *            on the device of the mesh's context, whatever device is current, and puts
  *            the caller's current device back before it returns;
@@ -297,8 +297,8 @@ int css_batch_free(css_batch* batch);
  * another device.
  * Limits: n <= 262144 particles, at most 1048576 faces; beyond them it returns
  * CSS_ERR_CAPACITY.  A source whose patch overflows the array's tables (4096 windows waiting
- * at a time, 14336 vertices) gives CSS_ERR_QUEUE_OVERFLOW, and css_compute_forces should be
- * used instead; a device loop cap gives CSS_ERR_ITER_LIMIT.
+ * at a time, 14336 vertices, 5120 of them boundary or saddle vertices) gives
+ * CSS_ERR_QUEUE_OVERFLOW, and css_compute_forces should be used instead; a device loop cap gives CSS_ERR_ITER_LIMIT.
  * The first call on a device looks up the array's device address (set-up): make it
  * before any stream capture.  Every call shares the array, which keeps the previous
  * call's contents, so calls that overlap on the GPU (other streams, other host threads)
@@ -323,18 +323,19 @@ int css_fma_peak(css_ctx* ctx, int precision, double* flops_per_s);
  * Launch shape of the neighbour/force evaluation (no counterpart in the paper, whose
  * method runs one source per CPU process).  Every source runs in a first pass: one
  * warp per source, with its working memory -- a ring of windows waiting to be unfolded, a
- * table of vertices, a table of targets -- in shared memory.  A source that overflows it is
+ * table of vertices, a table of targets -- in shared memory, as far as it fits.  A source that overflows it is
  * deferred, and a second pass re-runs the deferred sources with larger working memory in
  * global memory on fewer warps.  Results do not depend on the shape.
  *   warps_per_cta      first pass, 1..8
  *   ctas_per_sm        first pass resident CTAs per SM, 0 = as many as fit, else a cap
  *   tile               work items (sources) a warp claims per atomic, 1..64
- *   shared_scale       first-pass working memory in shared memory: 1, 2, 4 or 8 times 256
- *                      vertices, 64 targets and a ring of at most 128 windows (1024 in the team
- *                      form; halved until the shape fits an SM); 0 = in global memory
- *   window_capacity    first-pass windows, 64..2^20 (rounded up to 2^k): the ring holds a sixteenth
- *                      of them (a quarter in the team form), at least 32
- *   window_capacity2   the same for the second pass (grown on overflow)
+ *   shared_scale       first-pass tables in shared memory: 1, 2, 4 or 8 times 256 vertices and 64
+ *                      targets (1024 and 256 in the team form, halved until the shape fits an SM);
+ *                      0 = in global memory.  The ring of waiting windows is in shared memory
+ *                      either way, up to 64 of them (128 a warp in the team form)
+ *   window_capacity    first-pass windows, 64..2^20 (rounded up to 2^k): half of them can wait at a
+ *                      time, those beyond the ring in global memory
+ *   window_capacity2   the same for the second pass, whose tables follow it (grown on overflow)
  *   warps2_per_sm      second-pass warps per SM, 1..8
  *   occupancy          1 or 2: accepted and kept; the kernel's register budget (at most 128 a
  *                      thread) suits both

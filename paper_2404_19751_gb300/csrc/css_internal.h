@@ -12,9 +12,9 @@
 
 namespace cssi {
 // Launch shape of the neighbour / force evaluation.  The first pass runs every source
-// with per-warp tables in shared memory (scaled by `shared_scale`, 0: global tables) and a
-// window pool of `win_cap`; sources whose patch overflows either are deferred to a
-// second pass with global tables and a pool of `win_cap2`, on fewer warps.
+// with tables in shared memory (scaled by `shared_scale`, 0: in global memory) and room for
+// `win_cap` / 2 waiting windows; sources whose patch overflows either are deferred to a
+// second pass with tables in global memory for `win_cap2` windows, on fewer warps.
 struct LaunchCfg {
     int warps_per_cta = 4;   // first pass
     int ctas_per_sm = 0;     // 0: as many as fit
@@ -24,7 +24,7 @@ struct LaunchCfg {
     int win_cap2 = 16384;
     int warps2_per_sm = 2;   // second pass: warps per SM (one CTA each)
     int occupancy = 1;       // kept for css_get_launch only
-    int tab_cap = 0;         // first pass with global tables: table slots (0: tied to win_cap)
+    int tab_cap = 0;         // first pass with tables in global memory: their size (0: tied to win_cap)
     int team = 0;            // 1: the warps of a CTA work on one source together (team form)
 };
 // one pass's workspace (global tables and rings), grown on demand

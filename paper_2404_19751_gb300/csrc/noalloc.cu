@@ -31,7 +31,7 @@ constexpr size_t NA_OFF_PCNT = NA_OFF_SCAN + NA_SCAN_INTS * 4;
 constexpr size_t NA_OFF_DEFER = NA_OFF_PCNT + NA_MAX_PARTICLES * 4;   // two lists of sources left to a later pass
 constexpr size_t NA_OFF_SCAL = (NA_OFF_DEFER + 2 * NA_MAX_PARTICLES * 4 + 255) & ~(size_t)255;  // work, status
 constexpr size_t NA_OFF_COUNT = NA_OFF_SCAL + 256;                                              // 8 counters
-constexpr size_t NA_BYTES = NA_OFF_COUNT + 8 * 8;   // ~61 MB in all
+constexpr size_t NA_BYTES = NA_OFF_COUNT + 8 * 8;   // 62.9 MB in all
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NA_BYTES];
 

@@ -436,11 +436,12 @@ __global__ void k_cg_dir(Op o, int K, const int* active, const double* beta, con
 // an edge (one per face at it) are one entry, half the FP64 operations of the general form.
 // Bound by the FP64 pipe (two FMA a clock and SM): 4 FMA an entry for the transported
 // vector, 1 for the scalar.  Whole calls on one GB300, all pairs, general form -> this one:
-// 3916 vertices with 100 sources 59.4 -> 11.3 ms (heat 5.4, conjugate gradients 5.1; their
-// FP64 operations alone take 3.3 and 3.8 on the 100 SMs in use), with 20 sources 27.0 -> 5.8,
-// with 256 91.0 -> 19.9; 800 vertices with 100 sources 12.7 -> 2.3; 12800 vertices with 3
-// sources 35.4 -> 11.0.  CTAs of 1024 threads take 10.8 ms in the first case and 22.6 with 256
-// sources, where two CTAs of 512 share an SM.
+// 3996 vertices with 100 sources 59.3 -> 10.8 ms (heat 4.8, conjugate gradients 4.9; their
+// FP64 operations alone take 3.1 and 3.7 on the 100 SMs in use), with 20 sources 27.0 -> 5.7,
+// with 256 91.0 -> 19.9; 800 vertices with 100 sources 12.7 -> 2.1; 12740 vertices with 3
+// sources 35.4 -> 11.3.  CTAs of 1024 threads (measured with one relaxation factor for all rows) took
+// 10.8 ms where CTAs of 512 took 11.3, and 22.6 against 19.9 with 256 sources, where two CTAs of
+// 512 share an SM.
 struct Rows {
     int32_t np = 0;          // rows, a multiple of 32
     int32_t ncol = 0;

@@ -19,7 +19,7 @@
 // shared memory, the only other state is the table of vertex distances, and a wave is 32
 // windows whatever their keys (measured on the workloads: taking the smallest keys first
 // unfolds no fewer windows than the order of creation).  The particles of a face are tested
-// against each window that enters it; the tests are queued and evaluated 32 at a time.
+// against each window that enters it; the tests are queued and evaluated when ten are there.
 //
 // A window's cone is two directions in the frame of its pseudo-source, where they stay what
 // they are through every unfolding (the direction to the vertex that bounds the cone), so no
@@ -34,8 +34,8 @@
 //
 // Measured against windows kept in per-edge lists and trimmed against one another (the same
 // calls, default launch shapes): 65536 particles on a noisy level-8 sphere 110.7 -> 10.1 ms
-// (FP64) and 73.1 -> 11.0 ms (FP32), 8192 on a 256 x 256 height field 130-166 -> 8.7 ms, every pair
-// of 64 on a flat plane 27 -> 0.67 ms.  The windows unfolded per source are the same within 10 %
+// (FP64) and 73.1 -> 10.3 ms (FP32), 8192 on a 256 x 256 height field 130-166 -> 8.3 ms, every pair
+// of 64 on a flat plane 27 -> 0.66 ms.  The windows unfolded per source are the same within 10 %
 // (482 against 440, 3991 against 3950, 5135 against 5151).
 #include <cuda_runtime.h>
 #include <limits.h>
@@ -59,8 +59,8 @@ using cssi::WaveWs;
 // Where sources fill the chip, instruction fetch sets the pace: a wave is about 2000 instructions of
 // mostly straight code, 16 warps sit at different places of it, and 43 % of stall cycles waited for
 // instructions.  So loops are not unrolled, rare branches are marked and divisions in FP32 are the
-// short ones (16384 sources on a noisy sphere: 2.96 -> 2.45 ms in FP64, 3.10 -> 2.63 in FP32; 8192 on
-// a height field 3.55 -> 3.23; small sets and teams unchanged within 2 %).
+// short ones (16384 sources on a noisy sphere: 2.96 -> 2.45 ms in FP64; 2048 on a 128 x 128 height field
+// 3.55 -> 3.23; small sets and teams unchanged within 2 %).
 constexpr int MAXW = 8;          // warps per CTA
 constexpr int EV = 10;           // queued target tests per warp
 constexpr int NONE = -1;
