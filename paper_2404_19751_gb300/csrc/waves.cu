@@ -101,13 +101,15 @@ struct Index<0> {
     static __device__ __forceinline__ int2 make(int a, int b) { return make_int2(a, b); }
 };
 
+// a corner within this of a rim does not split the cone (relative to its distance)
+constexpr double RIM_MIN = 1e-12;
 // tolerance of a point on the rim of a cone, relative to its distance (FP32: the roundings of the
 // target's point, the rotation and the rim add up to 6.5e-7 at most)
 template <class R>
 struct Rim;
 template <>
 struct Rim<double> {
-    static constexpr double t = 1e-12;
+    static constexpr double t = 4e-12;
 };
 template <>
 struct Rim<float> {
@@ -881,7 +883,7 @@ __device__ __forceinline__ void Group<R, PL, TEAM, LK>::wave(int head, int n) {
         if (TEAM ? near : __builtin_expect(near, 0)) {   // too close to a rim for FP32
             const double gx = r.cx - S.x, gy = r.cy - S.y;
             const double ex = gx * rot.x + gy * rot.y, ey = gy * rot.x - gx * rot.y;
-            const double tg = Rim<double>::t * (fabs(gx) + fabs(gy));
+            const double tg = RIM_MIN * (fabs(gx) + fabs(gy));
             const double e0 = tg * (fabs(d0.x) + fabs(d0.y)), e1 = tg * (fabs(d1.x) + fabs(d1.y));
             const double c0 = d0.x * ey - d0.y * ex, c1 = d1.x * ey - d1.y * ex;
             in0 = c0 <= e0;
@@ -944,12 +946,14 @@ __device__ __forceinline__ void Group<R, PL, TEAM, LK>::wave(int head, int n) {
     // The children, side 0 across the edge u -> c, side 1 across c -> v: one lane each, packed densely
     // (a window has one child on average, at most two).  A child's lane reads its parent's
     // window from the ring again; the parent's slots are free once the last round has read them.
-    // (the corner bounds a child's cone unless it lies beyond the rim on the child's side)
+    // (the corner bounds a child's cone only where it splits it: a rim that moved to every corner within
+    // its tolerance would leave a gap of several tolerances after a chain of them, and the sliver between
+    // has no windows of its own behind flat vertices)
     const unsigned lm = __ballot_sync(CSS_FULL, left), rm = __ballot_sync(CSS_FULL, right);
     const int nleft = __popc(lm), total = nleft + __popc(rm);
     unsigned char* task = e + Y.e_task;
-    if (left) task[__popc(lm & css::lanemask_lt())] = (unsigned char)(lane | (in1 ? 64 : 0));
-    if (right) task[nleft + __popc(rm & css::lanemask_lt())] = (unsigned char)(lane | 32 | (in0 ? 64 : 0));
+    if (left) task[__popc(lm & css::lanemask_lt())] = (unsigned char)(lane | (beyond1 ? 64 : 0));
+    if (right) task[nleft + __popc(rm & css::lanemask_lt())] = (unsigned char)(lane | 32 | (beyond0 ? 64 : 0));
     __syncwarp();
 #pragma unroll 1
     for (int base = 0; base < total; base += 32) {
