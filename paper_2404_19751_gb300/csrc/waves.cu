@@ -568,10 +568,12 @@ __device__ __forceinline__ void Group<R, PL, TEAM, LK>::seed(int f0, double b1, 
     // the source from the corner's own weights (no cancellation next to a corner): (hx, hy) in the
     // frame of half-edge h, lx from its end; (ex, ey) the frame's x axis in the face's layout
     const int k0 = hh - 3 * f0;
-    const double wt[3] = {1.0 - b1 - b2, b1, b2};
+    // (weights below zero by rounding are zero for all three lanes: a source that lies on an edge for one
+    // and beside it for the others would see its corners in different directions)
+    const double wt[3] = {fmax(1.0 - b1 - b2, 0.0), fmax(b1, 0.0), fmax(b2, 0.0)};
     const double wa = k0 == 0 ? wt[0] : (k0 == 1 ? wt[1] : wt[2]), wb = k0 == 0 ? wt[1] : (k0 == 1 ? wt[2] : wt[0]);
     const double wc = k0 == 0 ? wt[2] : (k0 == 1 ? wt[0] : wt[1]);
-    const double hx = wb * r.L + wc * r.cx, lx = wa * r.L + wc * (r.L - r.cx), hy = fmax(wc * r.cy, 0.0);
+    const double hx = wb * r.L + wc * r.cx, lx = wa * r.L + wc * (r.L - r.cx), hy = wc * r.cy;
     double ax, ay, bx, by;
     unit_corner(m, f0, k0, ax, ay);
     unit_corner(m, f0, k0 + 1, bx, by);

@@ -34,7 +34,7 @@ def _near_vertices(m, edges, rng):
 
 @pytest.mark.parametrize("prec", ["fp64", "fp32"])
 @pytest.mark.parametrize("moved", [0.0, 0.1])
-@pytest.mark.parametrize("edges", [False])
+@pytest.mark.parametrize("edges", [False, True])
 def test_every_pair_next_to_vertices(edges, moved, prec):
     ctx = css.create(0)
     for seed in range(8):
