@@ -332,7 +332,8 @@ int css_fma_peak(css_ctx* ctx, int precision, double* flops_per_s);
  *   shared_scale       first-pass tables in shared memory: 1, 2, 4 or 8 times 256 vertices and 64
  *                      targets (1024 and 256 in the team form, halved until the shape fits an SM);
  *                      0 = in global memory.  The ring of waiting windows is in shared memory
- *                      either way, up to 64 of them (128 a warp in the team form)
+ *                      either way, up to 64 of them (128 a warp in the team form, 64 for FP32
+ *                      beside tables in shared memory)
  *   window_capacity    first-pass windows, 64..2^20 (rounded up to 2^k): half of them can wait at a
  *                      time, those beyond the ring in global memory
  *   window_capacity2   the same for the second pass, whose tables follow it (grown on overflow)

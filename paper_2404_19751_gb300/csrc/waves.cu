@@ -1403,18 +1403,21 @@ size_t dyn_bytes(const WaveLay& y, int warps, bool shared, bool team) {
 }  // namespace
 
 // Capacities of one source's working memory.  The ring holds 64 waiting windows in shared memory
-// (a team's 128 a warp), the rest of half the windows waits in a spill area in global memory.
+// (a team's 128 a warp, 64 in the FP32 form beside tables in shared memory), the rest of half the
+// windows waits in a spill area in global memory.
 // Tables in shared memory: 256 vertices (a team's 1024) and 64 targets (256) times the scale; in
 // global memory they follow the table capacity (0: the windows).  A team's tables and ring are
 // halved until the shape fits an SM.
 // 64 slots: a small patch has 60-100 windows waiting (CPU counts: 71 icosphere, 101 noisy sphere at
 // most), a wave takes 32 and makes as many; 14 KB a warp in all then leave room for 16 warps.
+// FP32 teams of 8 with 64 slots a warp go two to an SM (200 sources with 400 faces each on a smooth sphere
+// 0.130 ms, 0.226 with 128 slots; 300 with 1000 0.322, 0.466; 100 with 1000 0.261, 0.234).
 WaveLay wave_layout(int precision, int win_cap, int tab_cap, int shared_scale, int warps, int team) {
     const bool f32 = precision == CSS_FP32;
     const int tab = tab_cap > 0 ? tab_cap : win_cap;
     int wait = win_cap / 2;
     if (!shared_scale) wait = std::min(wait, std::max(32, tab / 4));
-    int rl = std::min(log2_up(wait), team ? log2_up(128 * warps) : 6);
+    int rl = std::min(log2_up(wait), team ? log2_up((f32 && shared_scale ? 64 : 128) * warps) : 6);
     int vl = shared_scale ? log2_up((team ? 1024 : 256) * shared_scale) : log2_up(std::max(64, tab / 2));
     int tl = shared_scale ? log2_up((team ? 256 : 64) * shared_scale) : log2_up(std::max(64, tab / 4));
     WaveLay y;
